@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "nolsm_internal.cuh"
+#include "oz_path.cuh"
 #include "prep.cuh"
 #include "tc_path.cuh"
 
@@ -245,7 +246,6 @@ __device__ double block_sum(double v, double* red) {
 
 // ------------------------------------------------------------------------------------ a4-a7 (FP64)
 struct NsArgs {
-  int32_t j0, j1;
   const int32_t* sub_n; const int32_t* nbf;
   const int64_t* a_off; const int64_t* c_off;
   const double* A; const double* Q; const double* Sc; const double* Hc; const double* lam;
@@ -254,7 +254,7 @@ struct NsArgs {
   double mu, tol;
   int32_t max_iter;
   const int32_t* budget;       // per-submatrix step cap (nullable)
-  const int32_t* list;         // work list (nullable: [j0, j1))
+  const int32_t* list;         // work list; only submatrices whose status is kSubRefine are taken
   int32_t count;
   double* ws; int64_t slot_elems;
   int32_t* next;               // work counter
@@ -271,9 +271,13 @@ __global__ void __launch_bounds__(256) k_ns_fp64(NsArgs g) {
   double* T = X + g.slot_elems;
   double* Xn = T + g.slot_elems;
   for (;;) {
-    if (threadIdx.x == 0) {
-      const int k = atomicAdd(g.next, 1);
-      job = g.list ? (k < g.count ? g.list[k] : -1) : (g.j0 + k < g.j1 ? g.j0 + k : -1);
+    if (threadIdx.x == 0) {   // the next submatrix that the tensor-core kernel left
+      int J;
+      do {
+        const int k = atomicAdd(g.next, 1);
+        J = k < g.count ? g.list[k] : -1;
+      } while (J >= 0 && g.status[J] != kSubRefine);
+      job = J;
     }
     __syncthreads();
     const int J = job;
@@ -663,33 +667,64 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   int dev = 0, sms = 0;
   NOLSM_CUDA_TRY(cudaGetDevice(&dev));
   NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int slots = (int)std::min<int64_t>(2 * sms, spec.list ? spec.count : j1 - j0);
-  if (slots <= 0) return NOLSM_OK;
+  const int32_t work = spec.list ? spec.count : (int32_t)(j1 - j0);
+  if (work <= 0) return NOLSM_OK;
+  const int slots = (int)std::min<int64_t>(2 * sms, work);
   int32_t maxn = 0;
   for (int64_t J = j0; J < j1; ++J) maxn = std::max(maxn, plan->h_sub_n[J]);
   const int64_t slot_elems = (int64_t)maxn * maxn;
   NOLSM_TRY(ensure(plan, plan->ws_ns, sizeof(double) * 3 * (size_t)slot_elems * slots));
+  if (!spec.list && (plan->oz_j0 != j0 || plan->oz_j1 != j1)) {   // the range, largest first
+    std::vector<int32_t> ord((size_t)work);
+    for (int32_t k = 0; k < work; ++k) ord[(size_t)k] = (int32_t)j0 + k;
+    std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
+    plan->oz_j0 = -1;
+    NOLSM_TRY(ensure(plan, plan->oz_order, sizeof(int32_t) * (size_t)plan->n_mol));
+    NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->oz_order.p, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, st));
+    NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is a host temporary
+    plan->oz_j0 = j0;
+    plan->oz_j1 = j1;
+  }
+  // the iteration on the tensor cores (oz_path.cu); the plain kernel after it takes what is left
+  OzSolve z;
+  z.order = spec.list ? spec.list : plan->oz_order.as<int32_t>();
+  z.count = work;
+  z.max_n = maxn;
+  z.R = (maxn + 127) & ~127;
+  z.LD = (maxn + 63) & ~63;
+  z.clusters = std::min(work, oz_clusters(maxn, dev, sms));
+  const size_t plane = (size_t)z.R * z.LD;
+  NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * plane * oz_planes() * z.clusters));
+  NOLSM_TRY(ensure(plan, plan->oz_xd, sizeof(double) * plane * z.clusters));
+  z.planes = plan->oz_planes.as<uint16_t>();
+  z.xd = plan->oz_xd.as<double>();
+  z.sub_n = plan->sub_n.as<int32_t>(); z.nbf = plan->sub_b.as<int32_t>();
+  z.a_off = plan->a_off.as<int64_t>(); z.c_off = plan->c_off.as<int64_t>();
+  z.A = plan->prep64.A.as<double>(); z.Q = plan->Q.as<double>(); z.Sc = plan->Sc.as<double>();
+  z.Hc = plan->Hc.as<double>(); z.lam = spec.lam ? spec.lam : plan->lam.as<double>();
+  z.lam_g = plan->lam.as<double>();
+  z.prep_status = plan->prep_status.as<int32_t>();
+  z.mu = mu; z.tol = o.tol_ns; z.max_iter = o.max_iter; z.budget = spec.budget;
+  z.Dc = plan->Dc.as<double>(); z.tS = plan->t_S.as<double>(); z.tH = plan->t_H.as<double>();
+  z.iters = plan->iters.as<int32_t>(); z.status = plan->status.as<int32_t>();
+  z.rsteps = plan->rsteps.as<int32_t>(); z.nbelow = plan->nbelow.as<int32_t>();
+  NOLSM_TRY(launch_ns_oz(z, st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
   NsArgs g;
-  g.j0 = (int32_t)j0; g.j1 = (int32_t)j1;
-  g.sub_n = plan->sub_n.as<int32_t>(); g.nbf = plan->sub_b.as<int32_t>();
-  g.a_off = plan->a_off.as<int64_t>(); g.c_off = plan->c_off.as<int64_t>();
-  g.A = plan->prep64.A.as<double>(); g.Q = plan->Q.as<double>(); g.Sc = plan->Sc.as<double>();
-  g.Hc = plan->Hc.as<double>(); g.lam = spec.lam ? spec.lam : plan->lam.as<double>();
-  g.lam_g = plan->lam.as<double>();
-  g.prep_status = plan->prep_status.as<int32_t>();
+  g.sub_n = z.sub_n; g.nbf = z.nbf;
+  g.a_off = z.a_off; g.c_off = z.c_off;
+  g.A = z.A; g.Q = z.Q; g.Sc = z.Sc; g.Hc = z.Hc; g.lam = z.lam; g.lam_g = z.lam_g;
+  g.prep_status = z.prep_status;
   g.mu = mu; g.tol = o.tol_ns;
   g.max_iter = o.max_iter;
-  g.budget = spec.budget; g.list = spec.list; g.count = spec.count;
+  g.budget = z.budget; g.list = z.order; g.count = work;
   g.ws = plan->ws_ns.as<double>(); g.slot_elems = slot_elems;
   g.next = plan->counter.as<int32_t>();
-  g.Dc = plan->Dc.as<double>(); g.tS = plan->t_S.as<double>(); g.tH = plan->t_H.as<double>();
-  g.iters = plan->iters.as<int32_t>(); g.status = plan->status.as<int32_t>();
-  g.rsteps = plan->rsteps.as<int32_t>();
-  g.nbelow = plan->nbelow.as<int32_t>();
+  g.Dc = z.Dc; g.tS = z.tS; g.tH = z.tH; g.iters = z.iters; g.status = z.status;
+  g.rsteps = z.rsteps; g.nbelow = z.nbelow;
   k_ns_fp64<<<slots, 256, 0, st>>>(g);
   NOLSM_LAUNCH_CHECK();
-  plan->stats.launches += 1;
+  plan->stats.launches += 3;
   return NOLSM_OK;
 }
 

@@ -149,6 +149,9 @@ struct nolsm_plan {
   nolsm::DevBuf prep_order;         // submatrices of one chunk, largest first (mixed preparation)
   nolsm::DevBuf ws_ysym;            // L^-1 T_J(H0) of one preparation chunk (symmetric form)
   nolsm::DevBuf ws_ns;              // per-CTA Newton-Schulz buffers (FP64 path)
+  nolsm::DevBuf oz_planes, oz_xd;   // FP64 path on the tensor cores: digit planes, final X (per cluster)
+  nolsm::DevBuf oz_order;           // submatrices [oz_j0, oz_j1), largest first
+  int64_t oz_j0 = -1, oz_j1 = -1;
   void* tc = nullptr;               // tensor-core path state (tc_path.cu)
 
   // tracing: accumulated stats and the events that time one ABI call's phases
