@@ -542,23 +542,20 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
     pa.Q = plan->Q.as<double>(); pa.lam = plan->lam.as<double>(); pa.prep_status = plan->prep_status.as<int32_t>();
     int chunk_max_n = 1;
     for (int64_t k = J; k < e; ++k) chunk_max_n = std::max(chunk_max_n, plan->h_sub_n[k]);
-    if (keep_fp64_A) {
-      NOLSM_TRY(launch_prepare(pa, (int)(e - J), chunk_max_n, true, P.A.p, st));
-      plan->stats.launches += 2;
-    } else if (cls == kPrepNS) {
-      // the coupled Newton-Schulz inverse square root on the tensor cores (A_J and X = T_J(S)^-1 in FP32),
-      // then the refinement of the centre columns of T_J(S)^-1 with X, then the FP64 preparation of what
-      // either of them flagged
-      const int64_t nbc = plan->h_c_off[e] - plan->h_c_off[J];
-      NOLSM_TRY(ensure(plan, plan->ws_refine, (sizeof(double) + sizeof(float)) * (size_t)std::max<int64_t>(nbc, 1)));
-      NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)n2));
-      std::vector<int32_t> ord((size_t)(e - J));
+    // the chunk's submatrices, largest first
+    std::vector<int32_t> ord;
+    auto sort_chunk = [&]() -> nolsm_status {
+      ord.resize((size_t)(e - J));
       for (int64_t k = J; k < e; ++k) ord[(size_t)(k - J)] = (int32_t)k;
       std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
       NOLSM_TRY(ensure(plan, plan->prep_order, sizeof(int32_t) * ord.size()));
-      NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->prep_order.p, ord.data(), sizeof(int32_t) * ord.size(),
-                                     cudaMemcpyHostToDevice, st));
-      NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is a host temporary
+      NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->prep_order.p, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, st));
+      NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is host memory
+      return NOLSM_OK;
+    };
+    // T_J(S)^-1 (and A_J unless Aout is null) in FP32 by the inverse square root on the tensor cores
+    auto tensor_inverse = [&](float* Aout) -> nolsm_status {
+      NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)n2));
       NsInvArgs ia;
       ia.order = plan->prep_order.as<int32_t>();
       ia.count = (int32_t)(e - J);
@@ -568,7 +565,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       ia.ws = g.ws;
       ia.a_base = g.a_base;
       ia.chunk_n2 = n2;
-      ia.Aout = P.A.as<float>();
+      ia.Aout = Aout;
       ia.Xout = plan->ws_l32.as<float>();
       ia.prep_out = plan->prep_status.as<int32_t>();
       ia.tol_inv = kNsInvTol;
@@ -576,7 +573,49 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       tmark(plan, st);
       NOLSM_TRY(launch_ns_inverse(plan, ia, st));
       tmark(plan, st);
-      pa.order = ia.order;
+      return NOLSM_OK;
+    };
+    if (keep_fp64_A) {
+      // the FP32 inverse refined with exact digit products on the tensor cores (oz_path.cu); the FP64 Cholesky
+      // factorisation of what that left, in particular overlaps that are not positive definite
+      if (chunk_max_n <= prepare_fp64_max_n()) {
+        NOLSM_TRY(sort_chunk());
+        NOLSM_TRY(tensor_inverse(nullptr));
+        int dev = 0, sms = 0;
+        NOLSM_CUDA_TRY(cudaGetDevice(&dev));
+        NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        OzSolve z{};
+        z.order = plan->prep_order.as<int32_t>();
+        z.count = (int32_t)(e - J);
+        z.max_n = chunk_max_n;
+        z.R = (chunk_max_n + 127) & ~127;
+        z.LD = (chunk_max_n + 63) & ~63;
+        z.clusters = std::min(z.count, oz_clusters(chunk_max_n, dev, sms));
+        NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * (size_t)z.R * z.LD * oz_planes(1) * z.clusters));
+        z.planes = plan->oz_planes.as<uint16_t>();
+        z.sub_n = pa.sub_n; z.nbf = pa.nbf; z.sub_c0 = pa.sub_c0;
+        z.a_off = pa.a_off; z.c_off = pa.c_off;
+        z.prep_status = z.prep_out = pa.prep_status;
+        z.ws = g.ws; z.a_base = g.a_base; z.chunk_n2 = n2;
+        z.X32 = plan->ws_l32.as<float>();
+        z.Aout = P.A.as<double>();
+        z.Qout = pa.Q;
+        NOLSM_TRY(launch_inverse_oz(z, st));
+        pa.only_flagged = 1;
+        plan->stats.launches += 4;
+      }
+      NOLSM_TRY(launch_prepare(pa, (int)(e - J), chunk_max_n, true, P.A.p, st));
+      NOLSM_TRY(launch_gershgorin(pa, (int)(e - J), P.A.as<double>(), st));
+      plan->stats.launches += 3;
+    } else if (cls == kPrepNS) {
+      // the coupled Newton-Schulz inverse square root on the tensor cores (A_J and X = T_J(S)^-1 in FP32),
+      // then the refinement of the centre columns of T_J(S)^-1 with X, then the FP64 preparation of what
+      // either of them flagged
+      const int64_t nbc = plan->h_c_off[e] - plan->h_c_off[J];
+      NOLSM_TRY(ensure(plan, plan->ws_refine, (sizeof(double) + sizeof(float)) * (size_t)std::max<int64_t>(nbc, 1)));
+      NOLSM_TRY(sort_chunk());
+      NOLSM_TRY(tensor_inverse(P.A.as<float>()));
+      pa.order = plan->prep_order.as<int32_t>();
       pa.L32 = plan->ws_l32.as<float>();
       pa.c_base = plan->h_c_off[J];
       pa.Qp = plan->ws_refine.as<float2>();
@@ -602,17 +641,8 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       pa.Qp = plan->ws_refine.as<float2>();
       pa.W32 = reinterpret_cast<float*>(pa.Qp + std::max<int64_t>(nbc, 1));
       pa.fallback_max_n = sym ? 0 : prepare_fp64_max_n();   // no FP64 fallback for the symmetric form
-      {   // CTAs take the chunk's submatrices largest first, so that the last wave is made of small ones
-        std::vector<int32_t> ord((size_t)(e - J));
-        for (int64_t k = J; k < e; ++k) ord[(size_t)(k - J)] = (int32_t)k;
-        std::stable_sort(ord.begin(), ord.end(),
-                         [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
-        NOLSM_TRY(ensure(plan, plan->prep_order, sizeof(int32_t) * ord.size()));
-        NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->prep_order.p, ord.data(), sizeof(int32_t) * ord.size(),
-                                       cudaMemcpyHostToDevice, st));
-        NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is a host temporary
-        pa.order = plan->prep_order.as<int32_t>();
-      }
+      NOLSM_TRY(sort_chunk());   // CTAs take the largest first, so that the last wave is made of small ones
+      pa.order = plan->prep_order.as<int32_t>();
       NOLSM_TRY(launch_prepare_mixed(pa, (int)(e - J), chunk_max_n, P.A.as<float>(), st));
       plan->stats.launches += 3;
     }
@@ -686,7 +716,7 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
     plan->oz_j1 = j1;
   }
   // the iteration on the tensor cores (oz_path.cu); the plain kernel after it takes what is left
-  OzSolve z;
+  OzSolve z{};
   z.order = spec.list ? spec.list : plan->oz_order.as<int32_t>();
   z.count = work;
   z.max_n = maxn;
@@ -694,7 +724,7 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   z.LD = (maxn + 63) & ~63;
   z.clusters = std::min(work, oz_clusters(maxn, dev, sms));
   const size_t plane = (size_t)z.R * z.LD;
-  NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * plane * oz_planes() * z.clusters));
+  NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * plane * oz_planes(0) * z.clusters));
   NOLSM_TRY(ensure(plan, plan->oz_xd, sizeof(double) * plane * z.clusters));
   z.planes = plan->oz_planes.as<uint16_t>();
   z.xd = plan->oz_xd.as<double>();

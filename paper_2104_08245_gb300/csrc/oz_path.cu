@@ -19,8 +19,12 @@
 // memory after every product, which also carries the parts of the defect and the overflow flags; every role then
 // takes the same decision by itself. All waits are bounded.
 //
-// What the fixed point does not hold is left to the plain FP64 kernel (k_ns_fp64), which runs afterwards on the
-// submatrices still marked kSubRefine: non-finite input, entries that outgrow every exponent tried, an
+// The second mode prepares A_J = T_J(S)^-1 T_J(H0) and the centre columns of T_J(S)^-1 for the same path, from the FP32
+// inverse X of the inverse-square-root kernel (good to about 1e-6): R = I - T_J(S) X, V = I + R (I + R), X <- X V, whose
+// error is about R^3 (again from R when ||R||_F was above kOzLast), then A_J = X T_J(H0).
+//
+// What the fixed point does not hold is left to the FP64 kernels (k_ns_fp64; in the second mode k_prepare), which run
+// afterwards on the submatrices still marked kSubRefine: non-finite input, entries that outgrow every exponent tried, an
 // accumulator at 2^24, or a wait that ran out.
 #include <cuda_fp16.h>
 
@@ -44,6 +48,12 @@ constexpr int kRegsLaunch = 168, kRegsLow = 56, kRegsEpi = 224;
 static_assert(128 * kRegsLow + kOzEpi * kRegsEpi <= kOzThreads * kRegsLaunch, "register split above the launch");
 constexpr uint64_t kOzWaitNs = 2000000000ull;
 constexpr int kExTries = 4;                  // exponents tried per submatrix, each 3 above the last
+// Inverse mode: after an update from ||R||_F at most kOzLast the inverse is done (its cube, spread over n^2 entries, is
+// below 1e-16); ||R||_F at or above kOzFar, or no end after kOzRounds updates: the FP64 Cholesky takes the submatrix
+constexpr float kOzLast = 1.5e-5f, kOzFar = 0.5f;
+constexpr int kOzRounds = 4;
+// operands in scratch: X, X', T; in inverse mode X, X', two that hold S (then V), R, H in turn, and I + R
+constexpr int sets(int mode) { return mode == 0 ? 3 : 5; }
 
 template <int kB_, int kD_>
 struct Digits {
@@ -75,6 +85,13 @@ struct OzArgs {
   int32_t R, LD;
   double* Dc; double* tS; double* tH; int32_t* iters; int32_t* status; int32_t* rsteps; int32_t* nbelow;
   uint64_t wait_ns;
+  // inverse mode: the chunk's T_J(S), T_J(H0) (FP64, at a_off[J] - a_base and chunk_n2 further), X (FP32, at
+  // a_off[J] - a_base), and the outputs
+  const double* ws; int64_t a_base, chunk_n2;
+  const float* X32;
+  const int32_t* sub_c0;
+  double* Aout; double* Qout;
+  int32_t* prep_out;
 };
 
 // What the two CTAs tell each other at the end of a product (double buffered by its parity)
@@ -157,40 +174,69 @@ __device__ __forceinline__ void st_global_256(void* p, const uint32_t (&v)[8]) {
                : "memory");
 }
 
-// The balanced digits of two entries as packed FP16 pairs, out[p] for digit p. bias makes every digit but the
-// first non-negative; 1024 + u is the FP16 number with bits 0x6400 + u (u <= 1024).
+// The balanced digits of two entries as packed FP16 pairs, out[p] for digit p. The bias makes every digit non-negative
+// (u <= 2^kB below 1024), and 1024 + u is the FP16 number with bits 0x6400 | u.
 template <class Dg>
 __device__ __forceinline__ void digits2(long long a, long long b, uint32_t (&out)[Dg::kD]) {
   constexpr int kB = Dg::kB, kD = Dg::kD;
   constexpr uint32_t half = 1u << (kB - 1), mask = (1u << kB) - 1;
   long long bias = 0;
 #pragma unroll
-  for (int p = 1; p < kD; ++p) bias += (long long)half << (kB * (kD - 1 - p));
-  a = (a << (Dg::F - Dg::U)) + bias;
-  b = (b << (Dg::F - Dg::U)) + bias;
-  const uint32_t off = 0x64006400u;
+  for (int p = 0; p < kD; ++p) bias += (long long)half << (kB * (kD - 1 - p));
+  const unsigned long long x = (unsigned long long)(a << (Dg::F - Dg::U)) + (unsigned long long)bias;
+  const unsigned long long y = (unsigned long long)(b << (Dg::F - Dg::U)) + (unsigned long long)bias;
   const __half2 sub = __half2half2(__ushort_as_half((unsigned short)(0x6400u + half)));
 #pragma unroll
   for (int p = 0; p < kD; ++p) {
     const int sh = kB * (kD - 1 - p);
-    uint32_t u = (uint32_t)(a >> sh), w = (uint32_t)(b >> sh);
-    if (p == 0) {
-      u += half;
-      w += half;
-    } else {
-      u &= mask;
-      w &= mask;
-    }
-    const uint32_t pk = (u + (w << 16)) + off;
+    const uint32_t m = p == 0 ? 0x03FF03FFu : mask * 0x00010001u;
+    const uint32_t pk = (__byte_perm((uint32_t)(x >> sh), (uint32_t)(y >> sh), 0x5410) & m) | 0x64006400u;
     const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&pk), sub);
     out[p] = *reinterpret_cast<const uint32_t*>(&d);
   }
 }
 
+// x 2^k rounded to the nearest integer (halves away from zero), by integer operations; |x| 2^k below 2^62.
+__device__ __forceinline__ long long to_fixed(double x, int k) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7FF), sh = e - 1075 + k;
+  unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
+  if (sh >= 0) m <<= sh & 15;
+  else m = sh < -60 ? 0ull : ((m >> (-sh - 1)) + 1) >> 1;
+  return b < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ long long to_fixed(float x, int k) {
+  const int b = __float_as_int(x), e = (b >> 23) & 0xFF, sh = e - 150 + k;
+  unsigned long long m = ((uint32_t)b & 0x7FFFFFu) | (e ? 1u << 23 : 0u);
+  if (sh >= 0) m <<= sh & 63;
+  else m = sh < -30 ? 0ull : ((m >> (-sh - 1)) + 1) >> 1;
+  return b < 0 ? -(long long)m : (long long)m;
+}
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// The MMAs of one 16-wide k step of a tile with kRows rows: every digit pair (p, q) with p + q < kD into accumulator
+// p + q. The descriptors differ by constants alone: a thread that computes them at run time issues an MMA every 85
+// cycles, and one of 128 x 64 takes 48 (32 with 64 rows).
+template <class Dg, int kRows>
+__device__ __forceinline__ void digit_pairs(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t id, bool first) {
+  constexpr int kD = Dg::kD;
+#pragma unroll
+  for (int p = 0; p < kD; ++p)
+#pragma unroll
+    for (int q = 0; q + p < kD; ++q)
+      tc::mma_f16(tmem + 64 * (p + q), ad + ((p * kRows * 64) >> 4), bd + ((q * 4096) >> 4), id, p > 0 || !first ? 1u : 0u);
+}
+
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
 
-template <class Dg>
+// kMode 0: the sign iteration; 1: the inverse of T_J(S) and A_J
+template <class Dg, int kMode>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     k_ns_oz(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA64,
             const __grid_constant__ CUtensorMap mapB, OzArgs g) {
@@ -198,7 +244,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
   extern __shared__ uint8_t smraw[];
   uint8_t* stage_mem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   __shared__ OzShared sh;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = (int)cta_rank(), cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -225,35 +271,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
   cluster_sync();   // the peer's barriers are initialised before anything arrives on them
   const uint32_t tmem = sh.tmem;
   const size_t plane_elems = (size_t)g.R * g.LD;
-  const int zc = cid * 3 * kD;                 // first plane of this cluster
+  const int zc = cid * sets(kMode) * kD;       // first plane of this cluster
   bool armed[3] = {false, false, false};
   uint32_t arm_phase[3] = {0, 0, 0};
   uint32_t kcount = 0, tcount = 0, ev = 0;     // stages, tiles and meetings so far (per role)
 
-  // Every role follows the same course: per submatrix the start (meeting), products in pairs (a meeting each) and
-  // the end (meeting); after a meeting each takes the next step from the records.
-  struct Course { int n, n16, nrb, ncb, cur, steps, cap, tries, status; bool last, gave_up; };
+  // Every role follows the same course: per submatrix the start, then products, a meeting after each (mode 0: and the
+  // end); after a meeting each takes the next step from the records.
+  struct Course { int n, n16, nrb, ncb, cur, sp, steps, cap, tries, status; bool last, gave_up; };
   Course c;
+  const bool mma_warp = warp == 1;
   auto meet = [&](Record& r) -> bool {         // waits for the meeting's end; false: give up
-    const bool ok = !sh.err && wait_cluster(&sh.done, ev & 1, 8 * g.wait_ns);
+    bool ok = !sh.err && wait_cluster(&sh.done, ev & 1, 8 * g.wait_ns);
+    if (mma_warp) ok = __all_sync(0xffffffffu, ok);
     r = sh.rec[ev & 1];
     ++ev;
     return ok && !((r.bad[0] | r.bad[1]) & 4);
   };
   auto begin = [&](int J) -> bool {            // false: not taken here
-    if (g.prep_status[J] != kSubOk) return false;
+    if (g.prep_status[J] != (kMode == 0 ? kSubOk : kSubPending)) return false;
     c.n = g.sub_n[J];
     c.n16 = (c.n + 15) & ~15;
     c.nrb = (c.n16 + 127) / 128;
     c.ncb = (c.n16 + 63) / 64;
-    c.cap = g.budget ? min(g.max_iter, g.budget[J]) : g.max_iter;
+    c.cap = kMode == 0 && g.budget ? min(g.max_iter, g.budget[J]) : g.max_iter;
     c.tries = 0;
     c.gave_up = false;
     return c.cap > 0;
   };
-  auto reset = [&]() { c.cur = 0; c.steps = 0; c.last = false; c.status = kSubNotConv; };
-  // after the start or a product X T; true: go on with X X
-  auto after_x = [&](const Record& r) -> int { // 0: go on, 1: start again, 2: finish
+  // cur: which of the two X operands; sp: the operand that holds S (inverse mode: 2, R in 3, or the reverse)
+  auto reset = [&]() { c.cur = 0; c.sp = 2; c.steps = 0; c.last = false; c.status = kSubNotConv; };
+  // after the start or a new X. 0: go on, 1: start again (larger exponents), 2: finish
+  auto after_x = [&](const Record& r) -> int {
     const uint32_t bad = r.bad[0] | r.bad[1];
     if (bad & 2) c.gave_up = true;
     else if (bad & 1) {
@@ -262,21 +311,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     }
     return (c.gave_up || c.last) ? 2 : 0;
   };
-  auto after_p = [&](const Record& r) {        // after a product X X: the stopping rule
-    const float defect = sqrtf((r.part[0] + r.part[1]) / (float)c.n);
+  auto after_p = [&](const Record& r) {        // after X X (mode 0): the stopping rule; after S X: how far X is off
+    const float sum = r.part[0] + r.part[1];
     c.steps += 1;
-    if (defect <= (float)g.tol) {
-      c.last = true;
-      c.status = kSubOk;
-    } else if (c.steps >= c.cap) {
-      c.last = true;
+    if constexpr (kMode == 0) {
+      if (sqrtf(sum / (float)c.n) <= (float)g.tol) {
+        c.last = true;
+        c.status = kSubOk;
+      } else if (c.steps >= c.cap) {
+        c.last = true;
+      }
+    } else {
+      const float far = sqrtf(sum);
+      if (!(far < kOzFar) || (far > kOzLast && c.steps >= kOzRounds)) c.gave_up = true;
+      else if (far <= kOzLast) c.last = true;
     }
   };
   auto tail64 = [&](int mb) { return c.n16 - 128 * mb <= 64; };
 
   if (warp < 4) {
     tc::setmaxnreg_dec<kRegsLow>();
-    if ((warp == 0 || warp == 1) && lane == 0) {
+    if ((warp == 0 && lane == 0) || warp == 1) {   // one thread loads; the MMA warp runs converged, one lane issues
       // one product: A in operand set za, B in zb
       auto product = [&](int sa, int sb) -> bool {
         const int n32 = (c.n16 + 31) / 32;
@@ -298,25 +353,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
             }
           } else {
             const uint32_t id = tc::idesc(0, 0, 0, 1, rows, min(64, c.n16 - 64 * cb));
-            if (!tc::mbar_wait(&sh.acce, (tcount & 1) ^ 1, tc::globaltimer() + g.wait_ns)) return false;
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(&sh.acce, (tcount & 1) ^ 1, tc::globaltimer() + g.wait_ns)))
+              return false;
             tc::tc_fence_after();
             for (int ks = 0; ks < n32; ++ks, ++kcount) {
               const int st = kcount % kStages;
-              if (!tc::mbar_wait(&sh.full[st], (kcount / kStages) & 1, tc::globaltimer() + g.wait_ns)) return false;
+              if (!__all_sync(0xffffffffu, tc::mbar_wait(&sh.full[st], (kcount / kStages) & 1, tc::globaltimer() + g.wait_ns)))
+                return false;
               tc::tc_fence_after();
-              const uint32_t a0 = tc::smem_u32(stage_mem + st * Dg::kStage);
+              const uint32_t a0 = __shfl_sync(0xffffffffu, tc::smem_u32(stage_mem + st * Dg::kStage), 0);
               const uint64_t ad = sdesc_sw64(a0), bd = tc::sdesc_sw128(a0 + Dg::kABytes, 4096, 1024);
-              for (int kk = 0; kk < 2 && 32 * ks + 16 * kk < c.n16; ++kk) {
-#pragma unroll
-                for (int p = 0; p < kD; ++p)
-#pragma unroll
-                  for (int q = 0; q + p < kD; ++q)
-                    tc::mma_f16(tmem + 64 * (p + q), ad + ((p * rows * 64 + kk * 32) >> 4),
-                                bd + ((q * 4096 + kk * 2048) >> 4), id, (ks > 0 || kk > 0 || p > 0) ? 1u : 0u);
+              if (elect_one()) {
+                for (int kk = 0; kk < 2 && 32 * ks + 16 * kk < c.n16; ++kk) {
+                  const uint64_t ak = ad + ((kk * 32) >> 4), bk = bd + ((kk * 2048) >> 4);
+                  if (m64) digit_pairs<Dg, 64>(tmem, ak, bk, id, ks == 0 && kk == 0);
+                  else digit_pairs<Dg, 128>(tmem, ak, bk, id, ks == 0 && kk == 0);
+                }
+                tc::mma_commit(&sh.empty[st]);
               }
-              tc::mma_commit(&sh.empty[st]);
+              __syncwarp();
             }
-            tc::mma_commit(&sh.accf);
+            if (elect_one()) tc::mma_commit(&sh.accf);
+            __syncwarp();
             ++tcount;
           }
         }
@@ -336,13 +394,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
             continue;
           }
           if (go == 2) break;
-          if (!(ok = product(c.cur, c.cur) && meet(r))) break;
-          tc::fence_proxy_async_global();
-          after_p(r);
-          if (!(ok = product(c.cur, 2))) break;
-          c.cur ^= 1;
+          if constexpr (kMode == 0) {
+            if (!(ok = product(c.cur, c.cur) && meet(r))) break;
+            tc::fence_proxy_async_global();
+            after_p(r);
+            if (!(ok = product(c.cur, 2))) break;
+            c.cur ^= 1;
+          } else {
+            if (!(ok = product(c.sp, c.cur) && meet(r))) break;      // R = I - S X
+            tc::fence_proxy_async_global();
+            after_p(r);
+            if (c.gave_up) break;
+            if (!(ok = product(5 - c.sp, 4) && meet(r))) break;      // V = I + R (I + R)
+            tc::fence_proxy_async_global();
+            if (!(ok = product(c.cur, c.sp))) break;                 // X' = X V
+            c.cur ^= 1;
+            c.sp = 5 - c.sp;                                         // S again (or H) in R's place
+          }
         }
-        if (!ok || !meet(r)) {
+        if (kMode == 1 && ok && !c.gave_up) ok = product(c.cur, c.sp);   // A_J = X H
+        if (!ok || ((kMode == 0 || !c.gave_up) && !meet(r))) {
           sh.err = 1;
           break;
         }
@@ -354,7 +425,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     uint16_t* const planes = g.planes + (size_t)zc * plane_elems;
     double* const xd = g.xd + (size_t)cid * plane_elems;
     const uint32_t rec0 = tc::smem_u32(&sh.rec[0]), done0 = tc::smem_u32(&sh.done);
-    int ex = 1, et = 2;
+    int ex = 1, et = 2, es = 1, eh = 1;          // exponents of X, T (mode 0), S and H (inverse mode)
 
     // the CTA's part of the meeting: sums over its threads to both CTAs' records, then the arrivals
     auto tell = [&](float part, uint32_t bad, double s0, double s1, double s2, bool sums) {
@@ -395,61 +466,100 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
       }
     };
 
-    // a4: X_0 = (A - mu I) / alpha as digits, this CTA's half of the rows; false: not representable
-    auto start = [&](int J) -> uint32_t {
-      const int n = c.n, n16 = c.n16;
-      const double* A = g.A + g.a_off[J];
-      const double alpha = scale_alpha(g.lam, g.lam_g, J, g.mu);
-      const double inv = 1.0 / alpha;
-      if (c.tries == 0) {
-        uint32_t mx = 0;                       // the largest |A_ij| by its leading bits
-        for (int e = etid; e < n * n; e += kOzEpi) mx = max(mx, (uint32_t)__double2hiint(__ldg(A + e)) & 0x7FFFFFFFu);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (lane == 0) sh.red[ew] = __uint_as_float(mx);
-        oz_bar();
-        for (int w = 0; w < 8; ++w) mx = max(mx, __float_as_uint(sh.red[w]));
-        oz_bar();
-        const double big = (__hiloint2double((int)mx, -1) + fabs(g.mu)) * fabs(inv);
-        if (!isfinite(inv) || !isfinite(big) || big > 1e6) return 2;
-        int e = 0;
-        frexp(big, &e);                        // big < 2^e
-        ex = max(1, e);
-      } else {
-        ex += 3;
+    // the largest |M_ij|, rounded up, of n x n entries (or, step n + 1, of the diagonal): by its leading bits
+    auto largest = [&](const auto* M, int n, int step) -> double {
+      uint32_t mx = 0;
+#pragma unroll 8
+      for (int e = etid * step; e < n * n; e += kOzEpi * step) {
+        if constexpr (sizeof(*M) == 8) mx = max(mx, (uint32_t)__double2hiint(__ldg(M + e)) & 0x7FFFFFFFu);
+        else mx = max(mx, __float_as_uint(__ldg(M + e)) & 0x7FFFFFFFu);
       }
-      et = ex + 1;
-      const double up = pow2(U - ex);
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      if (lane == 0) sh.red[ew] = __uint_as_float(mx);
+      oz_bar();
+      for (int w = 0; w < 8; ++w) mx = max(mx, __float_as_uint(sh.red[w]));
+      oz_bar();
+      return sizeof(*M) == 8 ? __hiloint2double((int)mx, -1) : (double)__uint_as_float(mx);
+    };
+    auto exponent = [](double big) {             // big < 2^e
+      int e = 0;
+      frexp(big, &e);
+      return e;
+    };
+    // (M - mu I) inv (n x n, row-major) as the digits of operand `set` with exponent e, zero up to n16 rows and
+    // columns: this CTA's half of the rows
+    auto fill = [&](const auto* __restrict__ M, double mu, double inv, int set, int e) {
+      const int n = c.n, n16 = c.n16;
+      uint16_t* dst = planes + (size_t)set * kD * plane_elems;
       const int half = (n16 / 16 + 1) / 2 * 16;
-      const int r0 = rank ? half : 0, r1 = rank ? n16 : half, w2 = ((n + 63) & ~63) / 2;
-      for (int i = r0 + ew; i < r1; i += 8)
+      const int r0 = rank ? half : 0, r1 = rank ? n16 : half, w2 = n16 / 2;
+      // four rows of a warp together: eight loads in flight per lane
+      for (int i0 = r0 + 4 * ew; i0 < r1; i0 += 32)
         for (int j = lane; j < w2; j += 32) {
-          long long v[2];
+          long long v[4][2];
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int col = 2 * j + u;
-            v[u] = 0;
-            if (i < n && col < n) {
-              const double x = (__ldg(A + (size_t)i * n + col) - (i == col ? g.mu : 0.0)) * inv;
-              v[u] = __double2ll_rn(x * up);
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int i = i0 + a, col = 2 * j + u;
+              v[a][u] = 0;
+              if (i < n && col < n) {
+                auto x = __ldg(M + (size_t)i * n + col);
+                if constexpr (kMode == 0) x = (x - (i == col ? mu : 0.0)) * inv;
+                v[a][u] = to_fixed(x, U - e);
+              }
             }
-          }
-          uint32_t d[kD];
-          digits2<Dg>(v[0], v[1], d);
 #pragma unroll
-          for (int p = 0; p < kD; ++p)
-            *reinterpret_cast<uint32_t*>(planes + p * plane_elems + (size_t)i * g.LD + 2 * j) = d[p];
+          for (int a = 0; a < 4; ++a) {
+            if (i0 + a >= r1) break;
+            uint32_t d[kD];
+            digits2<Dg>(v[a][0], v[a][1], d);
+#pragma unroll
+            for (int p = 0; p < kD; ++p)
+              *reinterpret_cast<uint32_t*>(dst + p * plane_elems + (size_t)(i0 + a) * g.LD + 2 * j) = d[p];
+          }
         }
+    };
+    // The operands of a new submatrix (or of another attempt with larger exponents). Mode 0, a4: X_0 = (A - mu I) / alpha.
+    // Inverse mode: X and S. Returns 2 when they cannot be represented.
+    auto start = [&](int J) -> uint32_t {
+      if constexpr (kMode == 0) {
+        const double* A = g.A + g.a_off[J];
+        const double inv = 1.0 / scale_alpha(g.lam, g.lam_g, J, g.mu);
+        // the Gershgorin interval bounds every entry of A - mu I by its alpha, and alpha is at least 1/1.7 of that
+        if (!isfinite(inv) || !isfinite(g.lam_g[2 * J]) || !isfinite(g.lam_g[2 * J + 1])) return 2;
+        ex = 1 + 3 * c.tries;
+        et = ex + 1;
+        fill(A, g.mu, inv, 0, ex);
+      } else {
+        const int64_t at = g.a_off[J] - g.a_base;
+        if (c.tries == 0) {
+          // positive definite matrices have their largest entry on the diagonal (with anything else R gets large)
+          const double bx = largest(g.X32 + at, c.n, c.n + 1), bs = largest(g.ws + at, c.n, c.n + 1);
+          if (!isfinite(bx) || !isfinite(bs) || bx > 1e6 || bs > 1e6) return 2;
+          ex = max(1, exponent(bx) + 1);
+          es = max(-8, exponent(bs) + 1);
+        } else {
+          ex += 3;
+        }
+        fill(g.X32 + at, 0.0, 1.0, 0, ex);
+        fill(g.ws + at, 0.0, 1.0, 2, es);
+      }
       return 0;
     };
 
-    // drains this CTA's tiles of one product. kind 0: T = 3I - P and the defect; 1: X' = P / 2 as digits; 2: X' as
-    // FP64 (the last). shift: left shift of the accumulators' sum to the output's units.
-    auto drain = [&](int kind, int so, float& part, uint32_t& bad) -> bool {
+    // Drains this CTA's tiles of one product P into operand `so` (digits) or an FP64 array. Mode 0: kT (T = 3I - P and
+    // the defect's sum), kX (P / 2), kXd (P / 2 in FP64: the last). Inverse mode: kR (R = I - P and I + R, the sum of
+    // R^2), kV (I + P), kX (P; with last_q its centre columns in FP64 too), kA (P in FP64).
+    enum : int { kT, kX, kXd, kR, kV, kA };
+    auto drain = [&](int kind, int so, int J, bool last_q, float& part, uint32_t& bad) -> bool {
       const int n = c.n, n16 = c.n16;
-      const int s = kind == 0 ? 2 * ex - et : et - 1;
-      const long long one = kind == 0 ? 1ll << (U - et) : 0;
-      const float down = pow2f(et - U);
-      const double downd = pow2(ex - U);
+      // exponents of the product's two operands together, and of the output
+      const int ein = kMode == 0 ? (kind == kT ? 2 * ex : ex + et) : (kind == kR ? es + ex : kind == kX ? ex + 1 : kind == kA ? ex + eh : 1);
+      const int eo = kMode == 0 ? (kind == kT ? et : ex + 1) : (kind == kR ? 0 : kind == kX ? ex : kind == kA ? ex + eh : 1);
+      const int s = ein - eo;
+      const long long one = 1ll << (U - eo);
+      const float down = pow2f(eo - U);
       // the first accumulator (2^(2 kB - 2) times the product) below this: no wrap in 64 bits
       const float most0 = fminf(pow2f(62 - kB * (kD - 2)), pow2f(3 - s + 2 * (kB - 1)));
       const int shl = U + s - Dg::G;           // from the last accumulator but one to the output's units
@@ -466,71 +576,118 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
         long long v[32];
         uint32_t ov = 0;
         float big0 = 0.0f, big = 0.0f;         // the largest first accumulator, and of the next (all but the last two)
-        if (rbase < n16) {
+        if (rbase < n16 && colg < n16) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
+            if (colg + 16 * h >= n16) {        // columns the MMAs left out hold anything
+#pragma unroll
+              for (int j = 0; j < 16; ++j) v[16 * h + j] = 0;
+              break;
+            }
             uint32_t r[kD][16];
 #pragma unroll
             for (int l = 0; l < kD; ++l) tmem_ld16(ta + 64 * l + 16 * h, r[l]);
             tc::tmem_wait_ld();
+            // sum of the accumulators in units of the last but one: those up to 30 bits above it as 32 x 32 -> 64 bit
+            // multiply-adds, the rest into the high word
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              long long a = 0;
+              int a[kD];
 #pragma unroll
-              for (int l = 0; l + 1 < kD; ++l) {
-                const float f = colg + 16 * h + j < n ? __uint_as_float(r[l][j]) : 0.0f;
+              for (int l = 0; l < kD; ++l) {
+                const float f = __uint_as_float(r[l][j]);
                 if (l == 0) big0 = fmaxf(big0, fabsf(f));
                 else if (l < kD - 2) big = fmaxf(big, fabsf(f));
-                a = (a << kB) + (long long)__float2int_rn(f);
+                a[l] = __float2int_rn(f);
               }
-              a += (__float2int_rn(__uint_as_float(r[kD - 1][j])) + (1 << (kB - 1))) >> kB;
-              a = shl >= 0 ? a << shl : (a + (1ll << (-shl - 1))) >> -shl;
-              v[16 * h + j] = a;
+              long long w = (long long)a[kD - 2] + ((a[kD - 1] + (1 << (kB - 1))) >> kB);
+              int hi = 0;
+#pragma unroll
+              for (int l = kD - 3; l >= 0; --l) {
+                const int up = kB * (kD - 2 - l);
+                if (up <= 30) w += (long long)a[l] * (1 << (up & 31));
+                else hi += (int)((uint32_t)a[l] << ((up - 32) & 31));
+              }
+              w += (long long)hi << 32;
+              v[16 * h + j] = shl >= 0 ? w << shl : (w + (1ll << (-shl - 1))) >> -shl;
             }
           }
         }
         tc::tc_fence_before();
         tc::mbar_arrive(&sh.acce);
-        if (rbase < n16) {
+        if (rbase < n16 && colg < n16) {
+          const bool rin = rok && row < n;
+          if (rin && !(big < 16777216.0f)) bad |= 2;
+          if (rin && !(big0 < most0)) bad |= 1;
+          // rows and columns from n to n16 are zeros of themselves, their operands' being zeros
+          const bool dia = rin && row >= colg && row < colg + 32 && kind != kX && kind != kXd && kind != kA;
+          float sq = 0.0f;
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
-            const int col = colg + j;
-            const bool in = row < n && col < n && rok;
             long long a = v[j];
-            if (kind == 0) {
-              const long long e = (row == col ? one : 0) - a;      // (I - P)_ij
-              const float ef = in ? down * (float)e : 0.0f;
-              part = fmaf(ef, ef, part);
-              a = e + (row == col ? 2 * one : 0);
+            if (kind == kT || kind == kR) {
+              a = -a;
+              if (dia) a += row == colg + j ? one : 0;               // (I - P)_ij
+              const float ef = down * (float)a;
+              sq = fmaf(ef, ef, sq);
+              if (dia && kind == kT) a += row == colg + j ? 2 * one : 0;
+            } else if (kind == kV) {
+              if (dia) a += row == colg + j ? one : 0;
             }
-            a = in ? a : 0;
             const int hi = (int)(a >> 32);
             ov |= (uint32_t)(hi ^ (hi >> 31));
             v[j] = a;
           }
-          const bool over = (ov >> (U - 32)) != 0;
-          if (rok && row < n && !(big < 16777216.0f)) bad |= 2;
-          if (over || (rok && row < n && !(big0 < most0))) bad |= 1;
-          if (rok && colg < n16) {
-            if (kind == 2) {
+          if (rin) part += sq;
+          if (rin && (ov >> (U - 32)) != 0 && kind != kXd && kind != kA) bad |= 1;
+          auto put = [&](int set) {
+            uint16_t* dst = planes + (size_t)set * kD * plane_elems + (size_t)row * g.LD + colg;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t o[kD][8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                uint32_t d[kD];
+                digits2<Dg>(v[16 * h + 2 * j], v[16 * h + 2 * j + 1], d);
+#pragma unroll
+                for (int p = 0; p < kD; ++p) o[p][j] = d[p];
+              }
+#pragma unroll
+              for (int p = 0; p < kD; ++p) st_global_256(dst + p * plane_elems + 16 * h, o[p]);
+            }
+          };
+          if (rok) {
+            if (kMode == 0 && kind == kXd) {
+              const double to = pow2(ex - U);
               double* dst = xd + (size_t)row * g.LD + colg;
 #pragma unroll
               for (int j = 0; j < 32; j += 2)
-                *reinterpret_cast<double2*>(dst + j) = make_double2((double)v[j] * downd, (double)v[j + 1] * downd);
+                *reinterpret_cast<double2*>(dst + j) = make_double2((double)v[j] * to, (double)v[j + 1] * to);
+            } else if (kMode == 1 && kind == kA) {
+              if (rin) {
+                const double to = pow2(eo - U);
+                double* dst = g.Aout + g.a_off[J] + (size_t)row * n + colg;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  if (colg + j < n) dst[j] = (double)v[j] * to;
+              }
             } else {
-              uint16_t* dst = planes + (size_t)so * kD * plane_elems + (size_t)row * g.LD + colg;
+              put(so);
+            }
+            if (kMode == 1 && kind == kR) {    // I + R, exponent 1
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                uint32_t o[kD][8];
+              for (int j = 0; j < 32; ++j)
+                v[j] = (v[j] + (dia && row == colg + j ? 1ll << U : 0) + 1) >> 1;
+              put(4);
+            }
+            if (kMode == 1 && kind == kX && last_q && rin) {
+              const int c0 = g.sub_c0[J], b = g.nbf[J];
+              const double to = pow2(ex - U);
+              double* Q = g.Qout + g.c_off[J] + (size_t)row * b;
+              if (colg < c0 + b && colg + 32 > c0) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  uint32_t d[kD];
-                  digits2<Dg>(v[16 * h + 2 * j], v[16 * h + 2 * j + 1], d);
-#pragma unroll
-                  for (int p = 0; p < kD; ++p) o[p][j] = d[p];
-                }
-#pragma unroll
-                for (int p = 0; p < kD; ++p) st_global_256(dst + p * plane_elems + 16 * h, o[p]);
+                for (int j = 0; j < 32; ++j)
+                  if (colg + j >= c0 && colg + j < c0 + b) Q[colg + j - c0] = (double)v[j] * to;
               }
             }
           }
@@ -561,16 +718,57 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
         if (go == 2) break;
         float part = 0.0f;
         bad = 0;
-        ok = drain(0, 2, part, bad);
-        tell(part, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
-        if (!(ok = meet(r) && ok)) break;
-        const uint32_t bad_p = (r.bad[0] | r.bad[1]) & 3;   // an overflow in T counts with X T's
-        after_p(r);
-        bad = bad_p;
-        ok = drain(c.last ? 2 : 1, c.cur ^ 1, part, bad);
-        tell(0.0f, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
-        if (!ok) break;
-        c.cur ^= 1;
+        if constexpr (kMode == 0) {
+          ok = drain(kT, 2, J, false, part, bad);
+          tell(part, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          if (!(ok = meet(r) && ok)) break;
+          bad = (r.bad[0] | r.bad[1]) & 3;     // an overflow in T counts with X T's
+          after_p(r);
+          ok = drain(c.last ? kXd : kX, c.cur ^ 1, J, false, part, bad);
+          tell(0.0f, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          if (!ok) break;
+          c.cur ^= 1;
+        } else {
+          if (c.steps == 0 && c.tries == 0) {  // while the MMAs form S X
+            const double bh = largest(g.ws + g.chunk_n2 + g.a_off[J] - g.a_base, c.n, 1);
+            if (!isfinite(bh) || bh > 1e6) bad = 2;
+            eh = max(-8, exponent(bh));
+          }
+          ok = drain(kR, 5 - c.sp, J, false, part, bad);
+          tell(part, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          if (!(ok = meet(r) && ok)) break;
+          uint32_t all = (r.bad[0] | r.bad[1]) & 3;
+          after_p(r);
+          if (c.gave_up) break;
+          bad = all;
+          ok = drain(kV, c.sp, J, false, part, bad);
+          tell(0.0f, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          if (!(ok = meet(r) && ok)) break;
+          bad = (r.bad[0] | r.bad[1]) & 3;
+          const int64_t at = g.a_off[J] - g.a_base;
+          // into R's place, while the MMAs form X V: S for another round, or H for A_J
+          fill(g.ws + at + (c.last ? g.chunk_n2 : 0), 0.0, 1.0, 5 - c.sp, c.last ? eh : es);
+          ok = drain(kX, c.cur ^ 1, J, c.last, part, bad);
+          tell(0.0f, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          if (!ok) break;
+          c.cur ^= 1;
+          c.sp = 5 - c.sp;
+        }
+      }
+      if constexpr (kMode == 1) {
+        float part = 0.0f;
+        bad = 0;
+        if (ok && !c.gave_up) {
+          ok = drain(kA, 0, J, false, part, bad);
+          tell(0.0f, bad | (ok ? 0u : 4u), 0.0, 0.0, 0.0, false);
+          ok = meet(r) && ok;
+        }
+        if (!ok) {
+          if (etid == 0) sh.err = 1;
+          break;
+        }
+        if (rank == 0 && etid == 0) g.prep_out[J] = c.gave_up || (r.bad[0] | r.bad[1]) ? kSubRefine : kSubOk;
+        continue;
       }
       if (!ok) {
         // the peer waits for this CTA's part of a meeting at most for its own limit
@@ -641,10 +839,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
   cluster_sync();   // no CTA leaves while its peer may still write to its shared memory
 }
 
-// Every submatrix of the work starts as kSubRefine: what k_ns_oz does not finish, k_ns_fp64 takes
+// Mode 0: every submatrix of the work starts as kSubRefine, and what k_ns_oz does not finish k_ns_fp64 takes. Inverse
+// mode: those whose FP32 inverse is there start as kSubPending, the others as kSubRefine (k_prepare takes both).
+template <int kMode>
 __global__ void k_oz_pending(int32_t count, const int32_t* __restrict__ order, int32_t* __restrict__ status) {
   for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x)
-    status[order[e]] = kSubRefine;
+    status[order[e]] = kMode == 1 && status[order[e]] == kSubOk ? kSubPending : kSubRefine;
 }
 
 // How many two-CTA clusters of the kernel run at once on the device (asked once per device).
@@ -663,8 +863,8 @@ int active_clusters(int dev, int sms) {
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaFuncSetAttribute(&k_ns_oz<Dg>, cudaFuncAttributeMaxDynamicSharedMemorySize, Dg::kSmem) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, &k_ns_oz<Dg>, &cfg) != cudaSuccess || n < 1) {
+  if (cudaFuncSetAttribute(&k_ns_oz<Dg, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, Dg::kSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, &k_ns_oz<Dg, 0>, &cfg) != cudaSuccess || n < 1) {
     cudaGetLastError();
     n = std::max(1, sms / 2);
   }
@@ -672,9 +872,9 @@ int active_clusters(int dev, int sms) {
   return n;
 }
 
-template <class Dg>
+template <class Dg, int kMode>
 nolsm_status launch(const OzSolve& a, cudaStream_t st) {
-  const auto kernel = &k_ns_oz<Dg>;
+  const auto kernel = &k_ns_oz<Dg, kMode>;
   cudaFuncAttributes at{};
   NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(kernel)));
   if (at.numRegs != kRegsLaunch) {
@@ -683,7 +883,7 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
     return NOLSM_ERR_UNSUPPORTED;
   }
   NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Dg::kSmem));
-  const uint64_t depth = (uint64_t)a.clusters * 3 * Dg::kD;
+  const uint64_t depth = (uint64_t)a.clusters * sets(kMode) * Dg::kD;
   CUtensorMap mA, mA64, mB;
   if (!tmap::make_3d(&mA, a.planes, 2, (uint64_t)a.LD, (uint64_t)a.R, depth, 32, 128, CU_TENSOR_MAP_SWIZZLE_64B, Dg::kD) ||
       !tmap::make_3d(&mA64, a.planes, 2, (uint64_t)a.LD, (uint64_t)a.R, depth, 32, 64, CU_TENSOR_MAP_SWIZZLE_64B, Dg::kD) ||
@@ -691,7 +891,7 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
     set_error("cuTensorMapEncodeTiled rejected the digit planes (R %d, LD %d, clusters %d)", a.R, a.LD, a.clusters);
     return NOLSM_ERR_CUDA;
   }
-  OzArgs g;
+  OzArgs g{};
   g.count = a.count; g.order = a.order;
   g.sub_n = a.sub_n; g.nbf = a.nbf; g.a_off = a.a_off; g.c_off = a.c_off;
   g.A = a.A; g.Q = a.Q; g.Sc = a.Sc; g.Hc = a.Hc; g.lam = a.lam; g.lam_g = a.lam_g;
@@ -701,7 +901,11 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
   g.Dc = a.Dc; g.tS = a.tS; g.tH = a.tH; g.iters = a.iters; g.status = a.status; g.rsteps = a.rsteps;
   g.nbelow = a.nbelow;
   g.wait_ns = kOzWaitNs;
-  k_oz_pending<<<std::min(256, (a.count + 255) / 256), 256, 0, st>>>(a.count, a.order, a.status);
+  g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2; g.X32 = a.X32; g.sub_c0 = a.sub_c0;
+  g.Aout = a.Aout; g.Qout = a.Qout; g.prep_out = a.prep_out;
+  if (kMode == 1) g.max_iter = 1;
+  k_oz_pending<kMode><<<std::min(256, (a.count + 255) / 256), 256, 0, st>>>(a.count, a.order,
+                                                                            kMode == 0 ? a.status : a.prep_out);
   NOLSM_LAUNCH_CHECK();
   kernel<<<2 * std::min(a.clusters, a.count), kOzThreads, Dg::kSmem, st>>>(mA, mA64, mB, g);
   NOLSM_LAUNCH_CHECK();
@@ -710,14 +914,18 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
 
 }  // namespace
 
-int oz_planes() { return 3 * Digits<8, 8>::kD; }
+int oz_planes(int mode) { return sets(mode) * Digits<8, 8>::kD; }
 
 int oz_clusters(int max_n, int dev, int sms) {
   return max_n <= kOzNineBits ? active_clusters<Digits<9, 7>>(dev, sms) : active_clusters<Digits<8, 8>>(dev, sms);
 }
 
 nolsm_status launch_ns_oz(const OzSolve& a, cudaStream_t st) {
-  return a.max_n <= kOzNineBits ? launch<Digits<9, 7>>(a, st) : launch<Digits<8, 8>>(a, st);
+  return a.max_n <= kOzNineBits ? launch<Digits<9, 7>, 0>(a, st) : launch<Digits<8, 8>, 0>(a, st);
+}
+
+nolsm_status launch_inverse_oz(const OzSolve& a, cudaStream_t st) {
+  return a.max_n <= kOzNineBits ? launch<Digits<9, 7>, 1>(a, st) : launch<Digits<8, 8>, 1>(a, st);
 }
 
 }  // namespace nolsm

@@ -18,13 +18,20 @@ struct OzSolve {
   const int32_t* prep_status;
   double mu, tol;
   int32_t max_iter; const int32_t* budget;
-  uint16_t* planes; double* xd; int32_t R, LD, clusters;   // scratch: oz_planes() planes of R x LD per cluster, R x LD
+  uint16_t* planes; double* xd; int32_t R, LD, clusters;   // scratch: oz_planes(mode) planes of R x LD per cluster, R x LD
   double* Dc; double* tS; double* tH; int32_t* iters; int32_t* status; int32_t* rsteps; int32_t* nbelow;
+  // launch_inverse_oz: the chunk's T_J(S), T_J(H0) (FP64, at a_off[J] - a_base and chunk_n2 further) and T_J(S)^-1 in
+  // FP32 (at a_off[J] - a_base), where prep_out[J] is kSubOk
+  const double* ws; int64_t a_base, chunk_n2; const float* X32; const int32_t* sub_c0;
+  double* Aout; double* Qout; int32_t* prep_out;
 };
-int oz_planes();
+int oz_planes(int mode);
 // how many clusters run at once (the scratch is sized for them)
 int oz_clusters(int max_n, int dev, int sms);
 // Leaves status[J] = kSubRefine for the submatrices k_ns_fp64 has to take.
 nolsm_status launch_ns_oz(const OzSolve& a, cudaStream_t st);
+// A_J in FP64 to Aout + a_off[J] and the centre columns of T_J(S)^-1 to Qout + c_off[J], prep_out[J] = kSubOk; kSubRefine
+// or kSubPending where k_prepare has to take the submatrix.
+nolsm_status launch_inverse_oz(const OzSolve& a, cudaStream_t st);
 
 }  // namespace nolsm

@@ -6,6 +6,8 @@ namespace nolsm {
 
 // internal preparation status: the submatrix is prepared again with the FP64 factorisation
 constexpr int32_t kSubRefine = 64;
+// FP64 preparation: the FP32 inverse is there, the refined one is not (yet)
+constexpr int32_t kSubPending = 65;
 
 struct PrepArgs {
   int32_t j0;                 // first submatrix of the chunk (one CTA per submatrix)
@@ -45,6 +47,8 @@ struct SymArgs {
 
 // a2-a3 for `count` submatrices starting at g.j0 (largest dimension max_n); A in FP64 (fp64_A) or FP32.
 nolsm_status launch_prepare(const PrepArgs& g, int count, int max_n, bool fp64_A, void* Acache, cudaStream_t st);
+// Gershgorin intervals of A_J (FP64) for the submatrices whose preparation succeeded.
+nolsm_status launch_gershgorin(const PrepArgs& g, int count, const double* A, cudaStream_t st);
 // The same with the FP32 factor and iterative refinement of Q (A in FP32), followed by the FP64
 // preparation of the submatrices it flagged.
 nolsm_status launch_prepare_mixed(const PrepArgs& g, int count, int max_n, float* Acache, cudaStream_t st);

@@ -976,7 +976,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_prepare(PrepArgs g, TA* __restr
   __shared__ int s_bad;
   __shared__ float rlo[kThreads], rhi[kThreads];
   const int J = g.j0 + blockIdx.x;
-  if (g.only_flagged && g.prep_status[J] != kSubRefine) return;
+  if (g.only_flagged && g.prep_status[J] != kSubRefine && g.prep_status[J] != kSubPending) return;
   const int n = g.sub_n[J];
   const int bJ = g.nbf[J];
   const int c0 = g.sub_c0[J];
@@ -996,6 +996,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_prepare(PrepArgs g, TA* __restr
   solve_Q(S, n, c0, bJ, g.Q + g.c_off[J], reinterpret_cast<double (*)[kMaxB + 1]>(raw), Xs);
   __syncthreads();
   gershgorin(A, n, g.lam + 2 * J, rlo, rhi);
+}
+
+__global__ void __launch_bounds__(kThreads) k_gershgorin(PrepArgs g, const double* __restrict__ A) {
+  __shared__ float rlo[kThreads], rhi[kThreads];
+  const int J = g.j0 + (int)blockIdx.x;
+  if (g.prep_status[J] == kSubOk) gershgorin(A + g.a_off[J], g.sub_n[J], g.lam + 2 * J, rlo, rhi);
 }
 
 __global__ void __launch_bounds__(kThreads, 4) k_prepare_mixed(PrepArgs g, float* __restrict__ Acache) {
@@ -1379,6 +1385,12 @@ nolsm_status launch_prepare(const PrepArgs& g, int count, int max_n, bool fp64_A
     NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_prepare<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_prepare<float><<<count, kThreads, smem, st>>>(g, static_cast<float*>(Acache));
   }
+  NOLSM_LAUNCH_CHECK();
+  return NOLSM_OK;
+}
+
+nolsm_status launch_gershgorin(const PrepArgs& g, int count, const double* A, cudaStream_t st) {
+  k_gershgorin<<<count, kThreads, 0, st>>>(g, A);
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }

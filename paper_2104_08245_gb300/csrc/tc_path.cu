@@ -134,7 +134,7 @@ struct TcArgs {
   // chunk_n2 further), the outputs and the iteration's stopping rule
   const double* ws;
   int64_t a_base, chunk_n2;
-  float* Aout;                // FP32 A_J at a_off[J]
+  float* Aout;                // FP32 A_J at a_off[J]; null: T_J(S)^-1 alone
   float* Xout;                // FP32 T_J(S)^-1 at a_off[J] - a_base
   int32_t* prep_out;          // kSubOk, or kSubRefine when the iteration failed (FP64 preparation next)
   float tol_inv;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           // Z in 1 or 4 (ping-pong: every row tile of T Z reads all of Z; until the first Z update the pair
           // holds T_0 = 2 Z_1, hence the factor zs), T and then X in 2; T_J(H0) goes into Y's pair once Y is
           // no longer needed
-          d.last = st.kind == 4;
+          d.last = st.kind == 4 || (st.kind == 3 && !g.Aout);
           d.scale = 0.5f;
           d.fo = st.fcur;
           switch (st.kind) {
@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
       }
       epi_bar<kEpiThreads>();   // dred free again; st.last visible to every epilogue thread
       // step 0 the last: Y_0 is not needed, T_J(H0) takes its pair now (else after the last Z update)
-      if (st.last) fill_pair(base, n, n64, H);
+      if (st.last && g.Aout) fill_pair(base, n, n64, H);
     };
 
     // a4 for a new submatrix of slot s: X_0 = (A - mu I) / alpha in the main format, zero padded
@@ -1074,7 +1074,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           default: break;
         }
       }
-      if (kMode == 1 && d.kind == 2 && st.last) {
+      if (kMode == 1 && d.kind == 2 && st.last && g.Aout) {
         // the iteration's last Z update is done: T_J(H0) into Y's pair (Y was last read by this step's
         // V = Z Y) for A_J = X T_J(H0), written now so that it is not held through the iteration
         const int J = st.job;
@@ -1146,7 +1146,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
             g.prep_out[sf.job] = sf.status;
             const double n3 = (double)sf.n * sf.n * sf.n;
             // step 0 needs one product (Y_1), every further step three but the last two (no Y update); then X, A
-            const double prods = 3.0 * sf.steps - 1.0;
+            const double prods = 3.0 * sf.steps - (g.Aout ? 1.0 : 2.0);
             atomicAdd(&g.flops[0], 2.0 * n3 * prods);
             atomicAdd(&g.flops[1], 6.0 * n3 * prods);
           }

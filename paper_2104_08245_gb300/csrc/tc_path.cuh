@@ -23,7 +23,7 @@ struct NsInvArgs {
   int32_t max_n;
   const double* ws;
   int64_t a_base, chunk_n2;
-  float* Aout;
+  float* Aout;                  // null: T_J(S)^-1 alone
   float* Xout;
   int32_t* prep_out;
   float tol_inv;
