@@ -611,15 +611,10 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       // the coupled Newton-Schulz inverse square root on the tensor cores (A_J and X = T_J(S)^-1 in FP32),
       // then the refinement of the centre columns of T_J(S)^-1 with X, then the FP64 preparation of what
       // either of them flagged
-      const int64_t nbc = plan->h_c_off[e] - plan->h_c_off[J];
-      NOLSM_TRY(ensure(plan, plan->ws_refine, (sizeof(double) + sizeof(float)) * (size_t)std::max<int64_t>(nbc, 1)));
       NOLSM_TRY(sort_chunk());
       NOLSM_TRY(tensor_inverse(P.A.as<float>()));
       pa.order = plan->prep_order.as<int32_t>();
       pa.L32 = plan->ws_l32.as<float>();
-      pa.c_base = plan->h_c_off[J];
-      pa.Qp = plan->ws_refine.as<float2>();
-      pa.W32 = reinterpret_cast<float*>(pa.Qp + std::max<int64_t>(nbc, 1));
       pa.fallback_max_n = prepare_fp64_max_n();
       NOLSM_TRY(launch_ns_qrefine(pa, (int)(e - J), chunk_max_n, plan->max_b, P.A.as<float>(), st));
       plan->stats.launches += 2;

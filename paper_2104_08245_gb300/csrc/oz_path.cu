@@ -213,12 +213,6 @@ __device__ __forceinline__ long long to_fixed(float x, int k) {
   return b < 0 ? -(long long)m : (long long)m;
 }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
 // The MMAs of one 16-wide k step of a tile with kRows rows: every digit pair (p, q) with p + q < kD into accumulator
 // p + q. The descriptors differ by constants alone: a thread that computes them at run time issues an MMA every 85
 // cycles, and one of 128 x 64 takes 48 (32 with 64 rows).
@@ -363,7 +357,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
               tc::tc_fence_after();
               const uint32_t a0 = __shfl_sync(0xffffffffu, tc::smem_u32(stage_mem + st * Dg::kStage), 0);
               const uint64_t ad = sdesc_sw64(a0), bd = tc::sdesc_sw128(a0 + Dg::kABytes, 4096, 1024);
-              if (elect_one()) {
+              if (tc::elect_one()) {
                 for (int kk = 0; kk < 2 && 32 * ks + 16 * kk < c.n16; ++kk) {
                   const uint64_t ak = ad + ((kk * 32) >> 4), bk = bd + ((kk * 2048) >> 4);
                   if (m64) digit_pairs<Dg, 64>(tmem, ak, bk, id, ks == 0 && kk == 0);
@@ -373,7 +367,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
               }
               __syncwarp();
             }
-            if (elect_one()) tc::mma_commit(&sh.accf);
+            if (tc::elect_one()) tc::mma_commit(&sh.accf);
             __syncwarp();
             ++tcount;
           }
@@ -640,22 +634,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
           }
           if (rin) part += sq;
           if (rin && (ov >> (U - 32)) != 0 && kind != kXd && kind != kA) bad |= 1;
-          auto put = [&](int set) {
-            uint16_t* dst = planes + (size_t)set * kD * plane_elems + (size_t)row * g.LD + colg;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              uint32_t o[kD][8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                uint32_t d[kD];
-                digits2<Dg>(v[16 * h + 2 * j], v[16 * h + 2 * j + 1], d);
-#pragma unroll
-                for (int p = 0; p < kD; ++p) o[p][j] = d[p];
-              }
-#pragma unroll
-              for (int p = 0; p < kD; ++p) st_global_256(dst + p * plane_elems + 16 * h, o[p]);
-            }
-          };
           if (rok) {
             if (kMode == 0 && kind == kXd) {
               const double to = pow2(ex - U);
@@ -672,13 +650,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                   if (colg + j < n) dst[j] = (double)v[j] * to;
               }
             } else {
-              put(so);
-            }
-            if (kMode == 1 && kind == kR) {    // I + R, exponent 1
+              // the digits; after R also those of I + R (exponent 1)
+              int set = so;
+#pragma unroll 1
+              for (int again = kMode == 1 && kind == kR ? 1 : 0; again >= 0; --again) {
+                uint16_t* dst = planes + (size_t)set * kD * plane_elems + (size_t)row * g.LD + colg;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                v[j] = (v[j] + (dia && row == colg + j ? 1ll << U : 0) + 1) >> 1;
-              put(4);
+                for (int h = 0; h < 2; ++h) {
+                  uint32_t o[kD][8];
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) {
+                    uint32_t d[kD];
+                    digits2<Dg>(v[16 * h + 2 * j], v[16 * h + 2 * j + 1], d);
+#pragma unroll
+                    for (int p = 0; p < kD; ++p) o[p][j] = d[p];
+                  }
+#pragma unroll
+                  for (int p = 0; p < kD; ++p) st_global_256(dst + p * plane_elems + 16 * h, o[p]);
+                }
+                if (kMode == 1 && again) {
+                  set = 4;
+#pragma unroll
+                  for (int j = 0; j < 32; ++j) v[j] = (v[j] + (dia && row == colg + j ? 1ll << U : 0) + 1) >> 1;
+                }
+              }
             }
             if (kMode == 1 && kind == kX && last_q && rin) {
               const int c0 = g.sub_c0[J], b = g.nbf[J];

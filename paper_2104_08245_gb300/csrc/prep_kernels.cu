@@ -25,6 +25,7 @@
 
 #include "nolsm_internal.cuh"
 #include "prep.cuh"
+#include "tc_split.cuh"
 
 namespace nolsm {
 
@@ -855,14 +856,6 @@ __device__ __forceinline__ float2 split_f64(double s) {
   return make_float2(hi, lo);
 }
 
-// s + c <- s + c + p with s = fl(s + p) and the rounding error of that sum added to c (Knuth's TwoSum).
-__device__ __forceinline__ void two_sum(float& s, float& c, float p) {
-  const float t = s + p;
-  const float z = t - s;
-  c += (s - (t - z)) + (p - z);
-  s = t;
-}
-
 // R = E_c - S q (S the full symmetric T_J(S) in FP64, q given as hi + lo FP32 pairs), written to R in
 // FP32, in double-FP32 arithmetic (the compensated dot product of Ogita, Rump and Oishi): the hi*hi
 // products are split exactly (fmaf) and summed with TwoSum, the hi*lo and lo*hi products summed plainly.
@@ -922,36 +915,47 @@ __device__ void residual_df(const double* __restrict__ S, int n, int c0, int b, 
 }
 
 // Gershgorin interval of A (n x n, FP32 or FP64) widened by its rounding, into lam[2J], lam[2J+1].
-template <typename TA>
+template <typename TA, int kT = kThreads>
 __device__ void gershgorin(const TA* __restrict__ A, int n, double* lam, float* rlo, float* rhi) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float lo = INFINITY, hi = -INFINITY;
-  for (int i0 = 4 * warp; i0 < n; i0 += 4 * (kThreads / 32)) {   // four rows per warp pass, lanes along them
-    float r[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int j = lane; j < n; j += 32) {
+  constexpr int kR = sizeof(TA) == 4 ? 8 : 4;   // rows per warp pass, lanes along them, 4 kR loads in flight
+  for (int i0 = kR * warp; i0 < n; i0 += kR * (kT / 32)) {
+    float r[kR];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u;
-        if (i < n && j != i) r[u] += fabsf((float)A[(size_t)i * n + j]);
-      }
+    for (int u = 0; u < kR; ++u) r[u] = 0.0f;
+    for (int j0 = lane; j0 < n; j0 += 128) {
+      TA v[kR][4];
+#pragma unroll
+      for (int u = 0; u < kR; ++u)
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const int i = i0 + u, j = j0 + 32 * w;
+          v[u][w] = i < n && j < n && j != i ? A[(size_t)i * n + j] : TA(0);
+        }
+#pragma unroll
+      for (int u = 0; u < kR; ++u)
+#pragma unroll
+        for (int w = 0; w < 4; ++w) r[u] += fabsf((float)v[u][w]);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < kR; ++u)
       for (int o = 16; o > 0; o >>= 1) r[u] += __shfl_xor_sync(0xffffffffu, r[u], o);
+    // lane u takes row u's end points
+    float d = 0.0f, rr = 0.0f;
+    const int i = i0 + lane;
+    if (lane < kR && i < n) d = (float)A[(size_t)i * n + i];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u;
-      if (i < n) {
-        const float d = (float)A[(size_t)i * n + i];
-        lo = fminf(lo, d - r[u]);
-        hi = fmaxf(hi, d + r[u]);
-      }
+    for (int u = 0; u < kR; ++u) rr = lane == u ? r[u] : rr;
+    if (lane < kR && i < n) {
+      lo = fminf(lo, d - rr);
+      hi = fmaxf(hi, d + rr);
     }
   }
   rlo[threadIdx.x] = lo;
   rhi[threadIdx.x] = hi;
   __syncthreads();
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
+  for (int s = kT / 2; s > 0; s >>= 1) {
     if (threadIdx.x < s) {
       rlo[threadIdx.x] = fminf(rlo[threadIdx.x], rlo[threadIdx.x + s]);
       rhi[threadIdx.x] = fmaxf(rhi[threadIdx.x], rhi[threadIdx.x + s]);
@@ -1121,99 +1125,221 @@ __global__ void __launch_bounds__(kThreads, 4) k_prepare_mixed(PrepArgs g, float
   if (tid == 0) g.prep_status[J] = ok ? kSubOk : (n <= g.fallback_max_n ? kSubRefine : kSubNotSpd);
 }
 
-// One row i of R = E_c - T_J(S) q for CN centre columns: S_i[k] at Si[k] (kCol false: Si is row i, each lane
-// streams its own row through L1) or at Si[k n] (kCol: Si is column i of the symmetric T_J(S), the lanes of a
-// warp read consecutive entries; better for long rows, whose lines leave L1 before their reuse); against q
-// (float2 hi/lo pairs, rows of stride bJ), products and sums in double-FP32 arithmetic (each product's
-// rounding error by FMA, each sum's by TwoSum); column c is on the diagonal of E_c when c == ce. Writes w[c]
-// (FP32) when rv.
-template <int CN, bool kCol>
-__device__ __forceinline__ void residual_row(const double* __restrict__ Si, const float2* __restrict__ q, int n,
-                                             int bJ, bool rv, int ce, float* __restrict__ w) {
-  float sh[CN], sl[CN];
+constexpr int kQThreads = 256, kQWarps = kQThreads / 32;
+constexpr int RPL = 2;          // rows per lane
+constexpr float kQBig = 6.0f;   // offset of the residual's leading sums (see residual_part)
+
+// This warp's share (rows k0 <= k < k1 of the symmetric T_J(S)) of (T_J(S) q)_ic for its lanes' rows i and NP pairs
+// of columns. The lanes read T_J(S) along its rows, coalesced. Each product a v, a and v as two FP32 words, is added
+// to a running sum t that starts at kQBig: t' = fl(t + a v), and what that rounded off is a v - (t' - t), exact to one
+// rounding because t is the larger (Dekker's Fast2Sum with the product inside the second FMA). t moves in steps of
+// ulp(kQBig) = 2^-21, so the remainders l stay near 2^-19 and their FP32 sum is good to 2^-43 per term: the residual
+// keeps about 1e-12 of |T_J(S)| |q|. Six packed operations per pair of columns instead of eleven per column.
+template <int NP>
+__device__ __forceinline__ void residual_part(const double* __restrict__ S, int n, int k0, int k1, const int (&row)[RPL],
+                                              const float* __restrict__ qh, const float* __restrict__ ql,
+                                              uint64_t (&t)[RPL][NP], uint64_t (&l)[RPL][NP]) {
+  const uint64_t neg = pair2(-1.0f, -1.0f);
 #pragma unroll
-  for (int c = 0; c < CN; ++c) sh[c] = sl[c] = 0.0f;
-#pragma unroll 4
-  for (int k = 0; k < n; ++k) {
-    const float2 a = split_f64(Si[kCol ? (size_t)k * n : (size_t)k]);
-    const float2* qk = q + (size_t)k * bJ;
+  for (int r = 0; r < RPL; ++r)
 #pragma unroll
-    for (int c = 0; c < CN; ++c) {
-      const float2 v = qk[c];
-      const float pr = a.x * v.x;
-      sl[c] += fmaf(a.x, v.x, -pr);
-      two_sum(sh[c], sl[c], pr);
-      sl[c] = fmaf(a.x, v.y, fmaf(a.y, v.x, sl[c]));
+    for (int p = 0; p < NP; ++p) {
+      t[r][p] = pair2(kQBig, kQBig);
+      l[r][p] = 0;
     }
-  }
-  if (rv) {
+  constexpr int kU = 4;   // rows k per step: their loads run one step ahead of the arithmetic
+  double nx[kU][RPL];
 #pragma unroll
-    for (int c = 0; c < CN; ++c) w[c] = ((c == ce ? 1.0f : 0.0f) - sh[c]) - sl[c];
+  for (int u = 0; u < kU; ++u)
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) nx[u][r] = k0 + u < k1 ? __ldg(S + (size_t)(k0 + u) * n + row[r]) : 0.0;
+  for (int k = k0; k < k1; k += kU) {
+    double sv[kU][RPL];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        sv[u][r] = nx[u][r];
+        nx[u][r] = k + kU + u < k1 ? __ldg(S + (size_t)(k + kU + u) * n + row[r]) : 0.0;
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      uint64_t ax[RPL], ay[RPL];
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const float2 a = split_f64(sv[u][r]);
+        ax[r] = pair2(a.x, a.x);
+        ay[r] = pair2(a.y, a.y);
+      }
+      const int kk = min(k + u, k1 - 1);   // past k1 the entries of T_J(S) are zeros
+      const uint64_t* vh = reinterpret_cast<const uint64_t*>(qh + kk * 2 * NP);
+      const uint64_t* vl = reinterpret_cast<const uint64_t*>(ql + kk * 2 * NP);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const uint64_t x = vh[p], y = vl[p];
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+          const uint64_t tn = fma2(ax[r], x, t[r][p]);
+          const uint64_t nh = fma2(tn, neg, t[r][p]);   // t - t'
+          l[r][p] = add2(l[r][p], fma2(ax[r], x, nh));
+          l[r][p] = fma2(ax[r], y, l[r][p]);
+          l[r][p] = fma2(ay[r], x, l[r][p]);
+          t[r][p] = tn;
+        }
+      }
+    }
   }
 }
 
-// One row i of the correction X R (kCol false: xi is row i of X) or X^T R (kCol: xi is column i; X =
-// T_J(S)^-1 is symmetric up to its rounding, so its transpose serves as the approximate inverse as well) for
-// CN columns of R (FP32, rows of stride bJ): four interleaved FP32 partial sums along k per column, added at
-// the end; d[c] for c < CN.
-template <int CN, bool kCol>
-__device__ __forceinline__ void update_row(const float* __restrict__ xi, const float* __restrict__ R, int n, int bJ,
-                                           float (&d)[8]) {
-  float acc[4][CN];
+// This warp's share of (X^T R)_ic likewise (X = T_J(S)^-1 is symmetric up to its rounding, so its transpose serves as
+// the approximate inverse as well and is read coalesced), in FP32.
+template <int NP>
+__device__ __forceinline__ void update_part(const float* __restrict__ X, int n, int k0, int k1, const int (&row)[RPL],
+                                            const float* __restrict__ R, uint64_t (&d)[RPL][NP]) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int r = 0; r < RPL; ++r)
 #pragma unroll
-    for (int c = 0; c < CN; ++c) acc[u][c] = 0.0f;
-  int k = 0;
-  for (; k + 4 <= n; k += 4) {
+    for (int p = 0; p < NP; ++p) d[r][p] = 0;
+  constexpr int kU = 8;
+  float nx[kU][RPL];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float x = xi[kCol ? (size_t)(k + u) * n : (size_t)(k + u)];
-      const float* rk = R + (size_t)(k + u) * bJ;
+  for (int u = 0; u < kU; ++u)
 #pragma unroll
-      for (int c = 0; c < CN; ++c) acc[u][c] = fmaf(x, rk[c], acc[u][c]);
+    for (int r = 0; r < RPL; ++r) nx[u][r] = k0 + u < k1 ? __ldg(X + (size_t)(k0 + u) * n + row[r]) : 0.0f;
+  for (int k = k0; k < k1; k += kU) {
+    float xv[kU][RPL];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        xv[u][r] = nx[u][r];
+        nx[u][r] = k + kU + u < k1 ? __ldg(X + (size_t)(k + kU + u) * n + row[r]) : 0.0f;
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const uint64_t* rv = reinterpret_cast<const uint64_t*>(R + min(k + u, k1 - 1) * 2 * NP);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const uint64_t x = rv[p];
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) d[r][p] = fma2(pair2(xv[u][r], xv[u][r]), x, d[r][p]);
+      }
     }
   }
-  for (; k < n; ++k) {
-    const float x = xi[kCol ? (size_t)k * n : (size_t)k];
-    const float* rk = R + (size_t)k * bJ;
-#pragma unroll
-    for (int c = 0; c < CN; ++c) acc[0][c] = fmaf(x, rk[c], acc[0][c]);
-  }
-#pragma unroll
-  for (int c = 0; c < CN; ++c) d[c] = (acc[0][c] + acc[1][c]) + (acc[2][c] + acc[3][c]);
 }
+
+// One group of up to 2 NP centre columns: R = E - T_J(S) q, then q += X^T R. Chunks of 32 RPL rows; every warp takes
+// n / kQWarps of the products of all rows of a chunk, and the shares meet in shared memory (red). Shared: qh, ql, R
+// [n][qs], red [kQWarps][32 RPL][2 NP] twice.
+template <int NP>
+__device__ void refine_group(const double* __restrict__ S, const float* __restrict__ X, int n, int cn, int ce,
+                             double* __restrict__ q, int qstride, float* __restrict__ qh, float* __restrict__ ql,
+                             float* __restrict__ R, float* __restrict__ red, float& dmax, double& qmax, bool& finite) {
+  constexpr int kRows = 32 * RPL, kCols = 2 * NP, qs = kCols;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (n + kQWarps - 1) / kQWarps, k0 = min(n, per * warp), k1 = min(n, k0 + per);
+  float* red2 = red + kQWarps * kRows * kCols;
+  for (int e = tid; e < n * qs; e += kQThreads) {
+    const int i = e / qs, c = e - i * qs;
+    const float2 v = c < cn ? split_f64(q[(size_t)i * qstride + c]) : make_float2(0.0f, 0.0f);
+    qh[e] = v.x;
+    ql[e] = v.y;
+  }
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {   // 0: the residual, 1: the update
+    for (int i0 = 0; i0 < n; i0 += kRows) {
+      int row[RPL];
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) row[r] = min(n - 1, i0 + 32 * r + lane);
+      uint64_t t[RPL][NP], l[RPL][NP];
+      if (pass == 0) residual_part<NP>(S, n, k0, k1, row, qh, ql, t, l);
+      else update_part<NP>(X, n, k0, k1, row, R, t);
+#pragma unroll
+      for (int r = 0; r < RPL; ++r)
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const int at = (warp * kCols + 2 * p) * kRows + 32 * r + lane;
+          const float2 a = unpair2(t[r][p]);
+          red[at] = pass == 0 ? a.x - kQBig : a.x;
+          red[at + kRows] = pass == 0 ? a.y - kQBig : a.y;
+          if (pass == 0) {
+            const float2 b = unpair2(l[r][p]);
+            red2[at] = b.x;
+            red2[at + kRows] = b.y;
+          }
+        }
+      __syncthreads();
+      for (int e = tid; e < kRows * kCols; e += kQThreads) {
+        const int c = e / kRows, i = i0 + (e & (kRows - 1));
+        if (i >= n || c >= cn) continue;
+        if (pass == 0) {
+          // the shares of t are multiples of 2^-21 below 4: E minus their sum is exact near the solution
+          float hi = i == ce + c ? 1.0f : 0.0f, lo = 0.0f;
+#pragma unroll
+          for (int w = 0; w < kQWarps; ++w) {
+            const float h = red[w * kRows * kCols + e], z = hi - h;
+            lo += (hi - z) - h;                       // what the subtraction rounded off (nothing, normally)
+            hi = z;
+            lo -= red2[w * kRows * kCols + e];
+          }
+          R[(size_t)i * qs + c] = hi + lo;
+        } else {
+          float d = 0.0f;
+#pragma unroll
+          for (int w = 0; w < kQWarps; ++w) d += red[w * kRows * kCols + e];
+          const size_t at = (size_t)i * qstride + c;
+          const double qe = q[at] + (double)d;
+          q[at] = qe;
+          finite = finite && isfinite(d) && isfinite(qe);
+          dmax = fmaxf(dmax, fabsf(d));
+          qmax = fmax(qmax, fabs(qe));
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Columns of a group: at most eight (two rows a lane); fewer for large n, so that qh, ql and R (12
+// bytes a row and column) and the shares leave room for two CTAs on an SM.
+__host__ __device__ inline size_t qrefine_bytes(int n, int g) { return (size_t)12 * n * g + (size_t)4096 * g; }
+__host__ __device__ inline int qrefine_cols(int n) {
+  int g = 8;
+  while (g > 2 && qrefine_bytes(n, g) > 110 * 1024) g -= 2;
+  return g;
+}
+static_assert(2 * kQWarps * 64 * sizeof(float) == 4096, "shares of one column");
 
 // After the tensor-core inverse square root (Eqs. inv1-inv3), which leaves X = T_J(S)^-1 in FP32 (in g.L32,
 // accurate to about 1e-6 of its norm) and A_J in Acache: the centre columns of T_J(S)^-1 by iterative
-// refinement with X as the approximate inverse (for n above 256 its transpose, read coalesced: X is symmetric up
-// to its rounding), q <- q + X (E_c - T_J(S) q) from q = X[:, centre], the
-// residual in double-FP32 arithmetic (as in k_prepare_mixed), until the correction is below 1e-6 of q; then
+// refinement with X as the approximate inverse, q <- q + X^T (E_c - T_J(S) q) from q = X[:, centre], the
+// residual in double-FP32 arithmetic (residual_part), until the correction is below 1e-6 of q; then
 // the Gershgorin interval of A_J. A submatrix the inverse kernel flagged, or whose refinement does not
 // contract, is left flagged for the FP64 preparation.
-__global__ void __launch_bounds__(kThreads) k_ns_qrefine(PrepArgs g, const float* __restrict__ Acache) {
-  extern __shared__ __align__(16) float Wsh[];   // the residual, n x b
-  __shared__ float rlo[kThreads], rhi[kThreads];
-  __shared__ float red_d[kThreads / 32];
-  __shared__ double red_q[kThreads / 32];
+// Bound: T_J(S), X and A_J are read once each (0.47 MB at n = 172); the eight warps share every row's products, so
+// that a submatrix's chain is n / 8 products long instead of n.
+__global__ void __launch_bounds__(kQThreads, 2) k_ns_qrefine(PrepArgs g, const float* __restrict__ Acache) {
+  extern __shared__ __align__(16) float qsm[];
+  __shared__ float rlo[kQThreads], rhi[kQThreads];
+  __shared__ float red_d[kQWarps];
+  __shared__ double red_q[kQWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int J = g.order ? g.order[blockIdx.x] : g.j0 + (int)blockIdx.x;
   if (g.prep_status[J] != kSubOk) return;
   const int n = g.sub_n[J], bJ = g.nbf[J], c0 = g.sub_c0[J], nbc = n * bJ;
   const double* S = g.ws + (g.a_off[J] - g.a_base);
   const float* X = g.L32 + (g.a_off[J] - g.a_base);
-  float2* qp = g.Qp + (g.c_off[J] - g.c_base);
   double* q = g.Q + g.c_off[J];
-  for (int e = tid; e < nbc; e += kThreads) {
+  for (int e = tid; e < nbc; e += kQThreads) {
     const int i = e / bJ, c = e - i * bJ;
     q[e] = (double)X[(size_t)i * n + c0 + c];
   }
   if (g.cond) {   // cond(T_J(S)) >= max_i S_ii (T_J(S)^-1)_ii
     float mx = 0.0f;
-    for (int i = tid; i < n; i += kThreads) mx = fmaxf(mx, (float)S[(size_t)i * n + i] * X[(size_t)i * n + i]);
+    for (int i = tid; i < n; i += kQThreads) mx = fmaxf(mx, (float)S[(size_t)i * n + i] * X[(size_t)i * n + i]);
     rhi[tid] = mx;
     __syncthreads();
-    for (int s = kThreads / 2; s > 0; s >>= 1) {
+    for (int s = kQThreads / 2; s > 0; s >>= 1) {
       if (tid < s) rhi[tid] = fmaxf(rhi[tid], rhi[tid + s]);
       __syncthreads();
     }
@@ -1221,71 +1347,20 @@ __global__ void __launch_bounds__(kThreads) k_ns_qrefine(PrepArgs g, const float
   }
   __syncthreads();
   bool conv = false;
-  constexpr int kWarps = kThreads / 32;
-  // rows of T_J(S) and X read along the row by each lane up to 256 columns, as columns (coalesced) beyond
-  const bool col = n > 256;
+  const int gmax = qrefine_cols(n);
   for (int it = 0; it < kRefineMax && !conv; ++it) {
-    for (int e = tid; e < nbc; e += kThreads) qp[e] = split_f64(q[e]);
-    __syncthreads();
-    // R = E_c - T_J(S) q: one row per lane (for n above 256 read as the column of the symmetric T_J(S):
-    // coalesced), the row's products along k in double-FP32 arithmetic (as residual_df), up to 8 centre columns
-    // per sweep; every lane reads the same entries of q
-    for (int i0 = 32 * warp; i0 < n; i0 += 32 * kWarps) {
-      const int i = i0 + lane;
-      const bool rv = i < n;
-      const double* Si = col ? S + (rv ? i : 0) : S + (size_t)(rv ? i : 0) * n;   // row i (or column i)
-      for (int cg = 0; cg < bJ; cg += 8) {
-        float* w = Wsh + (size_t)(rv ? i : 0) * bJ + cg;
-        const float2* qc = qp + cg;
-        const int ce = i - c0 - cg;   // row i holds the 1 of E_c's column cg + c when c == ce
-        switch (min(8, bJ - cg)) {
-          case 1: col ? residual_row<1, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<1, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 2: col ? residual_row<2, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<2, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 3: col ? residual_row<3, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<3, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 4: col ? residual_row<4, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<4, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 5: col ? residual_row<5, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<5, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 6: col ? residual_row<6, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<6, false>(Si, qc, n, bJ, rv, ce, w); break;
-          case 7: col ? residual_row<7, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<7, false>(Si, qc, n, bJ, rv, ce, w); break;
-          default: col ? residual_row<8, true>(Si, qc, n, bJ, rv, ce, w) : residual_row<8, false>(Si, qc, n, bJ, rv, ce, w); break;
-        }
-      }
-    }
-    __syncthreads();
-    // q <- q + X R (for n above 256 X^T R, one column of X per lane: coalesced), R from shared memory (the
-    // same entries for every lane)
     float dmax = 0.0f;
     double qmax = 0.0;
     bool finite = true;
-    for (int i0 = 32 * warp; i0 < n; i0 += 32 * kWarps) {
-      const int i = i0 + lane;
-      const bool rv = i < n;
-      const float* xi = col ? X + (rv ? i : 0) : X + (size_t)(rv ? i : 0) * n;
-      for (int cg = 0; cg < bJ; cg += 8) {
-        const int cn = min(8, bJ - cg);
-        float d[8];
-        switch (cn) {
-          case 1: col ? update_row<1, true>(xi, Wsh + cg, n, bJ, d) : update_row<1, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 2: col ? update_row<2, true>(xi, Wsh + cg, n, bJ, d) : update_row<2, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 3: col ? update_row<3, true>(xi, Wsh + cg, n, bJ, d) : update_row<3, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 4: col ? update_row<4, true>(xi, Wsh + cg, n, bJ, d) : update_row<4, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 5: col ? update_row<5, true>(xi, Wsh + cg, n, bJ, d) : update_row<5, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 6: col ? update_row<6, true>(xi, Wsh + cg, n, bJ, d) : update_row<6, false>(xi, Wsh + cg, n, bJ, d); break;
-          case 7: col ? update_row<7, true>(xi, Wsh + cg, n, bJ, d) : update_row<7, false>(xi, Wsh + cg, n, bJ, d); break;
-          default: col ? update_row<8, true>(xi, Wsh + cg, n, bJ, d) : update_row<8, false>(xi, Wsh + cg, n, bJ, d); break;
-        }
-        if (rv) {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            if (c < cn) {
-              const size_t e = (size_t)i * bJ + cg + c;
-              const double qe = q[e] + (double)d[c];
-              q[e] = qe;
-              finite = finite && isfinite(d[c]) && isfinite(qe);
-              dmax = fmaxf(dmax, fabsf(d[c]));
-              qmax = fmax(qmax, fabs(qe));
-            }
-          }
-        }
+    for (int cg = 0; cg < bJ; cg += gmax) {
+      const int cn = min(gmax, bJ - cg), ce = c0 + cg;   // row i holds the 1 of E_c's column c when i == ce + c
+      const int qs = (cn + 1) & ~1;
+      float *qh = qsm, *ql = qh + n * qs, *R = ql + n * qs, *red = R + n * qs;
+      switch (qs) {
+        case 2: refine_group<1>(S, X, n, cn, ce, q + cg, bJ, qh, ql, R, red, dmax, qmax, finite); break;
+        case 4: refine_group<2>(S, X, n, cn, ce, q + cg, bJ, qh, ql, R, red, dmax, qmax, finite); break;
+        case 6: refine_group<3>(S, X, n, cn, ce, q + cg, bJ, qh, ql, R, red, dmax, qmax, finite); break;
+        default: refine_group<4>(S, X, n, cn, ce, q + cg, bJ, qh, ql, R, red, dmax, qmax, finite); break;
       }
     }
     if (!finite) dmax = INFINITY;
@@ -1300,7 +1375,7 @@ __global__ void __launch_bounds__(kThreads) k_ns_qrefine(PrepArgs g, const float
     __syncthreads();
     float dm = 0.0f;
     double qm = 0.0;
-    for (int w2 = 0; w2 < kWarps; ++w2) {
+    for (int w2 = 0; w2 < kQWarps; ++w2) {
       dm = fmaxf(dm, red_d[w2]);
       qm = fmax(qm, red_q[w2]);
     }
@@ -1310,7 +1385,7 @@ __global__ void __launch_bounds__(kThreads) k_ns_qrefine(PrepArgs g, const float
     conv = (double)dm <= kRefineTol * qm || (it == 0 && (double)dm <= kNsOneStep * qm);
     __syncthreads();
   }
-  if (conv) gershgorin(Acache + g.a_off[J], n, g.lam + 2 * J, rlo, rhi);
+  if (conv) gershgorin<float, kQThreads>(Acache + g.a_off[J], n, g.lam + 2 * J, rlo, rhi);
   if (tid == 0) g.prep_status[J] = conv ? kSubOk : (n <= g.fallback_max_n ? kSubRefine : kSubNotSpd);
 }
 
@@ -1365,7 +1440,7 @@ size_t smem_fp64(int max_n) { return sizeof(double) * (size_t)std::max(max_n, 2 
 size_t smem_mixed(int max_n) {
   return sizeof(float) * std::max((size_t)(std::max(max_n, 2 * NB) + 36) * Ld<float>::v, (size_t)kRtSmem);
 }
-constexpr size_t kSmemLimit = 200 * 1024;
+constexpr size_t kSmemLimit = 200 * 1024, kSmemLimitQ = 222 * 1024;
 
 }  // namespace
 
@@ -1405,13 +1480,17 @@ nolsm_status launch_sym_finish(const SymArgs& g, int count, int max_n, int max_b
 }
 
 nolsm_status launch_ns_qrefine(const PrepArgs& g, int count, int max_n, int max_b, float* Acache, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (size_t)max_n * max_b;
-  if (smem > kSmemLimit) {
+  size_t smem = 0;   // the largest need of any dimension up to max_n: the group narrows as n grows
+  for (int n = max_n, g = qrefine_cols(n); g <= 8; g += 2) {
+    while (n > 1 && qrefine_cols(n) < g) --n;
+    smem = std::max(smem, qrefine_bytes(n, std::min(g, (max_b + 1) & ~1)));
+  }
+  if (smem > kSmemLimitQ) {
     set_error("submatrix dimension %d x %d centre columns exceed the refinement's shared memory", max_n, max_b);
     return NOLSM_ERR_UNSUPPORTED;
   }
   NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_ns_qrefine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_ns_qrefine<<<count, kThreads, smem, st>>>(g, Acache);
+  k_ns_qrefine<<<count, kQThreads, smem, st>>>(g, Acache);
   NOLSM_LAUNCH_CHECK();
   PrepArgs f = g;
   f.only_flagged = 1;
