@@ -47,7 +47,9 @@
 
 #include "nolsm_internal.cuh"
 #include "prep.cuh"
+#include "res_path.cuh"
 #include "tc_path.cuh"
+#include "tc_split.cuh"
 #include "tcgen05.cuh"
 #include "tmap.cuh"
 
@@ -90,13 +92,6 @@ static_assert(128 * kRegsLow + Shape<1>::kEpiThreads * kRegsEpi <= Shape<1>::kTh
 constexpr int kPlanes = 6;
 constexpr uint64_t kWaitNs = 2000000000ull;        // default limit per wait (2 s); one product takes < 1 ms
 
-enum : int { FMT_F16 = 0, FMT_BF16 = 1, FMT_E4M3 = 2 };
-
-struct Fmt {
-  int fmt;    // FMT_F16 / FMT_BF16 / FMT_E4M3
-  int terms;  // 1 or 3 (E4M3: 1)
-};
-
 // E4M3 operands carry a fixed power-of-two scale: the symmetric iterates have |x_ij| <= rho <= 1.7 (the
 // scale guard), so x * 2^7 stays below 218 of E4M3's 448 and values down to 2^-16 keep a subnormal; a
 // product of two scaled operands is scaled back by 2^-14.
@@ -130,6 +125,7 @@ struct TcArgs {
   const float* cond;          // preparation's cond(T_J(S)) estimate (nullable): above cond_max the submatrix
   float cond_max;             // is left to the FP64 path (its status stays as it is) when it has at most
   int32_t ill_max_n;          // ill_max_n rows (what the FP64 preparation takes)
+  int32_t above_n;            // sign mode: submatrices of at most this many rows are passed over (k_ns_res takes them)
   // inverse-square-root mode: the chunk's gathered T_J(S), T_J(H0) (FP64, at a_off[J] - a_base and
   // chunk_n2 further), the outputs and the iteration's stopping rule
   const double* ws;
@@ -194,36 +190,6 @@ struct Shared {
   float red[2][kMaxEpiWarps];    // defect partial sums, by product parity
   double dred[3][kMaxEpiWarps];
 };
-
-__device__ __forceinline__ float from_bits(uint16_t b, int fmt) {
-  if (fmt == FMT_BF16) return __bfloat162float(__ushort_as_bfloat16(b));
-  return __half2float(__ushort_as_half(b));
-}
-
-// Two values rounded to the 2-byte format (packed) and their low parts x - round(x) rounded likewise.
-__device__ __forceinline__ void split2(float a, float b, int fmt, uint32_t& hi, uint32_t& lo) {
-  if (fmt == FMT_BF16) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    lo = *reinterpret_cast<const uint32_t*>(&l);
-  } else {
-    const __half2 h = __floats2half2_rn(a, b);
-    const float2 hf = __half22float2(h);
-    const __half2 l = __floats2half2_rn(a - hf.x, b - hf.y);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    lo = *reinterpret_cast<const uint32_t*>(&l);
-  }
-}
-
-// s + c <- s + c + p with s = fl(s + p) and the rounding error of that sum added to c (Knuth's TwoSum).
-__device__ __forceinline__ void two_sum(float& s, float& c, float p) {
-  const float t = s + p;
-  const float z = t - s;
-  c += (s - (t - z)) + (p - z);
-  s = t;
-}
 
 // 32 consecutive values of one row as packed hi (and lo) pairs; the format a template parameter (one
 // branch per chunk, none per pair), the lo parts only when the format has them.
@@ -692,6 +658,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           start_inverse(s, J);
           break;
         }
+        if (g.sub_n[J] <= g.above_n) continue;
         if (g.cond && g.prep_status[J] == kSubOk && g.cond[J] > g.cond_max && g.sub_n[J] <= g.ill_max_n) continue;
         if (g.prep_status[J] != kSubOk) {
           if (tid == 128) {
@@ -939,7 +906,8 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
                     q4[j & 3] = fmaf(p, p, q4[j & 3]);
                     v[j] = -p;                                   // (3I - P)_ij
                   }
-                  part += (q4[0] + q4[1]) + (q4[2] + q4[3]);
+                  // lanes without a row hold whatever the tensor memory held before (0 times a NaN is one)
+                  if (rin) part += (q4[0] + q4[1]) + (q4[2] + q4[3]);
                 } else {
 #pragma unroll
                   for (int j = 0; j < 32; ++j) {
@@ -1383,6 +1351,12 @@ static nolsm_status run_buckets(int mode, int precision, bool fixed0, const TcMa
   return launch_shape(mode, s0, m, g, sms, st);
 }
 
+// Sign bucket 0 (n <= 192) has no shape to choose any more: the query reports 0 once it has run.
+static void resident_shape(int precision) {
+  std::lock_guard<std::mutex> lk(g_shape_mu);
+  g_shape[0][precision & 7][0] = 0;
+}
+
 int tc_shape_choice(int mode, int precision, int bucket) {
   if (mode < 0 || mode > 1 || bucket < 0 || bucket > 1) return -1;
   std::lock_guard<std::mutex> lk(g_shape_mu);
@@ -1405,15 +1379,23 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   int dev = 0, sms = 0;
   NOLSM_CUDA_TRY(cudaGetDevice(&dev));
   NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int32_t maxn = 0;
-  for (int64_t J = j0; J < j1; ++J) maxn = std::max(maxn, plan->h_sub_n[J]);
+  int32_t maxn = 0, minn = INT32_MAX;
+  for (int64_t J = j0; J < j1; ++J) {
+    maxn = std::max(maxn, plan->h_sub_n[J]);
+    minn = std::min(minn, plan->h_sub_n[J]);
+  }
   const int LD = (maxn + 63) & ~63, R = (maxn + 127) & ~127;
-  // one CTA per SM at most, each with kSlots submatrices in flight (one scratch sub-slot each)
   const int64_t work = spec.list ? spec.count : j1 - j0;
   if (work <= 0) return NOLSM_OK;
+  // submatrices of up to kResMaxN rows run with their operands on the SM (res_path.cu), the others, and E4M3, with
+  // operands in scratch
+  const bool f8 = mf.fmt == FMT_E4M3;
+  const int32_t above = f8 ? 0 : kResMaxN;
+  const bool streamed = maxn > above, resident = !f8 && minn <= kResMaxN;
+  // one CTA per SM at most, each with kSlots submatrices in flight (one scratch sub-slot each)
   const int ctas = (int)std::min<int64_t>(sms, (work + kSlots - 1) / kSlots);
   const int slots = ctas * kSlots;
-  if (!S->planes.p || S->R < R || S->LD < LD || S->slots < slots) {
+  if (streamed && (!S->planes.p || S->R < R || S->LD < LD || S->slots < slots)) {
     const int nR = std::max(R, S->R), nLD = std::max(LD, S->LD), nS = std::max(slots, S->slots);
     dev_free(plan, S->planes);
     NOLSM_TRY(dev_alloc(plan, S->planes, sizeof(uint16_t) * (size_t)kPlanes * nS * nR * nLD));
@@ -1436,20 +1418,6 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     S->ord_j1 = j1;
     S->ord_large = 0;
     while (S->ord_large < (int32_t)ord.size() && plan->h_sub_n[ord[(size_t)S->ord_large]] > 192) ++S->ord_large;
-  }
-  CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
-  if (!tmap::make_3d(&mS16, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
-                     CU_TENSOR_MAP_SWIZZLE_64B) ||
-      !tmap::make_3d(&mS16x2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
-                     CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mS2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
-                     CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mA, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 128) ||
-      !tmap::make_3d(&mB, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 64) ||
-      !tmap::make_3d(&mS, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
-                     CU_TENSOR_MAP_SWIZZLE_64B)) {
-    set_error("cuTensorMapEncodeTiled rejected the scratch layout (R %d, LD %d, slots %d)", S->R, S->LD, S->slots);
-    return NOLSM_ERR_CUDA;
   }
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(S->err.p, 0, sizeof(int32_t), st));
@@ -1488,15 +1456,7 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   g.cond = sym ? nullptr : prepared(plan, prep_class(o)).cond.as<float>();
   g.cond_max = cond_max(o.precision);
   g.ill_max_n = prepare_fp64_max_n();
-  // one-byte views of the same planes (rows of 2 LD bytes) for E4M3 operands, both loaded K-major (E4M3 runs
-  // in shape 0, whose B box is 256 rows)
-  TcMaps m{mA, mB, mS, {}, {}, mS16, mS2, mS16x2};
-  if (!tmap::make_3d(&m.mA8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128, 128) ||
-      !tmap::make_3d(&m.mB8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128,
-                     Shape<0>::kTileN)) {
-    set_error("cuTensorMapEncodeTiled rejected the one-byte scratch layout");
-    return NOLSM_ERR_CUDA;
-  }
+  g.above_n = above;
   // every submatrix of a launch starts as "timed out" (k_status_pending), the kernel overwrites what it takes
   int32_t* status = plan->status.as<int32_t>();
   auto pending = [&](const int32_t* list, int32_t count) -> nolsm_status {
@@ -1505,13 +1465,58 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     NOLSM_LAUNCH_CHECK();
     return NOLSM_OK;
   };
-  const bool f8 = mf.fmt == FMT_E4M3;
-  if (spec.list) {   // reruns: one launch in list order, shape 0
-    NOLSM_TRY(pending(spec.list, spec.count));
-    NOLSM_TRY(launch_shape(0, 0, m, g, sms, st));
-  } else {           // the largest-first order in its two buckets: n above 192, the rest
-    NOLSM_TRY(run_buckets(0, o.precision, f8, m, g, S->order.as<int32_t>(), S->ord_large, (int32_t)(j1 - j0), sms, st,
-                          pending));
+  const int32_t* order = spec.list ? spec.list : S->order.as<int32_t>();
+  NOLSM_TRY(pending(order, (int32_t)work));
+  if (streamed) {
+    CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
+    if (!tmap::make_3d(&mS16, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
+                       CU_TENSOR_MAP_SWIZZLE_64B) ||
+        !tmap::make_3d(&mS16x2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
+                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
+        !tmap::make_3d(&mS2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
+                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
+        !tmap::make_3d(&mA, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 128) ||
+        !tmap::make_3d(&mB, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 64) ||
+        !tmap::make_3d(&mS, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
+                       CU_TENSOR_MAP_SWIZZLE_64B)) {
+      set_error("cuTensorMapEncodeTiled rejected the scratch layout (R %d, LD %d, slots %d)", S->R, S->LD, S->slots);
+      return NOLSM_ERR_CUDA;
+    }
+    // one-byte views of the same planes (rows of 2 LD bytes) for E4M3 operands, both loaded K-major (E4M3 runs
+    // in shape 0, whose B box is 256 rows)
+    TcMaps m{mA, mB, mS, {}, {}, mS16, mS2, mS16x2};
+    if (!tmap::make_3d(&m.mA8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128, 128) ||
+        !tmap::make_3d(&m.mB8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128,
+                       Shape<0>::kTileN)) {
+      set_error("cuTensorMapEncodeTiled rejected the one-byte scratch layout");
+      return NOLSM_ERR_CUDA;
+    }
+    if (spec.list) {   // reruns and a bisection's later points: one launch in list order, shape 0
+      NOLSM_TRY(launch_shape(0, 0, m, g, sms, st));
+    } else {           // the largest-first order in its two buckets: n above 192, the rest (E4M3 only)
+      NOLSM_TRY(run_buckets(0, o.precision, f8, m, g, S->order.as<int32_t>(), S->ord_large,
+                            f8 ? (int32_t)work : S->ord_large, sms, st, pending));
+    }
+  }
+  if (resident) {
+    ResSolve r{};
+    r.order = spec.list ? spec.list : S->order.as<int32_t>() + S->ord_large;
+    r.count = spec.list ? spec.count : (int32_t)work - S->ord_large;
+    r.sub_n = g.sub_n; r.nbf = g.nbf; r.a_off = g.a_off; r.c_off = g.c_off;
+    r.A = g.A; r.Q = g.Q; r.Sc = g.Sc; r.Hc = g.Hc; r.lam = g.lam; r.lam_g = g.lam_g;
+    r.prep_status = g.prep_status;
+    r.mu = mu;
+    r.tol_ns = g.tol_ns; r.tol_accept = g.tol_accept;
+    r.max_iter = g.max_iter; r.refine_steps = g.refine_steps; r.budget = g.budget;
+    r.main_fmt = mf; r.refine_fmt = rf;
+    r.next = plan->counter.as<int32_t>() + 1; r.err = g.err;
+    r.Dc = g.Dc; r.tS = g.tS; r.tH = g.tH; r.iters = g.iters; r.status = g.status; r.rsteps = g.rsteps;
+    r.nbelow = g.nbelow;
+    r.wait_ns = g.wait_ns;
+    r.cond = g.cond; r.cond_max = g.cond_max; r.ill_max_n = g.ill_max_n;
+    NOLSM_TRY(launch_ns_res(r, sms, st));
+    resident_shape(o.precision);
+    plan->stats.launches += 1;
   }
   plan->stats.launches += 2;
   if (sym) {   // D_c = L^-T U and the traces
