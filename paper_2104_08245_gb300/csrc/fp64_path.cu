@@ -457,7 +457,8 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
   const int32_t n_mol = plan->n_mol;
   const size_t esz = keep_fp64_A ? sizeof(double) : sizeof(float);
   if (!P.A.p) {
-    NOLSM_TRY(dev_alloc(plan, P.A, esz * (size_t)std::max<int64_t>(plan->h_a_off[n_mol], 1)));
+    // 16 bytes more: bulk copies of A_J end on a 16-byte boundary
+    NOLSM_TRY(dev_alloc(plan, P.A, esz * (size_t)std::max<int64_t>(plan->h_a_off[n_mol], 1) + 16));
     P.done.assign(n_mol, 0);
     P.fp64 = keep_fp64_A;
   }

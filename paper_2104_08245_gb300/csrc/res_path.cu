@@ -42,15 +42,17 @@ constexpr int kQs = kResMaxN * 8;                 // staged columns of Q, FP32 [
 constexpr int kSplit = 4;                         // shares of the k range in X Q
 constexpr uint32_t kExtra = 4 * kQs + 8 * kSplit * kResMaxN * 8;   // Q, then the sums (hi, lo) of every share
 constexpr uint32_t kSmemR = kXBytes + kExtra + 1024;
+constexpr uint32_t kSmemI = kXBytes + 32 * 1024 + 2 * (16 * kResMaxN * 8 + 128) + 1024;   // inverse: FP32 staging of eight warps, the feed
 static_assert(kExtra >= 64 * 128, "the second row tile's A reads up to 64 rows past the last block");
-static_assert(kSmemR <= 227 * 1024, "shared memory");
+static_assert(kSmemR <= 227 * 1024 && kSmemI <= 227 * 1024 - 512, "shared memory");
+static_assert(kExtra >= 2 * (16 * kResMaxN * 8 + 128), "the feed's buffers share it");
 constexpr uint32_t kRing = 2 * kResMaxN;          // tensor memory column of the first Z accumulator
 constexpr uint64_t kWaitNsR = 2000000000ull;
 
 struct StepInfo { int term, n16, nrb, nch; Fmt f; };   // what the MMA warp needs of a step
 
 struct SharedR {
-  uint64_t xr, pf[2], tr[2], zf[2], ze[2], idle;
+  uint64_t xr, pf[2], tr[2], zf[2], ze[2], ld[2], idle;
   uint32_t tmem;
   int err, fetch;
   StepInfo mm;
@@ -105,6 +107,94 @@ __device__ __forceinline__ void product(uint32_t dt, uint32_t x0, int row0, uint
       }
     }
   }
+}
+
+// An n x n matrix (row-major, contiguous) from global into the operand in shared memory, by way of two staging buffers
+// that bulk copies fill: the shared memory of these kernels leaves the L1 some 20 KB, so that loads which count on
+// finding their lines there again fetch them several times over (45,000 cycles for the FP64 matrix at n = 172).
+// A row a warp, two adjacent columns a lane in up to three blocks of 64: every access to shared memory is free of bank
+// conflicts (with a 16-byte unit a lane the FP64 loads took 64 wavefronts a row, and 32,768 submatrices 12.2 ms in
+// k_inv_res instead of 9.8).
+// see(x, y, i, j): the entries (i, j) and (i, j + 1) in FP32, to be changed in place; zeros past the last column.
+constexpr uint32_t kFeed = 16 * kResMaxN * 8 + 128;   // a staging buffer: 16 rows in FP64, and what the widening adds
+__device__ __forceinline__ float narrow(float x, uint32_t&) { return x; }
+// x in FP32, halves away from zero, by integer operations (the conversion instruction runs on the FP64 pipe); below
+// 2^-126 a zero. big: the largest leading word, which tells whether an entry was out of FP32's range or not finite.
+__device__ __forceinline__ float narrow(double x, uint32_t& big) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), a = hi & 0x7FFFFFFFu;
+  big = max(big, a);
+  const uint32_t b = __funnelshift_l(lo, a, 3) + ((lo >> 28) & 1u) - (896u << 23);
+  return __uint_as_float(a < (897u << 20) ? 0u : (b | (hi & 0x80000000u)));
+}
+template <typename T, typename See>
+__device__ __forceinline__ uint32_t feed(uint8_t* X, const T* __restrict__ M, int n, int n64, Fmt f, uint8_t* stage,
+                                         uint64_t (&ld)[2], uint32_t& nld, uint64_t wait_ns, bool& bad, int etid, See&& see) {
+  const int ew = etid >> 5, lane = etid & 31;
+  const int R = (int)((kFeed - 128) / (n * sizeof(T))) & ~7, nc = (n + R - 1) / R;   // rows a buffer, the same for every warp
+  const bool even = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(M) & (2 * sizeof(T) - 1)) == 0;
+  uint32_t big = 0;
+  auto issue = [&](int c) {   // one thread: rows [c R, ...) widened to whole 16-byte units
+    const uintptr_t a = reinterpret_cast<uintptr_t>(M + (size_t)c * R * n), e = a + sizeof(T) * (size_t)min(R, n - c * R) * n;
+    const uint32_t bytes = (uint32_t)(((e + 15) & ~uintptr_t(15)) - (a & ~uintptr_t(15)));
+    uint64_t* bar = &ld[(nld + c) & 1];
+    tc::mbar_arrive_expect_tx(bar, bytes);
+    tc::bulk_load(stage + ((nld + c) & 1) * kFeed, reinterpret_cast<const void*>(a & ~uintptr_t(15)), bytes, bar);
+  };
+  if (etid == 0) {
+    issue(0);
+    if (nc > 1) issue(1);
+  }
+  const uint32_t unit = (lane >> 2) & 7, part = 4 * (lane & 3);
+  auto put = [&](int t, int i, uint32_t h, uint32_t l) {
+    uint8_t* at = X + t * kBlk + i * 128 + ((unit ^ (i & 7)) << 4) + part;
+    *reinterpret_cast<uint32_t*>(at) = h;
+    if (f.terms > 1) *reinterpret_cast<uint32_t*>(at + kPlane) = l;
+  };
+  for (int i = n + ew; i < n64; i += 8) {   // the rows of zeros
+    for (int t = 0; 64 * t < n64; ++t) put(t, i, 0, 0);
+  }
+#pragma unroll 1
+  for (int c = 0; c < nc; ++c) {
+    const uint32_t b = (nld + c) & 1;
+    if (!bad) bad = !tc::mbar_wait(&ld[b], ((nld + c) >> 1) & 1, tc::globaltimer() + wait_ns);
+    if (bad && etid == 0) tc::mbar_wait(&ld[b], ((nld + c) >> 1) & 1, tc::globaltimer() + 50000000ull);   // none left in flight
+    const T* rows = reinterpret_cast<const T*>(stage + b * kFeed + (reinterpret_cast<uintptr_t>(M + (size_t)c * R * n) & 15));
+    const int count = min(R, n - c * R);
+#pragma unroll 1
+    for (int r = ew; r < count; r += 8) {
+      const int i = c * R + r;
+      T x[3], y[3];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {   // past the row's end the last column again
+        const int j = 64 * t + 2 * lane;
+        if (even) {
+          struct alignas(2 * sizeof(T)) Pair { T x, y; };
+          const Pair v = *reinterpret_cast<const Pair*>(rows + r * n + min(j, n - 2));
+          x[t] = v.x;
+          y[t] = v.y;
+        } else {
+          x[t] = rows[r * n + min(j, n - 1)];
+          y[t] = rows[r * n + min(j + 1, n - 1)];
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int j = 64 * t + 2 * lane;
+        if (t > 0 && 64 * t >= n64) break;
+        float xf = narrow(x[t], big), yf = narrow(y[t], big);
+        if (j >= n) xf = 0.0f;
+        if (j + 1 >= n) yf = 0.0f;
+        see(xf, yf, i, j);
+        uint32_t h, l;
+        split2(xf, yf, f.fmt, h, l);
+        put(t, i, h, l);
+      }
+    }
+    bar_epi();   // the buffer has been read
+    if (etid == 0 && c + 2 < nc) issue(c + 2);
+  }
+  nld += nc;
+  return big;
 }
 
 // This lane's row of X (hi, with kLo lo) times eight columns of Q over k0 <= k < k1 (multiples of 16): FP32 sums of 16
@@ -164,7 +254,12 @@ __device__ __forceinline__ void xq_part(const uint8_t* __restrict__ X, int i, in
   }
 }
 
+// kFmt, kTerms: the main phase's operand format (the refinement's is FP16 in three terms). A template of it, and one site
+// each of T and of the Z blocks, because the epilogue's code has to stay in the instruction cache: with all four formats
+// at every site the code is 84 KB, against 62-74 KB.
+template <int kFmt, int kTerms>
 __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
+  constexpr bool kOne = kFmt == FMT_F16 && kTerms == 3;   // the main format is the refinement's
   extern __shared__ uint8_t smraw[];
   uint8_t* const X = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   float* const Qs = reinterpret_cast<float*>(X + kXBytes);
@@ -178,6 +273,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       tc::mbar_init(&sh.tr[t], kEpiR);
       tc::mbar_init(&sh.zf[t], 1);
       tc::mbar_init(&sh.ze[t], kEpiR);
+      tc::mbar_init(&sh.ld[t], 1);
     }
     tc::mbar_init(&sh.idle, 1);
     tc::fence_mbar_init();
@@ -242,8 +338,11 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
     // ------------------------------------------------ epilogue
     const int etid = tid - 128, ew = warp - 4, q = warp & 3, grp = ew >> 2;
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+    uint32_t nld = 0;
+    bool bad = false;
     for (;;) {
-      // ---- the next submatrix of at most kResMaxN rows
+      // ---- the next submatrix of at most kResMaxN rows (the last one's finish has used the feed's buffers)
+      tc::fence_proxy_async_smem();
       int J = -1;
       for (;;) {
         if (etid == 0) {
@@ -276,48 +375,18 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       {
         const float* __restrict__ A = g.A + g.a_off[J];
         const float inv = (float)(1.0 / scale_alpha(g.lam, g.lam_g, J, g.mu)), fmu = (float)g.mu;
-        const Fmt f = g.main_fmt;
-        // eight rows a warp pass; sixteen lanes along a row, four adjacent columns a lane, in three blocks of 64 columns:
-        // 48 loads in flight (no condition holds a load back), then 8-byte stores of hi and lo
-        for (int i0 = 8 * ew; i0 < n64; i0 += 64) {
-          float v[4][3][4];
-          const int jl = 4 * (lane & 15);
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const float* row = A + min(i0 + 2 * r + (lane >> 4), n - 1) * n;
-#pragma unroll
-            for (int t = 0; t < 3; ++t)
-#pragma unroll
-              for (int u = 0; u < 4; ++u) v[r][t][u] = __ldg(row + min(64 * t + jl + u, n - 1));
-          }
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const int i = i0 + 2 * r + (lane >> 4);
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-              float w[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int j = 64 * t + jl + u;
-                w[u] = i < n && j < n ? (v[r][t][u] - (i == j ? fmu : 0.0f)) * inv : 0.0f;
-              }
-              uint2 h, l;
-              split2(w[0], w[1], f.fmt, h.x, l.x);
-              split2(w[2], w[3], f.fmt, h.y, l.y);
-              uint8_t* at = X + unit_at(t, i, (lane & 15) >> 1) + 8 * (lane & 1);
-              if (64 * t < n64) {
-                *reinterpret_cast<uint2*>(at) = h;
-                if (f.terms > 1) *reinterpret_cast<uint2*>(at + kPlane) = l;
-              }
-            }
-          }
-        }
+        const Fmt f{kFmt, kTerms};
+        feed(X, A, n, n64, f, reinterpret_cast<uint8_t*>(Qs), sh.ld, nld, g.wait_ns, bad, etid,
+             [&](float& x, float& y, int i, int j) {
+               x = (i == j && i < n ? x - fmu : x) * inv;
+               y = (i == j + 1 && i < n ? y - fmu : y) * inv;
+             });
       }
       int phase = 0, refine_left = g.refine_steps, steps = 0, rsteps = 0, status = kSubNotConv;
       float dprev = INFINITY;
-      Fmt fcur = g.main_fmt;
-      bool last = false, bad = false;
-      if (etid == 0) sh.mm = StepInfo{0, n16, nrb, nch, fcur};
+      bool ref = kOne;   // X is in the refinement's format
+      bool last = false;
+      if (etid == 0) sh.mm = StepInfo{0, n16, nrb, nch, Fmt{kFmt, kTerms}};
       tc::fence_proxy_async_smem();
       tc::tc_fence_before();
       bar_epi();
@@ -354,14 +423,15 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
                 for (int u = 0; u < 32; ++u) r[u] = pick(u, lane, __float_as_uint(__uint_as_float(r[u]) - one), r[u]);
               }
               float sq = 0.0f;
-              scale_split<true>(r, -1.0f, fcur, h, l, sq);
+              if (!kOne && !ref) scale_split_t<kFmt, (kTerms > 1), true>(r, -1.0f, h, l, sq);
+              else scale_split_t<FMT_F16, true, true>(r, -1.0f, h, l, sq);
               if (row < n) part += sq;
               if (diag) {
                 uint32_t e = 0;
 #pragma unroll
                 for (int u = 0; u < 32; ++u) e = pick(u, lane, r[u], e);
                 uint32_t th, tl;
-                split2(row < n ? 2.0f - __uint_as_float(e) : 0.0f, 0.0f, fcur.fmt, th, tl);
+                split2(row < n ? 2.0f - __uint_as_float(e) : 0.0f, 0.0f, ref ? FMT_F16 : kFmt, th, tl);
                 const uint32_t sel = lane & 1 ? 0x5410u : 0x3254u;   // (low of x, low of t) or (low of t, high of x)
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
@@ -395,7 +465,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
         const float dd = sqrtf(dsum / (float)n);
         steps += 1;
         if (phase == 1) rsteps += 1;   // this step runs in the refinement format
-        Fmt fnxt = fcur;
+        bool rnxt = ref;
         status = kSubNotConv;
         if (!isfinite(dd)) {
           last = true;
@@ -408,7 +478,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
             } else {
               phase = 1;
               refine_left = g.refine_steps;
-              fnxt = g.refine_fmt;
+              rnxt = true;
             }
           }
         } else if (--refine_left <= 0) {
@@ -460,7 +530,10 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
             if (!bad) tc::mbar_arrive(&sh.ze[slot]);
             // rows and columns from n to n16 are zeros of themselves; columns past n16 hold anything and are not read
             float sq = 0.0f;
-            if (mine) scale_split<false>(r, 0.5f, fnxt, h, l, sq);
+            if (mine) {
+              if (!kOne && !rnxt) scale_split_t<kFmt, (kTerms > 1), false>(r, 0.5f, h, l, sq);
+              else scale_split_t<FMT_F16, true, false>(r, 0.5f, h, l, sq);
+            }
           };
           auto put = [&](int t, const uint32_t (&h)[16], const uint32_t (&l)[16]) {
             const int rbase = 128 * t + 32 * q, row = rbase + lane;
@@ -469,7 +542,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
             for (int u = 0; u < 4; ++u) {
               uint8_t* at = X + unit_at(c, row, 4 * grp + u);
               *reinterpret_cast<uint4*>(at) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
-              if (fnxt.terms > 1)
+              if (kTerms > 1 || rnxt)
                 *reinterpret_cast<uint4*>(at + kPlane) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
             }
           };
@@ -487,9 +560,9 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
           bad = true;
           break;
         }
-        fcur = fnxt;
+        ref = rnxt;
         if (!last) {
-          if (etid == 0) sh.mm.f = fcur;
+          if (etid == 0) sh.mm.f = ref ? Fmt{FMT_F16, 3} : Fmt{kFmt, kTerms};
           tc::fence_proxy_async_smem();
           bar_epi();
           tc::mbar_arrive(&sh.xr);
@@ -529,13 +602,8 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
           const int i = 32 * (it / kSplit) + lane, kq = it % kSplit;
           const int k0 = 16 * (units * kq / kSplit), k1 = 16 * (units * (kq + 1) / kSplit);
           uint64_t s[4], e[4];
-          if (fcur.fmt == FMT_BF16) {
-            if (fcur.terms > 1) xq_part<FMT_BF16, true>(X, i, k0, k1, Qs, s, e);
-            else xq_part<FMT_BF16, false>(X, i, k0, k1, Qs, s, e);
-          } else {
-            if (fcur.terms > 1) xq_part<FMT_F16, true>(X, i, k0, k1, Qs, s, e);
-            else xq_part<FMT_F16, false>(X, i, k0, k1, Qs, s, e);
-          }
+          if (!kOne && !ref) xq_part<kFmt, (kTerms > 1)>(X, i, k0, k1, Qs, s, e);
+          else xq_part<FMT_F16, true>(X, i, k0, k1, Qs, s, e);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const float2 a = unpair2(s[c]), d = unpair2(e[c]);
@@ -564,8 +632,8 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       double px = 0.0;   // the trace of the final X: (n - Tr X) / 2 eigenvalues lie below mu
       for (int i = etid; i < n; i += kEpiR) {
         const uint32_t at = unit_at(i >> 6, i, (i >> 3) & 7) + 2 * (i & 7);
-        float x = from_bits(*reinterpret_cast<const uint16_t*>(X + at), fcur.fmt);
-        if (fcur.terms > 1) x += from_bits(*reinterpret_cast<const uint16_t*>(X + kPlane + at), fcur.fmt);
+        float x = from_bits(*reinterpret_cast<const uint16_t*>(X + at), ref ? FMT_F16 : kFmt);
+        if (kTerms > 1 || ref) x += from_bits(*reinterpret_cast<const uint16_t*>(X + kPlane + at), ref ? FMT_F16 : kFmt);
         px += x;
       }
       for (int o = 16; o > 0; o >>= 1) {
@@ -607,22 +675,441 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
+// ------------------------------------------------------------------------------------ the inverse square root
+// a2-a3 for submatrices of up to 192 rows whose inverse square root converges in two steps (Eqs. inv1-inv3 with Z_0 = I),
+// with the same layout: T_0 = 3I - Y_0 stays in tensor memory as the A operand of every product of the iteration (all of
+// them are polynomials of T_J(S) and commute), and shared memory holds the other operand, overwritten column block by
+// column block by the product's result:
+//   Y_1 = T_0 Y_0 / 2,  T_1 = 3I - T_0 Y_1 / 2 (V_1 = Z_1 Y_1, Z_1 = T_0 / 2),  Z_2 = T_0 T_1 / 4,
+//   X = Z_2 Z_2 / c (P product; X in FP32 to memory and over its accumulators as the A operand),  A_J = X T_J(H0).
+// T_J(S) and T_J(H0) are read once and A_J and X written once, 0.71 MB at n = 172; nothing else moves. 27,000 submatrices
+// of 120-192 rows take 9.8 ms; k_ns_tc, which they used before, took 17.6 ms on them (every product's operands from L2 or
+// DRAM). At 6.5 TB/s the traffic alone would take 3.0 ms, the MMAs 2.9 ms: what bounds it is the epilogue, serial with
+// the products of one submatrix. Submatrices that need more steps are marked kSubAgain for k_ns_tc.
+struct InvInfo { int op, n16, nrb, nch; };   // op 0: T x B in column blocks, 1: B x B in row tiles, 2: the end
+
+struct SharedI {
+  uint64_t xr, pf[2], zf[2], ze[2], ld[2], idle;
+  uint32_t tmem;
+  int err, fetch;
+  InvInfo mm;
+  float red[8];
+};
+
+__global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
+  extern __shared__ uint8_t smraw[];
+  uint8_t* const X = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  __shared__ SharedI sh;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  if (tid == 0) {
+    tc::mbar_init(&sh.xr, kEpiR);
+    for (int t = 0; t < 2; ++t) {
+      tc::mbar_init(&sh.pf[t], 1);
+      tc::mbar_init(&sh.zf[t], 1);
+      tc::mbar_init(&sh.ze[t], kEpiR);
+      tc::mbar_init(&sh.ld[t], 1);
+    }
+    tc::mbar_init(&sh.idle, 1);
+    tc::fence_mbar_init();
+    sh.err = 0;
+  }
+  if (warp == 0) {
+    tc::tmem_alloc(&sh.tmem, 512);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = sh.tmem;
+  uint32_t nop = 0, np0 = 0, np1 = 0, nz = 0;   // products, P tiles and column blocks so far (per role)
+
+  if (warp < 4) {
+    tc::setmaxnreg_dec<kRegsLowR>();
+    if (warp == 1) {
+      auto wait = [&](uint64_t* b, uint32_t parity, int more) {
+        return (bool)__all_sync(0xffffffffu, tc::mbar_wait(b, parity, tc::globaltimer() + more * g.wait_ns));
+      };
+      const uint32_t x0 = __shfl_sync(0xffffffffu, tc::smem_u32(X), 0);
+      bool ok = true;
+      while (ok && !sh.err) {
+        if (!(ok = wait(&sh.xr, nop & 1, 8))) break;
+        ++nop;
+        tc::tc_fence_after();
+        const InvInfo m = sh.mm;
+        if (m.op == 2) break;
+        if (m.op == 1) {
+          const uint32_t id = tc::idesc(FMT_F16, FMT_F16, 0, 1, 128, m.n16);
+          for (int t = 0; t < m.nrb; ++t) {
+            if (tc::elect_one()) {
+              product<false>(tmem + kResMaxN * t, x0, 128 * t, 0, 0, m.n16, id, true);
+              tc::mma_commit(&sh.pf[t]);
+            }
+            __syncwarp();
+          }
+          continue;
+        }
+        for (int c = 0; c < m.nch && ok; ++c) {
+          const uint32_t id = tc::idesc(FMT_F16, FMT_F16, 0, 1, 128, min(64, m.n16 - 64 * c));
+          for (int t = 0; t < m.nrb; ++t, ++nz) {
+            const int slot = nz & 1;
+            if (!(ok = wait(&sh.ze[slot], ((nz >> 1) & 1) ^ 1, 1))) break;
+            tc::tc_fence_after();
+            if (tc::elect_one()) {
+              product<true>(tmem + kRing + 64 * slot, x0, 0, tmem + kResMaxN * t, c * kBlk, m.n16, id, true);
+              tc::mma_commit(&sh.zf[slot]);
+            }
+            __syncwarp();
+          }
+        }
+      }
+      if (!ok) sh.err = 1;
+    }
+  } else {
+    tc::setmaxnreg_inc<kRegsEpiR>();
+    const int etid = tid - 128, ew = warp - 4, q = warp & 3, grp = ew >> 2;
+    const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+    float* const wf = reinterpret_cast<float*>(X + kXBytes) + 1024 * ew;   // this warp's 32 x 32 staging
+    bool bad = false;
+    uint32_t nld = 0;
+    int kn = -1;   // thread 0: the next submatrix's place, once it has been drawn
+    // the operands are ready: product `op` may start
+    auto go = [&](int op, int n16, int nrb, int nch) {
+      if (etid == 0) sh.mm = InvInfo{op, n16, nrb, nch};
+      tc::fence_proxy_async_smem();
+      tc::tc_fence_before();
+      bar_epi();
+      tc::mbar_arrive(&sh.xr);
+    };
+    for (;;) {
+      if (etid == 0) {
+        const int k = kn >= 0 ? kn : atomicAdd(g.next, 1);
+        sh.fetch = (k < g.count && !sh.err) ? g.order[k] : -1;
+        kn = -1;
+      }
+      bar_epi();
+      const int J = sh.fetch;
+      bar_epi();
+      if (J < 0) {
+        go(2, 0, 0, 0);
+        break;
+      }
+      const int n = g.sub_n[J], n16 = (n + 15) & ~15, n64 = (n + 63) & ~63, nrb = (n + 127) / 128, nch = (n16 + 63) / 64;
+      const double* __restrict__ S = g.ws + (g.a_off[J] - g.a_base);
+      const double* __restrict__ H = S + g.chunk_n2;
+      auto total = [&](float p) -> float {   // sum over the epilogue's threads
+        for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+        if (lane == 0) sh.red[ew] = p;
+        bar_epi();
+        float d = 0.0f;
+        for (int w = 0; w < 8; ++w) d += sh.red[w];
+        bar_epi();
+        return d;
+      };
+      // a 32 x 32 chunk (row = lane) in FP32 to an n x n array, through the warp's staging so that a store
+      // instruction writes 32 consecutive entries of a row
+      auto out = [&](float* __restrict__ dst, int rbase, int col0, const uint32_t (&r)[32]) __attribute__((always_inline)) {
+        // pairs of entries: 2-entry unit p of row i at p ^ (i & 15)
+        __syncwarp();
+        float2* const wf2 = reinterpret_cast<float2*>(wf);
+#pragma unroll
+        for (int p = 0; p < 16; ++p)
+          wf2[lane * 16 + (p ^ (lane & 15))] = make_float2(__uint_as_float(r[2 * p]), __uint_as_float(r[2 * p + 1]));
+        __syncwarp();
+        const int rows = min(32, n - rbase), p = lane & 15, col = col0 + 2 * p;
+        float* at = dst + (size_t)(rbase + (lane >> 4)) * n + col;
+        if ((n & 1) == 0 && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {   // two rows an instruction, 8 bytes a lane
+          if (col < n) {
+#pragma unroll 8
+            for (int i = lane >> 4; i < rows; i += 2, at += 2 * n) *reinterpret_cast<float2*>(at) = wf2[i * 16 + (p ^ (i & 15))];
+          }
+        } else {
+          for (int i = lane >> 4; i < rows; i += 2, at += 2 * n) {
+            const float2 x = wf2[i * 16 + (p ^ (i & 15))];
+            if (col < n) at[0] = x.x;
+            if (col + 1 < n) at[1] = x.y;
+          }
+        }
+      };
+      if (etid == 0) tc::prefetch_l2(H, sizeof(double) * (size_t)n * n);
+      double tr = 0.0;   // c = Tr T_J(S) / n
+#pragma unroll
+      for (int k = 0; k < kResMaxN / 32; ++k) {
+        const int i = min(lane + 32 * k, n - 1);
+        const double d = __ldg(S + (size_t)i * n + i);
+        tr += lane + 32 * k < n ? d : 0.0;
+      }
+      for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+      const double cc = tr / n;
+      const float inv = (float)(1.0 / cc);
+      int status = kSubOk, steps = 1;
+      bool last0 = false;
+      // half 0: the iteration on Y_0 = T_J(S) / c, up to X; half 1: A_J = X T_J(H0). (One copy of the code for both and for
+      // every product: what the epilogue runs stays in the instruction cache.)
+#pragma unroll 1
+      for (int half = 0; half < (g.Aout ? 2 : 1) && status == kSubOk; ++half) {
+        const double* __restrict__ M = half ? H : S;
+        const float scale = half ? 1.0f : inv;
+        float part = 0.0f;   // ||I - Y_0||_F^2
+        const Fmt f3{FMT_F16, 3};
+        const uint32_t big = feed(X, M, n, n64, f3, X + kXBytes + 32 * 1024, sh.ld, nld, g.wait_ns, bad, etid,
+                                  [&](float& x, float& y, int i, int j) {
+                                    x *= scale;
+                                    y *= scale;
+                                    const float e0 = i == j ? 1.0f - x : x, e1 = i == j + 1 ? 1.0f - y : y;
+                                    part = fmaf(e0, e0, fmaf(e1, e1, part));
+                                  });
+        if (big >= (1151u << 20)) part = INFINITY;   // an entry beyond FP32, infinite or not a number
+        if (half == 0) {
+          const float d0 = sqrtf(total(part) / (float)n);   // its barriers also publish Y_0
+          last0 = d0 <= g.tol_inv;
+          if (!(cc > 0.0) || !isfinite(cc) || !isfinite(d0)) {   // the FP64 preparation takes it
+            status = kSubRefine;
+            break;
+          }
+          // T_0 = 3I - Y_0 into tensor memory (each lane its row); over Y_0 as well when step 0 is the last
+#pragma unroll 1
+          for (int t = 0; t < nrb; ++t) {
+            const int rbase = 128 * t + 32 * q, row = rbase + lane;
+            if (rbase >= n64) continue;
+#pragma unroll 1
+            for (int j = grp; 32 * j < n16; j += 2) {
+              uint32_t r[32], o[32], h[16], l[16];
+              const float d3 = row < n && 32 * j == rbase ? 3.0f : 0.0f;
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const uint8_t* at = X + unit_at(j >> 1, row, 4 * (j & 1) + u);
+                const uint4 a = *reinterpret_cast<const uint4*>(at), b = *reinterpret_cast<const uint4*>(at + kPlane);
+                const uint32_t hw[4] = {a.x, a.y, a.z, a.w}, lw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                  const float2 x = __half22float2(*reinterpret_cast<const __half2*>(&hw[w]));
+                  const float2 y = __half22float2(*reinterpret_cast<const __half2*>(&lw[w]));
+                  const float a0 = -(x.x + y.x), a1 = -(x.y + y.y);
+                  const int k = 8 * u + 2 * w;
+                  r[k] = pick(k, lane, __float_as_uint(d3 + a0), __float_as_uint(a0));
+                  r[k + 1] = pick(k + 1, lane, __float_as_uint(d3 + a1), __float_as_uint(a1));
+                }
+              }
+              float sq = 0.0f;
+              scale_split_t<FMT_F16, true, false>(r, 1.0f, h, l, sq);
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                o[u] = h[u];
+                o[16 + u] = l[u];
+              }
+              tc::tmem_st32(tmem + kResMaxN * t + lane_base + 32 * j, o);
+              if (last0) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  uint8_t* at = X + unit_at(j >> 1, row, 4 * (j & 1) + u);
+                  *reinterpret_cast<uint4*>(at) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+                  *reinterpret_cast<uint4*>(at + kPlane) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+                }
+              }
+            }
+          }
+          tc::tmem_wait_st();
+        }
+        // products with A in tensor memory, in column blocks: 0: Y_1 = P / 2, 1: T_1 = 3I - P / 2 and its defect, 2: Z_2 =
+        // P / 4, each over the operand; 4: A_J = P in FP32
+#pragma unroll 1
+        for (int s = half ? 4 : last0 ? 3 : 0; s != 3 && s < 5; ++s) {
+          const float m = s == 2 ? 0.25f : s == 1 ? -0.5f : 0.5f;
+          go(0, n16, nrb, nch);
+          float sum = 0.0f;
+#pragma unroll 1
+          for (int c = 0; c < nch; ++c) {
+            const int col0 = 64 * c + 32 * grp;
+            const bool cols = col0 < n16;
+            auto take = [&](int t, uint32_t (&h)[16], uint32_t (&l)[16]) __attribute__((always_inline)) {
+              const int slot = nz & 1;
+              if (!bad) bad = !tc::mbar_wait(&sh.zf[slot], (nz >> 1) & 1, tc::globaltimer() + g.wait_ns);
+              bad = __any_sync(0xffffffffu, bad);
+              ++nz;
+              tc::tc_fence_after();
+              uint32_t r[32];
+              const int rbase = 128 * t + 32 * q, row = rbase + lane;
+              const bool mine = rbase < n64 && cols && !bad;
+              if (mine) {
+                tc::tmem_ld32(tmem + kRing + 64 * slot + lane_base + 32 * grp, r);
+                tc::tmem_wait_ld();
+              }
+              tc::tc_fence_before();
+              if (!bad) tc::mbar_arrive(&sh.ze[slot]);
+              if (!mine) return;
+              if (s == 4) {
+                out(g.Aout + g.a_off[J], rbase, col0, r);
+                return;
+              }
+              if (col0 + 16 >= n16) {   // the MMAs left the second half out: it holds anything
+#pragma unroll
+                for (int u = 16; u < 32; ++u) r[u] = 0;
+              }
+              // T_1: off the diagonal -P / 2; on it first P - 2, whose -1/2-fold is 1 - P / 2, then 2 more
+              const bool diag = s == 1 && col0 == rbase;
+              if (diag) {
+                const float two = row < n ? 2.0f : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) r[u] = pick(u, lane, __float_as_uint(__uint_as_float(r[u]) - two), r[u]);
+              }
+              float sq = 0.0f;
+              scale_split_t<FMT_F16, true, true>(r, m, h, l, sq);
+              if (row < n) sum += sq;
+              if (diag) {
+                uint32_t e = 0;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) e = pick(u, lane, r[u], e);
+                uint32_t th, tl;
+                split2(row < n ? 2.0f - 0.5f * __uint_as_float(e) : 0.0f, 0.0f, FMT_F16, th, tl);
+                const uint32_t sel = lane & 1 ? 0x5410u : 0x3254u;
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                  h[u] = pick(u, lane >> 1, __byte_perm(h[u], th, sel), h[u]);
+                  l[u] = pick(u, lane >> 1, __byte_perm(l[u], tl, sel), l[u]);
+                }
+              }
+            };
+            auto put = [&](int t, const uint32_t (&h)[16], const uint32_t (&l)[16]) __attribute__((always_inline)) {
+              const int rbase = 128 * t + 32 * q, row = rbase + lane;
+              if (s == 4 || rbase >= n64 || !cols || bad) return;
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                uint8_t* at = X + unit_at(c, row, 4 * grp + u);
+                *reinterpret_cast<uint4*>(at) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+                *reinterpret_cast<uint4*>(at + kPlane) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+              }
+            };
+            // the operand's column block may be overwritten once the block's last product has completed
+            uint32_t h0[16], l0[16];
+            take(0, h0, l0);
+            if (nrb == 2) {
+              uint32_t h1[16], l1[16];
+              take(1, h1, l1);
+              put(1, h1, l1);
+            }
+            put(0, h0, l0);
+          }
+          if (s == 1) {
+            const float d1 = sqrtf(total(sum) / (float)n);
+            steps = 2;
+            if (!isfinite(d1)) status = kSubRefine;
+            else if (d1 > g.tol_inv) status = g.max_inv > 2 ? kSubAgain : kSubRefine;
+            if (status != kSubOk) break;
+          }
+        }
+        if (half == 1 || status != kSubOk) break;
+        if (etid == 0) {
+          kn = atomicAdd(g.next, 1);
+          if (kn < g.count) {
+            const int Jn = g.order[kn];
+            tc::prefetch_l2(g.ws + (g.a_off[Jn] - g.a_base), sizeof(double) * (size_t)g.sub_n[Jn] * g.sub_n[Jn]);
+          }
+        }
+        // X = Z Z / c, tile by tile: FP32 to memory, and over the accumulators as the next product's A
+        const float m = inv * (last0 ? 0.25f : 1.0f);
+        float* __restrict__ Xo = g.Xout + (g.a_off[J] - g.a_base);
+        go(1, n16, nrb, nch);
+#pragma unroll 1
+        for (int t = 0; t < nrb; ++t) {
+          if (!bad) bad = !tc::mbar_wait(&sh.pf[t], (t ? np1 : np0) & 1, tc::globaltimer() + g.wait_ns);
+          bad = __any_sync(0xffffffffu, bad);
+          ++(t ? np1 : np0);
+          tc::tc_fence_after();
+          const int rbase = 128 * t + 32 * q;
+          if (rbase < n64 && !bad) {
+            const uint32_t ta = tmem + kResMaxN * t + lane_base;
+#pragma unroll 1
+            for (int j = grp; 32 * j < n16; j += 2) {
+              uint32_t r[32], h[16], l[16], o[32];
+              tc::tmem_ld32(ta + 32 * j, r);
+              tc::tmem_wait_ld();
+              float sq = 0.0f;
+              scale_split_t<FMT_F16, true, false>(r, m, h, l, sq);
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                o[u] = h[u];
+                o[16 + u] = l[u];
+              }
+              tc::tmem_st32(ta + 32 * j, o);
+#pragma unroll
+              for (int u = 0; u < 32; ++u) r[u] = __float_as_uint(m * __uint_as_float(r[u]));
+              out(Xo, rbase, 32 * j, r);
+            }
+            tc::tmem_wait_st();
+          }
+        }
+        tc::tc_fence_before();
+        bar_epi();   // every P tile has been waited for: Z may be overwritten
+      }
+      if (bar_epi_or(bad)) {   // a wait ran out
+        if (etid == 0) {
+          sh.err = 1;
+          g.prep_out[J] = kSubTimeout;
+          atomicExch(g.err, 1);
+        }
+        go(2, 0, 0, 0);
+        break;
+      }
+      if (etid == 0) {
+        g.prep_out[J] = status;
+        if (status == kSubAgain) atomicAdd(g.again, 1);
+        else {
+          const double prods = 3.0 * steps - (g.Aout ? 1.0 : 2.0), n3 = (double)n * n * n;
+          atomicAdd(&g.flops[0], 2.0 * n3 * prods);
+          atomicAdd(&g.flops[1], 6.0 * n3 * prods);
+        }
+      }
+    }
+  }
+
+  __syncthreads();
+  if (sh.err && warp == 1 && lane == 0) {
+    tc::mma_commit(&sh.idle);
+    tc::mbar_wait(&sh.idle, 0, tc::globaltimer() + 50000000ull);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
 }  // namespace
+
+template <typename K>
+static nolsm_status ready(K* kernel, const char* name, uint32_t smem) {
+  cudaFuncAttributes at{};
+  NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(kernel)));
+  if (at.numRegs != kRegsLaunchR) {
+    set_error("%s was built with %d registers per thread; its register split needs exactly %d", name, at.numRegs,
+              kRegsLaunchR);
+    return NOLSM_ERR_UNSUPPORTED;
+  }
+  NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  return NOLSM_OK;
+}
 
 nolsm_status launch_ns_res(const ResSolve& a, int sms, cudaStream_t st) {
   if (a.count <= 0) return NOLSM_OK;
   ResSolve g = a;
   if (g.wait_ns == 0) g.wait_ns = kWaitNsR;
-  cudaFuncAttributes at{};
-  NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(&k_ns_res)));
-  if (at.numRegs != kRegsLaunchR) {
-    set_error("k_ns_res was built with %d registers per thread; its register split needs exactly %d", at.numRegs,
-              kRegsLaunchR);
-    return NOLSM_ERR_UNSUPPORTED;
-  }
-  NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_ns_res, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemR));
   NOLSM_CUDA_TRY(cudaMemsetAsync(g.next, 0, sizeof(int32_t), st));
-  k_ns_res<<<std::min(sms, a.count), kThreadsR, kSmemR, st>>>(g);
+  auto run = [&](auto* kernel) -> nolsm_status {
+    NOLSM_TRY(ready(kernel, "k_ns_res", kSmemR));
+    kernel<<<std::min(sms, a.count), kThreadsR, kSmemR, st>>>(g);
+    return NOLSM_OK;
+  };
+  if (a.main_fmt.fmt == FMT_BF16) NOLSM_TRY(a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_BF16, 3>) : run(&k_ns_res<FMT_BF16, 1>));
+  else NOLSM_TRY(a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_F16, 3>) : run(&k_ns_res<FMT_F16, 1>));
+  NOLSM_LAUNCH_CHECK();
+  return NOLSM_OK;
+}
+
+nolsm_status launch_inv_res(const InvSolve& a, int sms, cudaStream_t st) {
+  if (a.count <= 0) return NOLSM_OK;
+  InvSolve g = a;
+  if (g.wait_ns == 0) g.wait_ns = kWaitNsR;
+  NOLSM_TRY(ready(&k_inv_res, "k_inv_res", kSmemI));
+  NOLSM_CUDA_TRY(cudaMemsetAsync(g.next, 0, sizeof(int32_t), st));
+  k_inv_res<<<std::min(sms, a.count), kThreadsR, kSmemI, st>>>(g);
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }

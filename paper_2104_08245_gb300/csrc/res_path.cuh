@@ -16,7 +16,7 @@ struct ResSolve {
   double mu;
   float tol_ns, tol_accept;
   int32_t max_iter, refine_steps; const int32_t* budget;
-  Fmt main_fmt, refine_fmt;              // 2-byte formats
+  Fmt main_fmt;                          // a 2-byte format; the refinement's is FP16 in three terms
   int32_t* next; int32_t* err;           // work counter (reset by the launch), timeout flag
   double* Dc; double* tS; double* tH; int32_t* iters; int32_t* status; int32_t* rsteps; int32_t* nbelow;
   uint64_t wait_ns;                      // limit of a wait of one role on another, 0: 2 s
@@ -24,5 +24,21 @@ struct ResSolve {
 };
 // Every status of the work has been set to kSubTimeout before.
 nolsm_status launch_ns_res(const ResSolve& a, int sms, cudaStream_t st);
+
+// a2-a3 the same way, every submatrix of at most kResMaxN rows (see launch_ns_inverse for the fields): prep_out[J] =
+// kSubOk, kSubRefine, or kSubAgain where k_ns_tc has to take the submatrix (more than two steps); *again counts those.
+constexpr int32_t kSubAgain = 66;
+struct InvSolve {
+  const int32_t* order; int32_t count;
+  const int32_t* sub_n; const int64_t* a_off;
+  const double* ws; int64_t a_base, chunk_n2;
+  float* Aout; float* Xout;
+  int32_t* prep_out;
+  float tol_inv; int32_t max_inv;
+  int32_t* next; int32_t* err; int32_t* again;
+  double* flops;
+  uint64_t wait_ns;
+};
+nolsm_status launch_inv_res(const InvSolve& a, int sms, cudaStream_t st);
 
 }  // namespace nolsm

@@ -135,6 +135,7 @@ struct TcArgs {
   int32_t* prep_out;          // kSubOk, or kSubRefine when the iteration failed (FP64 preparation next)
   float tol_inv;
   int32_t max_inv;
+  int32_t again;              // only submatrices whose prep_out is kSubAgain (k_inv_res left them)
   double* flops;              // [2]: 2 n^3 per product (method count) and the split's issued flops, summed
 };
 
@@ -655,6 +656,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           break;
         }
         if constexpr (kMode == 1) {
+          if (g.again && g.prep_out[J] != kSubAgain) continue;
           start_inverse(s, J);
           break;
         }
@@ -1351,10 +1353,11 @@ static nolsm_status run_buckets(int mode, int precision, bool fixed0, const TcMa
   return launch_shape(mode, s0, m, g, sms, st);
 }
 
-// Sign bucket 0 (n <= 192) has no shape to choose any more: the query reports 0 once it has run.
-static void resident_shape(int precision) {
+// Bucket 0 (n <= 192) has no shape to choose (the sign but for E4M3 and the inverse run it in res_path.cu): the query
+// reports 0 once it has run.
+static void resident_shape(int mode, int precision) {
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  g_shape[0][precision & 7][0] = 0;
+  g_shape[mode][precision & 7][0] = 0;
 }
 
 int tc_shape_choice(int mode, int precision, int bucket) {
@@ -1508,14 +1511,14 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     r.mu = mu;
     r.tol_ns = g.tol_ns; r.tol_accept = g.tol_accept;
     r.max_iter = g.max_iter; r.refine_steps = g.refine_steps; r.budget = g.budget;
-    r.main_fmt = mf; r.refine_fmt = rf;
+    r.main_fmt = mf;
     r.next = plan->counter.as<int32_t>() + 1; r.err = g.err;
     r.Dc = g.Dc; r.tS = g.tS; r.tH = g.tH; r.iters = g.iters; r.status = g.status; r.rsteps = g.rsteps;
     r.nbelow = g.nbelow;
     r.wait_ns = g.wait_ns;
     r.cond = g.cond; r.cond_max = g.cond_max; r.ill_max_n = g.ill_max_n;
     NOLSM_TRY(launch_ns_res(r, sms, st));
-    resident_shape(o.precision);
+    resident_shape(0, o.precision);
     plan->stats.launches += 1;
   }
   plan->stats.launches += 2;
@@ -1544,69 +1547,102 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
   int dev = 0, sms = 0;
   NOLSM_CUDA_TRY(cudaGetDevice(&dev));
   NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int LD = (a.max_n + 63) & ~63, R = (a.max_n + 127) & ~127;
-  const int ctas = (int)std::min<int64_t>(sms, (a.count + kSlots - 1) / kSlots);
-  const int slots = ctas * kSlots;
-  if (!S->inv_planes.p || S->iR < R || S->iLD < LD || S->islots < slots) {
-    const int nR = std::max(R, S->iR), nLD = std::max(LD, S->iLD), nS = std::max(slots, S->islots);
-    dev_free(plan, S->inv_planes);
-    NOLSM_TRY(dev_alloc(plan, S->inv_planes, sizeof(uint16_t) * (size_t)kPlanesInv * nS * nR * nLD));
-    S->iR = nR;
-    S->iLD = nLD;
-    S->islots = nS;
-  }
   if (!S->err.p) NOLSM_TRY(dev_alloc(plan, S->err, sizeof(int32_t) * 4));
   if (!S->inv_flops.p) NOLSM_TRY(dev_alloc(plan, S->inv_flops, sizeof(double) * 2));
-  const uint64_t depth = (uint64_t)S->islots * kPlanesInv;
-  CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
-  if (!tmap::make_3d(&mS16, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
-                     CU_TENSOR_MAP_SWIZZLE_64B) ||
-      !tmap::make_3d(&mS16x2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
-                     CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mS2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
-                     CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mA, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 128) ||
-      !tmap::make_3d(&mB, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 64) ||
-      !tmap::make_3d(&mS, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
-                     CU_TENSOR_MAP_SWIZZLE_64B)) {
-    set_error("cuTensorMapEncodeTiled rejected the inverse scratch layout (R %d, LD %d, slots %d)", S->iR, S->iLD,
-              S->islots);
-    return NOLSM_ERR_CUDA;
-  }
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
-  NOLSM_CUDA_TRY(cudaMemsetAsync(S->err.p, 0, sizeof(int32_t), st));
+  NOLSM_CUDA_TRY(cudaMemsetAsync(S->err.p, 0, sizeof(int32_t) * 4, st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(S->inv_flops.p, 0, sizeof(double) * 2, st));
-  TcArgs g{};
-  g.j0 = 0; g.j1 = a.count;
-  g.order = a.order;
-  g.sub_n = plan->sub_n.as<int32_t>(); g.nbf = plan->sub_b.as<int32_t>();
-  g.a_off = plan->a_off.as<int64_t>(); g.c_off = plan->c_off.as<int64_t>();
-  g.main_fmt = Fmt{FMT_F16, 3}; g.refine_fmt = g.main_fmt;
-  g.planes = S->inv_planes.as<uint16_t>();
-  g.R = S->iR; g.LD = S->iLD;
-  g.next = plan->counter.as<int32_t>();
-  g.err = S->err.as<int32_t>();
-  g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2;
-  g.Aout = a.Aout; g.Xout = a.Xout; g.prep_out = a.prep_out;
-  g.tol_inv = a.tol_inv; g.max_inv = a.max_inv;
-  g.wait_ns = kWaitNs;
-  g.flops = S->inv_flops.as<double>();
-  // the largest-first order in its two buckets (n above 192, the rest), each in its tuned shape; every
-  // submatrix of a launch starts as "timed out" and the kernel overwrites what it takes. (The first call in a process
-  // also counts the flops of the shape measurements.)
-  TcMaps m{mA, mB, mS, mA, mB, mS16, mS2, mS16x2};
+  // every submatrix of a launch starts as "timed out" and the kernel overwrites what it takes. (The first call in a
+  // process also counts the flops of the shape measurements.)
   auto pending = [&](const int32_t* list, int32_t count) -> nolsm_status {
     k_status_pending<<<(unsigned)std::min(1024, (count + 255) / 256), 256, 0, st>>>(0, count, list, a.prep_out);
     NOLSM_LAUNCH_CHECK();
     return NOLSM_OK;
   };
-  NOLSM_TRY(run_buckets(1, NOLSM_FP16, false, m, g, a.order, a.n_large, a.count, sms, st, pending));
-  double fl[2];
-  NOLSM_CUDA_TRY(cudaMemcpyAsync(fl, S->inv_flops.p, sizeof(fl), cudaMemcpyDeviceToHost, st));
-  NOLSM_CUDA_TRY(cudaStreamSynchronize(st));
-  plan->stats.flops_prep_tensor += fl[0];
-  plan->stats.flops_prep_tensor_issued += fl[1];
-  plan->stats.launches += 2;
+  auto read_back = [&](int32_t* again) -> nolsm_status {   // flops, and what k_inv_res left; clears both
+    double fl[2];
+    NOLSM_CUDA_TRY(cudaMemcpyAsync(fl, S->inv_flops.p, sizeof(fl), cudaMemcpyDeviceToHost, st));
+    NOLSM_CUDA_TRY(cudaMemcpyAsync(again, S->err.as<int32_t>() + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    NOLSM_CUDA_TRY(cudaStreamSynchronize(st));
+    plan->stats.flops_prep_tensor += fl[0];
+    plan->stats.flops_prep_tensor_issued += fl[1];
+    return NOLSM_OK;
+  };
+  // n of at most kResMaxN: operands on the SM (res_path.cu)
+  const int32_t n_small = a.count - a.n_large;
+  if (n_small > 0) {
+    InvSolve r{};
+    r.order = a.order + a.n_large; r.count = n_small;
+    r.sub_n = plan->sub_n.as<int32_t>(); r.a_off = plan->a_off.as<int64_t>();
+    r.ws = a.ws; r.a_base = a.a_base; r.chunk_n2 = a.chunk_n2;
+    r.Aout = a.Aout; r.Xout = a.Xout; r.prep_out = a.prep_out;
+    r.tol_inv = a.tol_inv; r.max_inv = a.max_inv;
+    r.next = plan->counter.as<int32_t>() + 1;
+    r.err = S->err.as<int32_t>(); r.again = S->err.as<int32_t>() + 1;
+    r.flops = S->inv_flops.as<double>();
+    NOLSM_TRY(pending(r.order, n_small));
+    NOLSM_TRY(launch_inv_res(r, sms, st));
+    resident_shape(1, NOLSM_FP16);
+    plan->stats.launches += 2;
+  }
+  // the others, and those that need more than two steps, with operands in scratch
+  auto streamed = [&](const int32_t* order, int32_t n_large, int32_t count, int32_t again) -> nolsm_status {
+    const int max_n = again ? std::min(a.max_n, kResMaxN) : a.max_n;
+    const int LD = (max_n + 63) & ~63, R = (max_n + 127) & ~127;
+    const int slots = (int)std::min<int64_t>(sms, (count + kSlots - 1) / kSlots) * kSlots;
+    if (!S->inv_planes.p || S->iR < R || S->iLD < LD || S->islots < slots) {
+      const int nR = std::max(R, S->iR), nLD = std::max(LD, S->iLD), nS = std::max(slots, S->islots);
+      dev_free(plan, S->inv_planes);
+      NOLSM_TRY(dev_alloc(plan, S->inv_planes, sizeof(uint16_t) * (size_t)kPlanesInv * nS * nR * nLD));
+      S->iR = nR;
+      S->iLD = nLD;
+      S->islots = nS;
+    }
+    const uint64_t depth = (uint64_t)S->islots * kPlanesInv;
+    CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
+    if (!tmap::make_3d(&mS16, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
+                       CU_TENSOR_MAP_SWIZZLE_64B) ||
+        !tmap::make_3d(&mS16x2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
+                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
+        !tmap::make_3d(&mS2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
+                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
+        !tmap::make_3d(&mA, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 128) ||
+        !tmap::make_3d(&mB, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 64) ||
+        !tmap::make_3d(&mS, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
+                       CU_TENSOR_MAP_SWIZZLE_64B)) {
+      set_error("cuTensorMapEncodeTiled rejected the inverse scratch layout (R %d, LD %d, slots %d)", S->iR, S->iLD,
+                S->islots);
+      return NOLSM_ERR_CUDA;
+    }
+    TcArgs g{};
+    g.j0 = 0; g.j1 = count;
+    g.order = order;
+    g.sub_n = plan->sub_n.as<int32_t>(); g.nbf = plan->sub_b.as<int32_t>();
+    g.a_off = plan->a_off.as<int64_t>(); g.c_off = plan->c_off.as<int64_t>();
+    g.main_fmt = Fmt{FMT_F16, 3}; g.refine_fmt = g.main_fmt;
+    g.planes = S->inv_planes.as<uint16_t>();
+    g.R = S->iR; g.LD = S->iLD;
+    g.next = plan->counter.as<int32_t>();
+    g.err = S->err.as<int32_t>();
+    g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2;
+    g.Aout = a.Aout; g.Xout = a.Xout; g.prep_out = a.prep_out;
+    g.tol_inv = a.tol_inv; g.max_inv = a.max_inv;
+    g.again = again;
+    g.wait_ns = kWaitNs;
+    g.flops = S->inv_flops.as<double>();
+    const TcMaps m{mA, mB, mS, mA, mB, mS16, mS2, mS16x2};
+    plan->stats.launches += 2;
+    if (again) return launch_shape(1, 0, m, g, sms, st);
+    return run_buckets(1, NOLSM_FP16, false, m, g, order, n_large, count, sms, st, pending);
+  };
+  if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, a.n_large, 0));
+  int32_t again = 0;
+  NOLSM_TRY(read_back(&again));
+  if (again > 0) {
+    NOLSM_CUDA_TRY(cudaMemsetAsync(S->inv_flops.p, 0, sizeof(double) * 2, st));
+    NOLSM_TRY(streamed(a.order + a.n_large, 0, n_small, 1));
+    NOLSM_TRY(read_back(&again));
+  }
   return NOLSM_OK;
 }
 

@@ -95,6 +95,12 @@ template <int N>
 __device__ __forceinline__ void bulk_wait() {
   asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
 }
+// Untiled copy of whole 16-byte units from global to shared memory, complete on `bar`.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(smem_dst)),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
 // brings [p, p + bytes) (widened to whole 16-byte units) into L2
 __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
   const uint64_t a = reinterpret_cast<uint64_t>(p) & ~uint64_t(15), e = (reinterpret_cast<uint64_t>(p) + bytes) & ~uint64_t(15);
