@@ -337,7 +337,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
             for (int ks = 0; ks < n32; ++ks, ++kcount) {
               const int st = kcount % kStages;
               const uint32_t ph = (kcount / kStages) & 1;
-              if (!tc::mbar_wait(&sh.empty[st], ph ^ 1, tc::globaltimer() + g.wait_ns)) return false;
+              if (!tc::mbar_wait_ns(&sh.empty[st], ph ^ 1, g.wait_ns)) return false;
               uint8_t* sm = stage_mem + st * Dg::kStage;
               tc::mbar_arrive_expect_tx(&sh.full[st], kD * rows * 64 + Dg::kBBytes);
               armed[st] = true;
@@ -347,12 +347,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
             }
           } else {
             const uint32_t id = tc::idesc(0, 0, 0, 1, rows, min(64, c.n16 - 64 * cb));
-            if (!__all_sync(0xffffffffu, tc::mbar_wait(&sh.acce, (tcount & 1) ^ 1, tc::globaltimer() + g.wait_ns)))
+            if (!__all_sync(0xffffffffu, tc::mbar_wait_ns(&sh.acce, (tcount & 1) ^ 1, g.wait_ns)))
               return false;
             tc::tc_fence_after();
             for (int ks = 0; ks < n32; ++ks, ++kcount) {
               const int st = kcount % kStages;
-              if (!__all_sync(0xffffffffu, tc::mbar_wait(&sh.full[st], (kcount / kStages) & 1, tc::globaltimer() + g.wait_ns)))
+              if (!__all_sync(0xffffffffu, tc::mbar_wait_ns(&sh.full[st], (kcount / kStages) & 1, g.wait_ns)))
                 return false;
               tc::tc_fence_after();
               const uint32_t a0 = __shfl_sync(0xffffffffu, tc::smem_u32(stage_mem + st * Dg::kStage), 0);
@@ -559,7 +559,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
       const int shl = U + s - Dg::G;           // from the last accumulator but one to the output's units
       for (int t = rank; t < c.nrb * c.ncb; t += 2, ++tcount) {
         const int mb = t / c.ncb, cb = t - mb * c.ncb;
-        bool ok = tc::mbar_wait(&sh.accf, tcount & 1, tc::globaltimer() + g.wait_ns);
+        bool ok = tc::mbar_wait_ns(&sh.accf, tcount & 1, g.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) return false;
         tc::tc_fence_after();
         const bool m64 = tail64(mb);
@@ -822,10 +822,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
   if (sh.err) {
     if (warp == 0 && lane == 0)
       for (int s = 0; s < kStages; ++s)
-        if (armed[s]) tc::mbar_wait(&sh.full[s], arm_phase[s], tc::globaltimer() + 50000000ull);
+        if (armed[s]) tc::mbar_wait_ns(&sh.full[s], arm_phase[s], 50000000ull);
     if (warp == 1 && lane == 0) {
       tc::mma_commit(&sh.idle);
-      tc::mbar_wait(&sh.idle, 0, tc::globaltimer() + 50000000ull);
+      tc::mbar_wait_ns(&sh.idle, 0, 50000000ull);
     }
   }
   tc::tc_fence_before();

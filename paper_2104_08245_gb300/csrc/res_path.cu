@@ -71,14 +71,6 @@ __device__ __forceinline__ bool bar_epi_or(bool p) {
   return r != 0;
 }
 
-// u == k ? a : b as an instruction that the compiler does not fold into an indexed (local memory) array access: local
-// memory shares its bandwidth with the MMAs' operands
-__device__ __forceinline__ uint32_t pick(int u, int k, uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, %2;\n\tselp.b32 %0, %3, %4, p;\n\t}" : "=r"(r) : "r"(u), "r"(k), "r"(a), "r"(b));
-  return r;
-}
-
 // byte offset of the 16-byte unit u (eight columns) of row i in column block c of a plane
 __device__ __forceinline__ uint32_t unit_at(int c, int i, int u) { return c * kBlk + i * 128 + ((u ^ (i & 7)) << 4); }
 
@@ -156,8 +148,8 @@ __device__ __forceinline__ uint32_t feed(uint8_t* X, const T* __restrict__ M, in
 #pragma unroll 1
   for (int c = 0; c < nc; ++c) {
     const uint32_t b = (nld + c) & 1;
-    if (!bad) bad = !tc::mbar_wait(&ld[b], ((nld + c) >> 1) & 1, tc::globaltimer() + wait_ns);
-    if (bad && etid == 0) tc::mbar_wait(&ld[b], ((nld + c) >> 1) & 1, tc::globaltimer() + 50000000ull);   // none left in flight
+    if (!bad) bad = !tc::mbar_wait_ns(&ld[b], ((nld + c) >> 1) & 1, wait_ns);
+    if (bad && etid == 0) tc::mbar_wait_ns(&ld[b], ((nld + c) >> 1) & 1, 50000000ull);   // none left in flight
     const T* rows = reinterpret_cast<const T*>(stage + b * kFeed + (reinterpret_cast<uintptr_t>(M + (size_t)c * R * n) & 15));
     const int count = min(R, n - c * R);
 #pragma unroll 1
@@ -294,7 +286,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
   if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     auto wait = [&](uint64_t* b, uint32_t parity, int more) {
-      return (bool)__all_sync(0xffffffffu, tc::mbar_wait(b, parity, tc::globaltimer() + more * g.wait_ns));
+      return (bool)__all_sync(0xffffffffu, tc::mbar_wait_ns(b, parity, more * g.wait_ns));
     };
     const uint32_t x0 = __shfl_sync(0xffffffffu, tc::smem_u32(X), 0);
     bool ok = true;
@@ -396,7 +388,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
         // ---- P -> T, tile by tile
         float part = 0.0f;
         for (int t = 0; t < nrb; ++t) {
-          if (!bad) bad = !tc::mbar_wait(&sh.pf[t], (t ? np1 : np0) & 1, tc::globaltimer() + g.wait_ns);
+          if (!bad) bad = !tc::mbar_wait_ns(&sh.pf[t], (t ? np1 : np0) & 1, g.wait_ns);
           bad = __any_sync(0xffffffffu, bad);
           ++(t ? np1 : np0);
           tc::tc_fence_after();
@@ -516,7 +508,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
           // row tile t's block out of its accumulator, halved and split
           auto take = [&](int t, uint32_t (&h)[16], uint32_t (&l)[16]) {
             const int slot = nz & 1;
-            if (!bad) bad = !tc::mbar_wait(&sh.zf[slot], (nz >> 1) & 1, tc::globaltimer() + g.wait_ns);
+            if (!bad) bad = !tc::mbar_wait_ns(&sh.zf[slot], (nz >> 1) & 1, g.wait_ns);
             bad = __any_sync(0xffffffffu, bad);
             ++nz;
             tc::tc_fence_after();
@@ -668,7 +660,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
   __syncthreads();
   if (sh.err && warp == 1 && lane == 0) {
     tc::mma_commit(&sh.idle);
-    tc::mbar_wait(&sh.idle, 0, tc::globaltimer() + 50000000ull);
+    tc::mbar_wait_ns(&sh.idle, 0, 50000000ull);
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -727,7 +719,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
     tc::setmaxnreg_dec<kRegsLowR>();
     if (warp == 1) {
       auto wait = [&](uint64_t* b, uint32_t parity, int more) {
-        return (bool)__all_sync(0xffffffffu, tc::mbar_wait(b, parity, tc::globaltimer() + more * g.wait_ns));
+        return (bool)__all_sync(0xffffffffu, tc::mbar_wait_ns(b, parity, more * g.wait_ns));
       };
       const uint32_t x0 = __shfl_sync(0xffffffffu, tc::smem_u32(X), 0);
       bool ok = true;
@@ -923,7 +915,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
             const bool cols = col0 < n16;
             auto take = [&](int t, uint32_t (&h)[16], uint32_t (&l)[16]) __attribute__((always_inline)) {
               const int slot = nz & 1;
-              if (!bad) bad = !tc::mbar_wait(&sh.zf[slot], (nz >> 1) & 1, tc::globaltimer() + g.wait_ns);
+              if (!bad) bad = !tc::mbar_wait_ns(&sh.zf[slot], (nz >> 1) & 1, g.wait_ns);
               bad = __any_sync(0xffffffffu, bad);
               ++nz;
               tc::tc_fence_after();
@@ -1011,7 +1003,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
         go(1, n16, nrb, nch);
 #pragma unroll 1
         for (int t = 0; t < nrb; ++t) {
-          if (!bad) bad = !tc::mbar_wait(&sh.pf[t], (t ? np1 : np0) & 1, tc::globaltimer() + g.wait_ns);
+          if (!bad) bad = !tc::mbar_wait_ns(&sh.pf[t], (t ? np1 : np0) & 1, g.wait_ns);
           bad = __any_sync(0xffffffffu, bad);
           ++(t ? np1 : np0);
           tc::tc_fence_after();
@@ -1065,7 +1057,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
   __syncthreads();
   if (sh.err && warp == 1 && lane == 0) {
     tc::mma_commit(&sh.idle);
-    tc::mbar_wait(&sh.idle, 0, tc::globaltimer() + 50000000ull);
+    tc::mbar_wait_ns(&sh.idle, 0, 50000000ull);
   }
   tc::tc_fence_before();
   __syncthreads();

@@ -7,20 +7,24 @@
 // three-term split hi*hi + hi*lo + lo*hi with x = hi + lo (hi = round(x), lo = round(x - hi)),
 // accumulated in FP32 in tensor memory.
 //
-// One persistent CTA per SM keeps two submatrices in flight ("slots", taken largest first from a
-// work counter) and interleaves their products: while the tensor cores run a product of one slot,
-// the epilogue drains, rounds and stores the previous product of the other, so neither the operand
-// fill nor the epilogue of a product serialises the CTA. Operands live in per-slot scratch in global
-// memory (L2-resident) as 2-byte planes [X0 hi, X0 lo, X1 hi, X1 lo, T hi, T lo], each R x LD
-// (R = n rounded up to 128 rows, LD = n rounded up to 64 columns, zero padded). Output tiles are
-// 128 rows x up to 256 columns; the K dimension streams in slices of 64 through a two-stage TMA
-// pipeline with 128-byte swizzle; the epilogue writes the rounded planes back with TMA stores.
-// Warp roles: warp 0 (one thread) schedules the products of both slots and issues their TMA loads,
-// publishing one descriptor per product in a small ring; warp 1 (one thread) issues tcgen05.mma in
-// that order; warps 4-11 (two groups of four, even and odd 32-column chunks) drain the
-// double-buffered TMEM accumulators (2 x 256 columns), decide convergence and start and finish the
-// slots' submatrices. All waits are bounded by the global timer; a wait that runs out marks the
-// submatrices in flight as timed out.
+// Submatrices of more than 192 rows (and all of them in E4M3) run here; the others keep their operands on the SM
+// (res_path.cu). One persistent CTA per SM; a group of 1, 2, 4 or 8 CTAs (group_size) shares two submatrices in flight
+// ("slots", taken largest first from a work counter) and deals their products' tiles, and the rows of a start or a
+// finish, among its CTAs. While the tensor cores run a product of one slot, the epilogues drain, round and store the
+// previous product of the other, and the group meets. Operands live in per-slot scratch in global memory as 2-byte
+// planes [X0 hi, X0 lo, X1 hi, X1 lo, T hi, T lo], each R x LD (R = n rounded up to 128 rows, LD = n rounded up to 64
+// columns, zero padded). What bounds it: with two submatrices on every SM the planes (4 MB a submatrix at n = 650) miss
+// L2, and each product's operands come from DRAM several times over; the groups keep the planes in flight within L2
+// (512 submatrices of n = 600-713: 233 GB through DRAM before, 41 GB since; 40 -> 12.9 ms). What is left at 2.4 times
+// the MMAs' own time is the phases' latency (first slices, last tile's epilogue, the group's meeting) and, below
+// n = 256, the start and finish of a submatrix.
+// Output tiles are 128 rows x up to 256 columns; the K dimension streams in slices of 32 through a four-stage TMA
+// pipeline; the epilogue writes the rounded planes back with TMA stores.
+// Warp roles: warp 0 (one thread) schedules the phases of the slots, decides convergence and publishes one descriptor
+// per phase in a small ring; warp 2 issues the loads and warp 1 tcgen05.mma, both converged with one elected lane;
+// warps 4-11 (two groups of four, even and odd 32-column chunks) drain the double-buffered TMEM accumulators
+// (2 x 256 columns) and start and finish the submatrices. All waits are bounded by the global timer; a wait that runs
+// out marks the submatrices in flight as timed out.
 //
 // The same kernel, instantiated in its second mode, prepares A_J = T_J(S)^-1 T_J(H0) on the tensor cores
 // by the coupled Newton-Schulz iteration for the inverse square root (Eqs. inv1-inv3): with Y_0 = T_J(S)/c
@@ -57,17 +61,15 @@ namespace nolsm {
 
 namespace {
 
-constexpr int kStages = 2;
-constexpr uint32_t kABytes = 128 * 64 * 2;        // one A plane slice: 128 rows x 64 K
+constexpr int kStages = 4;                        // K slices of 32 in flight
+constexpr uint32_t kABytes = 128 * 32 * 2;        // one A plane slice: 128 rows x 32 K
+constexpr uint32_t kBBlock = 32 * 64 * 2;         // one B plane slice of a column block: 32 K x 64 columns
 constexpr int kMaxEpiWarps = 12;
 
-// The two launch shapes. Warp 0 issues the TMA loads, warp 1 the MMAs; the epilogue warps from warp 4 on
-// come in groups of four (each group covers the 128 TMEM lanes) and deal a tile's 32-column chunks round
-// robin. Shape 0: 384 threads, two groups, tiles of 128 x up to 256 columns. Shape 1: 512 threads, three
-// groups, tiles of 128 x up to 192 columns (so that the twelve 4 KB staging buffers fit beside the two
-// operand stages), with a register split (below). Which one runs a bucket of submatrices is measured
-// (tc_shape): shape 0 wins for the sign iteration, shape 1 for the inverse square root, whose per-submatrix
-// start (operand pairs from T_J(S)) and T_J(H0) weigh more against its few products.
+// The two launch shapes. The epilogue warps from warp 4 on come in groups of four (each group covers the 128 TMEM lanes)
+// and deal a tile's 32-column chunks round robin. Shape 0: 384 threads, two groups, tiles of 128 x up to 256 columns.
+// Shape 1: 512 threads, three groups, tiles of 128 x up to 192 columns (so that the twelve 4 KB staging buffers fit
+// beside the operand stages). Which one runs a bucket of submatrices is measured (bucket_shape).
 template <int kShape>
 struct Shape {
   static constexpr int kThreads = kShape == 0 ? 384 : 512;
@@ -75,20 +77,20 @@ struct Shape {
   static constexpr int kEpiThreads = 32 * kEpiWarps;
   static constexpr int kGroups = kEpiWarps / 4;
   static constexpr int kTileN = kShape == 0 ? 256 : 192;       // N of one MMA
-  static constexpr uint32_t kBBytes = 64 * kTileN * 2;        // one B plane slice: 64 K x up to kTileN columns
-  static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;
+  static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBlock * (kTileN / 64);   // hi and lo
   static constexpr uint32_t kStgTotal = 4096 * kEpiWarps;    // a 4 KB hi/lo staging buffer per epilogue warp
   static constexpr int kSmemBytes = kStages * kStageBytes + kStgTotal + 1024;
+  // registers per thread: of the launch, of the first warpgroup, of the epilogue
+  static constexpr int kRegsLaunch = kShape == 0 ? 168 : 128, kRegsLow = kShape == 0 ? 72 : 56, kRegsEpi = kShape == 0 ? 216 : 152;
 };
 static_assert(Shape<1>::kEpiWarps <= kMaxEpiWarps && Shape<0>::kEpiWarps <= kMaxEpiWarps, "epilogue warps");
 static_assert(Shape<0>::kSmemBytes <= 227 * 1024 && Shape<1>::kSmemBytes <= 227 * 1024, "shared memory");
-// Register split of the 512-thread shape: the launch gives every thread kRegsLaunch registers (512 x 128 = the
-// SM's 65,536); the first warpgroup (TMA and MMA threads) releases down to kRegsLow and the three epilogue
-// warpgroups take kRegsEpi: 128 x 56 + 384 x 152 = 65,536, so the increase never waits on registers that do
-// not exist.
-constexpr int kRegsLaunch = 128, kRegsLow = 56, kRegsEpi = 152;
-static_assert(128 * kRegsLow + Shape<1>::kEpiThreads * kRegsEpi <= Shape<1>::kThreads * kRegsLaunch,
-              "register split above the launch");
+// The first warpgroup (TMA and MMA threads) releases registers down to kRegsLow and the epilogue warpgroups take
+// kRegsEpi, within what the launch gives the block, so the increase never waits on registers that do not exist.
+template <int kShape>
+constexpr bool split_fits = 128 * Shape<kShape>::kRegsLow + Shape<kShape>::kEpiThreads * Shape<kShape>::kRegsEpi <=
+                            Shape<kShape>::kThreads * Shape<kShape>::kRegsLaunch;
+static_assert(split_fits<0> && split_fits<1>, "register split above the launch");
 constexpr int kPlanes = 6;
 constexpr uint64_t kWaitNs = 2000000000ull;        // default limit per wait (2 s); one product takes < 1 ms
 
@@ -137,7 +139,13 @@ struct TcArgs {
   int32_t max_inv;
   int32_t again;              // only submatrices whose prep_out is kSubAgain (k_inv_res left them)
   double* flops;              // [2]: 2 n^3 per product (method count) and the split's issued flops, summed
+  int32_t group;              // CTAs that share a submatrix (the grid is a multiple of it)
+  struct GroupSlot* groups;   // [grid / group * kSlots], zeroed before the launch
 };
+
+// Views of the operand planes: A slices of 128 rows x 32 K, B slices of 32 K x 64 or 128 columns, of one plane or of hi
+// and lo; the epilogue's stores; E4M3's slices of 128 bytes.
+struct TcMaps { CUtensorMap A, A2, B, B2, Bx2, B2x2, S, S2, A8, B8; };
 
 // Epilogue of a product: what is done with the accumulator P
 enum : int {
@@ -151,11 +159,33 @@ constexpr int kPlanesInv = 10;   // inverse mode: plane pairs Y (then T_J(H0)), 
 constexpr int kSlots = 2;   // submatrices in flight per CTA (their products interleave)
 constexpr int kRing = 4;    // product descriptors between the scheduler and the MMA / epilogue warps
 
-// Iteration state of one in-flight submatrix. Written by the epilogue (thread 128) before it arrives
-// on the slot's epi_done barrier; read by the scheduler after waiting on that barrier.
+// The CTAs of a group run the same sequence of phases in each of the group's slots: a phase (a fetch, a turn, a fill or
+// a product) ends when every CTA of the group has arrived on count, and then every scheduler derives the next one from
+// the same numbers. Per (group, slot) in global memory:
+constexpr int kMaxGroup = 16;
+struct alignas(128) GroupSlot {
+  uint32_t count;                // arrivals so far
+  int32_t next;                  // fetch: the next submatrix, or -1
+  float part[2][kMaxGroup];      // the CTAs' shares of the defect, by the phase's parity
+  double tr[3][kMaxGroup];       // turn: their shares of the traces
+};
+
+// What a descriptor asks for
+enum : int {
+  kOpFetch = 0,   // (no descriptor) the first CTA of the group draws the next submatrix
+  kOpTurn = 1,    // finish the slot's submatrix and start the next
+  kOpFill = 2,    // inverse mode: T_J(H0) into Y's pair
+  kOpProd = 3     // a product
+};
+
+// Iteration state of one in-flight submatrix: the scheduler's.
 struct SlotState {
-  int job;                       // submatrix index, -1 when the slot has retired
-  int n, n64, R, nrb, ncb, nks;  // dimension and tiling
+  int job, fin;                  // submatrix index, -1 for none; the one that a turn finishes
+  int next;                      // fetch: the next one, as drawn by this CTA
+  int op, rot;                   // phase under way; the CTA of tile 0 of the next product
+  uint32_t seq, epar;            // phases begun; parity of this CTA's next epi_done
+  bool alive, local;             // not retired; this CTA's epilogue is still to report
+  int n, n64, R, nrb, ncb;       // dimension and tiling
   int kind;                      // next product: 0 (X X) or 1 (X T)
   int cur;                       // which X plane pair holds the current iterate
   int phase, refine_left, steps, rsteps, status, last;
@@ -171,9 +201,12 @@ struct SlotState {
 // One product as scheduled by the producer: read in order by the MMA issuer and the epilogue.
 struct Desc {
   int term;                      // 1: no more products, exit
-  int slot, kind, last;
+  int op, slot, kind, par;       // kOp*; parity of the phase
+  int job, fin;                  // the submatrix (turn: to start), the one that a turn finishes
+  int t0;                        // this CTA's first tile (then every group-th)
+  int fill;                      // inverse mode: plane that T_J(H0) goes to at the product's end, -1: none
   Fmt f, fo;                     // format of the operands; of the operand the epilogue writes
-  int n, n64, nrb, ncb, nks;
+  int n, n64, nrb, ncb;
   int za, zb, zo;                // plane indices (hi planes) of A, B and the output
   int epi;                       // kEpi*
   float scale;                   // kEpiScale, kEpiX
@@ -182,80 +215,74 @@ struct Desc {
 
 struct Shared {
   uint64_t full[kStages], empty[kStages], accf[2], acce[2], idle;
-  uint64_t epi_done[kSlots], desc_full[kRing];
+  uint64_t epi_done[kSlots], desc_full[kRing], desc_free[kRing];
   uint32_t tmem;
   int err;
-  int fetch;
   SlotState slot[kSlots];
+  float part[kSlots];            // a group of one: its GroupSlot's part and tr
+  double tr[kSlots][3];
+  float cinv[kSlots];            // inverse mode: 1 / c of the submatrix just started
   Desc ring[kRing];
   float red[2][kMaxEpiWarps];    // defect partial sums, by product parity
   double dred[3][kMaxEpiWarps];
 };
 
-// 32 consecutive values of one row as packed hi (and lo) pairs; the format a template parameter (one
-// branch per chunk, none per pair), the lo parts only when the format has them.
+// Eight rows of X a warp (2-byte hi and, with kLo, lo planes, columns k0 .. k0 + kn - 1, kn a multiple of 32) times 8
+// columns of Q in FP32 (staged from row k0 on): four lanes a row, each 8 adjacent columns of every 32, so that a load
+// reads 64 consecutive bytes of a row. FP32 sums of 8 products, each added to s + e with TwoSum; then the four lanes'
+// sums together, the same in each of them.
+__device__ __forceinline__ int qs_at(int k) { return 8 * k + 4 * (k >> 3); }   // four lanes' rows in different banks
 template <int kFmt, bool kLo>
-__device__ __forceinline__ void split_pack_t(const float (&v)[32], uint32_t (&h)[16], uint32_t (&l)[16]) {
+__device__ __forceinline__ void xq_rows(const uint16_t* __restrict__ xh, const uint16_t* __restrict__ xl, int kn,
+                                        const float* __restrict__ Qs, int part, uint64_t (&s)[4], uint64_t (&e)[4]) {
+  const uint64_t neg = pair2(-1.0f, -1.0f);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (kLo) {
-      split2(v[2 * j], v[2 * j + 1], kFmt, h[j], l[j]);
-    } else if (kFmt == FMT_BF16) {
-      const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-      h[j] = *reinterpret_cast<const uint32_t*>(&b);
-    } else {
-      const __half2 b = __floats2half2_rn(v[2 * j], v[2 * j + 1]);
-      h[j] = *reinterpret_cast<const uint32_t*>(&b);
-    }
-  }
-}
-__device__ __forceinline__ void split_pack(const float (&v)[32], Fmt f, uint32_t (&h)[16], uint32_t (&l)[16]) {
-  if (f.fmt == FMT_BF16) {
-    if (f.terms > 1) split_pack_t<FMT_BF16, true>(v, h, l);
-    else split_pack_t<FMT_BF16, false>(v, h, l);
-  } else {
-    if (f.terms > 1) split_pack_t<FMT_F16, true>(v, h, l);
-    else split_pack_t<FMT_F16, false>(v, h, l);
-  }
-}
-
-// One row of X (2-byte hi and, with kLo, lo planes; n64 columns, zero padded) times 8 columns of Q in
-// FP32 (rows of stride bp, zero padded to n64 rows): FP32 partial sums of 16 products, each added to
-// sh + sl with TwoSum. The row is read in 32-column pieces, eight 16-byte loads in flight.
-template <int kFmt, bool kLo>
-__device__ __forceinline__ void xq_row(const uint16_t* __restrict__ xh, const uint16_t* __restrict__ xl, int n64,
-                                       const float* __restrict__ Qs, int bp, float (&sh)[8], float (&sl)[8]) {
-#pragma unroll
-  for (int c = 0; c < 8; ++c) sh[c] = sl[c] = 0.0f;
-  for (int k0 = 0; k0 < n64; k0 += 32) {
+  for (int c = 0; c < 4; ++c) s[c] = e[c] = 0;
+  auto add = [&](int c, uint64_t p) {   // TwoSum in pairs
+    const uint64_t t = add2(s[c], p), z = fma2(s[c], neg, t);
+    e[c] = add2(e[c], add2(fma2(fma2(z, neg, t), neg, s[c]), fma2(z, neg, p)));
+    s[c] = t;
+  };
+#pragma unroll 1
+  for (int k0 = 8 * part; k0 < kn; k0 += 128) {
     uint4 hv[4], lv[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      hv[t] = *reinterpret_cast<const uint4*>(xh + k0 + 8 * t);
-      lv[t] = kLo ? *reinterpret_cast<const uint4*>(xl + k0 + 8 * t) : make_uint4(0, 0, 0, 0);
+    for (int t = 0; t < 4; ++t) {   // (past the end the last piece again)
+      const int k = min(k0 + 32 * t, kn - 32 + 8 * part);
+      hv[t] = *reinterpret_cast<const uint4*>(xh + k);
+      lv[t] = kLo ? *reinterpret_cast<const uint4*>(xl + k) : make_uint4(0, 0, 0, 0);
     }
-    float p[8];
 #pragma unroll
-    for (int u = 0; u < 32; ++u) {
-      if ((u & 15) == 0) {
+    for (int t = 0; t < 4; ++t) {
+      const int k = k0 + 32 * t;
+      if (k >= kn) break;
+      uint64_t p[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int c = 0; c < 8; ++c) p[c] = 0.0f;
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t h = u < 2 ? hv[t].x : u < 4 ? hv[t].y : u < 6 ? hv[t].z : hv[t].w;
+        const uint32_t l = u < 2 ? lv[t].x : u < 4 ? lv[t].y : u < 6 ? lv[t].z : lv[t].w;
+        float x = from_bits((uint16_t)(h >> (16 * (u & 1))), kFmt);
+        if (kLo) x += from_bits((uint16_t)(l >> (16 * (u & 1))), kFmt);
+        const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u);
+        const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u + 4);
+        const uint64_t xx = pair2(x, x);
+        p[0] = fma2(xx, qa.x, p[0]);
+        p[1] = fma2(xx, qa.y, p[1]);
+        p[2] = fma2(xx, qb.x, p[2]);
+        p[3] = fma2(xx, qb.y, p[3]);
       }
-      const uint4 h4 = hv[u >> 3], l4 = lv[u >> 3];
-      const int w = (u & 7) >> 1, sft = 16 * (u & 1);
-      const uint32_t hw = w == 0 ? h4.x : w == 1 ? h4.y : w == 2 ? h4.z : h4.w;
-      const uint32_t lw = w == 0 ? l4.x : w == 1 ? l4.y : w == 2 ? l4.z : l4.w;
-      float x = from_bits((uint16_t)(hw >> sft), kFmt);
-      if (kLo) x += from_bits((uint16_t)(lw >> sft), kFmt);
-      const float4 qa = *reinterpret_cast<const float4*>(Qs + (size_t)(k0 + u) * bp);
-      const float4 qb = *reinterpret_cast<const float4*>(Qs + (size_t)(k0 + u) * bp + 4);
-      const float qv[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
 #pragma unroll
-      for (int c = 0; c < 8; ++c) p[c] = fmaf(x, qv[c], p[c]);
-      if ((u & 15) == 15) {
+      for (int c = 0; c < 4; ++c) add(c, p[c]);
+    }
+  }
 #pragma unroll
-        for (int c = 0; c < 8; ++c) two_sum(sh[c], sl[c], p[c]);
-      }
+  for (int o = 1; o < 4; o <<= 1) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint64_t so = __shfl_xor_sync(0xffffffffu, (unsigned long long)s[c], o);
+      const uint64_t eo = __shfl_xor_sync(0xffffffffu, (unsigned long long)e[c], o);
+      add(c, so);
+      e[c] = add2(e[c], eo);
     }
   }
 }
@@ -275,25 +302,15 @@ __device__ __forceinline__ bool epi_bar_or(bool p) {
   return r != 0;
 }
 
-// Whether row tile mb of a product is an M = 64 tile: the last one of a kind::f16 product whose n64 is an odd
-// multiple of 64 (n = 129..192 runs as 128 + 64 rows instead of 2 x 128). Its accumulator rows r sit in TMEM
-// lanes 32 (r / 16) + r % 16, the first 16 lanes of each warp's quarter.
-__device__ __forceinline__ bool tail64(const Desc& d, int mb) {
-  return d.f.fmt != FMT_E4M3 && d.fo.fmt != FMT_E4M3 && mb == d.nrb - 1 && (d.n64 & 127) == 64;
-}
-
 // kMode 0: the sign iteration (a4-a7); kMode 1: the inverse square root of T_J(S) and A_J (a2-a3); kShape:
 // the launch shape (Shape)
 template <int kMode, int kShape>
 __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
-    k_ns_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-            const __grid_constant__ CUtensorMap mapS, const __grid_constant__ CUtensorMap mapA8,
-            const __grid_constant__ CUtensorMap mapB8, const __grid_constant__ CUtensorMap mapS16,
-            const __grid_constant__ CUtensorMap mapS2, const __grid_constant__ CUtensorMap mapS16x2, TcArgs g) {
+    k_ns_tc(const __grid_constant__ TcMaps maps, TcArgs g) {
   constexpr int kPps = kMode == 0 ? kPlanes : kPlanesInv;   // planes per slot
   constexpr int kEpiWarps = Shape<kShape>::kEpiWarps, kEpiThreads = Shape<kShape>::kEpiThreads;
   constexpr int kGroups = Shape<kShape>::kGroups, kTileN = Shape<kShape>::kTileN;
-  constexpr uint32_t kBBytes = Shape<kShape>::kBBytes, kStageBytes = Shape<kShape>::kStageBytes;
+  constexpr uint32_t kStageBytes = Shape<kShape>::kStageBytes;
   constexpr uint32_t kStgTotal = Shape<kShape>::kStgTotal;
   extern __shared__ uint8_t smraw[];
   uint8_t* stage_mem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
@@ -310,18 +327,13 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
       tc::mbar_init(&sh.acce[b], kEpiThreads);
     }
     for (int s = 0; s < kSlots; ++s) tc::mbar_init(&sh.epi_done[s], kEpiThreads);
-    for (int r = 0; r < kRing; ++r) tc::mbar_init(&sh.desc_full[r], 1);
+    for (int r = 0; r < kRing; ++r) {
+      tc::mbar_init(&sh.desc_full[r], 1);
+      tc::mbar_init(&sh.desc_free[r], 3);   // loader, MMA issuer, epilogue
+    }
     tc::mbar_init(&sh.idle, 1);
     tc::fence_mbar_init();
     sh.err = 0;
-    tc::prefetch_tmap(&mapA);
-    tc::prefetch_tmap(&mapB);
-    tc::prefetch_tmap(&mapS);
-    tc::prefetch_tmap(&mapA8);
-    tc::prefetch_tmap(&mapB8);
-    tc::prefetch_tmap(&mapS16);
-    tc::prefetch_tmap(&mapS2);
-    tc::prefetch_tmap(&mapS16x2);
   }
   if (warp == 0) {
     tc::tmem_alloc(&sh.tmem, 512);
@@ -333,39 +345,305 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
   const uint32_t tmem = sh.tmem;
   const size_t plane_elems = (size_t)g.R * g.LD;
   uint8_t* const stg = stage_mem + kStages * kStageBytes;   // epilogue staging: 4 KB per epilogue warp
-  const int sub0 = blockIdx.x * kSlots;                      // scratch sub-slot of this CTA's slot 0
-  uint32_t arm_phase[kStages] = {0, 0};                      // producer: parity of the last load armed per stage
-  bool armed[kStages] = {false, false};
+  // the group's CTAs share its slots: rank 0 draws the submatrices, tiles and rows are dealt in turn
+  const int G = g.group, gid = blockIdx.x / G, rank = blockIdx.x - gid * G;
+  GroupSlot* const gs = g.groups + (size_t)gid * kSlots;
+  const int sub0 = gid * kSlots;                             // scratch sub-slot of the group's slot 0
+  uint32_t loads = 0;                                        // loader: K slices armed so far
 
   if (warp < 4) {
-  if constexpr (kShape == 1) tc::setmaxnreg_dec<kRegsLow>();   // the TMA / MMA warpgroup gives registers up
+  tc::setmaxnreg_dec<Shape<kShape>::kRegsLow>();   // the TMA / MMA warpgroup gives registers up
   if (warp == 0 && lane == 0) {
-    // ------------------------------------------------ producer: schedules the products of the slots
-    // a slot's next product is issued once the epilogue of its previous product (or its initialisation) has
-    // arrived on the slot's epi_done barrier; the live slots are polled round robin from the one after the
-    // last pick, and the first that is ready goes (no slot waits behind another's epilogue)
-    bool alive[kSlots];
-    uint32_t epar[kSlots];
+    // ------------------------------------------------ producer: schedules the phases of the slots
+    // a slot's next phase is issued once the previous one has ended in every CTA of the group; the live slots are
+    // polled round robin from the one after the last pick, and the first that is ready goes (no slot waits behind
+    // another's epilogue)
+    auto fetch = [&]() -> int {
+      for (;;) {
+        const int k = atomicAdd(g.next, 1);
+        if (k >= g.j1 - g.j0 || sh.err) return -1;
+        const int J = g.order[k];
+        if constexpr (kMode == 1) {
+          if (g.again && g.prep_out[J] != kSubAgain) continue;
+          return J;
+        }
+        if (g.sub_n[J] <= g.above_n) continue;
+        if (g.cond && g.prep_status[J] == kSubOk && g.cond[J] > g.cond_max && g.sub_n[J] <= g.ill_max_n) continue;
+        if (g.prep_status[J] == kSubOk) return J;
+        g.status[J] = g.prep_status[J];
+        g.iters[J] = 0;
+        g.rsteps[J] = 0;
+        g.tS[J] = 0.0;
+        g.tH[J] = 0.0;
+      }
+    };
+    auto begin_fetch = [&](int c) {
+      SlotState& st = sh.slot[c];
+      st.op = kOpFetch;
+      ++st.seq;
+      st.local = false;
+      if (rank == 0) {
+        st.next = fetch();
+        if (G > 1) __stcg(&gs[c].next, st.next);
+      }
+      if (G > 1) tc::red_release_gpu(&gs[c].count, 1u);
+    };
+    auto ready = [&](int c) -> bool {
+      SlotState& st = sh.slot[c];
+      if (st.local) {
+        if (!tc::mbar_test_wait(&sh.epi_done[c], st.epar)) return false;
+        st.epar ^= 1;
+        st.local = false;
+      }
+      return G == 1 || tc::reached_gpu(&gs[c].count, (uint32_t)G * st.seq);
+    };
+    auto defect = [&](int c) -> float {   // the phase's sum over the group, in an order that the slot does not change
+      if (G == 1) return sh.part[c];
+      float d = 0.0f;
+      for (int r = 0; r < G; ++r) d += __ldcg(&gs[c].part[sh.slot[c].seq & 1][r]);
+      return d;
+    };
+    // the phase under way in slot c has ended: its results, and the next phase's descriptor; false when that phase
+    // needs none (a fetch) or the slot has retired
+    auto advance = [&](int c, Desc& d) -> bool {
+      SlotState& st = sh.slot[c];
+      const int zb = (sub0 + c) * kPps;
+      d.term = 0;
+      d.slot = c;
+      d.fill = -1;
+      bool fill = false;
+      if (st.op == kOpFetch) {
+        const int J = rank == 0 ? st.next : __ldcg(&gs[c].next);
+        if (J < 0 && st.job < 0) {
+          st.alive = false;
+          return false;
+        }
+        d.op = st.op = kOpTurn;
+        d.fin = st.fin = kMode == 0 ? st.job : -1;
+        d.n = st.n; d.n64 = st.n64;
+        d.za = zb + 2 * st.cur;
+        d.f = st.fcur;
+        d.job = st.job = J;
+        // X_0 goes into the other pair: other CTAs of the group may still read the finished X. (E4M3 runs in groups of one.)
+        if (g.main_fmt.fmt == FMT_E4M3) st.cur = 0;
+        else st.cur ^= 1;
+        d.zo = zb + 2 * st.cur;
+        st.rot = c * (G / 2);
+      } else {
+        if (st.op == kOpTurn) {
+          if (kMode == 0 && st.fin >= 0) {
+            if (rank == 0) {
+              double t[3] = {0.0, 0.0, 0.0};
+              for (int r = 0; r < G; ++r)
+                for (int k = 0; k < 3; ++k) t[k] += G == 1 ? sh.tr[c][k] : __ldcg(&gs[c].tr[k][r]);
+              const int J = st.fin;
+              if (g.nbelow) g.nbelow[J] = (int32_t)lrint(0.5 * (st.n - t[2]));
+              int stt = st.status;
+              if (stt == kSubOk && !(isfinite(t[0]) && isfinite(t[1]))) stt = kSubNonFinite;
+              g.tS[J] = t[0];
+              g.tH[J] = t[1];
+              g.iters[J] = st.steps;
+              g.rsteps[J] = st.rsteps;
+              g.status[J] = stt;
+            }
+            st.fin = -1;
+          }
+          if (st.job < 0) {
+            st.alive = false;
+            return false;
+          }
+          st.n = g.sub_n[st.job];
+          st.n64 = (st.n + 63) & ~63;
+          st.R = (st.n + 127) & ~127;
+          st.nrb = st.R / 128; st.ncb = (st.n64 + kTileN - 1) / kTileN;
+          st.dprev = INFINITY;
+          st.last = 0;
+          st.rsteps = 0;
+          if constexpr (kMode == 0) {
+            st.kind = 0;
+            st.phase = 0; st.refine_left = g.refine_steps; st.steps = 0;
+            st.status = kSubNotConv;
+            st.fcur = g.main_fmt; st.fnxt = g.main_fmt;
+          } else {
+            st.yc = 0; st.zc = 1; st.cinv = sh.cinv[c]; st.zs = 0.5f;
+            st.steps = 1; st.status = kSubOk;
+            st.fcur = Fmt{FMT_F16, 3}; st.fnxt = st.fcur;
+            const float d0 = sqrtf(defect(c) / (float)st.n);   // not finite when c was not positive
+            st.zdone = 1;
+            st.last = d0 <= g.tol_inv ? 1 : 0;
+            st.kind = st.last ? 3 : 1;     // step 0 the last: X = Z_1 Z_1 / c next; else Y_1 = Y_0 T_0 / 2
+            fill = st.last && g.Aout;      // Y_0 is not needed: T_J(H0) takes its pair (else after the last Z update)
+            if (!isfinite(d0)) {           // the FP64 preparation takes it
+              st.status = kSubRefine;
+              st.kind = 5;
+            }
+          }
+        } else if (st.op == kOpProd) {
+          if constexpr (kMode == 1) {
+            switch (st.kind) {
+              case 0: {
+                const float dd = sqrtf(defect(c) / (float)st.n);
+                st.steps += 1;
+                if (!isfinite(dd) || (dd > g.tol_inv && st.steps >= g.max_inv)) {
+                  st.status = kSubRefine;   // diverged or too slow: the FP64 preparation takes it
+                  st.last = 1;
+                } else if (dd <= g.tol_inv) {
+                  st.last = 1;                // this step's Z update is the last product of the iteration
+                }
+                st.kind = st.last ? 2 : 1;
+                break;
+              }
+              case 1:   // after Y's update: Z's, unless the step's Z update was made at the start
+                if (st.ncb != 1) st.yc = st.yc == 0 ? 3 : 0;
+                st.kind = st.zdone ? 0 : 2;
+                st.zdone = 0;
+                break;
+              case 2: st.zc = st.zc == 1 ? 4 : 1; st.zs = 1.0f; st.kind = st.last ? 3 : 0; break;
+              case 3: st.kind = g.Aout ? 4 : 5; break;
+              default: st.kind = 5; break;
+            }
+          } else if (st.kind == 0) {
+            // defect of X_step and the decision about the following steps
+            const float dd = sqrtf(defect(c) / (float)st.n);
+            const int steps = st.steps + 1;
+            if (st.phase == 1) st.rsteps += 1;   // this step ran in the refinement format
+            int last_ = 0, status = kSubNotConv;
+            Fmt nxt = st.fcur;
+            if (!isfinite(dd)) {
+              last_ = 1;
+              status = kSubNonFinite;
+            } else if (st.phase == 0) {
+              // E4M3 iterates carry a rounding error of up to 2^-4 relative, which holds the defect at a floor
+              // near 0.05, well above tol_ns: their phase ends at twice that floor, or when the defect has
+              // stopped falling (below 0.25, where the exact iteration would at least halve it every step)
+              const bool f8_end = st.fcur.fmt == FMT_E4M3 && (dd <= kF8Switch || (dd < 0.25f && dd > 0.5f * st.dprev));
+              if (dd <= g.tol_ns || f8_end) {
+                if (g.refine_steps == 0) {
+                  last_ = 1;
+                  status = dd <= g.tol_accept ? kSubOk : kSubNotConv;
+                } else {
+                  st.phase = 1;
+                  st.refine_left = g.refine_steps;
+                  nxt = g.refine_fmt;
+                }
+              }
+            } else if (--st.refine_left <= 0) {
+              if (dd <= g.tol_accept) {
+                last_ = 1;
+                status = kSubOk;
+              } else if (dd < st.dprev) {
+                st.refine_left = 1;   // still converging: one more step (bounded by the step cap below)
+              } else {
+                last_ = 1;
+                status = kSubNotConv;
+              }
+            }
+            const int cap = g.budget ? min(g.max_iter, g.budget[st.job]) : g.max_iter;
+            if (!last_ && steps >= cap) {
+              last_ = 1;
+              status = kSubNotConv;
+            }
+            st.dprev = dd;
+            st.steps = steps;
+            st.last = last_;
+            st.status = status;
+            st.fnxt = nxt;
+            st.kind = 1;
+          } else {
+            // after X T: X_{k+1} is the current X (ping-pong unless written in place), in the next format
+            if (st.ncb != 1) st.cur ^= 1;
+            st.fcur = st.fnxt;
+            st.kind = st.last ? 5 : 0;
+          }
+        }
+        if (st.kind == 5) {   // the submatrix is done
+          if (kMode == 1) {
+            if (rank == 0) {
+              g.prep_out[st.job] = st.status;
+              const double n3 = (double)st.n * st.n * st.n;
+              // step 0 needs one product (Y_1), every further step three but the last two (no Y update); then X, A
+              const double prods = 3.0 * st.steps - (g.Aout ? 1.0 : 2.0);
+              atomicAdd(&g.flops[0], 2.0 * n3 * prods);
+              atomicAdd(&g.flops[1], 6.0 * n3 * prods);
+            }
+            st.job = -1;
+          }
+          begin_fetch(c);
+          return false;
+        }
+        d.job = st.job;
+        d.n = st.n; d.n64 = st.n64; d.nrb = st.nrb; d.ncb = st.ncb;
+        d.f = st.fcur;
+        d.kind = st.kind;
+        if (fill) {
+          d.op = st.op = kOpFill;
+          d.fill = zb;
+        } else {
+          d.op = st.op = kOpProd;
+          d.t0 = (rank - st.rot + G) % G;
+          st.rot = (st.rot + st.nrb * st.ncb) % G;
+          d.pscale = 1.0f;
+          if constexpr (kMode == 0) {   // the epilogue derives epi and scale from the kind
+            d.fo = st.kind == 0 ? st.fcur : st.fnxt;
+            d.za = zb + 2 * st.cur;
+            d.zb = st.kind == 0 ? d.za : zb + 4;
+            // X_{k+1} overwrites X_k when one column tile covers the matrix: row block mb of X_k is read
+            // (as the A operand) only by tile (mb, 0), whose loads have completed before its epilogue writes
+            d.zo = st.kind == 0 ? zb + 4 : (st.ncb == 1 ? d.za : zb + 2 * (st.cur ^ 1));
+          } else {
+            // pairs: Y in 0 (updated in place when one column tile covers the matrix, else ping-pong with 3),
+            // Z in 1 or 4 (ping-pong: every row tile of T Z reads all of Z; until the first Z update the pair
+            // holds T_0 = 2 Z_1, hence the factor zs), T and then X in 2; T_J(H0) goes into Y's pair once Y is
+            // no longer needed
+            d.scale = 0.5f;
+            d.fo = st.fcur;
+            switch (st.kind) {
+              case 0:  // V = Z Y -> T = 3I - V
+                d.za = zb + 2 * st.zc; d.zb = zb + 2 * st.yc; d.zo = zb + 4; d.epi = kEpiT; d.pscale = st.zs; break;
+              case 1:  // Y' = 1/2 Y T (row block mb of Y is read only by tile (mb, 0), as for X X T); at step 0
+                       // T_0 is in Z's pair
+                d.za = zb + 2 * st.yc; d.zb = st.zdone ? zb + 2 * st.zc : zb + 4;
+                d.zo = st.ncb == 1 ? d.za : zb + 2 * (st.yc == 0 ? 3 : 0);
+                d.epi = kEpiScale; break;
+              case 2:  // Z' = 1/2 T Z; after the last one Y (last read by this step's V = Z Y) makes room for T_J(H0)
+                d.za = zb + 4; d.zb = zb + 2 * st.zc; d.zo = zb + 2 * (st.zc == 1 ? 4 : 1); d.epi = kEpiScale;
+                d.scale = 0.5f * st.zs;
+                if (st.last && g.Aout) d.fill = zb + 2 * st.yc;
+                break;
+              case 3:  // X = Z Z / c = T_J(S)^-1
+                d.za = zb + 2 * st.zc; d.zb = d.za; d.zo = zb + 4; d.epi = kEpiX; d.scale = st.cinv * st.zs * st.zs;
+                break;
+              default:  // A_J = X T_J(H0)
+                d.za = zb + 4; d.zb = zb + 2 * st.yc; d.zo = zb + 4; d.epi = kEpiA; break;
+            }
+          }
+        }
+      }
+      ++st.seq;
+      st.local = true;
+      d.par = st.seq & 1;
+      return true;
+    };
+
     for (int c = 0; c < kSlots; ++c) {
-      alive[c] = true;
-      epar[c] = 0;
+      sh.slot[c].job = sh.slot[c].fin = -1;
+      sh.slot[c].alive = true;
+      sh.slot[c].seq = sh.slot[c].epar = 0;
+      sh.slot[c].cur = 0;
+      begin_fetch(c);
     }
-    uint32_t kcount = 0;
+    uint32_t kcount = 0, i = 0;
     int s = 0;
-    for (uint32_t i = 0;; ++i) {
+    for (;;) {
       int pick = -1;
       const uint64_t deadline = tc::globaltimer() + 4 * g.wait_ns;
       for (;;) {
         bool any = false;
         for (int t = 0; t < kSlots && pick < 0; ++t) {
           const int c = (s + t) % kSlots;
-          if (!alive[c]) continue;
+          if (!sh.slot[c].alive) continue;
           any = true;
-          if (!tc::mbar_test_wait(&sh.epi_done[c], epar[c])) continue;
-          epar[c] ^= 1;
-          tc::fence_proxy_async_global();   // the epilogue's plane writes, before TMA reads them
-          if (sh.slot[c].job >= 0) pick = c;
-          else alive[c] = false;
+          if (ready(c)) pick = c;
         }
         if (pick >= 0 || !any || sh.err) break;
         if (tc::globaltimer() > deadline) {
@@ -374,171 +652,149 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
         }
       }
       Desc d;
-      d.term = pick < 0 ? 1 : 0;
+      d.term = 1;
       if (pick >= 0) {
-        const SlotState& st = sh.slot[pick];
-        d.slot = pick;
-        d.kind = st.kind;
-        d.f = st.fcur;
-        d.n = st.n; d.n64 = st.n64; d.nrb = st.nrb; d.ncb = st.ncb; d.nks = st.nks;
-        const int zb = (sub0 + pick) * kPps;
-        d.pscale = 1.0f;
-        if constexpr (kMode == 0) {   // the epilogue derives epi and scale from the kind
-          d.last = st.kind == 1 && st.last;
-          d.fo = st.kind == 0 ? st.fcur : st.fnxt;
-          d.za = zb + 2 * st.cur;
-          d.zb = st.kind == 0 ? d.za : zb + 4;
-          // X_{k+1} overwrites X_k when one column tile covers the matrix: row block mb of X_k is read
-          // (as the A operand) only by tile (mb, 0), whose loads have completed before its epilogue writes
-          d.zo = st.kind == 0 ? zb + 4 : (st.ncb == 1 ? d.za : zb + 2 * (st.cur ^ 1));
-        } else {
-          // pairs: Y in 0 (updated in place when one column tile covers the matrix, else ping-pong with 3),
-          // Z in 1 or 4 (ping-pong: every row tile of T Z reads all of Z; until the first Z update the pair
-          // holds T_0 = 2 Z_1, hence the factor zs), T and then X in 2; T_J(H0) goes into Y's pair once Y is
-          // no longer needed
-          d.last = st.kind == 4 || (st.kind == 3 && !g.Aout);
-          d.scale = 0.5f;
-          d.fo = st.fcur;
-          switch (st.kind) {
-            case 0:  // V = Z Y -> T = 3I - V
-              d.za = zb + 2 * st.zc; d.zb = zb + 2 * st.yc; d.zo = zb + 4; d.epi = kEpiT; d.pscale = st.zs; break;
-            case 1:  // Y' = 1/2 Y T (row block mb of Y is read only by tile (mb, 0), as for X X T); at step 0
-                     // T_0 is in Z's pair
-              d.za = zb + 2 * st.yc; d.zb = st.zdone ? zb + 2 * st.zc : zb + 4;
-              d.zo = st.ncb == 1 ? d.za : zb + 2 * (st.yc == 0 ? 3 : 0);
-              d.epi = kEpiScale; break;
-            case 2:  // Z' = 1/2 T Z
-              d.za = zb + 4; d.zb = zb + 2 * st.zc; d.zo = zb + 2 * (st.zc == 1 ? 4 : 1); d.epi = kEpiScale;
-              d.scale = 0.5f * st.zs; break;
-            case 3:  // X = Z Z / c = T_J(S)^-1
-              d.za = zb + 2 * st.zc; d.zb = d.za; d.zo = zb + 4; d.epi = kEpiX; d.scale = st.cinv * st.zs * st.zs;
-              break;
-            default:  // A_J = X T_J(H0)
-              d.za = zb + 4; d.zb = zb + 2 * st.yc; d.zo = zb + 4; d.epi = kEpiA; break;
-          }
-        }
+        s = (pick + 1) % kSlots;
+        if (!advance(pick, d)) continue;
       }
-      sh.ring[i % kRing] = d;
-      tc::mbar_arrive(&sh.desc_full[i % kRing]);
-      if (d.term) break;
-      const int two = d.f.terms > 1 ? 2 : 1;
-      const bool f8 = d.f.fmt == FMT_E4M3;
-      const int nks = f8 ? k8_extent(d.n64) / 128 : d.nks;   // E4M3: 128-byte K slices
-      for (int mb = 0; mb < d.nrb && !sh.err; ++mb)
-        for (int cb = 0; cb < d.ncb && !sh.err; ++cb) {
-          const int nt = min(kTileN, d.n64 - kTileN * cb);
-          // an M = 64 tile loads 64 rows of A (the B map's 64 x 64 box)
-          const bool m64 = tail64(d, mb);
-          const uint32_t abytes = m64 ? kABytes / 2 : kABytes;
-          // E4M3: both operands K-major (the symmetric iterate is its own transpose); the B box is always
-          // kTileN rows (rows past R are zero-filled by the copy)
-          const uint32_t bytes = f8 ? kABytes + (uint32_t)kTileN * 128u : (uint32_t)two * (abytes + (uint32_t)nt * 128u);
-          for (int ks = 0; ks < nks; ++ks) {
-            const int st = kcount % kStages;
-            const uint32_t ph = (kcount / kStages) & 1;
-            if (!tc::mbar_wait(&sh.empty[st], ph ^ 1, tc::globaltimer() + g.wait_ns)) { sh.err = 1; break; }
-            uint8_t* sm = stage_mem + st * kStageBytes;
-            tc::mbar_arrive_expect_tx(&sh.full[st], bytes);
-            armed[st] = true;
-            arm_phase[st] = ph;
-            if (f8) {
-              tc::tma_load_3d(sm, &mapA8, &sh.full[st], 128 * ks, 128 * mb, d.za);
-              tc::tma_load_3d(sm + 2 * kABytes, &mapB8, &sh.full[st], 128 * ks, kTileN * cb, d.zb);
-            } else {
-              for (int z = 0; z < two; ++z) {
-                tc::tma_load_3d(sm + z * kABytes, m64 ? &mapB : &mapA, &sh.full[st], 64 * ks, 128 * mb, d.za + z);
-                uint8_t* bdst = sm + 2 * kABytes + z * kBBytes;
-                for (int c = 0; c < nt / 64; ++c)
-                  tc::tma_load_3d(bdst + c * 8192, &mapB, &sh.full[st], kTileN * cb + 64 * c, 64 * ks, d.zb + z);
-              }
-            }
-            ++kcount;
-          }
-        }
-      s = (pick + 1) % kSlots;
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------ MMA issuer: the products in the scheduler's order
-    uint32_t kcount = 0, tcount = 0;
-    for (uint32_t i = 0; !sh.err; ++i) {
-      if (!tc::mbar_wait(&sh.desc_full[i % kRing], (i / kRing) & 1, tc::globaltimer() + 8 * g.wait_ns)) {
+      if (i >= kRing && !tc::mbar_wait_ns(&sh.desc_free[i % kRing], ((i / kRing) & 1) ^ 1, 8 * g.wait_ns)) {
         sh.err = 1;
         break;
       }
-      const Desc d = sh.ring[i % kRing];
+      sh.ring[i % kRing] = d;
+      tc::mbar_arrive(&sh.desc_full[i % kRing]);
+      ++i;
       if (d.term) break;
-      const bool f8 = d.f.fmt == FMT_E4M3;
-      const int nks = f8 ? k8_extent(d.n64) / 128 : d.nks;
-      // kind::f16 products run over n16 = n rounded up to 16 in N and K (the loads stay whole 64-wide slices):
-      // the operands' rows and columns past n are zero, so the entries the trimmed product leaves out are 0
-      const int n16 = (d.n + 15) & ~15;
-      for (int mb = 0; mb < d.nrb && !sh.err; ++mb)
-        for (int cb = 0; cb < d.ncb && !sh.err; ++cb) {
-          const int nt = min(kTileN, d.n64 - kTileN * cb);
-          const int ntu = min(nt, n16 - kTileN * cb);
-          // kind::f16: A K-major, B MN-major; kind::f8f6f4 (E4M3 = 0): both K-major
-          const uint32_t id = f8 ? tc::idesc(0, 0, 0, 0, 128, nt)
-                                 : tc::idesc(d.f.fmt, d.f.fmt, 0, 1, tail64(d, mb) ? 64 : 128, ntu);
-          const int buf = tcount & 1;
-          if (!tc::mbar_wait(&sh.acce[buf], ((tcount >> 1) & 1) ^ 1, tc::globaltimer() + g.wait_ns)) {
-            sh.err = 1;
-            break;
-          }
-          tc::tc_fence_after();
-          const uint32_t dt = tmem + (uint32_t)buf * 256;
-          for (int ks = 0; ks < nks; ++ks) {
-            const int st = kcount % kStages;
-            const uint32_t ph = (kcount / kStages) & 1;
-            if (!tc::mbar_wait(&sh.full[st], ph, tc::globaltimer() + g.wait_ns)) { sh.err = 1; break; }
-            tc::tc_fence_after();
-            const uint32_t a0 = tc::smem_u32(stage_mem + st * kStageBytes);
-            const uint32_t b0 = a0 + 2 * kABytes;
-            if (f8) {   // four K = 32 steps of 32 bytes through the 128-byte slice
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                tc::mma_f8(dt, tc::sdesc_sw128(a0 + kk * 32, 16, 1024), tc::sdesc_sw128(b0 + kk * 32, 16, 1024), id,
-                           (ks > 0 || kk > 0) ? 1u : 0u);
-              tc::mma_commit(&sh.empty[st]);
-              ++kcount;
-              continue;
-            }
-            const int kku = min(4, (n16 - 64 * ks) / 16);   // K = 16 steps below n16 (at least one)
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              if (kk >= kku) break;
-              const uint64_t ah = tc::sdesc_sw128(a0 + kk * 32, 16, 1024);
-              const uint64_t bh = tc::sdesc_sw128(b0 + kk * 2048, 8192, 1024);
-              tc::mma_f16(dt, ah, bh, id, (ks > 0 || kk > 0) ? 1u : 0u);
-              if (d.f.terms > 1) {
-                const uint64_t al = tc::sdesc_sw128(a0 + kABytes + kk * 32, 16, 1024);
-                const uint64_t bl = tc::sdesc_sw128(b0 + kBBytes + kk * 2048, 8192, 1024);
-                tc::mma_f16(dt, ah, bl, id, 1u);
-                tc::mma_f16(dt, al, bh, id, 1u);
+    }
+  } else if (warp == 2) {
+    // ------------------------------------------------ loader: the K slices of the products, in the scheduler's order.
+    // (The whole warp runs the loop and one elected lane issues: from one lane's branch a TMA instruction took some 140
+    // cycles and an MMA 85, together more than the MMAs of a slice.)
+    auto wait = [&](uint64_t* b, uint32_t parity, int more) {
+      return (bool)__all_sync(0xffffffffu, tc::mbar_wait_ns(b, parity, more * g.wait_ns));
+    };
+    bool ok = true;
+    for (uint32_t i = 0; ok && !sh.err; ++i) {
+      if (!(ok = wait(&sh.desc_full[i % kRing], (i / kRing) & 1, 8))) break;
+      const Desc& d = sh.ring[i % kRing];
+      if (d.term) break;
+      if (d.op == kOpProd) {
+        tc::fence_proxy_async_global();   // the epilogues' plane writes, before TMA reads them
+        const bool f8 = d.f.fmt == FMT_E4M3, two = d.f.terms > 1;
+        const int nks = f8 ? k8_extent(d.n64) / 128 : (d.n + 31) / 32, tiles = d.nrb * d.ncb, ncb = d.ncb, za = d.za, zb = d.zb;
+        const CUtensorMap* const ma = two ? &maps.A2 : &maps.A;
+        const CUtensorMap* const mb1 = two ? &maps.B2 : &maps.B;
+        const CUtensorMap* const mb2 = two ? &maps.B2x2 : &maps.Bx2;
+        const uint32_t aoff = two ? 2 * kABytes : kABytes, boff = two ? 2 * kBBlock : kBBlock;
+        for (int ti = d.t0; ti < tiles && ok; ti += G) {
+          const int mb = ti / ncb, cb = ti - mb * ncb;
+          const int nb = min(kTileN, d.n64 - kTileN * cb) / 64, c0 = kTileN / 64 * cb;
+          // E4M3: both operands K-major (the symmetric iterate is its own transpose), 128-byte K slices; the B box is
+          // always kTileN rows (rows past R are zero-filled by the copy)
+          const uint32_t bytes = f8 ? 128 * 128 + (uint32_t)kTileN * 128u : aoff + nb * boff;
+          for (int ks = 0; ks < nks; ++ks, ++loads) {
+            const uint32_t st = loads % kStages;
+            if (!(ok = wait(&sh.empty[st], ((loads / kStages) & 1) ^ 1, 1))) break;
+            if (tc::elect_one()) {
+              uint8_t* const sm = stage_mem + st * kStageBytes;
+              uint64_t* const bar = &sh.full[st];
+              tc::mbar_arrive_expect_tx(bar, bytes);
+              if (f8) {
+                tc::tma_load_3d(sm, &maps.A8, bar, 128 * ks, 128 * mb, za);
+                tc::tma_load_3d(sm + 128 * 128, &maps.B8, bar, 128 * ks, kTileN * cb, zb);
+              } else {
+                tc::tma_load_3d(sm, ma, bar, 32 * ks, 128 * mb, za);
+                if (nb >= 2) tc::tma_load_4d(sm + aoff, mb2, bar, 0, 32 * ks, zb, c0);
+                if (nb == 4) tc::tma_load_4d(sm + aoff + 2 * boff, mb2, bar, 0, 32 * ks, zb, c0 + 2);
+                if (nb & 1) tc::tma_load_4d(sm + aoff + (nb - 1) * boff, mb1, bar, 0, 32 * ks, zb, c0 + nb - 1);
               }
             }
-            tc::mma_commit(&sh.empty[st]);
-            ++kcount;
+            __syncwarp();
           }
-          tc::mma_commit(&sh.accf[buf]);
-          ++tcount;
         }
+      }
+      if (lane == 0) tc::mbar_arrive(&sh.desc_free[i % kRing]);
     }
+    if (!ok) sh.err = 1;
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer: the products in the scheduler's order
+    auto wait = [&](uint64_t* b, uint32_t parity, int more) {
+      return (bool)__all_sync(0xffffffffu, tc::mbar_wait_ns(b, parity, more * g.wait_ns));
+    };
+    const uint32_t sm0 = __shfl_sync(0xffffffffu, tc::smem_u32(stage_mem), 0);
+    uint32_t kcount = 0, tcount = 0;
+    bool ok = true;
+    for (uint32_t i = 0; ok && !sh.err; ++i) {
+      if (!(ok = wait(&sh.desc_full[i % kRing], (i / kRing) & 1, 8))) break;
+      const Desc& d = sh.ring[i % kRing];
+      if (d.term) break;
+      if (d.op == kOpProd) {
+        const bool f8 = d.f.fmt == FMT_E4M3, two = d.f.terms > 1;
+        // kind::f16 products run over n16 = n rounded up to 16 in N and K (the loads are whole slices of 32 and blocks of
+        // 64): the operands' rows and columns past n are zero, so the entries the trimmed product leaves out are 0
+        const int n16 = (d.n + 15) & ~15, n64 = d.n64, tiles = d.nrb * d.ncb, ncb = d.ncb;
+        const int nks = f8 ? k8_extent(n64) / 128 : (d.n + 31) / 32;
+        const uint32_t aoff = two ? 2 * kABytes : kABytes, boff = two ? 2 * kBBlock : kBBlock;
+        const uint64_t ad0 = f8 ? tc::sdesc_sw128(sm0, 16, 1024) : tc::sdesc_sw64(sm0, 16, 512);
+        const uint64_t bd0 = f8 ? tc::sdesc_sw128(sm0 + 128 * 128, 16, 1024) : tc::sdesc_sw128(sm0 + aoff, boff, 1024);
+        for (int ti = d.t0; ti < tiles && ok; ti += G, ++tcount) {
+          const int mb = ti / ncb, cb = ti - mb * ncb;
+          const int nt = min(kTileN, n64 - kTileN * cb);
+          // kind::f16: A K-major, B MN-major; kind::f8f6f4 (E4M3 = 0): both K-major
+          const uint32_t id = f8 ? tc::idesc(0, 0, 0, 0, 128, nt)
+                                 : tc::idesc(d.f.fmt, d.f.fmt, 0, 1, 128, min(nt, n16 - kTileN * cb));
+          const int buf = tcount & 1;
+          if (!(ok = wait(&sh.acce[buf], ((tcount >> 1) & 1) ^ 1, 1))) break;
+          tc::tc_fence_after();
+          const uint32_t dt = tmem + (uint32_t)buf * 256;
+          for (int ks = 0; ks < nks; ++ks, ++kcount) {
+            const uint32_t st = kcount % kStages;
+            if (!(ok = wait(&sh.full[st], (kcount / kStages) & 1, 1))) break;
+            tc::tc_fence_after();
+            if (tc::elect_one()) {
+              const uint64_t ad = ad0 + ((st * kStageBytes) >> 4), bd = bd0 + ((st * kStageBytes) >> 4);
+              if (f8) {   // four K = 32 steps of 32 bytes through the 128-byte slice
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) tc::mma_f8(dt, ad + 2 * kk, bd + 2 * kk, id, (ks > 0 || kk > 0) ? 1u : 0u);
+              } else {
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk) {   // K = 16 steps below n16 (at least one)
+                  if (kk == 1 && 32 * ks + 16 >= n16) break;
+                  const uint64_t ah = ad + 2 * kk, bh = bd + 128 * kk;
+                  tc::mma_f16(dt, ah, bh, id, (ks > 0 || kk > 0) ? 1u : 0u);
+                  if (two) {
+                    tc::mma_f16(dt, ah, bh + (kBBlock >> 4), id, 1u);
+                    tc::mma_f16(dt, ah + (kABytes >> 4), bh, id, 1u);
+                  }
+                }
+              }
+              tc::mma_commit(&sh.empty[st]);
+              if (ks == nks - 1) tc::mma_commit(&sh.accf[buf]);
+            }
+            __syncwarp();
+          }
+        }
+      }
+      if (lane == 0) tc::mbar_arrive(&sh.desc_free[i % kRing]);
+    }
+    if (!ok) sh.err = 1;
   }
   } else {
-  if constexpr (kShape == 1) tc::setmaxnreg_inc<kRegsEpi>();   // to the epilogue groups
+  tc::setmaxnreg_inc<Shape<kShape>::kRegsEpi>();   // to the epilogue groups
   {
     // ------------------------------------------------ epilogue: drains products, decides, finishes and starts slots
     const int etid = tid - 128;              // 0..255
     const int q = warp & 3;                  // TMEM lane quarter of this warp
     const int grp = (warp - 4) >> 2;         // epilogue group: chunks grp, grp + 3, ... of a tile
     uint32_t tcount = 0;
+    int share = 0;   // this CTA's place in the group for the slot at hand: its rows and sums
 
     // One FP64 n x n matrix M (row-major) as an n64 x n64 operand (zero padded) into the 3-term FP16 planes
     // hi, lo (hi + plane_elems): four rows per warp pass, 8 consecutive columns per lane, the pass's 32 loads
     // all issued before its first store, then 16-byte stores.
     auto fill_pair = [&](uint16_t* hi, int n, int n64, const double* __restrict__ M) {
       uint16_t* lo = hi + plane_elems;
-      for (int i0 = 4 * (warp - 4); i0 < n64; i0 += 4 * kEpiWarps) {
+      for (int i0 = 4 * (kEpiWarps * share + warp - 4); i0 < n64; i0 += 4 * kEpiWarps * G) {
         for (int j0 = 8 * lane; j0 < n64; j0 += 256) {
           float vv[4][8];
 #pragma unroll
@@ -566,11 +822,9 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
     // V_0 = Y_0 = T_J(S) / c and T_0 = 3I - Y_0 are written directly (pairs 0 and 1, Z's pair: Z_1 = T_0 / 2,
     // the factor 1/2 applied by the products that read Z until its first update), with the defect
     // ||I - Y_0||_F / sqrt(n); only Y_1 = Y_0 T_0 / 2 needs the tensor cores.
-    auto start_inverse = [&](int s, int J) {
-      SlotState& st = sh.slot[s];
-      const int n = g.sub_n[J], n64 = (n + 63) & ~63, R = (n + 127) & ~127;
+    auto start_inverse = [&](int s, int J) -> float {
+      const int n = g.sub_n[J], n64 = (n + 63) & ~63;
       const double* S = g.ws + (g.a_off[J] - g.a_base);
-      const double* H = S + g.chunk_n2;
       // the trace of T_J(S) (every warp sums it alike, lanes along the diagonal)
       double tr = 0.0;
       for (int i = lane; i < n; i += 32) tr += S[(size_t)i * n + i];
@@ -580,7 +834,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
       uint16_t* base = g.planes + (size_t)(sub0 + s) * kPps * plane_elems;
       float dpart = 0.0f;   // this thread's share of ||I - Y_0||_F^2
       // Y_0 and T_0 from one read of T_J(S): the same pass pattern as fill_pair, two pairs out
-      for (int i0 = 4 * (warp - 4); i0 < n64; i0 += 4 * kEpiWarps) {
+      for (int i0 = 4 * (kEpiWarps * share + warp - 4); i0 < n64; i0 += 4 * kEpiWarps * G) {
         for (int j0 = 8 * lane; j0 < n64; j0 += 256) {
           float sv[4][8];   // the pass's 32 loads, all issued before its first store
 #pragma unroll
@@ -616,67 +870,18 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           }
         }
       }
-      for (int o = 16; o > 0; o >>= 1) dpart += __shfl_xor_sync(0xffffffffu, dpart, o);
-      if (lane == 0) sh.dred[0][warp - 4] = dpart;
-      epi_bar<kEpiThreads>();
-      if (tid == 128) {
-        float dsum = 0.0f;
-        for (int w = 0; w < kEpiWarps; ++w) dsum += (float)sh.dred[0][w];
-        const float d0 = sqrtf(dsum / (float)n);
-        st.job = J;
-        st.n = n; st.n64 = n64; st.R = R;
-        st.nrb = R / 128; st.ncb = (n64 + kTileN - 1) / kTileN; st.nks = n64 / 64;
-        st.yc = 0; st.zc = 1; st.cinv = inv; st.zs = 0.5f;
-        st.steps = 1; st.rsteps = 0; st.status = kSubOk;
-        st.fcur = Fmt{FMT_F16, 3}; st.fnxt = st.fcur;
-        st.dprev = INFINITY;
-        if (!(c > 0.0) || !isfinite(c) || !isfinite(d0)) st.status = kSubRefine;   // the FP64 preparation takes it
-        st.last = d0 <= g.tol_inv ? 1 : 0;
-        st.kind = st.last ? 3 : 1;     // step 0 the last: X = Z_1 Z_1 / c next; else Y_1 = Y_0 T_0 / 2
-        st.zdone = 1;
-      }
-      epi_bar<kEpiThreads>();   // dred free again; st.last visible to every epilogue thread
-      // step 0 the last: Y_0 is not needed, T_J(H0) takes its pair now (else after the last Z update)
-      if (st.last && g.Aout) fill_pair(base, n, n64, H);
+      if (!(c > 0.0) || !isfinite(c)) dpart = INFINITY;   // the scheduler leaves it to the FP64 preparation
+      if (tid == 128) sh.cinv[s] = inv;
+      return dpart;
     };
 
     // a4 for a new submatrix of slot s: X_0 = (A - mu I) / alpha in the main format, zero padded
-    auto start_slot = [&](int s) {
-      SlotState& st = sh.slot[s];
-      for (;;) {
-        if (tid == 128) {
-          const int k = atomicAdd(g.next, 1);
-          sh.fetch = (k < g.j1 - g.j0 && !sh.err) ? g.order[k] : -1;
-        }
-        epi_bar<kEpiThreads>();
-        const int J = sh.fetch;
-        epi_bar<kEpiThreads>();
-        if (J < 0) {
-          if (tid == 128) st.job = -1;
-          break;
-        }
-        if constexpr (kMode == 1) {
-          if (g.again && g.prep_out[J] != kSubAgain) continue;
-          start_inverse(s, J);
-          break;
-        }
-        if (g.sub_n[J] <= g.above_n) continue;
-        if (g.cond && g.prep_status[J] == kSubOk && g.cond[J] > g.cond_max && g.sub_n[J] <= g.ill_max_n) continue;
-        if (g.prep_status[J] != kSubOk) {
-          if (tid == 128) {
-            g.status[J] = g.prep_status[J];
-            g.iters[J] = 0;
-            g.rsteps[J] = 0;
-            g.tS[J] = 0.0;
-            g.tH[J] = 0.0;
-          }
-          continue;
-        }
+    auto start_sign = [&](int zo, int J) {
         const int n = g.sub_n[J], n64 = (n + 63) & ~63, R = (n + 127) & ~127;
         const float* A = g.A + g.a_off[J];
         const double alpha = scale_alpha(g.lam, g.lam_g, J, g.mu);
         const float inv = (float)(1.0 / alpha), fmu = (float)g.mu;
-        uint16_t* hi = g.planes + (size_t)(sub0 + s) * kPps * plane_elems;
+        uint16_t* hi = g.planes + (size_t)zo * plane_elems;
         uint16_t* lo = hi + plane_elems;
         const Fmt f = g.main_fmt;
         if (f.fmt == FMT_E4M3) {
@@ -684,7 +889,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           // the other X plane and of T (their products write only the first n64 columns)
           const int k8 = k8_extent(n64);
           uint8_t* p8 = reinterpret_cast<uint8_t*>(hi);
-          for (int e = etid; e < R * k8; e += kEpiThreads) {
+          for (int e = etid + kEpiThreads * share; e < R * k8; e += kEpiThreads * G) {
             const int i = e / k8, j = e - i * k8;
             float x = 0.0f;
             if (i < n && j < n) x = (A[(size_t)i * n + j] - (i == j ? fmu : 0.0f)) * inv;
@@ -698,7 +903,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           // four rows per warp pass, 8 consecutive columns per lane (all 32 loads in flight together, then
           // 16-byte stores of hi and lo); rows and columns n..n64 are the zero padding; rows from n64 on
           // only feed product rows that are never read back
-          for (int i0 = 4 * (warp - 4); i0 < n64; i0 += 4 * kEpiWarps) {
+          for (int i0 = 4 * (kEpiWarps * share + warp - 4); i0 < n64; i0 += 4 * kEpiWarps * G) {
             for (int j0 = 8 * lane; j0 < n64; j0 += 256) {
               float v[4][8];
 #pragma unroll
@@ -724,99 +929,86 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
             }
           }
         }
-        if (tid == 128) {
-          st.job = J;
-          st.n = n; st.n64 = n64; st.R = R;
-          st.nrb = R / 128; st.ncb = (n64 + kTileN - 1) / kTileN; st.nks = n64 / 64;
-          st.kind = 0; st.cur = 0;
-          st.phase = 0; st.refine_left = g.refine_steps; st.steps = 0; st.rsteps = 0;
-          st.status = kSubNotConv; st.last = 0;
-          st.dprev = INFINITY;
-          st.fcur = g.main_fmt; st.fnxt = g.main_fmt;
-        }
-        break;
-      }
-      tc::fence_proxy_async_global();
-      tc::mbar_arrive(&sh.epi_done[s]);
     };
 
     // a7 for the finished submatrix of slot s: centre columns of T_J(D) = 1/2 (I - X) T_J(S)^-1 and the
     // FP64 partial traces
-    auto finish_slot = [&](int s) {
-      epi_bar<kEpiThreads>();   // the slot state written by thread 128 and the final X of every group are visible
-      SlotState& st = sh.slot[s];
-      const int J = st.job, n = st.n, b = g.nbf[J];
+    auto finish_sign = [&](const Desc& d) {
+      const int J = d.fin, n = d.n, b = g.nbf[J];
+      // this CTA's rows
+      const int rows = 32 * (((n + 31) / 32 + G - 1) / G), r0 = min(n, rows * share), r1 = min(n, r0 + rows);
       // the final X_k, hi (+ lo) in the last product's output format
-      const uint16_t* xh = g.planes + ((size_t)(sub0 + s) * kPps + 2 * st.cur) * plane_elems;
+      const uint16_t* xh = g.planes + (size_t)d.za * plane_elems;
       const uint16_t* xl = xh + plane_elems;
-      const Fmt xfmt = st.fcur;
+      const Fmt xfmt = d.f;
       const double* Q = g.Q + g.c_off[J];
       const double* Sc = g.Sc + g.c_off[J];
       const double* Hc = g.Hc + g.c_off[J];
       double* Dc = g.Dc + g.c_off[J];
-      // X Q with one row of X per lane (32 consecutive rows per warp), Q in FP32 in the staging buffers (idle
-      // between products), zero padded to bp = 8 ceil(b / 8) columns and n64 rows so that the inner loop has
-      // no conditions; the sums (hi, lo) then go through shared memory to the FP64 step, which runs
-      // element by element. Larger cases take the same sums with Q read from global memory.
-      const int n64 = st.n64, bp = (b + 7) & ~7;
-      float* Qs = reinterpret_cast<float*>(stg);
-      const size_t qs_bytes = (size_t)n64 * bp * sizeof(float);
-      const bool fast = qs_bytes + (size_t)n * b * sizeof(float2) <= kStgTotal;
-      float2* Ps = reinterpret_cast<float2*>(stg + qs_bytes);
+      // X Q eight columns at a time, Q in FP32 in the staging buffers (idle between products; in pieces of kRowsQ rows
+      // when there are more), zero padded; the sums (hi, lo) of up to kRowsP rows of X then go through shared memory to
+      // the FP64 step, which runs entry by entry
+      constexpr int kRowsP = 128, kRowsQ = (int)((kStgTotal - 64 * kRowsP) / 34) & ~31;
+      static_assert(4 * (8 * kRowsQ + 4 * (kRowsQ / 8)) + 64 * kRowsP <= kStgTotal, "staging");
+      const int n64 = d.n64;
+      float* const Qs = reinterpret_cast<float*>(stg);
+      float2* const Ps = reinterpret_cast<float2*>(stg + kStgTotal - 64 * kRowsP);
       double ps = 0.0, ph = 0.0;
-      if (fast) {
-        for (int e = etid; e < n64 * bp; e += kEpiThreads) {
-          const int k = e / bp, c = e - k * bp;
-          Qs[e] = (k < n && c < b) ? (float)Q[(size_t)k * b + c] : 0.0f;
-        }
-        epi_bar<kEpiThreads>();
-        for (int i0 = 32 * (warp - 4); i0 < n; i0 += kEpiThreads) {
-          const int i = i0 + lane;
-          const size_t ro = (size_t)(i < n ? i : 0) * g.LD;
-          for (int cg = 0; cg < b; cg += 8) {
-            float sh_[8], sl_[8];
-            if (xfmt.fmt == FMT_BF16) {
-              if (xfmt.terms > 1) xq_row<FMT_BF16, true>(xh + ro, xl + ro, n64, Qs + cg, bp, sh_, sl_);
-              else xq_row<FMT_BF16, false>(xh + ro, xl + ro, n64, Qs + cg, bp, sh_, sl_);
-            } else {
-              if (xfmt.terms > 1) xq_row<FMT_F16, true>(xh + ro, xl + ro, n64, Qs + cg, bp, sh_, sl_);
-              else xq_row<FMT_F16, false>(xh + ro, xl + ro, n64, Qs + cg, bp, sh_, sl_);
+      for (int cg = 0; cg < b; cg += 8) {
+        const int cn = min(8, b - cg);
+        for (int rr = r0; rr < r1; rr += kRowsP) {
+          const int rn = min(kRowsP, r1 - rr);
+          for (int k0 = 0; k0 < n64; k0 += kRowsQ) {
+            const int kn = min(kRowsQ, n64 - k0);
+            if (rr == r0 || n64 > kRowsQ) {
+              epi_bar<kEpiThreads>();   // the last piece has been used
+              for (int e = etid; e < kn * 8; e += kEpiThreads) {
+                const int k = k0 + (e >> 3), c = e & 7;
+                Qs[qs_at(e >> 3) + c] = k < n && c < cn ? (float)Q[(size_t)k * b + cg + c] : 0.0f;
+              }
+              epi_bar<kEpiThreads>();
             }
-            if (i < n) {
+            for (int it = warp - 4; 8 * it < rn; it += kEpiWarps) {
+              const int row = 8 * it + (lane >> 2), part = lane & 3;
+              const size_t ro = (size_t)min(rr + row, n - 1) * g.LD + k0;
+              uint64_t s[4], e[4];
+              if (xfmt.fmt == FMT_BF16) {
+                if (xfmt.terms > 1) xq_rows<FMT_BF16, true>(xh + ro, xl + ro, kn, Qs, part, s, e);
+                else xq_rows<FMT_BF16, false>(xh + ro, xl + ro, kn, Qs, part, s, e);
+              } else {
+                if (xfmt.terms > 1) xq_rows<FMT_F16, true>(xh + ro, xl + ro, kn, Qs, part, s, e);
+                else xq_rows<FMT_F16, false>(xh + ro, xl + ro, kn, Qs, part, s, e);
+              }
+              if (part == 0) {
 #pragma unroll
-              for (int c = 0; c < 8; ++c)
-                if (cg + c < b) Ps[(size_t)i * b + cg + c] = make_float2(sh_[c], sl_[c]);
+                for (int c = 0; c < 8; ++c) {
+                  const float2 sv = unpair2(s[c >> 1]), ev = unpair2(e[c >> 1]);
+                  float2 p = c & 1 ? make_float2(sv.y, ev.y) : make_float2(sv.x, ev.x);
+                  if (k0 > 0) {
+                    const float2 o = Ps[row * 8 + c];
+                    two_sum(p.x, p.y, o.x);
+                    p.y += o.y;
+                  }
+                  Ps[row * 8 + c] = p;
+                }
+              }
             }
           }
-        }
-        epi_bar<kEpiThreads>();
-        for (int e = etid; e < n * b; e += kEpiThreads) {
-          const float2 p = Ps[e];
-          const double dv = 0.5 * (Q[e] - ((double)p.x + (double)p.y));
-          Dc[e] = dv;
-          ps += dv * Sc[e];
-          ph += dv * Hc[e];
-        }
-      } else {
-        for (int e = etid; e < n * b; e += kEpiThreads) {
-          const int i = e / b, c = e - i * b;
-          float sum = 0.0f, cmp = 0.0f;
-          for (int k = 0; k < n; ++k) {
-            const float x = from_bits(xh[(size_t)i * g.LD + k], xfmt.fmt) +
-                            (xfmt.terms > 1 ? from_bits(xl[(size_t)i * g.LD + k], xfmt.fmt) : 0.0f);
-            const float qv = (float)Q[(size_t)k * b + c];
-            const float p = x * qv;
-            cmp += fmaf(x, qv, -p);
-            two_sum(sum, cmp, p);
+          epi_bar<kEpiThreads>();
+          for (int e = etid; e < rn * cn; e += kEpiThreads) {
+            const int i = e / cn, c = e - i * cn;
+            const float2 p = Ps[i * 8 + c];
+            const size_t at = (size_t)(rr + i) * b + cg + c;
+            const double dv = 0.5 * (Q[at] - ((double)p.x + (double)p.y));
+            Dc[at] = dv;
+            ps += dv * Sc[at];
+            ph += dv * Hc[at];
           }
-          const double dv = 0.5 * (Q[e] - ((double)sum + (double)cmp));
-          Dc[e] = dv;
-          ps += dv * Sc[e];
-          ph += dv * Hc[e];
+          epi_bar<kEpiThreads>();
         }
       }
       double px = 0.0;   // the trace of the final X: (n - Tr X) / 2 eigenvalues lie below mu
-      for (int i = etid; i < n; i += kEpiThreads) {
+      for (int i = r0 + etid; i < r1; i += kEpiThreads) {
         float x = from_bits(xh[(size_t)i * g.LD + i], xfmt.fmt);
         if (xfmt.terms > 1) x += from_bits(xl[(size_t)i * g.LD + i], xfmt.fmt);
         px += x;
@@ -832,54 +1024,77 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
         sh.dred[2][warp - 4] = px;
       }
       epi_bar<kEpiThreads>();
-      if (tid == 128) {
-        double ts = 0.0, th = 0.0, tx = 0.0;
-        for (int w = 0; w < kEpiWarps; ++w) {
-          ts += sh.dred[0][w];
-          th += sh.dred[1][w];
-          tx += sh.dred[2][w];
-        }
-        if (g.nbelow) g.nbelow[J] = (int32_t)lrint(0.5 * (n - tx));
-        int stt = st.status;
-        if (stt == kSubOk && !(isfinite(ts) && isfinite(th))) stt = kSubNonFinite;
-        g.tS[J] = ts;
-        g.tH[J] = th;
-        g.iters[J] = st.steps;
-        g.rsteps[J] = st.rsteps;
-        g.status[J] = stt;
+      if (tid < 131 && tid >= 128) {
+        double t = 0.0;
+        for (int w = 0; w < kEpiWarps; ++w) t += sh.dred[tid - 128][w];
+        if (G > 1) __stcg(&gs[d.slot].tr[tid - 128][share], t);
+        else sh.tr[d.slot][tid - 128] = t;
       }
       epi_bar<kEpiThreads>();   // staging and dred free again
     };
 
-    for (int c = 0; c < kSlots; ++c) start_slot(c);
+    // this CTA's part of a phase is done: its share of the defect (thread 128), and the arrival. Every thread's writes
+    // precede the barrier.
+    auto arrive = [&](const Desc& d, float part) {
+      if (tid == 128) {
+        if (G > 1) {
+          __stcg(&gs[d.slot].part[d.par][share], part);
+          tc::red_release_gpu(&gs[d.slot].count, 1u);
+        } else {
+          sh.part[d.slot] = part;
+        }
+      }
+      tc::mbar_arrive(&sh.epi_done[d.slot]);
+    };
+
     for (uint32_t i = 0;; ++i) {
       // every epilogue thread waits for the descriptor; a wait that ran out in any of them ends all
-      const bool got = tc::mbar_wait(&sh.desc_full[i % kRing], (i / kRing) & 1, tc::globaltimer() + 8 * g.wait_ns);
+      const bool got = tc::mbar_wait_ns(&sh.desc_full[i % kRing], (i / kRing) & 1, 8 * g.wait_ns);
       if (epi_bar_or<kEpiThreads>(!got || sh.err)) {
         if (tid == 128) sh.err = 1;
         break;
       }
       const Desc d = sh.ring[i % kRing];
       if (d.term) break;
-      SlotState& st = sh.slot[d.slot];
-      const int n = d.n, n64 = d.n64;
+      const int n = d.n, n64 = d.n64, n16 = (n + 15) & ~15;
+      share = (rank - d.slot * (G / 2) + G) % G;
+      if (d.op != kOpProd) {
+        float dpart = 0.0f;
+        if (d.op == kOpFill) {
+          fill_pair(g.planes + (size_t)d.fill * plane_elems, n, n64, g.ws + (g.a_off[d.job] - g.a_base) + g.chunk_n2);
+        } else {
+          if constexpr (kMode == 0) {
+            if (d.fin >= 0) finish_sign(d);
+            if (d.job >= 0) start_sign(d.zo, d.job);
+          } else {
+            dpart = start_inverse(d.slot, d.job);
+          }
+        }
+        tc::fence_proxy_async_global();
+        for (int o = 16; o > 0; o >>= 1) dpart += __shfl_xor_sync(0xffffffffu, dpart, o);
+        if (lane == 0) sh.red[i & 1][warp - 4] = dpart;
+        epi_bar<kEpiThreads>();
+        float dsum = 0.0f;
+        if (tid == 128)
+          for (int w = 0; w < kEpiWarps; ++w) dsum += sh.red[i & 1][w];
+        arrive(d, dsum);
+        if (tid == 128) tc::mbar_arrive(&sh.desc_free[i % kRing]);
+        continue;
+      }
       // the sign iteration's epilogues are fixed by the product kind (no descriptor fields needed)
       const int epi = kMode == 0 ? (d.kind == 0 ? kEpiT : kEpiScale) : d.epi;
       const float escale = kMode == 0 ? 0.5f : (epi == kEpiA ? 1.0f : d.scale);
       float part = 0.0f;
       bool bad = false;   // a wait of this warp ran out: keep the barrier schedule, skip the work
-      for (int mb = 0; mb < d.nrb; ++mb)
-        for (int cb = 0; cb < d.ncb; ++cb) {
+      for (int ti = d.t0; ti < d.nrb * d.ncb; ti += G) {
+          const int mb = ti / d.ncb, cb = ti - mb * d.ncb;
           const int nt = min(kTileN, n64 - kTileN * cb);
           const int buf = tcount & 1;
-          if (!bad) bad = !tc::mbar_wait(&sh.accf[buf], (tcount >> 1) & 1, tc::globaltimer() + g.wait_ns);
+          if (!bad) bad = !tc::mbar_wait_ns(&sh.accf[buf], (tcount >> 1) & 1, g.wait_ns);
           bad = __any_sync(0xffffffffu, bad);   // tcgen05.ld needs the whole warp
           tc::tc_fence_after();
-          // an M = 64 tile: 16 rows per warp quarter, in its lanes 0-15
-          const bool m64 = tail64(d, mb);
-          const int rbase = 128 * mb + (m64 ? 16 : 32) * q;
+          const int rbase = 128 * mb + 32 * q;
           const int row = rbase + lane;
-          const bool rok = !m64 || lane < 16;
           const bool live = rbase < n64 && !bad;   // rows >= n64 are never read back
           const int nch = nt / 32;
           const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)buf * 256;
@@ -889,119 +1104,119 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
           const float sc = (d.f.fmt == FMT_E4M3 ? kF8Down : 1.0f) * (kMode == 1 && epi == kEpiT ? d.pscale : 1.0f);
           for (int c0 = grp; c0 < nch; c0 += kGroups) {
             const int col0 = kTileN * cb + 32 * c0;
-            float v[32];
-            if (live) {
-              tc::tmem_wait_ld();
-              // entries past n are written as zeros: the trimmed products leave the accumulator's columns
-              // past n16 as they were, and the next products' K and N never reach past n16
-              // a chunk inside the n columns that holds none of the warp's diagonal entries takes the short
-              // path (warp-uniform test): rows past n through a zero factor, no test per entry
-              const bool rin = rok && row < n;
-              const bool inner = col0 + 32 <= n && col0 != (rbase & ~31);
-              if (epi == kEpiT) {
-                if (inner) {
-                  const float s = rin ? sc : 0.0f;
-                  float q4[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // four partial sums: a dependence chain of 8, not 32
+            if (!live) continue;
+            tc::tmem_wait_ld();
+            // Zeros from column n16 on, where the trimmed product left the accumulator as it was: the next products'
+            // K and N reach to n64. Rows and columns from n to n16 are zeros already, the operands' being zeros.
+            if (col0 + 16 >= n16) {
+              const bool none = col0 >= n16;
 #pragma unroll
-                  for (int j = 0; j < 32; ++j) {
-                    const float p = s * __uint_as_float(r[j]);   // P_ij, off the diagonal: (I - P)_ij = -p
-                    q4[j & 3] = fmaf(p, p, q4[j & 3]);
-                    v[j] = -p;                                   // (3I - P)_ij
-                  }
-                  // lanes without a row hold whatever the tensor memory held before (0 times a NaN is one)
-                  if (rin) part += (q4[0] + q4[1]) + (q4[2] + q4[3]);
-                } else {
-#pragma unroll
-                  for (int j = 0; j < 32; ++j) {
-                    const int col = col0 + j;
-                    const bool in = rin && col < n;
-                    const float e = (row == col ? 1.0f : 0.0f) - sc * __uint_as_float(r[j]);  // (I - P)_ij
-                    if (in) part += e * e;
-                    v[j] = in ? e + (row == col ? 2.0f : 0.0f) : 0.0f;                 // (3I - P)_ij
-                  }
-                }
-              } else {
-                const float m = escale * sc;
-                if (col0 + 32 <= n) {
-                  const float mr = rin ? m : 0.0f;
-#pragma unroll
-                  for (int j = 0; j < 32; ++j) v[j] = mr * __uint_as_float(r[j]);
-                } else {
-#pragma unroll
-                  for (int j = 0; j < 32; ++j) v[j] = (rin && col0 + j < n) ? m * __uint_as_float(r[j]) : 0.0f;
-                }
-              }
-              if (c0 + kGroups < nch) tc::tmem_ld32(taddr + 32 * (c0 + kGroups), r);   // overlaps this chunk's work
+              for (int u = 0; u < 32; ++u) r[u] = u >= 16 || none ? 0u : r[u];
             }
-            if (kMode == 1 && live && epi >= kEpiX) {
+            const bool rin = row < n;
+            if (kMode == 1 && epi >= kEpiX) {
               // inverse mode: X or A_J in FP32, row-major n x n. The chunk goes through the warp's staging
               // buffer (row = lane, entry j at j ^ lane: no bank conflicts either way) so that each store
               // instruction writes 32 consecutive entries of one row
-              const int J = sh.slot[d.slot].job;
-              float* dst = epi == kEpiX ? g.Xout + (g.a_off[J] - g.a_base) : g.Aout + g.a_off[J];
+              float* dst = epi == kEpiX ? g.Xout + (g.a_off[d.job] - g.a_base) : g.Aout + g.a_off[d.job];
               float* wf = reinterpret_cast<float*>(stg + (size_t)(warp - 4) * 4096);
               if (lane == 0) tc::bulk_wait_read<0>();   // this warp's previous store has read the buffer
               __syncwarp();
 #pragma unroll
-              for (int j = 0; j < 32; ++j) wf[lane * 32 + (j ^ lane)] = v[j];
+              for (int j = 0; j < 32; ++j) wf[lane * 32 + (j ^ lane)] = escale * __uint_as_float(r[j]);
               __syncwarp();
-              const int nr = m64 ? 16 : 32;
-              for (int rr = 0; rr < nr; ++rr) {
-                const int orow = rbase + rr;
-                if (orow < n && col0 + lane < n) dst[(size_t)orow * n + col0 + lane] = wf[rr * 32 + (lane ^ rr)];
+              const int nr = min(32, n - rbase);
+              float* at = dst + (size_t)rbase * n + col0 + lane;
+              if (col0 + lane < n) {
+#pragma unroll 8
+                for (int rr = 0; rr < nr; ++rr, at += n) *at = wf[rr * 32 + (lane ^ rr)];
               }
               __syncwarp();   // the staging is free again
+              if (epi == kEpiA) {   // no operand to write
+                if (c0 + kGroups < nch) tc::tmem_ld32(taddr + 32 * (c0 + kGroups), r);
+                continue;
+              }
             }
-            if (kMode == 1 && epi == kEpiA) {
-              // no operand to write
-            } else if (d.fo.fmt == FMT_E4M3) {
+            // T: (3I - P)_ij = (I - P)_ij = -P_ij off the diagonal. On it (rows below n): P - 1 first, whose negative
+            // counts for the defect, then 2 more. sc is a power of two, so that P - 1 / sc is as exact as sc P - 1.
+            const int du = epi == kEpiT && col0 == (rbase & ~31) && rin ? row - col0 : -1;   // this row's diagonal entry
+            float m = escale * sc;
+            if (epi == kEpiT) {
+              m = -sc;
+              if (col0 == (rbase & ~31)) {
+                const float one = 1.0f / sc;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) r[u] = pick(u, du, __float_as_uint(__uint_as_float(r[u]) - one), r[u]);
+              }
+            }
+            if (kMode == 0 && kShape == 0 && d.fo.fmt == FMT_E4M3) {
               // E4M3 output (scaled by 2^7): this thread's 32 bytes of the row, two 16-byte stores into the
               // one-byte view of the plane (rows of 2 LD bytes)
-              if (live) {
-                uint32_t w8[8];
+              float q4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+              uint32_t w8[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const uint32_t p0 = __nv_cvt_float2_to_fp8x2(make_float2(kF8Up * v[4 * j], kF8Up * v[4 * j + 1]),
-                                                               __NV_SATFINITE, __NV_E4M3);
-                  const uint32_t p1 = __nv_cvt_float2_to_fp8x2(make_float2(kF8Up * v[4 * j + 2], kF8Up * v[4 * j + 3]),
-                                                               __NV_SATFINITE, __NV_E4M3);
-                  w8[j] = p0 | (p1 << 16);
+              for (int j = 0; j < 8; ++j) {
+                float v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  v[u] = m * __uint_as_float(r[4 * j + u]);
+                  q4[u] = fmaf(v[u], v[u], q4[u]);
+                  v[u] = kF8Up * __uint_as_float(pick(4 * j + u, du, __float_as_uint(v[u] + 2.0f), __float_as_uint(v[u])));
                 }
-                uint8_t* dst = reinterpret_cast<uint8_t*>(g.planes) + (size_t)d.zo * plane_elems * 2 +
-                               (size_t)row * (2 * g.LD) + col0;
-                reinterpret_cast<uint4*>(dst)[0] = make_uint4(w8[0], w8[1], w8[2], w8[3]);
-                reinterpret_cast<uint4*>(dst)[1] = make_uint4(w8[4], w8[5], w8[6], w8[7]);
+                const uint32_t p0 = __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
+                const uint32_t p1 = __nv_cvt_float2_to_fp8x2(make_float2(v[2], v[3]), __NV_SATFINITE, __NV_E4M3);
+                w8[j] = p0 | (p1 << 16);
               }
-            } else if (live) {
-              // each warp stores its own 32 rows x 32 columns through its own 4 KB staging buffer (hi rows, then
-              // lo rows; 64-byte swizzle: 16-byte unit c of row r at unit c ^ ((r >> 1) & 3)), with one TMA
-              // tensor store issued by its lane 0 for both planes (a box two planes deep): no barrier between
-              // warps, one store per chunk. An M = 64 tile has 16 rows per warp: its lo rows follow its 16 hi
-              // rows, and the 16-row box reads them there.
-              uint32_t h[16], l[16];
-              split_pack(v, d.fo, h, l);
-              uint8_t* wb = stg + (size_t)(warp - 4) * 4096;
-              if (lane == 0) tc::bulk_wait_read<0>();   // this warp's previous store has read the buffer
-              __syncwarp();
-              if (rok) {
-                uint4* dh = reinterpret_cast<uint4*>(wb + lane * 64);
+              if (rin) part += (q4[0] + q4[1]) + (q4[2] + q4[3]);
+              if (c0 + kGroups < nch) tc::tmem_ld32(taddr + 32 * (c0 + kGroups), r);
+              uint8_t* dst = reinterpret_cast<uint8_t*>(g.planes) + (size_t)d.zo * plane_elems * 2 +
+                             (size_t)row * (2 * g.LD) + col0;
+              reinterpret_cast<uint4*>(dst)[0] = make_uint4(w8[0], w8[1], w8[2], w8[3]);
+              reinterpret_cast<uint4*>(dst)[1] = make_uint4(w8[4], w8[5], w8[6], w8[7]);
+              continue;
+            }
+            uint32_t h[16], l[16];
+            float sq = 0.0f;
+            if constexpr (kMode == 1) scale_split_t<FMT_F16, true, true>(r, m, h, l, sq);
+            else scale_split<true>(r, m, d.fo, h, l, sq);
+            if (rin) part += sq;   // (lanes without a row hold anything; used after T alone)
+            if (epi == kEpiT && col0 == (rbase & ~31)) {
+              uint32_t e = 0;
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                  dh[c ^ ((lane >> 1) & 3)] = make_uint4(h[4 * c], h[4 * c + 1], h[4 * c + 2], h[4 * c + 3]);
-                if (d.fo.terms > 1) {
-                  uint4* dl = reinterpret_cast<uint4*>(wb + (m64 ? 1024 : 2048) + lane * 64);
+              for (int u = 0; u < 32; ++u) e = pick(u, du, r[u], e);
+              uint32_t th, tl;
+              split2(fmaf(m, __uint_as_float(e), 2.0f), 0.0f, kMode == 1 ? (int)FMT_F16 : d.fo.fmt, th, tl);
+              const uint32_t sel = du & 1 ? 0x5410u : 0x3254u;
+              const int dw = du >> 1;   // (-1 for none)
 #pragma unroll
-                  for (int c = 0; c < 4; ++c)
-                    dl[c ^ ((lane >> 1) & 3)] = make_uint4(l[4 * c], l[4 * c + 1], l[4 * c + 2], l[4 * c + 3]);
-                }
+              for (int u = 0; u < 16; ++u) {
+                h[u] = pick(u, dw, __byte_perm(h[u], th, sel), h[u]);
+                l[u] = pick(u, dw, __byte_perm(l[u], tl, sel), l[u]);
               }
-              tc::fence_proxy_async_smem();
-              __syncwarp();
-              if (lane == 0) {
-                const CUtensorMap* ms = d.fo.terms > 1 ? (m64 ? &mapS16x2 : &mapS2) : (m64 ? &mapS16 : &mapS);
-                tc::tma_store_3d(ms, wb, col0, rbase, d.zo);
-                tc::bulk_commit();
-              }
+            }
+            if (c0 + kGroups < nch) tc::tmem_ld32(taddr + 32 * (c0 + kGroups), r);   // overlaps the stores
+            // each warp stores its own 32 rows x 32 columns through its own 4 KB staging buffer (hi rows, then
+            // lo rows; 64-byte swizzle: 16-byte unit c of row r at unit c ^ ((r >> 1) & 3)), with one TMA
+            // tensor store issued by its lane 0 for both planes (a box two planes deep): no barrier between
+            // warps, one store per chunk
+            uint8_t* wb = stg + (size_t)(warp - 4) * 4096;
+            if (lane == 0) tc::bulk_wait_read<0>();   // this warp's previous store has read the buffer
+            __syncwarp();
+            uint4* dh = reinterpret_cast<uint4*>(wb + lane * 64);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              dh[c ^ ((lane >> 1) & 3)] = make_uint4(h[4 * c], h[4 * c + 1], h[4 * c + 2], h[4 * c + 3]);
+            if (kMode == 1 || d.fo.terms > 1) {
+              uint4* dl = reinterpret_cast<uint4*>(wb + 2048 + lane * 64);
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                dl[c ^ ((lane >> 1) & 3)] = make_uint4(l[4 * c], l[4 * c + 1], l[4 * c + 2], l[4 * c + 3]);
+            }
+            tc::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tc::tma_store_3d(kMode == 1 || d.fo.terms > 1 ? &maps.S2 : &maps.S, wb, col0, rbase, d.zo);
+              tc::bulk_commit();
             }
           }
           tc::tc_fence_before();
@@ -1017,127 +1232,27 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
         if (tid == 128) sh.err = 1;
         break;
       }
-      if (kMode == 1 && tid == 128) {
-        // inverse mode: the next product of the slot
-        switch (d.kind) {
-          case 0: {
-            float dsum = 0.0f;
-            for (int w = 0; w < kEpiWarps; ++w) dsum += sh.red[i & 1][w];
-            const float dd = sqrtf(dsum / (float)n);
-            st.steps += 1;
-            if (!isfinite(dd) || (dd > g.tol_inv && st.steps >= g.max_inv)) {
-              st.status = kSubRefine;   // diverged or too slow: the FP64 preparation takes it
-              st.last = 1;
-            } else if (dd <= g.tol_inv) {
-              st.last = 1;                // this step's Z update is the last product of the iteration
-            }
-            st.kind = st.last ? 2 : 1;
-            break;
-          }
-          case 1:   // after Y's update: Z's, unless the step's Z update was made at the start
-            if (st.ncb != 1) st.yc = st.yc == 0 ? 3 : 0;
-            st.kind = st.zdone ? 0 : 2;
-            st.zdone = 0;
-            break;
-          case 2: st.zc = st.zc == 1 ? 4 : 1; st.zs = 1.0f; st.kind = st.last ? 3 : 0; break;
-          case 3: st.kind = 4; break;
-          default: break;
-        }
+      if (kMode == 1 && d.fill >= 0) {
+        fill_pair(g.planes + (size_t)d.fill * plane_elems, n, n64, g.ws + (g.a_off[d.job] - g.a_base) + g.chunk_n2);
+        tc::fence_proxy_async_global();
+        epi_bar<kEpiThreads>();
       }
-      if (kMode == 1 && d.kind == 2 && st.last && g.Aout) {
-        // the iteration's last Z update is done: T_J(H0) into Y's pair (Y was last read by this step's
-        // V = Z Y) for A_J = X T_J(H0), written now so that it is not held through the iteration
-        const int J = st.job;
-        const double* H = g.ws + (g.a_off[J] - g.a_base) + g.chunk_n2;
-        uint16_t* yp = g.planes + ((size_t)(sub0 + d.slot) * kPps + 2 * st.yc) * plane_elems;
-        fill_pair(yp, n, n64, H);
-      }
-      if (kMode == 0 && tid == 128) {
-        if (d.kind == 0) {
-          // defect of X_step and the decision about the following steps
-          float dsum = 0.0f;
-          for (int w = 0; w < kEpiWarps; ++w) dsum += sh.red[i & 1][w];
-          const float dd = sqrtf(dsum / (float)n);
-          const int steps = st.steps + 1;
-          if (st.phase == 1) st.rsteps += 1;   // this step ran in the refinement format
-          int last_ = 0, status = kSubNotConv;
-          Fmt nxt = st.fcur;
-          if (!isfinite(dd)) {
-            last_ = 1;
-            status = kSubNonFinite;
-          } else if (st.phase == 0) {
-            // E4M3 iterates carry a rounding error of up to 2^-4 relative, which holds the defect at a floor
-            // near 0.05, well above tol_ns: their phase ends at twice that floor, or when the defect has
-            // stopped falling (below 0.25, where the exact iteration would at least halve it every step)
-            const bool f8_end = st.fcur.fmt == FMT_E4M3 && (dd <= kF8Switch || (dd < 0.25f && dd > 0.5f * st.dprev));
-            if (dd <= g.tol_ns || f8_end) {
-              if (g.refine_steps == 0) {
-                last_ = 1;
-                status = dd <= g.tol_accept ? kSubOk : kSubNotConv;
-              } else {
-                st.phase = 1;
-                st.refine_left = g.refine_steps;
-                nxt = g.refine_fmt;
-              }
-            }
-          } else if (--st.refine_left <= 0) {
-            if (dd <= g.tol_accept) {
-              last_ = 1;
-              status = kSubOk;
-            } else if (dd < st.dprev) {
-              st.refine_left = 1;   // still converging: one more step (bounded by the step cap below)
-            } else {
-              last_ = 1;
-              status = kSubNotConv;
-            }
-          }
-          const int cap = g.budget ? min(g.max_iter, g.budget[st.job]) : g.max_iter;
-          if (!last_ && steps >= cap) {
-            last_ = 1;
-            status = kSubNotConv;
-          }
-          st.dprev = dd;
-          st.steps = steps;
-          st.last = last_;
-          st.status = status;
-          st.fnxt = nxt;
-          st.kind = 1;
-        } else {
-          // after X T: X_{k+1} is the current X (ping-pong unless written in place), in the next format
-          if (d.ncb != 1) st.cur ^= 1;
-          st.fcur = st.fnxt;
-          st.kind = 0;
-        }
-      }
-      if (d.last) {
-        if constexpr (kMode == 1) {
-          if (tid == 128) {
-            const SlotState& sf = sh.slot[d.slot];
-            g.prep_out[sf.job] = sf.status;
-            const double n3 = (double)sf.n * sf.n * sf.n;
-            // step 0 needs one product (Y_1), every further step three but the last two (no Y update); then X, A
-            const double prods = 3.0 * sf.steps - (g.Aout ? 1.0 : 2.0);
-            atomicAdd(&g.flops[0], 2.0 * n3 * prods);
-            atomicAdd(&g.flops[1], 6.0 * n3 * prods);
-          }
-        } else {
-          finish_slot(d.slot);
-        }
-        start_slot(d.slot);
-      } else {
-        tc::mbar_arrive(&sh.epi_done[d.slot]);
-      }
+      float dsum = 0.0f;
+      if (tid == 128)
+        for (int w = 0; w < kEpiWarps; ++w) dsum += sh.red[i & 1][w];
+      arrive(d, dsum);
+      if (tid == 128) tc::mbar_arrive(&sh.desc_free[i % kRing]);
     }
     if (sh.err && tid == 128) {
       // a wait ran out: the submatrices in flight are reported as timed out
-      for (int s = 0; s < kSlots; ++s) {
-        const int J = sh.slot[s].job;
+      for (int s = 0; s < 2 * kSlots; ++s) {
+        const int J = s & 1 ? sh.slot[s >> 1].fin : sh.slot[s >> 1].job;
         if (J >= 0 && kMode == 1) {
           g.prep_out[J] = kSubTimeout;
         } else if (J >= 0) {
           g.status[J] = kSubTimeout;
-          g.iters[J] = sh.slot[s].steps;
-          g.rsteps[J] = sh.slot[s].rsteps;
+          g.iters[J] = sh.slot[s >> 1].steps;
+          g.rsteps[J] = sh.slot[s >> 1].rsteps;
           g.tS[J] = 0.0;
           g.tH[J] = 0.0;
         }
@@ -1151,12 +1266,12 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
   // TMA loads and MMAs still in flight before the shared and tensor memory are released
   __syncthreads();
   if (sh.err) {
-    if (warp == 0 && lane == 0)
-      for (int s = 0; s < kStages; ++s)
-        if (armed[s]) tc::mbar_wait(&sh.full[s], arm_phase[s], tc::globaltimer() + 50000000ull);
+    if (warp == 2 && lane == 0)
+      for (uint32_t k = loads > kStages ? loads - kStages : 0; k < loads; ++k)
+        tc::mbar_wait_ns(&sh.full[k % kStages], (k / kStages) & 1, 50000000ull);
     if (warp == 1 && lane == 0) {
       tc::mma_commit(&sh.idle);
-      tc::mbar_wait(&sh.idle, 0, tc::globaltimer() + 50000000ull);
+      tc::mbar_wait_ns(&sh.idle, 0, 50000000ull);
     }
   }
   tc::tc_fence_before();
@@ -1178,10 +1293,11 @@ __global__ void k_status_pending(int32_t j0, int32_t count, const int32_t* __res
 // ==================================================================================== host side
 
 struct TcState {
-  DevBuf planes, order, err;
+  DevBuf planes, order, err, groups;
   int R = 0, LD = 0, slots = 0;
   int64_t ord_j0 = -1, ord_j1 = -1;
   int32_t ord_large = 0;          // how many of the cached order (a prefix) have n above 192
+  int32_t ord_mean = 0;           // their mean dimension
   DevBuf inv_planes, inv_flops;   // inverse mode: its own plane layout (kPlanesInv per slot), flop sums
   int iR = 0, iLD = 0, islots = 0;
 };
@@ -1197,6 +1313,7 @@ void tc_release(nolsm_plan* plan) {
   dev_free(plan, s->planes);
   dev_free(plan, s->order);
   dev_free(plan, s->err);
+  dev_free(plan, s->groups);
   dev_free(plan, s->inv_planes);
   dev_free(plan, s->inv_flops);
   delete s;
@@ -1219,15 +1336,13 @@ static bool formats(int precision, Fmt* main_fmt, Fmt* refine_fmt) {
   }
 }
 
-// The inverse kernel's register split (setmaxnreg) assumes the launch gives each of its 512 threads
-// kRegsLaunch registers; with fewer, the epilogue warpgroups' increase could never be granted, so the launch
-// is refused.
-static nolsm_status check_register_split(const void* fn) {
+// The register split (setmaxnreg) assumes that the launch gives each thread regs registers; with fewer, the epilogue
+// warpgroups' increase could never be granted, so the launch is refused.
+static nolsm_status check_register_split(const void* fn, int regs) {
   cudaFuncAttributes at{};
   NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, fn));
-  if (at.numRegs != kRegsLaunch) {
-    set_error("k_ns_tc was built with %d registers per thread; its register split needs exactly %d", at.numRegs,
-              kRegsLaunch);
+  if (at.numRegs != regs) {
+    set_error("k_ns_tc was built with %d registers per thread; its register split needs exactly %d", at.numRegs, regs);
     return NOLSM_ERR_UNSUPPORTED;
   }
   return NOLSM_OK;
@@ -1235,26 +1350,66 @@ static nolsm_status check_register_split(const void* fn) {
 
 // ------------------------------------------------------------------ launch shapes and their tuner
 
+// The maps of [planes][R][LD] 2-byte planes; one_byte: also as rows of 2 LD bytes for E4M3 (which runs in shape 0)
+static nolsm_status make_maps(TcMaps* m, void* base, int R, int LD, int planes, bool one_byte) {
+  const uint64_t r = (uint64_t)R, ld = (uint64_t)LD, z = (uint64_t)planes;
+  const CUtensorMapSwizzle sw64 = CU_TENSOR_MAP_SWIZZLE_64B;
+  bool ok = tmap::make_3d(&m->A, base, 2, ld, r, z, 32, 128, sw64) && tmap::make_3d(&m->A2, base, 2, ld, r, z, 32, 128, sw64, 2) &&
+            tmap::make_blocks(&m->B, base, ld, r, z, 32, 1, 1) && tmap::make_blocks(&m->B2, base, ld, r, z, 32, 2, 1) &&
+            tmap::make_blocks(&m->Bx2, base, ld, r, z, 32, 1, 2) && tmap::make_blocks(&m->B2x2, base, ld, r, z, 32, 2, 2) &&
+            tmap::make_3d(&m->S, base, 2, ld, r, z, 32, 32, sw64) && tmap::make_3d(&m->S2, base, 2, ld, r, z, 32, 32, sw64, 2);
+  m->A8 = m->A;
+  m->B8 = m->B;
+  if (one_byte)
+    ok = ok && tmap::make_3d(&m->A8, base, 1, 2 * ld, r, z, 128, 128) &&
+         tmap::make_3d(&m->B8, base, 1, 2 * ld, r, z, 128, Shape<0>::kTileN);
+  if (ok) return NOLSM_OK;
+  set_error("cuTensorMapEncodeTiled rejected the scratch layout (R %d, LD %d, planes %d)", R, LD, planes);
+  return NOLSM_ERR_CUDA;
+}
+
 using TcKernel = decltype(&k_ns_tc<0, 0>);
-struct TcMaps { CUtensorMap mA, mB, mS, mA8, mB8, mS16, mS2, mS16x2; };
 
 static TcKernel tc_kernel(int mode, int shape) {
   if (mode == 0) return shape == 0 ? &k_ns_tc<0, 0> : &k_ns_tc<0, 1>;
   return shape == 0 ? &k_ns_tc<1, 0> : &k_ns_tc<1, 1>;
 }
 
+// How many CTAs share a submatrix, by the mean dimension of a launch's submatrices above 192 rows: enough for the planes
+// of the submatrices in flight to stay in L2, few enough for a product's tiles (2 at n = 256, 18 at n = 650) to give
+// each CTA some. Measured, sign + inverse, ms, with 1 / 2 / 4 / 8 CTAs: 5,000 of n = 193-310 (mean 222) 24.4 / 23.0 /
+// 32.2 / 59.5; 512 merged sites of n = 200-400 13.6 / 7.4 / 6.8 / 8.4; 343 of n = 200-500 10.9 / 7.5 / 6.7 / 6.9; 512 of
+// n = 598-713 35.5 / 30.0 / 24.3 / 20.9, with 16 38.3.
+static int group_size(int mean_n) {
+  return mean_n <= 192 ? 1 : mean_n <= 256 ? 2 : mean_n <= 512 ? 4 : 8;
+}
+static int group_slots(int G, int64_t count, int sms) {
+  return (int)std::min<int64_t>(sms / G, (count + kSlots - 1) / kSlots) * kSlots;
+}
+
 // One launch of kernel (mode, shape) over the submatrices g.order[0, g.j1) (g.j0 = 0): one CTA per SM at most,
-// kSlots submatrices in flight in each; the work counter is reset first.
-static nolsm_status launch_shape(int mode, int shape, const TcMaps& m, const TcArgs& g, int sms, cudaStream_t st) {
+// kSlots submatrices in flight in each group of them; the work counter and the groups' are reset first. CTAs that wait
+// on one another have to run at the same time: a cooperative launch.
+static nolsm_status launch_shape(int mode, int shape, const TcMaps& m, TcArgs g, int sms, cudaStream_t st) {
   const TcKernel k = tc_kernel(mode, shape);
   const int threads = shape == 0 ? Shape<0>::kThreads : Shape<1>::kThreads;
   const int smem = shape == 0 ? Shape<0>::kSmemBytes : Shape<1>::kSmemBytes;
   NOLSM_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  if (shape == 1) NOLSM_TRY(check_register_split(reinterpret_cast<const void*>(k)));
+  NOLSM_TRY(check_register_split(reinterpret_cast<const void*>(k), shape == 0 ? Shape<0>::kRegsLaunch : Shape<1>::kRegsLaunch));
   NOLSM_CUDA_TRY(cudaMemsetAsync(g.next, 0, sizeof(int32_t), st));
-  const int ctas = (int)std::min<int64_t>(sms, ((int64_t)g.j1 + kSlots - 1) / kSlots);
-  k<<<ctas, threads, smem, st>>>(m.mA, m.mB, m.mS, m.mA8, m.mB8, m.mS16, m.mS2, m.mS16x2, g);
-  NOLSM_LAUNCH_CHECK();
+  const int slots = group_slots(g.group, g.j1, sms);
+  if (g.group > 1) NOLSM_CUDA_TRY(cudaMemsetAsync(g.groups, 0, sizeof(GroupSlot) * slots, st));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(slots / kSlots * g.group));
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = g.group > 1 ? 1 : 0;
+  NOLSM_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, m, g));
   return NOLSM_OK;
 }
 
@@ -1330,24 +1485,30 @@ static nolsm_status bucket_shape(int mode, int precision, int bucket, bool fixed
 // launch per bucket.
 template <typename Pending>
 static nolsm_status run_buckets(int mode, int precision, bool fixed0, const TcMaps& m, TcArgs g, const int32_t* order,
-                                int32_t n_large, int32_t count, int sms, cudaStream_t st, Pending pending) {
+                                int32_t n_large, int32_t count, int mean_n, int sms, cudaStream_t st, Pending pending) {
   if (count <= 0) return NOLSM_OK;
   int s1 = -1, s0 = -1;
+  const int g1 = fixed0 ? 1 : group_size(mean_n), g0 = 1;
+  g.group = g1;
   if (n_large > 0) NOLSM_TRY(bucket_shape(mode, precision, 1, fixed0, m, g, order, n_large, sms, st, pending, &s1));
+  g.group = g0;
   if (count > n_large)
     NOLSM_TRY(bucket_shape(mode, precision, 0, fixed0, m, g, order + n_large, count - n_large, sms, st, pending, &s0));
   g.j0 = 0;
-  if (n_large == 0 || n_large == count || s1 == s0) {
+  if (n_large == 0 || n_large == count || (s1 == s0 && g1 == g0)) {
+    g.group = n_large > 0 ? g1 : g0;
     g.order = order;
     g.j1 = count;
     NOLSM_TRY(pending(order, count));
     return launch_shape(mode, n_large > 0 ? s1 : s0, m, g, sms, st);
   }
   g.order = order;
+  g.group = g1;
   g.j1 = n_large;
   NOLSM_TRY(pending(order, n_large));
   NOLSM_TRY(launch_shape(mode, s1, m, g, sms, st));
   g.order = order + n_large;
+  g.group = g0;
   g.j1 = count - n_large;
   NOLSM_TRY(pending(order + n_large, count - n_large));
   return launch_shape(mode, s0, m, g, sms, st);
@@ -1395,18 +1556,8 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   const bool f8 = mf.fmt == FMT_E4M3;
   const int32_t above = f8 ? 0 : kResMaxN;
   const bool streamed = maxn > above, resident = !f8 && minn <= kResMaxN;
-  // one CTA per SM at most, each with kSlots submatrices in flight (one scratch sub-slot each)
-  const int ctas = (int)std::min<int64_t>(sms, (work + kSlots - 1) / kSlots);
-  const int slots = ctas * kSlots;
-  if (streamed && (!S->planes.p || S->R < R || S->LD < LD || S->slots < slots)) {
-    const int nR = std::max(R, S->R), nLD = std::max(LD, S->LD), nS = std::max(slots, S->slots);
-    dev_free(plan, S->planes);
-    NOLSM_TRY(dev_alloc(plan, S->planes, sizeof(uint16_t) * (size_t)kPlanes * nS * nR * nLD));
-    S->R = nR;
-    S->LD = nLD;
-    S->slots = nS;
-  }
   if (!S->err.p) NOLSM_TRY(dev_alloc(plan, S->err, sizeof(int32_t) * 4));
+  if (!S->groups.p) NOLSM_TRY(dev_alloc(plan, S->groups, sizeof(GroupSlot) * kSlots * sms));
   if (S->ord_j0 != j0 || S->ord_j1 != j1) {
     std::vector<int32_t> ord((size_t)(j1 - j0));
     for (int64_t J = j0; J < j1; ++J) ord[(size_t)(J - j0)] = (int32_t)J;
@@ -1420,7 +1571,21 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     S->ord_j0 = j0;
     S->ord_j1 = j1;
     S->ord_large = 0;
-    while (S->ord_large < (int32_t)ord.size() && plan->h_sub_n[ord[(size_t)S->ord_large]] > 192) ++S->ord_large;
+    int64_t sum = 0;
+    while (S->ord_large < (int32_t)ord.size() && plan->h_sub_n[ord[(size_t)S->ord_large]] > 192)
+      sum += plan->h_sub_n[ord[(size_t)S->ord_large++]];
+    S->ord_mean = S->ord_large > 0 ? (int32_t)(sum / S->ord_large) : 0;
+  }
+  // one CTA per SM at most, each group of them with kSlots submatrices in flight (one scratch sub-slot each)
+  const int group = f8 ? 1 : group_size(S->ord_mean);   // (E4M3: a turn writes the pair that it finishes)
+  const int slots = group_slots(group, work, sms);
+  if (streamed && (!S->planes.p || S->R < R || S->LD < LD || S->slots < slots)) {
+    const int nR = std::max(R, S->R), nLD = std::max(LD, S->LD), nS = std::max(slots, S->slots);
+    dev_free(plan, S->planes);
+    NOLSM_TRY(dev_alloc(plan, S->planes, sizeof(uint16_t) * (size_t)kPlanes * nS * nR * nLD));
+    S->R = nR;
+    S->LD = nLD;
+    S->slots = nS;
   }
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(S->err.p, 0, sizeof(int32_t), st));
@@ -1460,6 +1625,8 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   g.cond_max = cond_max(o.precision);
   g.ill_max_n = prepare_fp64_max_n();
   g.above_n = above;
+  g.group = group;
+  g.groups = S->groups.as<GroupSlot>();
   // every submatrix of a launch starts as "timed out" (k_status_pending), the kernel overwrites what it takes
   int32_t* status = plan->status.as<int32_t>();
   auto pending = [&](const int32_t* list, int32_t count) -> nolsm_status {
@@ -1471,34 +1638,13 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   const int32_t* order = spec.list ? spec.list : S->order.as<int32_t>();
   NOLSM_TRY(pending(order, (int32_t)work));
   if (streamed) {
-    CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
-    if (!tmap::make_3d(&mS16, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
-                       CU_TENSOR_MAP_SWIZZLE_64B) ||
-        !tmap::make_3d(&mS16x2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 16,
-                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-        !tmap::make_3d(&mS2, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
-                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-        !tmap::make_3d(&mA, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 128) ||
-        !tmap::make_3d(&mB, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 64, 64) ||
-        !tmap::make_3d(&mS, S->planes.p, 2, (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 32, 32,
-                       CU_TENSOR_MAP_SWIZZLE_64B)) {
-      set_error("cuTensorMapEncodeTiled rejected the scratch layout (R %d, LD %d, slots %d)", S->R, S->LD, S->slots);
-      return NOLSM_ERR_CUDA;
-    }
-    // one-byte views of the same planes (rows of 2 LD bytes) for E4M3 operands, both loaded K-major (E4M3 runs
-    // in shape 0, whose B box is 256 rows)
-    TcMaps m{mA, mB, mS, {}, {}, mS16, mS2, mS16x2};
-    if (!tmap::make_3d(&m.mA8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128, 128) ||
-        !tmap::make_3d(&m.mB8, S->planes.p, 1, 2 * (uint64_t)S->LD, (uint64_t)S->R, (uint64_t)S->slots * kPlanes, 128,
-                       Shape<0>::kTileN)) {
-      set_error("cuTensorMapEncodeTiled rejected the one-byte scratch layout");
-      return NOLSM_ERR_CUDA;
-    }
+    TcMaps m;
+    NOLSM_TRY(make_maps(&m, S->planes.p, S->R, S->LD, S->slots * kPlanes, f8));
     if (spec.list) {   // reruns and a bisection's later points: one launch in list order, shape 0
       NOLSM_TRY(launch_shape(0, 0, m, g, sms, st));
     } else {           // the largest-first order in its two buckets: n above 192, the rest (E4M3 only)
       NOLSM_TRY(run_buckets(0, o.precision, f8, m, g, S->order.as<int32_t>(), S->ord_large,
-                            f8 ? (int32_t)work : S->ord_large, sms, st, pending));
+                            f8 ? (int32_t)work : S->ord_large, S->ord_mean, sms, st, pending));
     }
   }
   if (resident) {
@@ -1548,6 +1694,7 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
   NOLSM_CUDA_TRY(cudaGetDevice(&dev));
   NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (!S->err.p) NOLSM_TRY(dev_alloc(plan, S->err, sizeof(int32_t) * 4));
+  if (!S->groups.p) NOLSM_TRY(dev_alloc(plan, S->groups, sizeof(GroupSlot) * kSlots * sms));
   if (!S->inv_flops.p) NOLSM_TRY(dev_alloc(plan, S->inv_flops, sizeof(double) * 2));
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(S->err.p, 0, sizeof(int32_t) * 4, st));
@@ -1589,7 +1736,8 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
   auto streamed = [&](const int32_t* order, int32_t n_large, int32_t count, int32_t again) -> nolsm_status {
     const int max_n = again ? std::min(a.max_n, kResMaxN) : a.max_n;
     const int LD = (max_n + 63) & ~63, R = (max_n + 127) & ~127;
-    const int slots = (int)std::min<int64_t>(sms, (count + kSlots - 1) / kSlots) * kSlots;
+    const int group = group_size(again ? 0 : a.mean_n);
+    const int slots = group_slots(group, count, sms);
     if (!S->inv_planes.p || S->iR < R || S->iLD < LD || S->islots < slots) {
       const int nR = std::max(R, S->iR), nLD = std::max(LD, S->iLD), nS = std::max(slots, S->islots);
       dev_free(plan, S->inv_planes);
@@ -1598,22 +1746,8 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
       S->iLD = nLD;
       S->islots = nS;
     }
-    const uint64_t depth = (uint64_t)S->islots * kPlanesInv;
-    CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
-    if (!tmap::make_3d(&mS16, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
-                       CU_TENSOR_MAP_SWIZZLE_64B) ||
-        !tmap::make_3d(&mS16x2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 16,
-                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-        !tmap::make_3d(&mS2, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
-                       CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-        !tmap::make_3d(&mA, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 128) ||
-        !tmap::make_3d(&mB, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 64, 64) ||
-        !tmap::make_3d(&mS, S->inv_planes.p, 2, (uint64_t)S->iLD, (uint64_t)S->iR, depth, 32, 32,
-                       CU_TENSOR_MAP_SWIZZLE_64B)) {
-      set_error("cuTensorMapEncodeTiled rejected the inverse scratch layout (R %d, LD %d, slots %d)", S->iR, S->iLD,
-                S->islots);
-      return NOLSM_ERR_CUDA;
-    }
+    TcMaps m;
+    NOLSM_TRY(make_maps(&m, S->inv_planes.p, S->iR, S->iLD, S->islots * kPlanesInv, false));
     TcArgs g{};
     g.j0 = 0; g.j1 = count;
     g.order = order;
@@ -1628,12 +1762,13 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     g.Aout = a.Aout; g.Xout = a.Xout; g.prep_out = a.prep_out;
     g.tol_inv = a.tol_inv; g.max_inv = a.max_inv;
     g.again = again;
+    g.group = group;
+    g.groups = S->groups.as<GroupSlot>();
     g.wait_ns = kWaitNs;
     g.flops = S->inv_flops.as<double>();
-    const TcMaps m{mA, mB, mS, mA, mB, mS16, mS2, mS16x2};
     plan->stats.launches += 2;
     if (again) return launch_shape(1, 0, m, g, sms, st);
-    return run_buckets(1, NOLSM_FP16, false, m, g, order, n_large, count, sms, st, pending);
+    return run_buckets(1, NOLSM_FP16, false, m, g, order, n_large, count, a.mean_n, sms, st, pending);
   };
   if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, a.n_large, 0));
   int32_t again = 0;
@@ -1744,16 +1879,8 @@ extern "C" nolsm_status nolsm_sign_noalloc(int32_t count, const int32_t* sub_n, 
   unsigned char* base = static_cast<unsigned char*>(addr);
   int32_t* ints = reinterpret_cast<int32_t*>(base + kNaPlanesBytes);
 
-  CUtensorMap mA, mB, mS, mS16, mS2, mS16x2;
-  if (!tmap::make_3d(&mS16, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 32, 16, CU_TENSOR_MAP_SWIZZLE_64B) ||
-      !tmap::make_3d(&mS16x2, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 32, 16, CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mS2, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B, 2) ||
-      !tmap::make_3d(&mA, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 64, 128) ||
-      !tmap::make_3d(&mB, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 64, 64) ||
-      !tmap::make_3d(&mS, base, 2, kNaLD, kNaR, (uint64_t)kNaSlots * kPlanes, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) {
-    set_error("nolsm_sign_noalloc: cuTensorMapEncodeTiled rejected the static scratch layout");
-    return NOLSM_ERR_CUDA;
-  }
+  TcMaps m;
+  NOLSM_TRY(make_maps(&m, base, kNaR, kNaLD, kNaSlots * kPlanes, false));
   k_noalloc_reset<<<(count + 255) / 256, 256, 0, st>>>(base, count, status);
   NOLSM_LAUNCH_CHECK();
   TcArgs g{};
@@ -1773,10 +1900,12 @@ extern "C" nolsm_status nolsm_sign_noalloc(int32_t count, const int32_t* sub_n, 
   g.err = ints + 3 * kNaMaxSub + 32;
   g.Dc = Dc; g.tS = t_S; g.tH = t_H; g.iters = iters; g.status = status;
   g.rsteps = ints + 2 * kNaMaxSub;
+  g.group = 1;
   g.nbelow = nullptr;
   g.wait_ns = opts->wait_ns > 0 ? (uint64_t)opts->wait_ns : kWaitNs;
   NOLSM_CUDA_TRY(cudaFuncSetAttribute((k_ns_tc<0, 0>), cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<0>::kSmemBytes));
-  k_ns_tc<0, 0><<<std::min(kNaSlots / kSlots, (count + kSlots - 1) / kSlots), Shape<0>::kThreads, Shape<0>::kSmemBytes, st>>>(mA, mB, mS, mA, mB, mS16, mS2, mS16x2, g);
+  NOLSM_TRY(check_register_split(reinterpret_cast<const void*>(&k_ns_tc<0, 0>), Shape<0>::kRegsLaunch));
+  k_ns_tc<0, 0><<<std::min(kNaSlots / kSlots, (count + kSlots - 1) / kSlots), Shape<0>::kThreads, Shape<0>::kSmemBytes, st>>>(m, g);
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }

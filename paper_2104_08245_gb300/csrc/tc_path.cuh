@@ -21,6 +21,7 @@ struct NsInvArgs {
   int32_t count;
   int32_t n_large;              // how many of them (a prefix of order) have n above 192
   int32_t max_n;
+  int32_t mean_n;               // of the n_large
   const double* ws;
   int64_t a_base, chunk_n2;
   float* Aout;                  // null: T_J(S)^-1 alone

@@ -70,6 +70,14 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   return d;
 }
 
+// u == k ? a : b as an instruction that the compiler does not fold into an indexed (local memory) array access: local
+// memory shares its bandwidth with the MMAs' operands
+__device__ __forceinline__ uint32_t pick(int u, int k, uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, %2;\n\tselp.b32 %0, %3, %4, p;\n\t}" : "=r"(r) : "r"(u), "r"(k), "r"(a), "r"(b));
+  return r;
+}
+
 // m times 32 accumulators of one row as packed hi (and lo) pairs, and with kSq the sum of the squares added to sq.
 template <int kFmt, bool kLo, bool kSq>
 __device__ __forceinline__ void scale_split_t(const uint32_t (&r)[32], float m, uint32_t (&h)[16], uint32_t (&l)[16],

@@ -63,6 +63,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   }
 }
 
+// The same with a limit from now on (ns); the timer is read only when the phase has not completed by then.
+__device__ __forceinline__ bool mbar_wait_ns(uint64_t* bar, uint32_t parity, uint64_t limit) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer();
+  for (;;) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (globaltimer() - t0 >= limit) return false;
+  }
+}
+
 // Register reallocation between warpgroups: every thread of the warpgroup executes the same instruction; a
 // decrease returns registers to the CTA's pool, an increase waits until the pool holds them.
 template <int N>
@@ -76,6 +86,13 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
       ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z,
+                                            int w) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w)
       : "memory");
 }
 // Tiled TMA store of a shared-memory box to global memory, tracked by the issuing thread's bulk groups.
@@ -105,6 +122,18 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint3
 __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
   const uint64_t a = reinterpret_cast<uint64_t>(p) & ~uint64_t(15), e = (reinterpret_cast<uint64_t>(p) + bytes) & ~uint64_t(15);
   if (e > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
+}
+// arrival at and reading of a counter in global memory that several CTAs share
+__device__ __forceinline__ void red_release_gpu(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// (polled relaxed, fenced once: an acquire per poll would drop the SM's L1 each time)
+__device__ __forceinline__ bool reached_gpu(const uint32_t* p, uint32_t v) {
+  uint32_t x;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+  if (x < v) return false;
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  return true;
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -217,6 +246,11 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, ui
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
+}
+
+// The same with 64-byte swizzling (mode 4): atoms of 8 rows of 64 bytes, 512-byte aligned.
+__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return (sdesc_sw128(saddr, lbo, sbo) & ~((uint64_t)7 << 61)) | ((uint64_t)4 << 61);
 }
 
 // Instruction descriptor of kind::f16 / kind::f8f6f4 with FP32 accumulation. fmt: kind::f16 0 = F16,

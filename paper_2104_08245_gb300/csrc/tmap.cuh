@@ -41,4 +41,18 @@ inline bool make_3d(CUtensorMap* map, void* base, int esize, uint64_t dim0, uint
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same planes of 2-byte elements ([planes][rows][ld], ld a multiple of 64) as columns in blocks of 64: a 4-D map
+// [ld / 64][planes][rows][64], whose box of `blocks` blocks by `depth` planes by `box1` rows lands block by block.
+inline bool make_blocks(CUtensorMap* map, void* base, uint64_t ld, uint64_t rows, uint64_t planes, uint32_t box1,
+                        uint32_t depth, uint32_t blocks) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[4] = {64, rows, planes, ld / 64};
+  cuuint64_t strides[3] = {ld * 2, ld * rows * 2, 128};
+  cuuint32_t box[4] = {64, box1, depth, blocks};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tmap

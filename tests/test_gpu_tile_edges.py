@@ -90,10 +90,8 @@ def clusters(sizes, pair, arg, seed=5):
     return types.SimpleNamespace(nbf=np.array(nbf, np.int32), S=csr("S"), H=csr("H"), n_occ=float(occ)), exact
 
 
-@pytest.mark.parametrize("prec,arg", [(p, a) for p in TOL for a in ((0.0005, 0.1, 0.6) if p == "fp64" else (1.2, 0.5, 0.25))])
-def test_every_tile_edge(nl, prec, arg):
-    sizes = SIZES_FP64 if prec == "fp64" else SIZES
-    sysm, exact = clusters(sizes, random_pair if prec == "fp64" else lattice_pair, arg)
+def solved(nl, prec, sizes, pair, arg):
+    sysm, exact = clusters(sizes, pair, arg)
     po = orc.build_plan(sysm.nbf, sysm.S.row_ptr, sysm.S.col_idx, sysm.H.row_ptr, sysm.H.col_idx)
     plan = nl.nolsm_build_submatrices(nl.DeviceSystem(sysm))
     r = nl.nolsm_solve_batch(plan, MU, nl.options(prec))
@@ -105,3 +103,16 @@ def test_every_tile_edge(nl, prec, arg):
         at += n
     print(f"{prec}, {arg}: max|dD| = {max(err.values()):.3e}")
     assert max(err.values()) <= TOL[prec], err
+
+
+@pytest.mark.parametrize("prec,arg", [(p, a) for p in TOL for a in ((0.0005, 0.1, 0.6) if p == "fp64" else (1.2, 0.5, 0.25))])
+def test_every_tile_edge(nl, prec, arg):
+    sizes = SIZES_FP64 if prec == "fp64" else SIZES
+    solved(nl, prec, sizes, random_pair if prec == "fp64" else lattice_pair, arg)
+
+
+@pytest.mark.parametrize("sizes", [(193, 255, 257), (321, 384, 385, 512), (448, 513, 640, 767, 961)])
+def test_groups_of_ctas(nl, sizes):
+    """Streamed submatrices shared by two, four and eight CTAs (by their mean dimension), with one to four column tiles,
+    and a Q of more rows than one staged piece."""
+    solved(nl, "bf16x3", sizes, lattice_pair, 0.5)
