@@ -493,7 +493,16 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
            (e == J || 2 * 8 * (plan->h_a_off[e + 1] - plan->h_a_off[J]) <= budget))
       ++e;
     const int64_t n2 = plan->h_a_off[e] - plan->h_a_off[J];
-    NOLSM_TRY(ensure(plan, plan->ws_dense, sizeof(double) * 2 * (size_t)n2));
+    // what the largest chunk of the range needs: a workspace that grew from one chunk to the next would be mapped anew
+    const int64_t cap = std::max(n2, std::min(plan->h_a_off[j1] - plan->h_a_off[J], budget / 16));
+    NOLSM_TRY(ensure(plan, plan->ws_dense, sizeof(double) * 2 * (size_t)cap));
+    // the chunk's submatrices, largest first: CTAs take them in this order, so that the last wave is made of small ones.
+    // Copied before the gather starts, as a copy from host memory waits for the stream.
+    std::vector<int32_t> ord;
+    largest_first(plan->h_sub_n, J, e - J, ord);
+    NOLSM_TRY(ensure(plan, plan->prep_order, sizeof(int32_t) * (size_t)std::max(j1 - J, e - J)));
+    NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->prep_order.p, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, st));
+    NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is host memory
     GatherArgs g{};
     g.n_mol = n_mol;
     g.nbf = plan->sys.nbf;
@@ -543,20 +552,9 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
     pa.Q = plan->Q.as<double>(); pa.lam = plan->lam.as<double>(); pa.prep_status = plan->prep_status.as<int32_t>();
     int chunk_max_n = 1;
     for (int64_t k = J; k < e; ++k) chunk_max_n = std::max(chunk_max_n, plan->h_sub_n[k]);
-    // the chunk's submatrices, largest first
-    std::vector<int32_t> ord;
-    auto sort_chunk = [&]() -> nolsm_status {
-      ord.resize((size_t)(e - J));
-      for (int64_t k = J; k < e; ++k) ord[(size_t)(k - J)] = (int32_t)k;
-      std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
-      NOLSM_TRY(ensure(plan, plan->prep_order, sizeof(int32_t) * ord.size()));
-      NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->prep_order.p, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, st));
-      NOLSM_CUDA_TRY(cudaStreamSynchronize(st));   // ord is host memory
-      return NOLSM_OK;
-    };
     // T_J(S)^-1 (and A_J unless Aout is null) in FP32 by the inverse square root on the tensor cores
     auto tensor_inverse = [&](float* Aout) -> nolsm_status {
-      NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)n2));
+      NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)cap));
       NsInvArgs ia;
       ia.order = plan->prep_order.as<int32_t>();
       ia.count = (int32_t)(e - J);
@@ -582,8 +580,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       // the FP32 inverse refined with exact digit products on the tensor cores (oz_path.cu); the FP64 Cholesky
       // factorisation of what that left, in particular overlaps that are not positive definite
       if (chunk_max_n <= prepare_fp64_max_n()) {
-        NOLSM_TRY(sort_chunk());
-        NOLSM_TRY(tensor_inverse(nullptr));
+          NOLSM_TRY(tensor_inverse(nullptr));
         int dev = 0, sms = 0;
         NOLSM_CUDA_TRY(cudaGetDevice(&dev));
         NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -614,7 +611,6 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       // the coupled Newton-Schulz inverse square root on the tensor cores (A_J and X = T_J(S)^-1 in FP32),
       // then the refinement of the centre columns of T_J(S)^-1 with X, then the FP64 preparation of what
       // either of them flagged
-      NOLSM_TRY(sort_chunk());
       NOLSM_TRY(tensor_inverse(P.A.as<float>()));
       pa.order = plan->prep_order.as<int32_t>();
       pa.L32 = plan->ws_l32.as<float>();
@@ -626,20 +622,19 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       const int64_t nbc = plan->h_c_off[e] - plan->h_c_off[J];
       NOLSM_TRY(ensure(plan, plan->ws_refine, (sizeof(double) + sizeof(float)) * (size_t)std::max<int64_t>(nbc, 1)));
       if (sym) {   // the factors stay for the finishing step D_c = L^-T U
-        NOLSM_TRY(ensure(plan, plan->ws_ysym, sizeof(float) * (size_t)n2));
+        NOLSM_TRY(ensure(plan, plan->ws_ysym, sizeof(float) * (size_t)cap));
         pa.L32 = plan->Lsym.as<float>() + plan->h_a_off[J];
         pa.sym = 1;
         pa.Ysym = plan->ws_ysym.as<float>();
         pa.Wc = plan->Wc.as<double>();
       } else {
-        NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)n2));
+        NOLSM_TRY(ensure(plan, plan->ws_l32, sizeof(float) * (size_t)cap));
         pa.L32 = plan->ws_l32.as<float>();
       }
       pa.c_base = plan->h_c_off[J];
       pa.Qp = plan->ws_refine.as<float2>();
       pa.W32 = reinterpret_cast<float*>(pa.Qp + std::max<int64_t>(nbc, 1));
       pa.fallback_max_n = sym ? 0 : prepare_fp64_max_n();   // no FP64 fallback for the symmetric form
-      NOLSM_TRY(sort_chunk());   // CTAs take the largest first, so that the last wave is made of small ones
       pa.order = plan->prep_order.as<int32_t>();
       NOLSM_TRY(launch_prepare_mixed(pa, (int)(e - J), chunk_max_n, P.A.as<float>(), st));
       plan->stats.launches += 3;
@@ -703,9 +698,8 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   const int64_t slot_elems = (int64_t)maxn * maxn;
   NOLSM_TRY(ensure(plan, plan->ws_ns, sizeof(double) * 3 * (size_t)slot_elems * slots));
   if (!spec.list && (plan->oz_j0 != j0 || plan->oz_j1 != j1)) {   // the range, largest first
-    std::vector<int32_t> ord((size_t)work);
-    for (int32_t k = 0; k < work; ++k) ord[(size_t)k] = (int32_t)j0 + k;
-    std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
+    std::vector<int32_t> ord;
+    largest_first(plan->h_sub_n, j0, work, ord);
     plan->oz_j0 = -1;
     NOLSM_TRY(ensure(plan, plan->oz_order, sizeof(int32_t) * (size_t)plan->n_mol));
     NOLSM_CUDA_TRY(cudaMemcpyAsync(plan->oz_order.p, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, st));

@@ -1559,9 +1559,8 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
   if (!S->err.p) NOLSM_TRY(dev_alloc(plan, S->err, sizeof(int32_t) * 4));
   if (!S->groups.p) NOLSM_TRY(dev_alloc(plan, S->groups, sizeof(GroupSlot) * kSlots * sms));
   if (S->ord_j0 != j0 || S->ord_j1 != j1) {
-    std::vector<int32_t> ord((size_t)(j1 - j0));
-    for (int64_t J = j0; J < j1; ++J) ord[(size_t)(J - j0)] = (int32_t)J;
-    std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return plan->h_sub_n[a] > plan->h_sub_n[b]; });
+    std::vector<int32_t> ord;
+    largest_first(plan->h_sub_n, j0, j1 - j0, ord);
     if (S->order.bytes < sizeof(int32_t) * ord.size()) {
       dev_free(plan, S->order);
       NOLSM_TRY(dev_alloc(plan, S->order, sizeof(int32_t) * (size_t)plan->n_mol));
