@@ -27,7 +27,7 @@ namespace nolsm {
 
 namespace {
 
-constexpr int kPowThreads = 256;
+constexpr int kPowThreads = 1024;   // at most (power_bounds)
 
 __device__ __forceinline__ float block_sum_f(float v, float* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -79,22 +79,50 @@ __global__ void __launch_bounds__(kPowThreads) k_power_bounds(PowArgs g, const T
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   float eu = 0.0f, ev = 0.0f;
   for (int it = 0; it < g.iters; ++it) {
-    // u2 = A u - lo u, v2 = hi v - A v: one warp per row, lanes along the row
-    for (int i = warp; i < n; i += nw) {
-      const TA* Ai = A + (size_t)i * n;
-      float au = 0.0f, av = 0.0f;
-      for (int k = lane; k < n; k += 32) {
-        const float a = (float)Ai[k];
-        au = fmaf(a, u[k], au);
-        av = fmaf(a, v[k], av);
+    // u2 = A u - lo u, v2 = hi v - A v: four rows a warp, lanes along them. Every iteration streams A (from DRAM once the
+    // submatrices in flight exceed L2), so what counts is loads in flight: 16 a lane here (343 submatrices of n =
+    // 200-500: 10.9 ms with a row a warp and some four loads in flight, 0.9 now).
+    for (int i0 = 4 * warp; i0 < n; i0 += 4 * nw) {
+      const TA* r[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = A + (size_t)min(i0 + q, n - 1) * n;
+      float au[4] = {0.0f, 0.0f, 0.0f, 0.0f}, av[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      int k = lane;
+      for (; k + 96 < n; k += 128) {
+        TA a[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) a[q][t] = r[q][k + 32 * t];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float uk = u[k + 32 * t], vk = v[k + 32 * t];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            au[q] = fmaf((float)a[q][t], uk, au[q]);
+            av[q] = fmaf((float)a[q][t], vk, av[q]);
+          }
+        }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        au += __shfl_xor_sync(0xffffffffu, au, o);
-        av += __shfl_xor_sync(0xffffffffu, av, o);
+      for (; k < n; k += 32) {
+        const float uk = u[k], vk = v[k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float a = (float)r[q][k];
+          au[q] = fmaf(a, uk, au[q]);
+          av[q] = fmaf(a, vk, av[q]);
+        }
       }
-      if (lane == 0) {
-        u2[i] = au - lo * u[i];
-        v2[i] = hi * v[i] - av;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        for (int o = 16; o > 0; o >>= 1) {
+          au[q] += __shfl_xor_sync(0xffffffffu, au[q], o);
+          av[q] += __shfl_xor_sync(0xffffffffu, av[q], o);
+        }
+        if (lane == 0 && i0 + q < n) {
+          u2[i0 + q] = au[q] - lo * u[i0 + q];
+          v2[i0 + q] = hi * v[i0 + q] - av[q];
+        }
       }
     }
     __syncthreads();
@@ -648,13 +676,17 @@ nolsm_status power_bounds(nolsm_plan* plan, int cls, int64_t j0, int64_t j1, con
   g.iters = 30;
   const int blocks = list ? count : (int)(b - a);
   if (blocks <= 0) return NOLSM_OK;
+  // Large submatrices, or too few to fill the SMs with small CTAs: 1,024 threads each, so that the loads in flight come
+  // from one submatrix (343 of n = 200-500: 256 threads 2.6, 512 1.6, 1,024 0.9 ms); else 256, whose barriers are cheaper
+  // (4,096 of n = 120-310: 0.1 ms below 512 threads, 1.1 ms below 1,024).
+  const int threads = plan->max_n > 320 || blocks <= 512 ? kPowThreads : 256;
   const size_t smem = sizeof(float) * 4 * (size_t)std::max(plan->max_n, 1);
   if (cls == kPrepFP64) {
     NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_power_bounds<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_power_bounds<double><<<blocks, kPowThreads, smem, st>>>(g, plan->prep64.A.as<double>());
+    k_power_bounds<double><<<blocks, threads, smem, st>>>(g, plan->prep64.A.as<double>());
   } else {
     NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_power_bounds<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_power_bounds<float><<<blocks, kPowThreads, smem, st>>>(g, prepared(plan, cls).A.as<float>());
+    k_power_bounds<float><<<blocks, threads, smem, st>>>(g, prepared(plan, cls).A.as<float>());
   }
   NOLSM_LAUNCH_CHECK();
   plan->stats.launches += 1;
