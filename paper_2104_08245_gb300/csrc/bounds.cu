@@ -297,228 +297,257 @@ __device__ MlpSmem load_params(const float* __restrict__ p, float* sm) {
     s.b1[e] = p[kOffB1 + e];
     s.b2[e] = p[kOffB2 + e];
   }
-  for (int e = threadIdx.x; e < kWidth * kWidth; e += blockDim.x) s.W2[(e >> 7) * kW2Ld + (e & 127)] = p[kOffW2 + e];
+  static_assert(kOffW2 % 4 == 0, "16-byte loads of W2");
+#pragma unroll 16
+  for (int e = 4 * threadIdx.x; e < kWidth * kWidth; e += 4 * kMlpThreads) {
+    const float4 w = *reinterpret_cast<const float4*>(p + kOffW2 + e);
+    float* d = s.W2 + (e >> 7) * kW2Ld + (e & 127);
+    d[0] = w.x;
+    d[1] = w.y;
+    d[2] = w.z;
+    d[3] = w.w;
+  }
   for (int e = threadIdx.x; e < kWidth * kOutputs; e += blockDim.x) s.W3[e] = p[kOffW3 + e];
   if (threadIdx.x < kOutputs) s.b3[threadIdx.x] = p[kOffB3 + threadIdx.x];
   __syncthreads();
   return s;
 }
 
-// y = W3^T tanh(W2^T tanh(W1^T x + b1) + b2) + b3 per sample; act (nullable) receives h1, h2.
+// A batch: rows start .. of (x, t) as they are (N = 0), or sample r of a minibatch: row (start + r) * 7919 + epoch *
+// 104729 (mod N).
+struct MlpBatch {
+  const float* x; const float* t;
+  int32_t N, start, epoch;
+  __device__ int64_t row(int r) const {
+    return N == 0 ? r : (((int64_t)(start + r) * 7919 + (int64_t)epoch * 104729) % N + N) % N;
+  }
+};
+
+// One sample by a warp, unit lane + 32 m of either layer: h1 = tanh(W1^T x + b1) (also to h1w, shared), h2 = tanh(W2^T h1 +
+// b2), y = W3^T h2 + b3 in every lane.
+__device__ __forceinline__ void mlp_sample(const MlpSmem& s, const float* __restrict__ x, int lane, float* h1w, float (&h1)[4],
+                                           float (&h2)[4], float (&y)[kOutputs]) {
+  float xv[kFeatures];
+#pragma unroll
+  for (int k = 0; k < kFeatures; ++k) xv[k] = x[k];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int u = lane + 32 * m;
+    float z = s.b1[u];
+#pragma unroll
+    for (int k = 0; k < kFeatures; ++k) z = fmaf(xv[k], s.W1[k * kWidth + u], z);
+    h1[m] = tanhf(z);
+    h1w[u] = h1[m];
+  }
+  __syncwarp();
+  float z[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) z[m] = s.b2[lane + 32 * m];
+#pragma unroll 8
+  for (int k = 0; k < kWidth; ++k) {
+    const float h = h1w[k];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) z[m] = fmaf(h, s.W2[k * kW2Ld + lane + 32 * m], z[m]);
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) h2[m] = tanhf(z[m]);
+#pragma unroll
+  for (int o = 0; o < kOutputs; ++o) {
+    float p = 0.0f;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) p = fmaf(h2[m], s.W3[(lane + 32 * m) * kOutputs + o], p);
+    for (int off = 16; off > 0; off >>= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
+    y[o] = p + s.b3[o];
+  }
+}
+
+// y per sample
 __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float* __restrict__ params, int32_t B,
-                                                             const float* __restrict__ x, float* __restrict__ y,
-                                                             float* __restrict__ act) {
+                                                             const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ __align__(16) float msm[];
   const MlpSmem s = load_params(params, msm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* h1w = s.wbuf + warp * 2 * kWidth;
   for (int b = blockIdx.x * 8 + warp; b < B; b += gridDim.x * 8) {
-    float xv[kFeatures];
-#pragma unroll
-    for (int k = 0; k < kFeatures; ++k) xv[k] = x[(size_t)b * kFeatures + k];
-    float h1[4], h2[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int u = lane + 32 * m;
-      float z = s.b1[u];
-#pragma unroll
-      for (int k = 0; k < kFeatures; ++k) z = fmaf(xv[k], s.W1[k * kWidth + u], z);
-      h1[m] = tanhf(z);
-      h1w[u] = h1[m];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int u = lane + 32 * m;
-      float z = s.b2[u];
-      for (int k = 0; k < kWidth; ++k) z = fmaf(h1w[k], s.W2[k * kW2Ld + u], z);
-      h2[m] = tanhf(z);
-    }
-    float yo[kOutputs];
-#pragma unroll
-    for (int o = 0; o < kOutputs; ++o) {
-      float p = 0.0f;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) p = fmaf(h2[m], s.W3[(lane + 32 * m) * kOutputs + o], p);
-      for (int off = 16; off > 0; off >>= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
-      yo[o] = p + s.b3[o];
-    }
+    float h1[4], h2[4], yo[kOutputs];
+    mlp_sample(s, x + (size_t)b * kFeatures, lane, s.wbuf + warp * 2 * kWidth, h1, h2, yo);
     if (lane == 0)
 #pragma unroll
       for (int o = 0; o < kOutputs; ++o) y[(size_t)b * kOutputs + o] = yo[o];
-    if (act) {
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        act[(size_t)b * 2 * kWidth + lane + 32 * m] = h1[m];
-        act[(size_t)b * 2 * kWidth + kWidth + lane + 32 * m] = h2[m];
-      }
-    }
     __syncwarp();
   }
 }
 
-// Per sample: dy = (y - t) / B, dz2 = (dy W3^T) * (1 - h2^2), dz1 = (dz2 W2^T) * (1 - h1^2); the loss
-// 1/(2B) sum (y - t)^2 is accumulated into loss (FP64).
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_backward(const float* __restrict__ params, int32_t B,
-                                                              const float* __restrict__ act,
-                                                              const float* __restrict__ y, const float* __restrict__ t,
-                                                              float* __restrict__ dz, float* __restrict__ dy,
-                                                              double* __restrict__ loss) {
+// A training step runs in three kernels (six launches of 50 us and their gaps before, 63 us a step of 1,024 samples, now
+// 29): forward and backward of a sample by one warp with the weights loaded once, the weight gradients, their sum and
+// Adam. The sums keep one order: samples of a chunk, then chunks.
+//
+// Per sample: y, dy = (y - t) / B, dz2 = (dy W3^T) * (1 - h2^2), dz1 = (dz2 W2^T) * (1 - h1^2); act receives h1, h2; the
+// loss 1/(2B) sum (y - t)^2 is accumulated into loss (FP64).
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_sample(const float* __restrict__ params, int32_t B, MlpBatch batch,
+                                                            float* __restrict__ act, float* __restrict__ dz,
+                                                            float* __restrict__ dy, double* __restrict__ loss) {
   extern __shared__ __align__(16) float msm[];
   const MlpSmem s = load_params(params, msm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* dz2w = s.wbuf + warp * 2 * kWidth;
+  float* h1w = s.wbuf + warp * 2 * kWidth;
+  float* dz2w = h1w + kWidth;
   double lsum = 0.0;
   for (int b = blockIdx.x * 8 + warp; b < B; b += gridDim.x * 8) {
-    float d[kOutputs];
+    const int64_t row = batch.row(b);
+    float h1[4], h2[4], d[kOutputs];
+    mlp_sample(s, batch.x + (size_t)row * kFeatures, lane, h1w, h1, h2, d);
 #pragma unroll
     for (int o = 0; o < kOutputs; ++o) {
-      const float r = y[(size_t)b * kOutputs + o] - t[(size_t)b * kOutputs + o];
+      const float r = d[o] - batch.t[(size_t)row * kOutputs + o];
       d[o] = r / (float)B;
       if (lane == 0) lsum += 0.5 * (double)r * (double)r / (double)B;
     }
-    const float* a = act + (size_t)b * 2 * kWidth;
+    float* a = act + (size_t)b * 2 * kWidth;
+    float* z = dz + (size_t)b * 2 * kWidth;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int u = lane + 32 * m;
       float g = 0.0f;
 #pragma unroll
       for (int o = 0; o < kOutputs; ++o) g = fmaf(d[o], s.W3[u * kOutputs + o], g);
-      const float h2 = a[kWidth + u];
-      const float z2 = g * (1.0f - h2 * h2);
+      const float z2 = g * (1.0f - h2[m] * h2[m]);
       dz2w[u] = z2;
-      dz[(size_t)b * 2 * kWidth + kWidth + u] = z2;
+      z[kWidth + u] = z2;
+      a[u] = h1[m];
+      a[kWidth + u] = h2[m];
     }
     __syncwarp();
+    float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 8
+    for (int u = 0; u < kWidth; ++u) {
+      const float w = dz2w[u];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int k = lane + 32 * m;
-      float g = 0.0f;
-      for (int u = 0; u < kWidth; ++u) g = fmaf(s.W2[k * kW2Ld + u], dz2w[u], g);
-      const float h1 = a[k];
-      dz[(size_t)b * 2 * kWidth + k] = g * (1.0f - h1 * h1);
+      for (int m = 0; m < 4; ++m) g[m] = fmaf(s.W2[(lane + 32 * m) * kW2Ld + u], w, g[m]);
     }
-    if (lane < kOutputs) dy[(size_t)b * kOutputs + lane] = d[lane];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) z[lane + 32 * m] = g[m] * (1.0f - h1[m] * h1[m]);
+#pragma unroll
+    for (int o = 0; o < kOutputs; ++o)
+      if (lane == o) dy[(size_t)b * kOutputs + o] = d[o];
     __syncwarp();
   }
   if (lane == 0 && lsum != 0.0) atomicAdd(loss, lsum);
 }
 
-// Partial weight gradients of one chunk of kChunk samples into part[chunk][kParams].
-__global__ void __launch_bounds__(256) k_mlp_wgrad(int32_t B, const float* __restrict__ x,
-                                                   const float* __restrict__ act, const float* __restrict__ dz,
-                                                   const float* __restrict__ dy, float* __restrict__ part) {
-  __shared__ __align__(16) float ha[kChunk][kWidth];   // h1, later h2
-  __shared__ __align__(16) float zb[kChunk][kWidth];   // dz2, later dz1
-  __shared__ float xs[kChunk][kFeatures];
-  __shared__ float ds[kChunk][kOutputs];
-  const int c0 = blockIdx.x * kChunk;
-  const int tid = threadIdx.x;
+// Partial weight gradients of one chunk of kChunk samples into part[chunk][kParams], in six blocks: W2 by 32 of its rows
+// (the first with b2), W1 with b1, W3 with b3. Bound by the latency of its loads; one block a chunk, 32 for a batch of
+// 1,024, took 21 us.
+constexpr int kSlices = 6;
+__global__ void __launch_bounds__(256) k_mlp_wgrad(int32_t B, MlpBatch batch, const float* __restrict__ act,
+                                                   const float* __restrict__ dz, const float* __restrict__ dy,
+                                                   float* __restrict__ part) {
+  __shared__ __align__(16) float zb[kChunk][kWidth];   // dz2, dz1 or h2
+  __shared__ __align__(16) float hb[kChunk][32];       // 32 of h1; x; dy
+  const int c0 = blockIdx.x * kChunk, slice = blockIdx.y, tid = threadIdx.x;
   float* out = part + (size_t)blockIdx.x * kParams;
+  const float* zsrc = slice < 4 ? dz + kWidth : slice == 4 ? dz : act + kWidth;
+#pragma unroll
   for (int e = tid; e < kChunk * kWidth; e += 256) {
     const int b = e >> 7, u = e & 127;
-    const bool ok = c0 + b < B;
-    ha[b][u] = ok ? act[(size_t)(c0 + b) * 2 * kWidth + u] : 0.0f;
-    zb[b][u] = ok ? dz[(size_t)(c0 + b) * 2 * kWidth + kWidth + u] : 0.0f;
+    zb[b][u] = c0 + b < B ? zsrc[(size_t)(c0 + b) * 2 * kWidth + u] : 0.0f;
   }
-  for (int e = tid; e < kChunk * kFeatures; e += 256) {
-    const int b = e / kFeatures, k = e - b * kFeatures;
-    xs[b][k] = c0 + b < B ? x[(size_t)(c0 + b) * kFeatures + k] : 0.0f;
-  }
-  for (int e = tid; e < kChunk * kOutputs; e += 256) {
-    const int b = e / kOutputs, o = e - b * kOutputs;
-    ds[b][o] = c0 + b < B ? dy[(size_t)(c0 + b) * kOutputs + o] : 0.0f;
+#pragma unroll
+  for (int e = tid; e < kChunk * 32; e += 256) {
+    const int b = e >> 5, k = e & 31;
+    float v = 0.0f;
+    if (c0 + b < B) {
+      if (slice < 4) v = act[(size_t)(c0 + b) * 2 * kWidth + 32 * slice + k];
+      else if (slice == 4 && k < kFeatures) v = batch.x[(size_t)batch.row(c0 + b) * kFeatures + k];
+      else if (slice == 5 && k < kOutputs) v = dy[(size_t)(c0 + b) * kOutputs + k];
+    }
+    hb[b][k] = v;
   }
   __syncthreads();
-  // gW2[i][j] = sum_b h1[b][i] dz2[b][j]: 8 x 8 outputs per thread
-  {
-    const int ti = tid >> 4, tj = tid & 15;
-    float acc[8][8];
+  if (slice < 4) {   // gW2[i][j] = sum_b h1[b][i] dz2[b][j]: 4 x 4 outputs per thread
+    const int i0 = 4 * (tid >> 5), j0 = tid & 31;
+    float acc[4][4];
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int c = 0; c < 8; ++c) acc[a][c] = 0.0f;
+      for (int c = 0; c < 4; ++c) acc[a][c] = 0.0f;
+#pragma unroll 4
     for (int b = 0; b < kChunk; ++b) {
-      float hv[8], zv[8];
+      const float4 h = *reinterpret_cast<const float4*>(&hb[b][i0]);
+      const float hv[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
-      for (int a = 0; a < 8; ++a) hv[a] = ha[b][ti + 16 * a];
+      for (int c = 0; c < 4; ++c) {
+        const float z = zb[b][j0 + 32 * c];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) zv[c] = zb[b][tj + 16 * c];
-#pragma unroll
-      for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[a][c] = fmaf(hv[a], zv[c], acc[a][c]);
+        for (int a = 0; a < 4; ++a) acc[a][c] = fmaf(hv[a], z, acc[a][c]);
+      }
     }
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int c = 0; c < 8; ++c) out[kOffW2 + (ti + 16 * a) * kWidth + tj + 16 * c] = acc[a][c];
-  }
-  // gb2[j] = sum_b dz2[b][j]
-  if (tid < kWidth) {
-    float s = 0.0f;
-    for (int b = 0; b < kChunk; ++b) s += zb[b][tid];
-    out[kOffB2 + tid] = s;
-  }
-  __syncthreads();
-  // second pass: h2 and dz1
-  for (int e = tid; e < kChunk * kWidth; e += 256) {
-    const int b = e >> 7, u = e & 127;
-    const bool ok = c0 + b < B;
-    ha[b][u] = ok ? act[(size_t)(c0 + b) * 2 * kWidth + kWidth + u] : 0.0f;
-    zb[b][u] = ok ? dz[(size_t)(c0 + b) * 2 * kWidth + u] : 0.0f;
-  }
-  __syncthreads();
-  // gW1[k][u] = sum_b x[b][k] dz1[b][u]
-  for (int e = tid; e < kFeatures * kWidth; e += 256) {
-    const int k = e >> 7, u = e & 127;
-    float s = 0.0f;
-    for (int b = 0; b < kChunk; ++b) s = fmaf(xs[b][k], zb[b][u], s);
-    out[kOffW1 + e] = s;
-  }
-  // gb1[u] = sum_b dz1[b][u]
-  if (tid < kWidth) {
-    float s = 0.0f;
-    for (int b = 0; b < kChunk; ++b) s += zb[b][tid];
-    out[kOffB1 + tid] = s;
-  }
-  // gW3[u][o] = sum_b h2[b][u] dy[b][o]
-  for (int e = tid; e < kWidth * kOutputs; e += 256) {
-    const int u = e / kOutputs, o = e - u * kOutputs;
-    float s = 0.0f;
-    for (int b = 0; b < kChunk; ++b) s = fmaf(ha[b][u], ds[b][o], s);
-    out[kOffW3 + e] = s;
-  }
-  // gb3[o] = sum_b dy[b][o]
-  if (tid < kOutputs) {
-    float s = 0.0f;
-    for (int b = 0; b < kChunk; ++b) s += ds[b][tid];
-    out[kOffB3 + tid] = s;
+      for (int c = 0; c < 4; ++c) out[kOffW2 + (32 * slice + i0 + a) * kWidth + j0 + 32 * c] = acc[a][c];
+    if (slice == 0 && tid < kWidth) {   // gb2[j] = sum_b dz2[b][j]
+      float v = 0.0f;
+      for (int b = 0; b < kChunk; ++b) v += zb[b][tid];
+      out[kOffB2 + tid] = v;
+    }
+  } else if (slice == 4) {
+    for (int e = tid; e < kFeatures * kWidth; e += 256) {   // gW1[k][u] = sum_b x[b][k] dz1[b][u]
+      const int k = e >> 7, u = e & 127;
+      float v = 0.0f;
+      for (int b = 0; b < kChunk; ++b) v = fmaf(hb[b][k], zb[b][u], v);
+      out[kOffW1 + e] = v;
+    }
+    if (tid < kWidth) {   // gb1[u] = sum_b dz1[b][u]
+      float v = 0.0f;
+      for (int b = 0; b < kChunk; ++b) v += zb[b][tid];
+      out[kOffB1 + tid] = v;
+    }
+  } else {
+    for (int e = tid; e < kWidth * kOutputs; e += 256) {   // gW3[u][o] = sum_b h2[b][u] dy[b][o]
+      const int u = e / kOutputs, o = e - u * kOutputs;
+      float v = 0.0f;
+      for (int b = 0; b < kChunk; ++b) v = fmaf(zb[b][u], hb[b][o], v);
+      out[kOffW3 + e] = v;
+    }
+    if (tid < kOutputs) {   // gb3[o] = sum_b dy[b][o]
+      float v = 0.0f;
+      for (int b = 0; b < kChunk; ++b) v += hb[b][tid];
+      out[kOffB3 + tid] = v;
+    }
   }
 }
 
-// grad[p] = sum over chunks (fixed order) of part[chunk][p]
-__global__ void k_mlp_reduce(int32_t chunks, const float* __restrict__ part, float* __restrict__ grad) {
+// Adam with bias correction (step >= 1).
+struct AdamArgs {
+  float* p; float* m; float* v;
+  int32_t step;
+  float lr, b1, b2, eps;
+};
+__device__ __forceinline__ void adam_update(const AdamArgs& a, int i, float gi) {
+  const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
+  const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+  a.m[i] = mi;
+  a.v[i] = vi;
+  const float mh = mi / (1.0f - powf(a.b1, (float)a.step));
+  const float vh = vi / (1.0f - powf(a.b2, (float)a.step));
+  a.p[i] -= a.lr * mh / (sqrtf(vh) + a.eps);
+}
+
+// grad[p] = sum over chunks (fixed order) of part[chunk][p]; with kAdam the step that it makes
+template <bool kAdam>
+__global__ void k_mlp_reduce(int32_t chunks, const float* __restrict__ part, float* __restrict__ grad, AdamArgs a) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= kParams) return;
   float s = 0.0f;
+#pragma unroll 16
   for (int c = 0; c < chunks; ++c) s += part[(size_t)c * kParams + p];
   grad[p] = s;
+  if (kAdam) adam_update(a, p, s);
 }
 
-// Adam with bias correction (step t >= 1).
-__global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                           float* __restrict__ v, int32_t t, float lr, float b1, float b2, float eps) {
+__global__ void k_mlp_adam(const float* __restrict__ g, AdamArgs a) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kParams) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.0f - b1) * gi;
-  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float mh = mi / (1.0f - powf(b1, (float)t));
-  const float vh = vi / (1.0f - powf(b2, (float)t));
-  p[i] -= lr * mh / (sqrtf(vh) + eps);
+  if (i < kParams) adam_update(a, i, g[i]);
 }
 
 // SplitMix64 (Steele, Lea and Flood; constants from its published definition) as a counter-based
@@ -542,16 +571,6 @@ __global__ void k_mlp_init(float* __restrict__ p, uint64_t seed) {
   p[i] = lim * (2.0f * u - 1.0f);
 }
 
-// Minibatch gather: sample r of the batch is idx = (start + r) * 7919 + epoch * 104729 (mod N).
-__global__ void k_mlp_batch(int32_t N, int32_t start, int32_t count, int32_t epoch, const float* __restrict__ x,
-                            const float* __restrict__ t, float* __restrict__ xb, float* __restrict__ tb) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= count) return;
-  const int64_t i = (((int64_t)(start + r) * 7919 + (int64_t)epoch * 104729) % N + N) % N;
-  for (int k = 0; k < kFeatures; ++k) xb[(size_t)r * kFeatures + k] = x[(size_t)i * kFeatures + k];
-  for (int o = 0; o < kOutputs; ++o) tb[(size_t)r * kOutputs + o] = t[(size_t)i * kOutputs + o];
-}
-
 }  // namespace
 
 }  // namespace nolsm
@@ -565,13 +584,12 @@ struct nolsm_mlp {
   float* v = nullptr;
   double* loss = nullptr;
   // per-sample workspaces for up to cap samples
-  float* act = nullptr; float* dz = nullptr; float* dy = nullptr; float* y = nullptr; float* part = nullptr;
-  float* xb = nullptr; float* tb = nullptr;
+  float* act = nullptr; float* dz = nullptr; float* dy = nullptr; float* part = nullptr;
   int32_t cap = 0;
   int32_t step = 0;   // Adam steps taken
   ~nolsm_mlp() {
     for (void* p : {(void*)params, (void*)grad, (void*)m, (void*)v, (void*)loss, (void*)act, (void*)dz, (void*)dy,
-                    (void*)y, (void*)part, (void*)xb, (void*)tb})
+                    (void*)part})
       if (p) cudaFree(p);
   }
 };
@@ -584,7 +602,7 @@ size_t mlp_smem_bytes() { return sizeof(float) * kMlpSmemFloats + 64; }
 
 nolsm_status mlp_reserve(nolsm_mlp* m, int32_t B) {
   if (B <= m->cap) return NOLSM_OK;
-  for (float** p : {&m->act, &m->dz, &m->dy, &m->y, &m->part, &m->xb, &m->tb}) {
+  for (float** p : {&m->act, &m->dz, &m->dy, &m->part}) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }
@@ -593,10 +611,7 @@ nolsm_status mlp_reserve(nolsm_mlp* m, int32_t B) {
   NOLSM_CUDA_TRY(cudaMalloc(&m->act, sizeof(float) * b * 2 * kWidth));
   NOLSM_CUDA_TRY(cudaMalloc(&m->dz, sizeof(float) * b * 2 * kWidth));
   NOLSM_CUDA_TRY(cudaMalloc(&m->dy, sizeof(float) * b * kOutputs));
-  NOLSM_CUDA_TRY(cudaMalloc(&m->y, sizeof(float) * b * kOutputs));
   NOLSM_CUDA_TRY(cudaMalloc(&m->part, sizeof(float) * chunks * kParams));
-  NOLSM_CUDA_TRY(cudaMalloc(&m->xb, sizeof(float) * b * kFeatures));
-  NOLSM_CUDA_TRY(cudaMalloc(&m->tb, sizeof(float) * b * kOutputs));
   m->cap = B;
   return NOLSM_OK;
 }
@@ -616,31 +631,35 @@ nolsm_status mlp_set_smem() {
   static bool done = false;
   if (!done) {
     NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()));
-    NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()));
+    NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_mlp_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem_bytes()));
     done = true;
   }
   return NOLSM_OK;
 }
 
-// forward (activations kept) + backward + weight gradients into m->grad; loss accumulated into m->loss
-nolsm_status mlp_grad(nolsm_mlp* m, int32_t B, const float* x, const float* t, cudaStream_t st) {
+AdamArgs adam_args(nolsm_mlp* m, float lr) { return AdamArgs{m->params, m->m, m->v, m->step, lr, 0.9f, 0.999f, 1e-8f}; }
+
+// forward + backward + weight gradients into m->grad, loss accumulated into m->loss; with lr > 0 also an Adam step
+nolsm_status mlp_grad(nolsm_mlp* m, int32_t B, const MlpBatch& batch, float lr, cudaStream_t st) {
   NOLSM_TRY(mlp_set_smem());
-  k_mlp_forward<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), st>>>(m->params, B, x, m->y, m->act);
-  NOLSM_LAUNCH_CHECK();
-  k_mlp_backward<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), st>>>(m->params, B, m->act, m->y, t, m->dz, m->dy,
-                                                                       m->loss);
+  k_mlp_sample<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), st>>>(m->params, B, batch, m->act, m->dz, m->dy, m->loss);
   NOLSM_LAUNCH_CHECK();
   const int chunks = (B + kChunk - 1) / kChunk;
-  k_mlp_wgrad<<<chunks, 256, 0, st>>>(B, x, m->act, m->dz, m->dy, m->part);
+  k_mlp_wgrad<<<dim3((unsigned)chunks, kSlices), 256, 0, st>>>(B, batch, m->act, m->dz, m->dy, m->part);
   NOLSM_LAUNCH_CHECK();
-  k_mlp_reduce<<<(kParams + 255) / 256, 256, 0, st>>>(chunks, m->part, m->grad);
+  if (lr > 0.0f) {
+    m->step += 1;
+    k_mlp_reduce<true><<<(kParams + 127) / 128, 128, 0, st>>>(chunks, m->part, m->grad, adam_args(m, lr));
+  } else {
+    k_mlp_reduce<false><<<(kParams + 127) / 128, 128, 0, st>>>(chunks, m->part, m->grad, AdamArgs{});
+  }
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }
 
 nolsm_status mlp_adam(nolsm_mlp* m, float lr, cudaStream_t st) {
   m->step += 1;
-  k_mlp_adam<<<(kParams + 255) / 256, 256, 0, st>>>(m->params, m->grad, m->m, m->v, m->step, lr, 0.9f, 0.999f, 1e-8f);
+  k_mlp_adam<<<(kParams + 255) / 256, 256, 0, st>>>(m->grad, adam_args(m, lr));
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }
@@ -737,8 +756,7 @@ nolsm_status mlp_bounds(nolsm_plan* plan, int64_t j0, int64_t j1, int32_t max_it
   NOLSM_TRY(mlp_set_smem());
   const int32_t B = (int32_t)(j1 - j0);
   k_mlp_forward<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), st>>>(
-      plan->mlp->params, B, plan->feat.as<float>() + (size_t)j0 * kFeatures, plan->mlp_y.as<float>() + (size_t)j0 * kOutputs,
-      nullptr);
+      plan->mlp->params, B, plan->feat.as<float>() + (size_t)j0 * kFeatures, plan->mlp_y.as<float>() + (size_t)j0 * kOutputs);
   NOLSM_LAUNCH_CHECK();
   k_mlp_bounds<<<(unsigned)((B + 255) / 256), 256, 0, st>>>((int32_t)j0, (int32_t)j1, plan->mlp_y.as<float>(),
                                                              plan->lam.as<double>(), max_iter, plan->lam_m.as<double>(),
@@ -823,7 +841,7 @@ nolsm_status nolsm_mlp_set_params(nolsm_mlp* mlp, const float* host_params) {
 nolsm_status nolsm_mlp_forward(nolsm_mlp* mlp, int32_t B, const float* x, float* y, nolsm_stream_t stream) {
   if (!mlp || !x || !y || B < 1) { set_error("nolsm_mlp_forward: invalid argument"); return NOLSM_ERR_ARG; }
   NOLSM_TRY(mlp_set_smem());
-  k_mlp_forward<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), (cudaStream_t)stream>>>(mlp->params, B, x, y, nullptr);
+  k_mlp_forward<<<mlp_grid(B), kMlpThreads, mlp_smem_bytes(), (cudaStream_t)stream>>>(mlp->params, B, x, y);
   NOLSM_LAUNCH_CHECK();
   NOLSM_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
   return NOLSM_OK;
@@ -835,7 +853,7 @@ nolsm_status nolsm_mlp_gradient(nolsm_mlp* mlp, int32_t B, const float* x, const
   cudaStream_t st = (cudaStream_t)stream;
   NOLSM_TRY(mlp_reserve(mlp, B));
   NOLSM_CUDA_TRY(cudaMemsetAsync(mlp->loss, 0, sizeof(double), st));
-  NOLSM_TRY(mlp_grad(mlp, B, x, t, st));
+  NOLSM_TRY(mlp_grad(mlp, B, MlpBatch{x, t, 0, 0, 0}, 0.0f, st));
   if (grad_host)
     NOLSM_CUDA_TRY(cudaMemcpyAsync(grad_host, mlp->grad, sizeof(float) * kParams, cudaMemcpyDeviceToHost, st));
   double l = 0.0;
@@ -866,10 +884,7 @@ nolsm_status nolsm_mlp_train(nolsm_mlp* mlp, int32_t N, const float* x, const fl
     NOLSM_CUDA_TRY(cudaMemsetAsync(mlp->loss, 0, sizeof(double), st));
     for (int32_t s = 0; s < steps; ++s) {
       const int32_t start = s * bs, cnt = std::min(bs, N - start);
-      k_mlp_batch<<<(cnt + 255) / 256, 256, 0, st>>>(N, start, cnt, e, x, t, mlp->xb, mlp->tb);
-      NOLSM_LAUNCH_CHECK();
-      NOLSM_TRY(mlp_grad(mlp, cnt, mlp->xb, mlp->tb, st));
-      NOLSM_TRY(mlp_adam(mlp, lr, st));
+      NOLSM_TRY(mlp_grad(mlp, cnt, MlpBatch{x, t, N, start, e}, lr, st));
     }
     if (epoch_loss) {
       double l = 0.0;
