@@ -50,12 +50,12 @@ struct GatherArgs {
   const int64_t* a_off; const int64_t* c_off;
   int64_t a_base;       // a_off of the chunk's first submatrix
   int64_t chunk_n2;     // sum of n^2 over the chunk (offset of the T(H0) half)
-  int64_t p0, p1;       // row bands [p0, p1) of the chunk
-  int32_t max_nq;       // largest |N(J)|: each warp's lookup tables hold 3 max_nq ints
+  int32_t j0;           // the chunk's first submatrix
+  int32_t max_nq;       // largest |N(J)|: entries of the lookup tables
+  int32_t unordered;    // N(J) is not in ascending order
   double* ws;           // [2*chunk_n2]
   double* Sc; double* Hc;
-  // elements generated from the geometry (gen != 0) instead of read from sval / hval
-  int gen;
+  // elements generated from the geometry instead of read from sval / hval
   const double* pos; double cell[3]; const double* onsite; const int64_t* onsite_off;
   double s_exp, hop, hop_len, aniso; const double* dirs;
 };
@@ -91,88 +91,115 @@ __device__ __forceinline__ double aniso_factor(const GatherArgs& g, int k, const
   return __dadd_rn(1.0, __dmul_rn(g.aniso, __dsub_rn(ua, uc)));
 }
 
+// A CTA per submatrix, a warp per band of rows. What bounds it is the writing of T_J(S) and T_J(H0), once the chain of
+// dependent loads ahead of a band is short: N(J) is read once into shared memory, and the stored blocks of block row I_a
+// are looked up in it, rather than N(J)'s columns in the block row by searches in global memory (262,144 submatrices of
+// n = 162: 110 GB, 39 ms then, 26 now; 32,768 uneven 5.0 and 3.5).
 constexpr int kGatherWarps = 8;
-constexpr int kGatherTableBytes = 32;   // per block column of a band: two int64 offsets, three int32, padding
+// bytes per block column: N(J) (molecule, first column, width; the molecules in order and their places); per warp the offsets of block (I_a, I_c) in the stored S
+// and H0 values (-1: no block); the block models of generated elements follow every warp's tables
+constexpr int kGatherTableBytes = 24 + 16 * kGatherWarps;
 
-__global__ void __launch_bounds__(32 * kGatherWarps) k_gather(GatherArgs g) {
+template <bool kGen>   // elements generated from the geometry
+__global__ void __launch_bounds__(32 * kGatherWarps, 4) k_gather(GatherArgs g) {
   extern __shared__ __align__(8) unsigned char gsm[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t p = g.p0 + (int64_t)blockIdx.x * kGatherWarps + w;
-  if (p >= g.p1) return;   // whole warps only; no block-wide barrier follows
-  // this warp's tables, one entry per block column c of the band (32 bytes each): the offsets of block
-  // (Ia, Ic) in the stored S and H0 values (-1: no block), its first column, its width and Ic; the block
-  // models of generated elements follow every warp's tables
-  int64_t* sbase = reinterpret_cast<int64_t*>(gsm + (size_t)w * kGatherTableBytes * g.max_nq);
-  int64_t* hbase = sbase + g.max_nq;
-  int32_t* coff = reinterpret_cast<int32_t*>(hbase + g.max_nq);
-  int32_t* bcs = coff + g.max_nq;
-  int32_t* mol = bcs + g.max_nq;
-  BlockModel* bm = reinterpret_cast<BlockModel*>(gsm + (size_t)kGatherWarps * kGatherTableBytes * g.max_nq) +
-                   w * g.max_nq;
-  const int J = owner_of(g.nb_ptr, g.n_mol, p);
+  const int J = g.j0 + (int)blockIdx.x;
   const int q0 = g.nb_ptr[J], nq = g.nb_ptr[J + 1] - q0;
-  const int Ia = g.nb_idx[p];
-  const int ba = g.nbf[Ia];
-  const int offa = g.nb_off[p];
-  const int n = g.sub_n[J];
-  for (int c = lane; c < nq; c += 32) {
+  int64_t* const sbase = reinterpret_cast<int64_t*>(gsm) + (size_t)2 * w * g.max_nq;
+  int64_t* const hbase = sbase + g.max_nq;
+  int32_t* const mol = reinterpret_cast<int32_t*>(gsm + (size_t)16 * kGatherWarps * g.max_nq);
+  int32_t* const coff = mol + g.max_nq;
+  int32_t* const bcs = coff + g.max_nq;
+  int32_t* const key = bcs + g.max_nq;
+  int32_t* const place = key + g.max_nq;
+  BlockModel* const bm = reinterpret_cast<BlockModel*>(gsm + (size_t)kGatherTableBytes * g.max_nq) + w * g.max_nq;
+  for (int c = threadIdx.x; c < nq; c += blockDim.x) {
     const int32_t Ic = g.nb_idx[q0 + c];
-    const int ss = find_sorted(g.sci, g.srp[Ia], g.srp[Ia + 1], Ic);
-    const int hs = find_sorted(g.hci, g.hrp[Ia], g.hrp[Ia + 1], Ic);
-    sbase[c] = ss < 0 ? -1 : (g.gen ? 0 : g.soff[ss]);
-    hbase[c] = hs < 0 ? -1 : (g.gen ? 0 : g.hoff[hs]);
+    mol[c] = Ic;
     coff[c] = g.nb_off[q0 + c];
     bcs[c] = g.nbf[Ic];
-    mol[c] = Ic;
-    if (g.gen && Ic != Ia) bm[c] = block_model(g, Ia, Ic, ba, g.nbf[Ic]);
   }
-  __syncwarp();
+  __syncthreads();
+  for (int c = threadIdx.x; c < nq; c += blockDim.x) {   // (a group's own molecules come ahead of the others)
+    const int32_t Ic = mol[c];
+    int at = c;
+    if (g.unordered) {
+      at = 0;
+      for (int x = 0; x < nq; ++x) at += mol[x] < Ic ? 1 : 0;
+    }
+    key[at] = Ic;
+    place[at] = c;
+  }
+  __syncthreads();
+  const int n = g.sub_n[J];
   const int c0 = g.sub_c0[J];
   const int bJ = g.sub_b[J];
   double* TS = g.ws + (g.a_off[J] - g.a_base);
   double* TH = TS + g.chunk_n2;
   double* Sc = g.Sc + g.c_off[J];
   double* Hc = g.Hc + g.c_off[J];
-  int c = 0;   // block column of col; columns advance by 32, blocks by at least one function
-  for (int col = lane; col < n; col += 32) {
-    while (c + 1 < nq && coff[c + 1] <= col) ++c;
-    const int bc = bcs[c], cc = col - coff[c];
-    const int64_t sb = sbase[c], hb = hbase[c];
-    const bool intra = mol[c] == Ia;
-    const bool centre = col >= c0 && col < c0 + bJ;
-    // the column's ba rows, four at a time: their loads issued together, then their stores
-    for (int r0 = 0; r0 < ba; r0 += 4) {
-      double vs[4], vh[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u;
-        vs[u] = vh[u] = 0.0;
-        if (r >= ba) continue;
-        if (!g.gen) {
-          if (sb >= 0) vs[u] = __ldg(g.sval + sb + r * bc + cc);
-          if (hb >= 0) vh[u] = __ldg(g.hval + hb + r * bc + cc);
-        } else if (intra) {   // intra-molecular: identity and the on-site energies
-          vs[u] = (sb >= 0 && r == cc) ? 1.0 : 0.0;
-          vh[u] = (hb >= 0 && r == cc) ? g.onsite[g.onsite_off[Ia] + r] : 0.0;
-        } else {
-          const BlockModel& m = bm[c];
-          vs[u] = sb >= 0 ? (g.aniso != 0.0 ? __dmul_rn(m.s, aniso_factor(g, 0, m, r, cc)) : m.s) : 0.0;
-          vh[u] = hb >= 0 ? (g.aniso != 0.0 ? __dmul_rn(m.h, aniso_factor(g, 1, m, r, cc)) : m.h) : 0.0;
-        }
+  for (int band = kGatherWarps * blockIdx.y + w; band < nq; band += kGatherWarps * gridDim.y) {
+    const int Ia = mol[band], ba = bcs[band], offa = coff[band];
+    // the warp's tables of the band
+    for (int c = lane; c < nq; c += 32) {
+      sbase[c] = hbase[c] = -1;
+      if (kGen && c != band) bm[c] = block_model(g, Ia, mol[c], ba, bcs[c]);
+    }
+    __syncwarp();
+    auto look_up = [&](const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, const int64_t* __restrict__ off,
+                       int64_t* base) {
+      for (int s = rp[Ia] + lane; s < rp[Ia + 1]; s += 32) {
+        const int64_t o = kGen ? 0 : off[s];
+        const int c = find_sorted(key, 0, nq, ci[s]);
+        if (c >= 0) base[place[c]] = o;
       }
+    };
+    look_up(g.srp, g.sci, g.soff, sbase);
+    look_up(g.hrp, g.hci, g.hoff, hbase);
+    __syncwarp();
+    int c = 0;   // block column of col; columns advance by 32, blocks by at least one function
+    for (int col = lane; col < n; col += 32) {
+      while (c + 1 < nq && coff[c + 1] <= col) ++c;
+      const int bc = bcs[c], cc = col - coff[c];
+      const int64_t sb = sbase[c], hb = hbase[c];
+      const bool intra = mol[c] == Ia;
+      const bool centre = col >= c0 && col < c0 + bJ;
+      // the column's ba rows, six at a time: their loads issued together, then their stores
+      for (int r0 = 0; r0 < ba; r0 += 6) {
+        double vs[6], vh[6];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u;
-        if (r >= ba) break;
-        const int64_t at = (int64_t)(offa + r) * n + col;
-        TS[at] = vs[u];
-        TH[at] = vh[u];
-        if (centre) {
-          Sc[(int64_t)(offa + r) * bJ + (col - c0)] = vs[u];
-          Hc[(int64_t)(offa + r) * bJ + (col - c0)] = vh[u];
+        for (int u = 0; u < 6; ++u) {
+          const int r = r0 + u;
+          vs[u] = vh[u] = 0.0;
+          if (r >= ba) continue;
+          if (!kGen) {
+            if (sb >= 0) vs[u] = __ldg(g.sval + sb + r * bc + cc);
+            if (hb >= 0) vh[u] = __ldg(g.hval + hb + r * bc + cc);
+          } else if (intra) {   // intra-molecular: identity and the on-site energies
+            vs[u] = (sb >= 0 && r == cc) ? 1.0 : 0.0;
+            vh[u] = (hb >= 0 && r == cc) ? g.onsite[g.onsite_off[Ia] + r] : 0.0;
+          } else {
+            const BlockModel& m = bm[c];
+            vs[u] = sb >= 0 ? (g.aniso != 0.0 ? __dmul_rn(m.s, aniso_factor(g, 0, m, r, cc)) : m.s) : 0.0;
+            vh[u] = hb >= 0 ? (g.aniso != 0.0 ? __dmul_rn(m.h, aniso_factor(g, 1, m, r, cc)) : m.h) : 0.0;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 6; ++u) {
+          const int r = r0 + u;
+          if (r >= ba) break;
+          const int64_t at = (int64_t)(offa + r) * n + col;
+          TS[at] = vs[u];
+          TH[at] = vh[u];
+          if (centre) {
+            Sc[(int64_t)(offa + r) * bJ + (col - c0)] = vs[u];
+            Hc[(int64_t)(offa + r) * bJ + (col - c0)] = vh[u];
+          }
         }
       }
     }
+    __syncwarp();   // the tables are free again
   }
 }
 
@@ -516,13 +543,11 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
     g.a_off = plan->a_off.as<int64_t>(); g.c_off = plan->c_off.as<int64_t>();
     g.a_base = plan->h_a_off[J];
     g.chunk_n2 = n2;
-    g.p0 = plan->h_nb_ptr[J];
+    g.j0 = (int32_t)J;
     g.ws = plan->ws_dense.as<double>();
     g.Sc = plan->Sc.as<double>(); g.Hc = plan->Hc.as<double>();
-    const int64_t bands = plan->h_nb_ptr[e] - plan->h_nb_ptr[J];
-    g.p1 = plan->h_nb_ptr[e];
     g.max_nq = max_nq;
-    g.gen = plan->gen ? 1 : 0;
+    g.unordered = plan->grouped ? 1 : 0;
     if (plan->gen) {
       const nolsm_element_model& m = plan->model;
       g.pos = m.pos; g.cell[0] = m.cell[0]; g.cell[1] = m.cell[1]; g.cell[2] = m.cell[2];
@@ -533,10 +558,17 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       return NOLSM_ERR_ARG;
     }
     pmark(plan, st);
-    const size_t gsm = (size_t)kGatherTableBytes * kGatherWarps * max_nq +
+    const size_t gsm = (size_t)kGatherTableBytes * max_nq +
                        (plan->gen ? sizeof(BlockModel) * kGatherWarps * (size_t)max_nq : 0);
-    if (gsm > 48 * 1024) NOLSM_CUDA_TRY(cudaFuncSetAttribute(k_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
-    k_gather<<<(unsigned)((bands + kGatherWarps - 1) / kGatherWarps), 32 * kGatherWarps, gsm, st>>>(g);
+    auto gather = [&](auto* kernel) -> nolsm_status {
+      if (gsm > 48 * 1024) NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
+      // with few submatrices the bands of each go to several CTAs (64 of 27 bands: 43 us with one each, 14 with four)
+      const unsigned spread = (unsigned)std::max<int64_t>(
+          1, std::min<int64_t>((max_nq + kGatherWarps - 1) / kGatherWarps, (16 * 152 + e - J - 1) / (e - J)));
+      kernel<<<dim3((unsigned)(e - J), spread), 32 * kGatherWarps, gsm, st>>>(g);
+      return NOLSM_OK;
+    };
+    NOLSM_TRY(plan->gen ? gather(&k_gather<true>) : gather(&k_gather<false>));
     NOLSM_LAUNCH_CHECK();
     pmark(plan, st);
     PrepArgs pa;
