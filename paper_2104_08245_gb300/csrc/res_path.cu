@@ -1044,7 +1044,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
       }
       if (etid == 0) {
         g.prep_out[J] = status;
-        if (status == kSubAgain) atomicAdd(g.again, 1);
+        if (status == kSubAgain) g.again_list[atomicAdd(g.again, 1)] = J;
         else {
           const double prods = 3.0 * steps - (g.Aout ? 1.0 : 2.0), n3 = (double)n * n * n;
           atomicAdd(&g.flops[0], 2.0 * n3 * prods);

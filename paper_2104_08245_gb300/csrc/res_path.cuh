@@ -26,7 +26,7 @@ struct ResSolve {
 nolsm_status launch_ns_res(const ResSolve& a, int sms, cudaStream_t st);
 
 // a2-a3 the same way, every submatrix of at most kResMaxN rows (see launch_ns_inverse for the fields): prep_out[J] =
-// kSubOk, kSubRefine, or kSubAgain where k_ns_tc has to take the submatrix (more than two steps); *again counts those.
+// kSubOk, kSubRefine, or kSubAgain where k_ns_tc has to take the submatrix (more than two steps); *again counts those, again_list names them.
 constexpr int32_t kSubAgain = 66;
 struct InvSolve {
   const int32_t* order; int32_t count;
@@ -35,7 +35,7 @@ struct InvSolve {
   float* Aout; float* Xout;
   int32_t* prep_out;
   float tol_inv; int32_t max_inv;
-  int32_t* next; int32_t* err; int32_t* again;
+  int32_t* next; int32_t* err; int32_t* again; int32_t* again_list;
   double* flops;
   uint64_t wait_ns;
 };

@@ -137,7 +137,6 @@ struct TcArgs {
   int32_t* prep_out;          // kSubOk, or kSubRefine when the iteration failed (FP64 preparation next)
   float tol_inv;
   int32_t max_inv;
-  int32_t again;              // only submatrices whose prep_out is kSubAgain (k_inv_res left them)
   double* flops;              // [2]: 2 n^3 per product (method count) and the split's issued flops, summed
   int32_t group;              // CTAs that share a submatrix (the grid is a multiple of it)
   struct GroupSlot* groups;   // [grid / group * kSlots], zeroed before the launch
@@ -363,10 +362,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
         const int k = atomicAdd(g.next, 1);
         if (k >= g.j1 - g.j0 || sh.err) return -1;
         const int J = g.order[k];
-        if constexpr (kMode == 1) {
-          if (g.again && g.prep_out[J] != kSubAgain) continue;
-          return J;
-        }
+        if constexpr (kMode == 1) return J;
         if (g.sub_n[J] <= g.above_n) continue;
         if (g.cond && g.prep_status[J] == kSubOk && g.cond[J] > g.cond_max && g.sub_n[J] <= g.ill_max_n) continue;
         if (g.prep_status[J] == kSubOk) return J;
@@ -1293,7 +1289,7 @@ __global__ void k_status_pending(int32_t j0, int32_t count, const int32_t* __res
 // ==================================================================================== host side
 
 struct TcState {
-  DevBuf planes, order, err, groups;
+  DevBuf planes, order, err, groups, again;
   int R = 0, LD = 0, slots = 0;
   int64_t ord_j0 = -1, ord_j1 = -1;
   int32_t ord_large = 0;          // how many of the cached order (a prefix) have n above 192
@@ -1314,6 +1310,7 @@ void tc_release(nolsm_plan* plan) {
   dev_free(plan, s->order);
   dev_free(plan, s->err);
   dev_free(plan, s->groups);
+  dev_free(plan, s->again);
   dev_free(plan, s->inv_planes);
   dev_free(plan, s->inv_flops);
   delete s;
@@ -1724,7 +1721,12 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     r.Aout = a.Aout; r.Xout = a.Xout; r.prep_out = a.prep_out;
     r.tol_inv = a.tol_inv; r.max_inv = a.max_inv;
     r.next = plan->counter.as<int32_t>() + 1;
+    if (S->again.bytes < sizeof(int32_t) * (size_t)n_small) {
+      dev_free(plan, S->again);
+      NOLSM_TRY(dev_alloc(plan, S->again, sizeof(int32_t) * (size_t)n_small));
+    }
     r.err = S->err.as<int32_t>(); r.again = S->err.as<int32_t>() + 1;
+    r.again_list = S->again.as<int32_t>();
     r.flops = S->inv_flops.as<double>();
     NOLSM_TRY(pending(r.order, n_small));
     NOLSM_TRY(launch_inv_res(r, sms, st));
@@ -1732,10 +1734,11 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     plan->stats.launches += 2;
   }
   // the others, and those that need more than two steps, with operands in scratch
-  auto streamed = [&](const int32_t* order, int32_t n_large, int32_t count, int32_t again) -> nolsm_status {
+  auto streamed = [&](const int32_t* order, int32_t count, bool again) -> nolsm_status {
     const int max_n = again ? std::min(a.max_n, kResMaxN) : a.max_n;
     const int LD = (max_n + 63) & ~63, R = (max_n + 127) & ~127;
-    const int group = group_size(again ? 0 : a.mean_n);
+    // the few that k_inv_res left: several CTAs each while there are enough, as the start of one dominates
+    const int group = !again ? group_size(a.mean_n) : 2 * count <= sms ? 4 : count <= sms ? 2 : 1;
     const int slots = group_slots(group, count, sms);
     if (!S->inv_planes.p || S->iR < R || S->iLD < LD || S->islots < slots) {
       const int nR = std::max(R, S->iR), nLD = std::max(LD, S->iLD), nS = std::max(slots, S->islots);
@@ -1760,21 +1763,20 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2;
     g.Aout = a.Aout; g.Xout = a.Xout; g.prep_out = a.prep_out;
     g.tol_inv = a.tol_inv; g.max_inv = a.max_inv;
-    g.again = again;
     g.group = group;
     g.groups = S->groups.as<GroupSlot>();
     g.wait_ns = kWaitNs;
     g.flops = S->inv_flops.as<double>();
     plan->stats.launches += 2;
     if (again) return launch_shape(1, 0, m, g, sms, st);
-    return run_buckets(1, NOLSM_FP16, false, m, g, order, n_large, count, a.mean_n, sms, st, pending);
+    return run_buckets(1, NOLSM_FP16, false, m, g, order, count, count, a.mean_n, sms, st, pending);
   };
-  if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, a.n_large, 0));
+  if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, false));
   int32_t again = 0;
   NOLSM_TRY(read_back(&again));
   if (again > 0) {
     NOLSM_CUDA_TRY(cudaMemsetAsync(S->inv_flops.p, 0, sizeof(double) * 2, st));
-    NOLSM_TRY(streamed(a.order + a.n_large, 0, n_small, 1));
+    NOLSM_TRY(streamed(S->again.as<int32_t>(), again, true));
     NOLSM_TRY(read_back(&again));
   }
   return NOLSM_OK;
