@@ -585,9 +585,18 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       const int units = n16 / 16, nitem = ((n + 31) / 32) * kSplit;   // of k: 16 at a time
       for (int cg = 0; cg < b; cg += 8) {
         const int cn = min(8, b - cg);
-        for (int e = etid; e < n16 * 8; e += kEpiR) {
-          const int k = e >> 3, c = e & 7;
-          Qs[e] = (k < n && c < cn) ? (float)Q[(size_t)k * b + cg + c] : 0.0f;
+        {   // all loads in flight together
+          double v[kResMaxN * 8 / kEpiR];
+#pragma unroll
+          for (int u = 0; u < kResMaxN * 8 / kEpiR; ++u) {
+            const int e = etid + u * kEpiR;
+            v[u] = __ldg(Q + (size_t)min(e >> 3, n - 1) * b + cg + min(e & 7, cn - 1));
+          }
+#pragma unroll
+          for (int u = 0; u < kResMaxN * 8 / kEpiR; ++u) {
+            const int e = etid + u * kEpiR, k = e >> 3;
+            if (k < n16) Qs[e] = k < n && (e & 7) < cn ? (float)v[u] : 0.0f;
+          }
         }
         bar_epi();
         for (int it = ew; it < nitem; it += 8) {

@@ -958,9 +958,18 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
             const int kn = min(kRowsQ, n64 - k0);
             if (rr == r0 || n64 > kRowsQ) {
               epi_bar<kEpiThreads>();   // the last piece has been used
-              for (int e = etid; e < kn * 8; e += kEpiThreads) {
-                const int k = k0 + (e >> 3), c = e & 7;
-                Qs[qs_at(e >> 3) + c] = k < n && c < cn ? (float)Q[(size_t)k * b + cg + c] : 0.0f;
+              for (int e0 = etid; e0 < kn * 8; e0 += 8 * kEpiThreads) {   // eight loads in flight
+                double v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int e = e0 + u * kEpiThreads;
+                  v[u] = __ldg(Q + (size_t)min(k0 + (e >> 3), n - 1) * b + cg + min(e & 7, cn - 1));
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int e = e0 + u * kEpiThreads, k = e >> 3;
+                  if (k < kn) Qs[qs_at(k) + (e & 7)] = k0 + k < n && (e & 7) < cn ? (float)v[u] : 0.0f;
+                }
               }
               epi_bar<kEpiThreads>();
             }
