@@ -50,11 +50,13 @@ typedef enum {
 } nolsm_status;
 
 /* Arithmetic of the sign-iteration products (a5/a6). The trace sums are FP64 in every mode. The overlap
- * factorisation is FP64 in NOLSM_FP64; the tensor-core modes factor T_J(S) in FP32, form A_J with FP32
+ * inverse is refined to FP64 in NOLSM_FP64; the tensor-core modes factor T_J(S) in FP32, form A_J with FP32
  * solves, and refine the centre columns of T_J(S)^-1 with a double-FP32 residual (about 48 bits) to about
  * 1e-12 relative; a submatrix whose refinement does not contract, or whose overlap is too ill-conditioned
  * for the FP32 factor, is prepared again with the FP64 factorisation.
- *   NOLSM_FP64       every step in FP64 on the CUDA cores (the plain reference path).
+ *   NOLSM_FP64       FP64 accuracy: the products of the sign iteration and of the inverse's refinement as exact
+ *                    sums of products of 8- or 9-bit digits on the tensor cores (64-bit fixed point); submatrices
+ *                    that the fixed point does not hold, by an FP64 factorisation and iteration on the CUDA cores.
  *   NOLSM_FP32       every Newton-Schulz product as a three-term split of FP16 tensor-core products
  *                    (hi*hi + hi*lo + lo*hi, FP32 accumulation): about 22 significant bits.
  *   NOLSM_BF16       Newton-Schulz products as single BF16 tensor-core products (FP32 accumulation)
@@ -521,8 +523,8 @@ nolsm_status nolsm_sign_noalloc(int32_t count, const int32_t* sub_n, const int32
  * comes in two shapes: 0 (384 threads, two epilogue groups, output tiles of 128 rows x up to 256 columns) and
  * 1 (512 threads, three epilogue groups, 128 x up to 192, a register split between warpgroups). Each solve
  * (kernel 0: sign iteration) or preparation chunk (kernel 1: inverse square root) splits its submatrices,
- * largest first, into two buckets, n above 192 (bucket 1) and the rest (bucket 0), and launches them once
- * together when both take the same shape, else once each. The first time a process
+ * largest first, into two buckets, n above 192 (bucket 1) and the rest (bucket 0). Bucket 0 has a kernel with one
+ * shape (reported as 0), but for E4M3. The first time a process
  * meets a (kernel, precision, bucket), both shapes run on that bucket's largest submatrices (32 per slot
  * of every SM), timed with CUDA events on the caller's stream, and the faster is kept for the life of the
  * process; the timed runs' results are computed again by the bucket's launch. Setting the environment

@@ -1,7 +1,6 @@
-// Geometry preparation (a1 gather, a2 FP64 Cholesky, a3 A = T_J(S)^-1 T_J(H0) and the centre
-// columns of T_J(S)^-1), the plain FP64 sign iteration (a4-a7), the trace reductions and the
-// write-back (a8). The FP64 sign iteration is the reference GPU path; the tensor-core paths reuse
-// everything here except the sign iteration itself.
+// Geometry preparation (a1 gather, a2-a3 dispatched to the preparation kernels), the FP64 solve (a4-a7: the exact digit
+// products of oz_path.cu, then the plain FP64 iteration here for what they leave), the trace reductions and the
+// write-back (a8).
 #include <algorithm>
 #include <cmath>
 

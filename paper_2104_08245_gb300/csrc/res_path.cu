@@ -8,11 +8,17 @@
 //   Z = T X      column block c (64) of every row tile     -> X' = Z / 2 over column block c of X
 // Z's column block c needs nothing of X but its column block c, so X' can overwrite it as soon as the block's products
 // are done. Tensor memory: T's two tiles take 2 x 192 columns, two Z accumulators 2 x 64.
+// With one term T commutes with X only to the rounding of T, and the product keeps the order X T of the streaming kernel
+// (T X differs from it as much as either does from the exact sign): T goes into the second plane as the B operand, Z over
+// the accumulators of P, and X' over tile t's rows of X once tile t's products are done.
 //
 // The streaming kernel (k_ns_tc), which these submatrices used before and larger ones still use, keeps the operands of
 // two submatrices per SM in global memory: 0.6 MB of TMA traffic a product at n = 172, more than the L2 holds over 152
-// SMs (14.6 GB of DRAM traffic on 4,096 submatrices). Here the products are bound by the MMAs, 12,100 cycles a step at
-// n = 172 in the three-term split, and the epilogue of T tile 0 and of the Z blocks runs beside them.
+// SMs (14.6 GB of DRAM traffic on 4,096 submatrices). Here a step takes some 17,000 cycles at n = 174 in the three-term
+// split, 12,100 of them the MMAs' own, the rest where the epilogue waits for them or they for it; with one term the
+// epilogue's (11,000 of 14,600 at n = 162), whose arithmetic on the two SM quarters that hold the second row tile counts.
+// 27,000 submatrices: 18.2 ms, some 31 with the streaming kernel. Twelve or sixteen epilogue warps instead of eight: 18.6 and
+// 26 ms (their registers spill); the MMAs unrolled over K: 19.0.
 //
 // Roles: warp 1 issues the MMAs (converged, one elected lane), warps 4-11 are the epilogue (two groups of four, even
 // and odd 32-column chunks), which also starts and finishes the submatrices. All waits are bounded.
@@ -52,7 +58,7 @@ constexpr uint64_t kWaitNsR = 2000000000ull;
 struct StepInfo { int term, n16, nrb, nch; Fmt f; };   // what the MMA warp needs of a step
 
 struct SharedR {
-  uint64_t xr, pf[2], tr[2], zf[2], ze[2], ld[2], idle;
+  uint64_t xr, pf[2], tr[2], zf[2], ze[2], zp[2], ld[2], idle;
   uint32_t tmem;
   int err, fetch;
   StepInfo mm;
@@ -264,6 +270,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       tc::mbar_init(&sh.pf[t], 1);
       tc::mbar_init(&sh.tr[t], kEpiR);
       tc::mbar_init(&sh.zf[t], 1);
+      tc::mbar_init(&sh.zp[t], 1);
       tc::mbar_init(&sh.ze[t], kEpiR);
       tc::mbar_init(&sh.ld[t], 1);
     }
@@ -305,6 +312,22 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
         }
         __syncwarp();
       }
+      if (kTerms == 1 && !three) {   // Z = X T, T in the second plane, over P's accumulators
+        for (int t = 0; t < m.nrb && ok; ++t) {
+          ok = wait(&sh.tr[t], (t ? np1 : np0) & 1, 1);
+          ++(t ? np1 : np0);
+        }
+        if (!ok) break;
+        tc::tc_fence_after();
+        for (int t = 0; t < m.nrb; ++t) {
+          if (tc::elect_one()) {
+            product<false>(tmem + kResMaxN * t, x0, 128 * t, 0, kPlane, m.n16, idp, false);
+            tc::mma_commit(&sh.zp[t]);
+          }
+          __syncwarp();
+        }
+        continue;
+      }
       for (int c = 0; c < m.nch && ok; ++c) {
         const uint32_t idz = tc::idesc(m.f.fmt, m.f.fmt, 0, 1, 128, min(64, m.n16 - 64 * c));
         for (int t = 0; t < m.nrb; ++t, ++nz) {
@@ -330,7 +353,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
     // ------------------------------------------------ epilogue
     const int etid = tid - 128, ew = warp - 4, q = warp & 3, grp = ew >> 2;
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-    uint32_t nld = 0;
+    uint32_t nld = 0, nq0 = 0, nq1 = 0;   // fills; one-term Z products of either row tile
     bool bad = false;
     for (;;) {
       // ---- the next submatrix of at most kResMaxN rows (the last one's finish has used the feed's buffers)
@@ -431,6 +454,14 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
                   l[u] = pick(u, lane >> 1, __byte_perm(l[u], tl, sel), l[u]);
                 }
               }
+              if (kTerms == 1 && !ref) {
+                if (j + 2 < nsub) tc::tmem_ld32(ta + 32 * (j + 2), r);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  *reinterpret_cast<uint4*>(X + kPlane + unit_at(j >> 1, row, 4 * (j & 1) + u)) =
+                      make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+                continue;
+              }
               uint32_t o[32];
 #pragma unroll
               for (int u = 0; u < 16; ++u) {
@@ -443,6 +474,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
             tc::tmem_wait_st();
           }
           tc::tc_fence_before();
+          if (kTerms == 1) tc::fence_proxy_async_smem();
           if (!bad) tc::mbar_arrive(&sh.tr[t]);
         }
         // ---- the defect of X and the decision about the following steps (every thread alike)
@@ -501,8 +533,39 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
             if (nn <= kResMaxN) tc::prefetch_l2(g.A + g.a_off[Jn], sizeof(float) * (size_t)nn * nn);
           }
         }
-        // ---- Z -> X', column block by column block (two 32-column chunks, one a group)
-        for (int c = 0; c < nch; ++c) {
+        // ---- one term: Z -> X', row tile by row tile. Tile t's rows of X are read by tile t's products alone; the lo plane
+        // of the refinement's format takes T's place once all of them have completed.
+        if (kTerms == 1 && !ref) {
+          for (int t = rnxt ? -nrb : 0; t < nrb; ++t) {
+            const int w = t < 0 ? t + nrb : t;
+            if (!bad) bad = !tc::mbar_wait_ns(&sh.zp[w], (w ? nq1 : nq0) & 1, g.wait_ns);
+            bad = __any_sync(0xffffffffu, bad);
+            tc::tc_fence_after();
+            const int rbase = 128 * w + 32 * q, row = rbase + lane;
+            if (t < 0 || rbase >= n64 || bad) continue;
+            const uint32_t ta = tmem + kResMaxN * w + lane_base;
+#pragma unroll 1
+            for (int j = grp; 32 * j < n16; j += 2) {
+              uint32_t r[32], h[16], l[16];
+              tc::tmem_ld32(ta + 32 * j, r);
+              tc::tmem_wait_ld();
+              float sq = 0.0f;
+              if (!rnxt) scale_split_t<kFmt, false, false>(r, 0.5f, h, l, sq);
+              else scale_split_t<FMT_F16, true, false>(r, 0.5f, h, l, sq);
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                uint8_t* at = X + unit_at(j >> 1, row, 4 * (j & 1) + u);
+                *reinterpret_cast<uint4*>(at) = make_uint4(h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
+                if (rnxt) *reinterpret_cast<uint4*>(at + kPlane) = make_uint4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+              }
+            }
+          }
+          ++nq0;
+          nq1 += nrb - 1;
+          tc::tc_fence_before();
+        }
+        // ---- else Z -> X', column block by column block (two 32-column chunks, one a group)
+        for (int c = 0; c < (kTerms == 1 && !ref ? 0 : nch); ++c) {
           const int col0 = 64 * c + 32 * grp;
           const bool cols = col0 < n16;
           // row tile t's block out of its accumulator, halved and split
