@@ -616,7 +616,7 @@ def main():
     tf = lambda fl, ms: fl / (ms / 1e3) / 1e12 if ms > 0 else 0.0
     peak = peaks["bf16_sustained"]
     chunks = max(1, int(st["factor_launches"]))
-    roof_sign = {"bound": "tensor" if not fp64_path else "alu", "kernel": "k_ns_tc (sign iteration)",
+    roof_sign = {"bound": "tensor" if not fp64_path else "alu", "kernel": "k_ns_res, k_ns_tc above 192 rows (sign iteration)",
                  "achieved": tf(fl_paper, ms_sign), "peak": peak, "unit": "TFLOP/s",
                  "frac": tf(fl_paper, ms_sign) / peak if peak else None,
                  "traffic": kernel_traffic("k_ns_tc", j1 - j0),
@@ -634,8 +634,8 @@ def main():
     if not fp64_path and args.inverse == "ns":
         ms_prep_kernel = mean("ms_prep_tensor")
         fl_prep = mean("flops_prep_tensor")
-        roof_prep = {"bound": "tensor", "kernel": "k_ns_tc<1> (inverse square root of T_J(S), Eqs. inv1-inv3, "
-                                                  "and A_J)",
+        roof_prep = {"bound": "tensor", "kernel": "k_inv_res, k_ns_tc<1> above 192 rows (inverse square root of "
+                                                  "T_J(S), Eqs. inv1-inv3, and A_J)",
                      "achieved": tf(fl_prep, ms_prep_kernel), "peak": peak, "unit": "TFLOP/s",
                      "frac": tf(fl_prep, ms_prep_kernel) / peak if peak else None,
                      "traffic": kernel_traffic("k_ns_tc_inv", (j1 - j0) / chunks), "launches_per_step": chunks,
