@@ -36,9 +36,7 @@
 // T_J(S) exceeds twice the mean (then the defect grows, and the submatrix, like any whose iteration does
 // not reach tol_inv within max_inv steps, is flagged for the FP64 preparation). X = T_J(S)^-1 is also
 // written in FP32 for the refinement of the centre columns of T_J(S)^-1.
-// This mode runs 512 threads: three epilogue groups (warps 4-15, every third chunk each), since the start
-// of a submatrix (three operand pairs from T_J(S)) and T_J(H0) weigh more against its few products; its
-// tiles are 128 x up to 192 columns, and the TMA / MMA warpgroup hands registers to the epilogue (setmaxnreg).
+// Submatrices of up to 192 rows come here only for what k_inv_res leaves (more than two steps).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
