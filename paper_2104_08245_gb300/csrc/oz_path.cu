@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "nolsm_internal.cuh"
 #include "oz_path.cuh"
@@ -487,21 +488,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
       uint16_t* dst = planes + (size_t)set * kD * plane_elems;
       const int half = (n16 / 16 + 1) / 2 * 16;
       const int r0 = rank ? half : 0, r1 = rank ? n16 : half, w2 = n16 / 2;
-      // four rows of a warp together: eight loads in flight per lane
+      // four rows of a warp together: eight loads in flight per lane (no condition holds one back)
       for (int i0 = r0 + 4 * ew; i0 < r1; i0 += 32)
         for (int j = lane; j < w2; j += 32) {
           long long v[4][2];
+          std::remove_cv_t<std::remove_reference_t<decltype(*M)>> x[4][2];
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) x[a][u] = __ldg(M + (size_t)min(i0 + a, n - 1) * n + min(2 * j + u, n - 1));
 #pragma unroll
           for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
               const int i = i0 + a, col = 2 * j + u;
-              v[a][u] = 0;
-              if (i < n && col < n) {
-                auto x = __ldg(M + (size_t)i * n + col);
-                if constexpr (kMode == 0) x = (x - (i == col ? mu : 0.0)) * inv;
-                v[a][u] = to_fixed(x, U - e);
-              }
+              if constexpr (kMode == 0) x[a][u] = (x[a][u] - (i == col ? mu : 0.0)) * inv;
+              v[a][u] = i < n && col < n ? to_fixed(x[a][u], U - e) : 0;
             }
 #pragma unroll
           for (int a = 0; a < 4; ++a) {
@@ -784,7 +786,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
           const double* xi = xd + (size_t)i * g.LD;
           double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
           int kk = 0;
-          for (; kk + 4 <= n; kk += 4) {
+#pragma unroll 4
+          for (; kk + 4 <= n; kk += 4) {   // 24 loads in flight: their latency is what a row of X costs
             const double2 xa = __ldcg(reinterpret_cast<const double2*>(xi + kk));
             const double2 xb = __ldcg(reinterpret_cast<const double2*>(xi + kk + 2));
             s0 = fma(xa.x, Q[(size_t)kk * b + col], s0);
