@@ -902,13 +902,17 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
               float v[4][8];
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
-                const int i = i0 + r;
+                const float* row = A + (size_t)min(i0 + r, n - 1) * n;   // (no condition holds a load back)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[r][u] = __ldg(row + min(j0 + u, n - 1));
+              }
+#pragma unroll
+              for (int r = 0; r < 4; ++r)
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                  const int j = j0 + u;
-                  v[r][u] = (i < n && j < n) ? (A[(size_t)i * n + j] - (i == j ? fmu : 0.0f)) * inv : 0.0f;
+                  const int i = i0 + r, j = j0 + u;
+                  v[r][u] = i < n && j < n ? (v[r][u] - (i == j ? fmu : 0.0f)) * inv : 0.0f;
                 }
-              }
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
                 const int i = i0 + r;
