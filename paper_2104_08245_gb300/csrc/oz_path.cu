@@ -17,7 +17,10 @@
 // brings in is used by every pair it belongs to (kD (kD + 1) / 2 MMAs per 2 kD tiles). Roles: warp 0 (one thread)
 // TMA loads, warp 1 (one thread) MMAs, warps 4-11 the epilogue. The CTAs meet on a barrier in each other's shared
 // memory after every product, which also carries the parts of the defect and the overflow flags; every role then
-// takes the same decision by itself. All waits are bounded.
+// takes the same decision by itself. All three roles of both CTAs arrive, loader and MMA warp when they begin to wait:
+// so none is more than one meeting behind (the records are kept for two), also where nothing else holds it, as in a
+// CTA that has no tile (n up to 64), between a finish and the next start, or after a start that gave up; and every role
+// has looked a submatrix's status up before an epilogue writes it. All waits are bounded.
 //
 // The second mode prepares A_J = T_J(S)^-1 T_J(H0) and the centre columns of T_J(S)^-1 for the same path, from the FP32
 // inverse X of the inverse-square-root kernel (good to about 1e-6): R = I - T_J(S) X, V = I + R (I + R), X <- X V, whose
@@ -248,7 +251,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     }
     tc::mbar_init(&sh.accf, 1);
     tc::mbar_init(&sh.acce, kOzEpi);
-    tc::mbar_init(&sh.done, 2);
+    tc::mbar_init(&sh.done, 6);                // loader, MMA warp and epilogue of both CTAs
     tc::mbar_init(&sh.idle, 1);
     tc::fence_mbar_init();
     sh.err = 0;
@@ -276,7 +279,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
   struct Course { int n, n16, nrb, ncb, cur, sp, steps, cap, tries, status; bool last, gave_up; };
   Course c;
   const bool mma_warp = warp == 1;
+  auto arrive = [&]() {                        // one thread of a role
+    const uint32_t done0 = tc::smem_u32(&sh.done);
+    for (uint32_t to = 0; to < 2; ++to) arrive_cluster(mapa(done0, to));
+  };
   auto meet = [&](Record& r) -> bool {         // waits for the meeting's end; false: give up
+    if (warp < 4 && lane == 0) arrive();       // (the epilogue has arrived in tell)
     bool ok = !sh.err && wait_cluster(&sh.done, ev & 1, 8 * g.wait_ns);
     if (mma_warp) ok = __all_sync(0xffffffffu, ok);
     r = sh.rec[ev & 1];
@@ -328,7 +336,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     tc::setmaxnreg_dec<kRegsLow>();
     if ((warp == 0 && lane == 0) || warp == 1) {   // one thread loads; the MMA warp runs converged, one lane issues
       // one product: A in operand set za, B in zb
-      auto product = [&](int sa, int sb) -> bool {
+      auto tiles = [&](int sa, int sb) -> bool {
         const int n32 = (c.n16 + 31) / 32;
         for (int t = rank; t < c.nrb * c.ncb; t += 2) {
           const int mb = t / c.ncb, cb = t - mb * c.ncb;
@@ -375,6 +383,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
         }
         return true;
       };
+      auto product = [&](int sa, int sb) -> bool {
+        if (tiles(sa, sb)) return true;
+        sh.err = 1;                            // a wait ran out: the others meet once more without this role, and leave
+        if (lane == 0) arrive();
+        return false;
+      };
       Record r;
       for (int k = cid; k < g.count; k += ncl) {
         if (!begin(g.order[k])) continue;
@@ -419,7 +433,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     const int etid = tid - 128, ew = warp - 4, q = warp & 3, grp = ew >> 2;
     uint16_t* const planes = g.planes + (size_t)zc * plane_elems;
     double* const xd = g.xd + (size_t)cid * plane_elems;
-    const uint32_t rec0 = tc::smem_u32(&sh.rec[0]), done0 = tc::smem_u32(&sh.done);
+    const uint32_t rec0 = tc::smem_u32(&sh.rec[0]);
     int ex = 1, et = 2, es = 1, eh = 1;          // exponents of X, T (mode 0), S and H (inverse mode)
 
     // the CTA's part of the meeting: sums over its threads to both CTAs' records, then the arrivals
@@ -457,7 +471,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
           st_cluster(at + 8 + 4 * rank, b);
           for (int u = 0; u < 3; ++u) st_cluster(at + 16 + 24 * rank + 8 * u, t[u]);
         }
-        for (uint32_t to = 0; to < 2; ++to) arrive_cluster(mapa(done0, to));
+        arrive();
       }
     };
 
