@@ -36,7 +36,7 @@ constexpr int kThreads = 128;   // several CTAs (submatrices) per SM overlap eac
 constexpr int kMaxB = 64;
 constexpr int kRefineMax = 4;   // refinement steps of Q before a submatrix falls back to the FP64 factor
 constexpr double kRefineTol = 1e-6;
-constexpr double kNsOneStep = 1e-5;   // k_ns_qrefine: a first correction below this ends the refinement
+constexpr double kNsOneStep = 8e-6;   // k_ns_qrefine: a first correction below this ends the refinement
 
 // Row stride of panels and tiles in shared memory: FP64 rows padded by one element (bank spread),
 // FP32 rows by four so that every row starts on a 16-byte boundary (vector loads).
@@ -1127,26 +1127,21 @@ __global__ void __launch_bounds__(kThreads, 4) k_prepare_mixed(PrepArgs g, float
 
 constexpr int kQThreads = 256, kQWarps = kQThreads / 32;
 constexpr int RPL = 2;          // rows per lane
-constexpr float kQBig = 6.0f;   // offset of the residual's leading sums (see residual_part)
 
 // This warp's share (rows k0 <= k < k1 of the symmetric T_J(S)) of (T_J(S) q)_ic for its lanes' rows i and NP pairs
-// of columns. The lanes read T_J(S) along its rows, coalesced. Each product a v, a and v as two FP32 words, is added
-// to a running sum t that starts at kQBig: t' = fl(t + a v), and what that rounded off is a v - (t' - t), exact to one
-// rounding because t is the larger (Dekker's Fast2Sum with the product inside the second FMA). t moves in steps of
-// ulp(kQBig) = 2^-21, so the remainders l stay near 2^-19 and their FP32 sum is good to 2^-43 per term: the residual
-// keeps about 1e-12 of |T_J(S)| |q|. Six packed operations per pair of columns instead of eleven per column.
+// of columns, as t + l. The lanes read T_J(S) along its rows, coalesced. Each product a v, a and v as two FP32 words, is
+// added to t with its own rounding error and the sum's in l (add_product2): about 48 bits of |T_J(S)| |q|, on every
+// overlap. (A Fast2Sum about an offset, six packed operations a pair of columns instead of twelve, kept 43 bits, and 21
+// where the products, which reach S_ii (T_J(S)^-1)_ii, leave the offset's range. Whole steps with it and now: 262,144
+// submatrices of n = 162 372.4 and 376.9 ms, 512 of 23 functions a molecule 23.2 and 24.0.)
 template <int NP>
 __device__ __forceinline__ void residual_part(const double* __restrict__ S, int n, int k0, int k1, const int (&row)[RPL],
                                               const float* __restrict__ qh, const float* __restrict__ ql,
                                               uint64_t (&t)[RPL][NP], uint64_t (&l)[RPL][NP]) {
-  const uint64_t neg = pair2(-1.0f, -1.0f);
 #pragma unroll
   for (int r = 0; r < RPL; ++r)
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      t[r][p] = pair2(kQBig, kQBig);
-      l[r][p] = 0;
-    }
+    for (int p = 0; p < NP; ++p) t[r][p] = l[r][p] = 0;
   constexpr int kU = 4;   // rows k per step: their loads run one step ahead of the arithmetic
   double nx[kU][RPL];
 #pragma unroll
@@ -1164,11 +1159,12 @@ __device__ __forceinline__ void residual_part(const double* __restrict__ S, int 
       }
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-      uint64_t ax[RPL], ay[RPL];
+      uint64_t ax[RPL], an[RPL], ay[RPL];
 #pragma unroll
       for (int r = 0; r < RPL; ++r) {
         const float2 a = split_f64(sv[u][r]);
         ax[r] = pair2(a.x, a.x);
+        an[r] = pair2(-a.x, -a.x);
         ay[r] = pair2(a.y, a.y);
       }
       const int kk = min(k + u, k1 - 1);   // past k1 the entries of T_J(S) are zeros
@@ -1179,12 +1175,9 @@ __device__ __forceinline__ void residual_part(const double* __restrict__ S, int 
         const uint64_t x = vh[p], y = vl[p];
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
-          const uint64_t tn = fma2(ax[r], x, t[r][p]);
-          const uint64_t nh = fma2(tn, neg, t[r][p]);   // t - t'
-          l[r][p] = add2(l[r][p], fma2(ax[r], x, nh));
+          add_product2(t[r][p], l[r][p], ax[r], an[r], x);
           l[r][p] = fma2(ax[r], y, l[r][p]);
           l[r][p] = fma2(ay[r], x, l[r][p]);
-          t[r][p] = tn;
         }
       }
     }
@@ -1260,8 +1253,8 @@ __device__ void refine_group(const double* __restrict__ S, const float* __restri
         for (int p = 0; p < NP; ++p) {
           const int at = (warp * kCols + 2 * p) * kRows + 32 * r + lane;
           const float2 a = unpair2(t[r][p]);
-          red[at] = pass == 0 ? a.x - kQBig : a.x;
-          red[at + kRows] = pass == 0 ? a.y - kQBig : a.y;
+          red[at] = a.x;
+          red[at + kRows] = a.y;
           if (pass == 0) {
             const float2 b = unpair2(l[r][p]);
             red2[at] = b.x;
@@ -1273,13 +1266,10 @@ __device__ void refine_group(const double* __restrict__ S, const float* __restri
         const int c = e / kRows, i = i0 + (e & (kRows - 1));
         if (i >= n || c >= cn) continue;
         if (pass == 0) {
-          // the shares of t are multiples of 2^-21 below 4: E minus their sum is exact near the solution
           float hi = i == ce + c ? 1.0f : 0.0f, lo = 0.0f;
 #pragma unroll
           for (int w = 0; w < kQWarps; ++w) {
-            const float h = red[w * kRows * kCols + e], z = hi - h;
-            lo += (hi - z) - h;                       // what the subtraction rounded off (nothing, normally)
-            hi = z;
+            two_sum(hi, lo, -red[w * kRows * kCols + e]);
             lo -= red2[w * kRows * kCols + e];
           }
           R[(size_t)i * qs + c] = hi + lo;
@@ -1380,8 +1370,9 @@ __global__ void __launch_bounds__(kQThreads, 2) k_ns_qrefine(PrepArgs g, const f
       qm = fmax(qm, red_q[w2]);
     }
     // converged when the correction is below 1e-6 of q, or after the first step when that correction (the
-    // error of X's columns, about the contraction factor ||I - X T_J(S)|| too) is below 1e-5 of q: the error
-    // left is then about its square, below 1e-10 of q
+    // error of X's columns, and the contraction factor ||I - X T_J(S)|| up to some 1.5 times as much) is below 8e-6 of q:
+    // the error left is below 1e-10 of q (1.06e-10 was left behind a first correction just below 1e-5: n = 46, pairs
+    // overlapping by 0.89). A line of 5e-6 would cost merged sites of n = 200-400 a second step, 12.5 ms instead of 10.7.
     conv = (double)dm <= kRefineTol * qm || (it == 0 && (double)dm <= kNsOneStep * qm);
     __syncthreads();
   }

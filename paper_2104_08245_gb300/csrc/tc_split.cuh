@@ -70,6 +70,17 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   return d;
 }
 
+// s + e <- s + e + a x in pairs, na = -a: the product's rounding error by FMA, the sum's by TwoSum, whatever the order of
+// magnitude of the two; e collects them in FP32.
+__device__ __forceinline__ void add_product2(uint64_t& s, uint64_t& e, uint64_t a, uint64_t na, uint64_t x) {
+  const uint64_t neg = pair2(-1.0f, -1.0f);
+  const uint64_t p = mul2(a, x), m = fma2(na, x, p);   // p - a x
+  const uint64_t t = add2(s, p), z = fma2(s, neg, t);  // t - s
+  const uint64_t d = add2(fma2(fma2(z, neg, t), neg, s), fma2(z, neg, p));
+  e = fma2(m, neg, add2(e, d));
+  s = t;
+}
+
 // u == k ? a : b as an instruction that the compiler does not fold into an indexed (local memory) array access: local
 // memory shares its bandwidth with the MMAs' operands
 __device__ __forceinline__ uint32_t pick(int u, int k, uint32_t a, uint32_t b) {
