@@ -1713,7 +1713,7 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     NOLSM_LAUNCH_CHECK();
     return NOLSM_OK;
   };
-  auto read_back = [&](int32_t* again) -> nolsm_status {   // flops, and what k_inv_res left; clears both
+  auto read_back = [&](int32_t* again) -> nolsm_status {   // adds up the flops; how many k_inv_res has left
     double fl[2];
     NOLSM_CUDA_TRY(cudaMemcpyAsync(fl, S->inv_flops.p, sizeof(fl), cudaMemcpyDeviceToHost, st));
     NOLSM_CUDA_TRY(cudaMemcpyAsync(again, S->err.as<int32_t>() + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1779,7 +1779,10 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
     g.wait_ns = kWaitNs;
     g.flops = S->inv_flops.as<double>();
     plan->stats.launches += 2;
-    if (again) return launch_shape(1, 0, m, g, sms, st);
+    if (again) {
+      NOLSM_TRY(pending(order, count));
+      return launch_shape(1, 0, m, g, sms, st);
+    }
     return run_buckets(1, NOLSM_FP16, false, m, g, order, count, count, a.mean_n, sms, st, pending);
   };
   if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, false));
