@@ -255,6 +255,29 @@ __device__ __forceinline__ void xq_part(const uint8_t* __restrict__ X, int i, in
   }
 }
 
+// The same with every product's rounding error (exact_xq): two products a step, as short in code as it can be.
+template <int kFmt, bool kLo>
+__device__ __forceinline__ void xq_exact(const uint8_t* __restrict__ X, int i, int k0, int k1, const float* __restrict__ Qs,
+                                         uint64_t (&s)[4], uint64_t (&e)[4]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) s[c] = e[c] = 0;
+#pragma unroll 1
+  for (int k = k0; k < k1; k += 2) {
+    const uint32_t at = unit_at(k >> 6, i, (k >> 3) & 7) + 2 * (k & 7);
+    const uint32_t h = *reinterpret_cast<const uint32_t*>(X + at), l = kLo ? *reinterpret_cast<const uint32_t*>(X + kPlane + at) : 0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float x = from_bits((uint16_t)(h >> (16 * u)), kFmt);
+      if (kLo) x += from_bits((uint16_t)(l >> (16 * u)), kFmt);
+      const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(Qs + (k + u) * 8);
+      const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(Qs + (k + u) * 8 + 4);
+      const uint64_t xx = pair2(x, x), xn = pair2(-x, -x), q[4] = {qa.x, qa.y, qb.x, qb.y};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) add_product2(s[c], e[c], xx, xn, q[c]);
+    }
+  }
+}
+
 // kFmt, kTerms: the main phase's operand format (the refinement's is FP16 in three terms). A template of it, and one site
 // each of T and of the Z blocks, because the epilogue's code has to stay in the instruction cache: with all four formats
 // at every site the code is 84 KB, against 62-74 KB.
@@ -648,6 +671,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       const double* __restrict__ Hc = g.Hc + g.c_off[J];
       double* __restrict__ Dc = g.Dc + g.c_off[J];
       double ps = 0.0, ph = 0.0;
+      const bool exact = exact_xq(n, b);
       const int units = n16 / 16, nitem = ((n + 31) / 32) * kSplit;   // of k: 16 at a time
       for (int cg = 0; cg < b; cg += 8) {
         const int cn = min(8, b - cg);
@@ -669,8 +693,13 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
           const int i = 32 * (it / kSplit) + lane, kq = it % kSplit;
           const int k0 = 16 * (units * kq / kSplit), k1 = 16 * (units * (kq + 1) / kSplit);
           uint64_t s[4], e[4];
-          if (!kOne && !ref) xq_part<kFmt, (kTerms > 1)>(X, i, k0, k1, Qs, s, e);
-          else xq_part<FMT_F16, true>(X, i, k0, k1, Qs, s, e);
+          if (!kOne && !ref) {
+            if (exact) xq_exact<kFmt, (kTerms > 1)>(X, i, k0, k1, Qs, s, e);
+            else xq_part<kFmt, (kTerms > 1)>(X, i, k0, k1, Qs, s, e);
+          } else {
+            if (exact) xq_exact<FMT_F16, true>(X, i, k0, k1, Qs, s, e);
+            else xq_part<FMT_F16, true>(X, i, k0, k1, Qs, s, e);
+          }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const float2 a = unpair2(s[c]), d = unpair2(e[c]);

@@ -43,9 +43,10 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdlib>
 #include <mutex>
-#include <cmath>
+#include <type_traits>
 
 #include "nolsm_internal.cuh"
 #include "prep.cuh"
@@ -226,10 +227,10 @@ struct Shared {
 
 // Eight rows of X a warp (2-byte hi and, with kLo, lo planes, columns k0 .. k0 + kn - 1, kn a multiple of 32) times 8
 // columns of Q in FP32 (staged from row k0 on): four lanes a row, each 8 adjacent columns of every 32, so that a load
-// reads 64 consecutive bytes of a row. FP32 sums of 8 products, each added to s + e with TwoSum; then the four lanes'
-// sums together, the same in each of them.
+// reads 64 consecutive bytes of a row. FP32 sums of 8 products, each added to s + e with TwoSum, or with kExact (exact_xq)
+// every product with its own rounding error; then the four lanes' sums together, the same in each of them.
 __device__ __forceinline__ int qs_at(int k) { return 8 * k + 4 * (k >> 3); }   // four lanes' rows in different banks
-template <int kFmt, bool kLo>
+template <int kFmt, bool kLo, bool kExact>
 __device__ __forceinline__ void xq_rows(const uint16_t* __restrict__ xh, const uint16_t* __restrict__ xl, int kn,
                                         const float* __restrict__ Qs, int part, uint64_t (&s)[4], uint64_t (&e)[4]) {
   const uint64_t neg = pair2(-1.0f, -1.0f);
@@ -240,17 +241,18 @@ __device__ __forceinline__ void xq_rows(const uint16_t* __restrict__ xh, const u
     e[c] = add2(e[c], add2(fma2(fma2(z, neg, t), neg, s[c]), fma2(z, neg, p)));
     s[c] = t;
   };
+  constexpr int kT = kExact ? 1 : 4;   // pieces of 32 columns together
 #pragma unroll 1
-  for (int k0 = 8 * part; k0 < kn; k0 += 128) {
-    uint4 hv[4], lv[4];
+  for (int k0 = 8 * part; k0 < kn; k0 += 32 * kT) {
+    uint4 hv[kT], lv[kT];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {   // (past the end the last piece again)
+    for (int t = 0; t < kT; ++t) {   // (past the end the last piece again)
       const int k = min(k0 + 32 * t, kn - 32 + 8 * part);
       hv[t] = *reinterpret_cast<const uint4*>(xh + k);
       lv[t] = kLo ? *reinterpret_cast<const uint4*>(xl + k) : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < kT; ++t) {
       const int k = k0 + 32 * t;
       if (k >= kn) break;
       uint64_t p[4] = {0, 0, 0, 0};
@@ -262,14 +264,15 @@ __device__ __forceinline__ void xq_rows(const uint16_t* __restrict__ xh, const u
         if (kLo) x += from_bits((uint16_t)(l >> (16 * (u & 1))), kFmt);
         const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u);
         const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u + 4);
-        const uint64_t xx = pair2(x, x);
-        p[0] = fma2(xx, qa.x, p[0]);
-        p[1] = fma2(xx, qa.y, p[1]);
-        p[2] = fma2(xx, qb.x, p[2]);
-        p[3] = fma2(xx, qb.y, p[3]);
+        const uint64_t xx = pair2(x, x), xn = pair2(-x, -x), q[4] = {qa.x, qa.y, qb.x, qb.y};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (kExact) add_product2(s[c], e[c], xx, xn, q[c]);
+          else p[c] = fma2(xx, q[c], p[c]);
+        }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) add(c, p[c]);
+      for (int c = 0; c < 4 && !kExact; ++c) add(c, p[c]);
     }
   }
 #pragma unroll
@@ -949,6 +952,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
       constexpr int kRowsP = 128, kRowsQ = (int)((kStgTotal - 64 * kRowsP) / 34) & ~31;
       static_assert(4 * (8 * kRowsQ + 4 * (kRowsQ / 8)) + 64 * kRowsP <= kStgTotal, "staging");
       const int n64 = d.n64;
+      const bool exact = exact_xq(n, b);
       float* const Qs = reinterpret_cast<float*>(stg);
       float2* const Ps = reinterpret_cast<float2*>(stg + kStgTotal - 64 * kRowsP);
       double ps = 0.0, ph = 0.0;
@@ -979,12 +983,17 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
               const int row = 8 * it + (lane >> 2), part = lane & 3;
               const size_t ro = (size_t)min(rr + row, n - 1) * g.LD + k0;
               uint64_t s[4], e[4];
+              auto sums = [&](auto sum) {
+                if (exact) sum(std::true_type{});
+                else sum(std::false_type{});
+              };
+              const uint16_t *h = xh + ro, *l = xl + ro;
               if (xfmt.fmt == FMT_BF16) {
-                if (xfmt.terms > 1) xq_rows<FMT_BF16, true>(xh + ro, xl + ro, kn, Qs, part, s, e);
-                else xq_rows<FMT_BF16, false>(xh + ro, xl + ro, kn, Qs, part, s, e);
+                if (xfmt.terms > 1) sums([&](auto x) { xq_rows<FMT_BF16, true, x.value>(h, l, kn, Qs, part, s, e); });
+                else sums([&](auto x) { xq_rows<FMT_BF16, false, x.value>(h, l, kn, Qs, part, s, e); });
               } else {
-                if (xfmt.terms > 1) xq_rows<FMT_F16, true>(xh + ro, xl + ro, kn, Qs, part, s, e);
-                else xq_rows<FMT_F16, false>(xh + ro, xl + ro, kn, Qs, part, s, e);
+                if (xfmt.terms > 1) sums([&](auto x) { xq_rows<FMT_F16, true, x.value>(h, l, kn, Qs, part, s, e); });
+                else sums([&](auto x) { xq_rows<FMT_F16, false, x.value>(h, l, kn, Qs, part, s, e); });
               }
               if (part == 0) {
 #pragma unroll
