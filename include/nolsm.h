@@ -55,8 +55,10 @@ typedef enum {
  * 1e-12 relative; a submatrix whose refinement does not contract, or whose overlap is too ill-conditioned
  * for the FP32 factor, is prepared again with the FP64 factorisation.
  *   NOLSM_FP64       FP64 accuracy: the products of the sign iteration and of the inverse's refinement as exact
- *                    sums of products of 8- or 9-bit digits on the tensor cores (64-bit fixed point); submatrices
- *                    that the fixed point does not hold, by an FP64 factorisation and iteration on the CUDA cores.
+ *                    sums of products of 8- or 9-bit digits on the tensor cores (64-bit fixed point, one exponent
+ *                    for all entries of a matrix); submatrices that the fixed point does not hold as accurately as
+ *                    FP64 does (overlaps of condition above some 50, iterates with entries of 2 or more), by an
+ *                    FP64 factorisation and iteration on the CUDA cores.
  *   NOLSM_FP32       every Newton-Schulz product as a three-term split of FP16 tensor-core products
  *                    (hi*hi + hi*lo + lo*hi, FP32 accumulation): about 22 significant bits.
  *   NOLSM_BF16       Newton-Schulz products as single BF16 tensor-core products (FP32 accumulation)

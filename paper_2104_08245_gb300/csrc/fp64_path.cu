@@ -476,7 +476,7 @@ static nolsm_status ensure(nolsm_plan* plan, DevBuf& b, size_t bytes) {
 constexpr float kNsInvTol = 1e-3f;
 constexpr int kNsInvMaxSteps = 40;
 
-nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStream_t st) {
+nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStream_t st, bool loose) {
   const bool keep_fp64_A = cls == kPrepFP64;
   const bool sym = cls == kPrepSym;
   Prepared& P = prepared(plan, cls);
@@ -512,10 +512,11 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
   const int64_t budget = (int64_t)1 << 34;  // bytes of gathered T_J(S), T_J(H0) per chunk (16 GB of the 288)
   int64_t J = j0;
   while (J < j1) {
-    while (J < j1 && P.done[J]) ++J;
+    auto done = [&](int64_t k) { return P.done[k] == kDone || (loose && P.done[k] == kDoneLoose); };
+    while (J < j1 && done(J)) ++J;
     if (J >= j1) break;
     int64_t e = J;
-    while (e < j1 && !P.done[e] &&
+    while (e < j1 && !done(e) &&
            (e == J || 2 * 8 * (plan->h_a_off[e + 1] - plan->h_a_off[J]) <= budget))
       ++e;
     const int64_t n2 = plan->h_a_off[e] - plan->h_a_off[J];
@@ -611,7 +612,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       // the FP32 inverse refined with exact digit products on the tensor cores (oz_path.cu); the FP64 Cholesky
       // factorisation of what that left, in particular overlaps that are not positive definite
       if (chunk_max_n <= prepare_fp64_max_n()) {
-          NOLSM_TRY(tensor_inverse(nullptr));
+        NOLSM_TRY(tensor_inverse(nullptr));
         int dev = 0, sms = 0;
         NOLSM_CUDA_TRY(cudaGetDevice(&dev));
         NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -628,6 +629,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
         z.a_off = pa.a_off; z.c_off = pa.c_off;
         z.prep_status = z.prep_out = pa.prep_status;
         z.ws = g.ws; z.a_base = g.a_base; z.chunk_n2 = n2;
+        z.loose = loose;
         z.X32 = plan->ws_l32.as<float>();
         z.Aout = P.A.as<double>();
         z.Qout = pa.Q;
@@ -687,7 +689,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       } else {
         plan->stats.flops_fp32 += 2.0 * (fma_fact + (sym ? 3.5 : 3.0) * m * m * b);
       }
-      P.done[k] = 1;
+      P.done[k] = loose ? kDoneLoose : kDone;
     }
     J = e;
   }
@@ -757,6 +759,7 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   z.Hc = plan->Hc.as<double>(); z.lam = spec.lam ? spec.lam : plan->lam.as<double>();
   z.lam_g = plan->lam.as<double>();
   z.prep_status = plan->prep_status.as<int32_t>();
+  z.loose = spec.loose;
   z.mu = mu; z.tol = o.tol_ns; z.max_iter = o.max_iter; z.budget = spec.budget;
   z.Dc = plan->Dc.as<double>(); z.tS = plan->t_S.as<double>(); z.tH = plan->t_H.as<double>();
   z.iters = plan->iters.as<int32_t>(); z.status = plan->status.as<int32_t>();

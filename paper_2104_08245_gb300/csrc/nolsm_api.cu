@@ -347,7 +347,7 @@ static nolsm_status solve_on_fp64(nolsm_plan* plan, double mu, const nolsm_optio
   for (size_t a = 0; a < subs.size();) {
     size_t b = a + 1;
     while (b < subs.size() && subs[b] == subs[b - 1] + 1) ++b;
-    NOLSM_TRY(prepare(plan, subs[a], (int64_t)subs[b - 1] + 1, kPrepFP64, st));
+    NOLSM_TRY(prepare(plan, subs[a], (int64_t)subs[b - 1] + 1, kPrepFP64, st, true));
     a = b;
   }
   if (!plan->ill_list.p) NOLSM_TRY(dev_alloc(plan, plan->ill_list, sizeof(int32_t) * (size_t)plan->n_mol));
@@ -359,6 +359,7 @@ static nolsm_status solve_on_fp64(nolsm_plan* plan, double mu, const nolsm_optio
   SolveSpec fs;
   fs.list = plan->ill_list.as<int32_t>();
   fs.count = (int32_t)subs.size();
+  fs.loose = true;
   NOLSM_TRY(solve_fp64(plan, mu, o64, j0, j1, fs, st));
   plan->stats.ill_conditioned += (int64_t)subs.size();
   return NOLSM_OK;

@@ -43,10 +43,11 @@ struct DevBuf {
 };
 
 // Geometry-dependent data of one precision class, computed once per plan (a1-a3 and the bounds).
+enum : uint8_t { kDone = 1, kDoneLoose = 2 };
 struct Prepared {
   bool fp64 = false;          // true: A held in FP64 (plain path); false: FP32 (tensor-core paths)
   DevBuf A;                   // A_J = T_J(S)^-1 T_J(H0), n_J x n_J row-major at a_off[J]
-  std::vector<uint8_t> done;  // host flag per submatrix: prepared
+  std::vector<uint8_t> done;  // host flag per submatrix: prepared (kDone), FP64 for a tensor-core mode alone (kDoneLoose)
   // tensor-core preparations: a lower estimate of cond(T_J(S)), (max_i L_ii / min_i L_ii)^2 from the FP32
   // Cholesky factor, max_i S_ii (T_J(S)^-1)_ii from the inverse square root (float per submatrix, device
   // and host copies; huge when the FP32 preparation failed)
@@ -187,7 +188,9 @@ inline int prep_class(const nolsm_options& o) {
   return o.inverse == NOLSM_INVERSE_NEWTON_SCHULZ ? kPrepNS : kPrepMixed;
 }
 inline Prepared& prepared(nolsm_plan* plan, int cls);
-nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStream_t st);
+// loose: FP64 class for a tensor-core mode that hands submatrices over (kFixedLoose); the FP64 class itself prepares
+// them again.
+nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStream_t st, bool loose = false);
 // a4 scale of submatrix J at mu: alpha = max(hi - mu, mu - lo) of the bound source's interval, but not
 // below 1/1.7 of the same from the Gershgorin interval [lg, hg], which contains the spectrum. Every
 // eigenvalue of X_0 then lies in [-1.7, 1.7] inside (-sqrt(3), sqrt(3)), where the Newton-Schulz map
@@ -205,6 +208,7 @@ struct SolveSpec {
   const int32_t* budget = nullptr;
   const int32_t* list = nullptr;
   int32_t count = 0;
+  bool loose = false;             // FP64: for a tensor-core mode (kFixedLoose)
 };
 nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int64_t j0, int64_t j1,
                         const SolveSpec& spec, cudaStream_t st);

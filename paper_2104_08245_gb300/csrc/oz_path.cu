@@ -26,9 +26,9 @@
 // inverse X of the inverse-square-root kernel (good to about 1e-6): R = I - T_J(S) X, V = I + R (I + R), X <- X V, whose
 // error is about R^3 (again from R when ||R||_F was above kOzLast), then A_J = X T_J(H0).
 //
-// What the fixed point does not hold is left to the FP64 kernels (k_ns_fp64; in the second mode k_prepare), which run
-// afterwards on the submatrices still marked kSubRefine: non-finite input, entries that outgrow every exponent tried, an
-// accumulator at 2^24, or a wait that ran out.
+// What the fixed point does not hold, or not as accurately (Fixed), is left to the FP64 kernels (k_ns_fp64; in the second
+// mode k_prepare), which run afterwards on the submatrices still marked kSubRefine: non-finite input, entries that outgrow
+// every exponent tried, an accumulator at 2^24, an FP32 inverse too far off, or a wait that ran out.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -51,10 +51,11 @@ constexpr int kOzEpi = 256;                  // epilogue threads (warps 4-11)
 constexpr int kRegsLaunch = 168, kRegsLow = 56, kRegsEpi = 224;
 static_assert(128 * kRegsLow + kOzEpi * kRegsEpi <= kOzThreads * kRegsLaunch, "register split above the launch");
 constexpr uint64_t kOzWaitNs = 2000000000ull;
-constexpr int kExTries = 4;                  // exponents tried per submatrix, each 3 above the last
-// Inverse mode: after an update from ||R||_F at most kOzLast the inverse is done (its cube, spread over n^2 entries, is
-// below 1e-16); ||R||_F at or above kOzFar, or no end after kOzRounds updates: the FP64 Cholesky takes the submatrix
-constexpr float kOzLast = 1.5e-5f, kOzFar = 0.5f;
+// Inverse mode: after an update from ||R||_F at most kOzLast the inverse is done: its cube is below 3.4e-15, and of that a
+// direction gets its share of some sqrt(n) (an X whose ||R||_F is that small has rounding errors in all of them; the
+// centre columns were 1.3e-16 off behind 1.35e-5). ||R||_F at or above Fixed::far, or no end after kOzRounds updates:
+// the FP64 Cholesky takes the submatrix
+constexpr float kOzLast = 1.5e-5f;
 constexpr int kOzRounds = 4;
 // operands in scratch: X, X', T; in inverse mode X, X', two that hold S (then V), R, H in turn, and I + R
 constexpr int sets(int mode) { return mode == 0 ? 3 : 5; }
@@ -89,6 +90,7 @@ struct OzArgs {
   int32_t R, LD;
   double* Dc; double* tS; double* tH; int32_t* iters; int32_t* status; int32_t* rsteps; int32_t* nbelow;
   uint64_t wait_ns;
+  Fixed lim;
   // inverse mode: the chunk's T_J(S), T_J(H0) (FP64, at a_off[J] - a_base and chunk_n2 further), X (FP32, at
   // a_off[J] - a_base), and the outputs
   const double* ws; int64_t a_base, chunk_n2;
@@ -309,7 +311,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     const uint32_t bad = r.bad[0] | r.bad[1];
     if (bad & 2) c.gave_up = true;
     else if (bad & 1) {
-      if (++c.tries < kExTries) return 1;
+      if (++c.tries < g.lim.tries) return 1;
       c.gave_up = true;
     }
     return (c.gave_up || c.last) ? 2 : 0;
@@ -318,7 +320,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     const float sum = r.part[0] + r.part[1];
     c.steps += 1;
     if constexpr (kMode == 0) {
-      if (sqrtf(sum / (float)c.n) <= (float)g.tol) {
+      if ((double)sqrtf(sum / (float)c.n) <= g.tol) {   // (the sum is good to 1e-6: a step more or less at that distance)
         c.last = true;
         c.status = kSubOk;
       } else if (c.steps >= c.cap) {
@@ -326,7 +328,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
       }
     } else {
       const float far = sqrtf(sum);
-      if (!(far < kOzFar) || (far > kOzLast && c.steps >= kOzRounds)) c.gave_up = true;
+      if (!(far < g.lim.far) || (far > kOzLast && c.steps >= kOzRounds)) c.gave_up = true;
       else if (far <= kOzLast) c.last = true;
     }
   };
@@ -913,6 +915,7 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
   g.Dc = a.Dc; g.tS = a.tS; g.tH = a.tH; g.iters = a.iters; g.status = a.status; g.rsteps = a.rsteps;
   g.nbelow = a.nbelow;
   g.wait_ns = kOzWaitNs;
+  g.lim = a.loose ? kFixedLoose : kFixedFp64;
   g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2; g.X32 = a.X32; g.sub_c0 = a.sub_c0;
   g.Aout = a.Aout; g.Qout = a.Qout; g.prep_out = a.prep_out;
   if (kMode == 1) g.max_iter = 1;

@@ -10,12 +10,25 @@ namespace nolsm {
 // K = 190 (seen on the 168-row water submatrices), although six of them would need a quarter fewer products.
 constexpr int kOzNineBits = 512;
 
+// What the fixed point takes: how many exponents of X are tried (each 3 above the last; what it drops and rounds grows
+// with their square), and the ||I - T_J(S) X||_F of the FP32 inverse, a measure of the overlap's condition, from which the
+// Cholesky factorisation prepares A_J instead (solving with the factor loses less than a product with the inverse).
+// kFixedFp64, the FP64 class: no more than what is as accurate as FP64 arithmetic. Distance of A_J, Q and D from
+// extended precision, relative to their largest entry, at n = 60 and 170, conditions 2 to 10: 1e-16 to 7e-16, with the
+// FP64 kernels 6e-16 to 4e-15; at 250 to 1,000, which these limits leave to the FP64 kernels: up to 4e-13, 2e-14, 8e-13
+// against 2e-13, 8e-14, 3e-13. The norm is 1e-5 to 5e-5 on water of any density, 1e-4 to 3e-4 at condition 50.
+// kFixedLoose, the submatrices that a tensor-core mode hands over: what keeps some twelve digits, for the six of the mode
+// (28 of 64 submatrices at condition 1,200: 14.5 ms a solve, 118 with the FP64 limits).
+struct Fixed { int tries; float far; };
+constexpr Fixed kFixedFp64{1, 2e-4f}, kFixedLoose{4, 0.5f};
+
 struct OzSolve {
   const int32_t* order; int32_t count;         // submatrices, largest first
   int32_t max_n;                               // largest dimension among them
   const int32_t* sub_n; const int32_t* nbf; const int64_t* a_off; const int64_t* c_off;
   const double* A; const double* Q; const double* Sc; const double* Hc; const double* lam; const double* lam_g;
   const int32_t* prep_status;
+  bool loose;                                  // kFixedLoose
   double mu, tol;
   int32_t max_iter; const int32_t* budget;
   uint16_t* planes; double* xd; int32_t R, LD, clusters;   // scratch: oz_planes(mode) planes of R x LD per cluster, R x LD
