@@ -469,6 +469,22 @@ static nolsm_status ensure(nolsm_plan* plan, DevBuf& b, size_t bytes) {
   return dev_alloc(plan, b, bytes);
 }
 
+// The digit kernels' operand planes for submatrices of up to max_n rows: R x LD each, for as many clusters as run at once
+static void oz_scratch(OzSolve* z, int max_n, int dev, int sms) {
+  z->max_n = max_n;
+  z->R = (max_n + 127) & ~127;
+  z->LD = (max_n + 63) & ~63;
+  z->clusters = std::min(z->count, oz_clusters(max_n, dev, sms));
+}
+
+// Workspaces of the tensor-core preparation that a later call allocates again, given back for an allocation that would
+// not fit beside them
+static void release_scratch(nolsm_plan* plan) {
+  dev_free(plan, plan->ws_l32);
+  dev_free(plan, plan->ws_ns);
+  tc_release(plan);
+}
+
 // Stopping rule of the tensor-core inverse square root: the step whose ||I - Z_k Y_k||_F / sqrt(n) is below
 // kNsInvTol is the last (the iteration converges quadratically, so its Z is about kNsInvTol^2 from the
 // limit, below the three-term products' own rounding); a submatrix still above it after kNsInvMaxSteps
@@ -510,9 +526,11 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
   int max_nq = 1;
   for (int64_t J = j0; J < j1; ++J) max_nq = std::max(max_nq, plan->h_nb_ptr[J + 1] - plan->h_nb_ptr[J]);
   const int64_t budget = (int64_t)1 << 34;  // bytes of gathered T_J(S), T_J(H0) per chunk (16 GB of the 288)
+  auto done = [&](int64_t k) { return P.done[k] == kDone || (loose && P.done[k] == kDoneLoose); };
+  int64_t left = 0;   // sum of n^2 over what is to be prepared
+  for (int64_t k = j0; k < j1; ++k) left += done(k) ? 0 : plan->h_a_off[k + 1] - plan->h_a_off[k];
   int64_t J = j0;
   while (J < j1) {
-    auto done = [&](int64_t k) { return P.done[k] == kDone || (loose && P.done[k] == kDoneLoose); };
     while (J < j1 && done(J)) ++J;
     if (J >= j1) break;
     int64_t e = J;
@@ -520,8 +538,9 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
            (e == J || 2 * 8 * (plan->h_a_off[e + 1] - plan->h_a_off[J]) <= budget))
       ++e;
     const int64_t n2 = plan->h_a_off[e] - plan->h_a_off[J];
-    // what the largest chunk of the range needs: a workspace that grew from one chunk to the next would be mapped anew
-    const int64_t cap = std::max(n2, std::min(plan->h_a_off[j1] - plan->h_a_off[J], budget / 16));
+    // what the largest chunk still to come needs: a workspace that grew from one chunk to the next would be mapped anew
+    const int64_t cap = std::max(n2, std::min(left, budget / 16));
+    left -= n2;
     NOLSM_TRY(ensure(plan, plan->ws_dense, sizeof(double) * 2 * (size_t)cap));
     // the chunk's submatrices, largest first: CTAs take them in this order, so that the last wave is made of small ones.
     // Copied before the gather starts, as a copy from host memory waits for the stream.
@@ -610,8 +629,9 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
     };
     if (keep_fp64_A) {
       // the FP32 inverse refined with exact digit products on the tensor cores (oz_path.cu); the FP64 Cholesky
-      // factorisation of what that left, in particular overlaps that are not positive definite
-      if (chunk_max_n <= prepare_fp64_max_n()) {
+      // factorisation of what that left, in particular overlaps that are not positive definite, and of everything when
+      // those kernels cannot run as built or their scratch does not fit on the device
+      auto by_digits = [&]() -> nolsm_status {
         NOLSM_TRY(tensor_inverse(nullptr));
         int dev = 0, sms = 0;
         NOLSM_CUDA_TRY(cudaGetDevice(&dev));
@@ -619,12 +639,9 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
         OzSolve z{};
         z.order = plan->prep_order.as<int32_t>();
         z.count = (int32_t)(e - J);
-        z.max_n = chunk_max_n;
-        z.R = (chunk_max_n + 127) & ~127;
-        z.LD = (chunk_max_n + 63) & ~63;
-        z.clusters = std::min(z.count, oz_clusters(chunk_max_n, dev, sms));
-        NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * (size_t)z.R * z.LD * oz_planes(1) * z.clusters));
-        z.planes = plan->oz_planes.as<uint16_t>();
+        oz_scratch(&z, chunk_max_n, dev, sms);
+        NOLSM_TRY(ensure(plan, plan->ws_ns, sizeof(uint16_t) * (size_t)z.R * z.LD * oz_planes(1) * z.clusters));
+        z.planes = plan->ws_ns.as<uint16_t>();
         z.sub_n = pa.sub_n; z.nbf = pa.nbf; z.sub_c0 = pa.sub_c0;
         z.a_off = pa.a_off; z.c_off = pa.c_off;
         z.prep_status = z.prep_out = pa.prep_status;
@@ -633,8 +650,13 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
         z.X32 = plan->ws_l32.as<float>();
         z.Aout = P.A.as<double>();
         z.Qout = pa.Q;
-        NOLSM_TRY(launch_inverse_oz(z, st));
-        pa.only_flagged = 1;
+        return launch_inverse_oz(z, st);
+      };
+      if (chunk_max_n <= prepare_fp64_max_n() && oz_ready(chunk_max_n) && ns_inverse_ready()) {
+        const nolsm_status s = by_digits();
+        if (s == NOLSM_ERR_OOM) release_scratch(plan);
+        else NOLSM_TRY(s);
+        pa.only_flagged = s == NOLSM_OK;
         plan->stats.launches += 4;
       }
       NOLSM_TRY(launch_prepare(pa, (int)(e - J), chunk_max_n, true, P.A.p, st));
@@ -729,7 +751,6 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   int32_t maxn = 0;
   for (int64_t J = j0; J < j1; ++J) maxn = std::max(maxn, plan->h_sub_n[J]);
   const int64_t slot_elems = (int64_t)maxn * maxn;
-  NOLSM_TRY(ensure(plan, plan->ws_ns, sizeof(double) * 3 * (size_t)slot_elems * slots));
   if (!spec.list && (plan->oz_j0 != j0 || plan->oz_j1 != j1)) {   // the range, largest first
     std::vector<int32_t> ord;
     largest_first(plan->h_sub_n, j0, work, ord);
@@ -744,15 +765,24 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   OzSolve z{};
   z.order = spec.list ? spec.list : plan->oz_order.as<int32_t>();
   z.count = work;
-  z.max_n = maxn;
-  z.R = (maxn + 127) & ~127;
-  z.LD = (maxn + 63) & ~63;
-  z.clusters = std::min(work, oz_clusters(maxn, dev, sms));
-  const size_t plane = (size_t)z.R * z.LD;
-  NOLSM_TRY(ensure(plan, plan->oz_planes, sizeof(uint16_t) * plane * oz_planes(0) * z.clusters));
-  NOLSM_TRY(ensure(plan, plan->oz_xd, sizeof(double) * plane * z.clusters));
-  z.planes = plan->oz_planes.as<uint16_t>();
-  z.xd = plan->oz_xd.as<double>();
+  oz_scratch(&z, maxn, dev, sms);
+  // One workspace for both kernels, the plain one starting when the other has ended: digit planes, then the final X;
+  // without room for those, what the plain kernel needs, and it takes everything.
+  const size_t plane = (size_t)z.R * z.LD, planes = sizeof(uint16_t) * plane * oz_planes(0) * z.clusters;
+  const size_t plain = sizeof(double) * 3 * (size_t)slot_elems * slots;
+  bool digits = oz_ready(maxn);
+  if (digits) {
+    nolsm_status s = ensure(plan, plan->ws_ns, std::max(plain, planes + sizeof(double) * plane * z.clusters));
+    if (s == NOLSM_ERR_OOM) {
+      release_scratch(plan);
+      s = ensure(plan, plan->ws_ns, std::max(plain, planes + sizeof(double) * plane * z.clusters));
+    }
+    if (s != NOLSM_ERR_OOM) NOLSM_TRY(s);
+    digits = s == NOLSM_OK;
+  }
+  if (!digits) NOLSM_TRY(ensure(plan, plan->ws_ns, plain));
+  z.planes = plan->ws_ns.as<uint16_t>();
+  z.xd = reinterpret_cast<double*>(plan->ws_ns.as<unsigned char>() + planes);
   z.sub_n = plan->sub_n.as<int32_t>(); z.nbf = plan->sub_b.as<int32_t>();
   z.a_off = plan->a_off.as<int64_t>(); z.c_off = plan->c_off.as<int64_t>();
   z.A = plan->prep64.A.as<double>(); z.Q = plan->Q.as<double>(); z.Sc = plan->Sc.as<double>();
@@ -764,7 +794,7 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   z.Dc = plan->Dc.as<double>(); z.tS = plan->t_S.as<double>(); z.tH = plan->t_H.as<double>();
   z.iters = plan->iters.as<int32_t>(); z.status = plan->status.as<int32_t>();
   z.rsteps = plan->rsteps.as<int32_t>(); z.nbelow = plan->nbelow.as<int32_t>();
-  NOLSM_TRY(launch_ns_oz(z, st));
+  NOLSM_TRY(digits ? launch_ns_oz(z, st) : leave_ns_oz(z, st));
   NOLSM_CUDA_TRY(cudaMemsetAsync(plan->counter.p, 0, sizeof(int32_t), st));
   NsArgs g;
   g.sub_n = z.sub_n; g.nbf = z.nbf;

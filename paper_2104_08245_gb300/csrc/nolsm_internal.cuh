@@ -151,8 +151,7 @@ struct nolsm_plan {
   nolsm::DevBuf ws_refine;          // q as FP32 pairs and FP32 corrections of Q for one chunk
   nolsm::DevBuf prep_order;         // submatrices of one chunk, largest first (mixed preparation)
   nolsm::DevBuf ws_ysym;            // L^-1 T_J(H0) of one preparation chunk (symmetric form)
-  nolsm::DevBuf ws_ns;              // per-CTA Newton-Schulz buffers (FP64 path)
-  nolsm::DevBuf oz_planes, oz_xd;   // FP64 path on the tensor cores: digit planes, final X (per cluster)
+  nolsm::DevBuf ws_ns;              // FP64 path: digit planes and final X per cluster, then buffers per CTA
   nolsm::DevBuf oz_order;           // submatrices [oz_j0, oz_j1), largest first
   int64_t oz_j0 = -1, oz_j1 = -1;
   void* tc = nullptr;               // tensor-core path state (tc_path.cu)

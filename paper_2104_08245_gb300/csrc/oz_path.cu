@@ -887,13 +887,26 @@ int active_clusters(int dev, int sms) {
 }
 
 template <class Dg, int kMode>
+bool split_fits() {
+  cudaFuncAttributes at{};
+  const bool ok = cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(&k_ns_oz<Dg, kMode>)) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok && at.numRegs == kRegsLaunch;
+}
+
+template <int kMode>
+nolsm_status pending(const OzSolve& a, cudaStream_t st) {
+  k_oz_pending<kMode><<<std::min(256, (a.count + 255) / 256), 256, 0, st>>>(a.count, a.order,
+                                                                            kMode == 0 ? a.status : a.prep_out);
+  NOLSM_LAUNCH_CHECK();
+  return NOLSM_OK;
+}
+
+template <class Dg, int kMode>
 nolsm_status launch(const OzSolve& a, cudaStream_t st) {
   const auto kernel = &k_ns_oz<Dg, kMode>;
-  cudaFuncAttributes at{};
-  NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(kernel)));
-  if (at.numRegs != kRegsLaunch) {
-    set_error("k_ns_oz was built with %d registers per thread; its register split needs exactly %d", at.numRegs,
-              kRegsLaunch);
+  if (!split_fits<Dg, kMode>()) {
+    set_error("k_ns_oz was not built with the %d registers per thread that its register split needs", kRegsLaunch);
     return NOLSM_ERR_UNSUPPORTED;
   }
   NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Dg::kSmem));
@@ -919,9 +932,7 @@ nolsm_status launch(const OzSolve& a, cudaStream_t st) {
   g.ws = a.ws; g.a_base = a.a_base; g.chunk_n2 = a.chunk_n2; g.X32 = a.X32; g.sub_c0 = a.sub_c0;
   g.Aout = a.Aout; g.Qout = a.Qout; g.prep_out = a.prep_out;
   if (kMode == 1) g.max_iter = 1;
-  k_oz_pending<kMode><<<std::min(256, (a.count + 255) / 256), 256, 0, st>>>(a.count, a.order,
-                                                                            kMode == 0 ? a.status : a.prep_out);
-  NOLSM_LAUNCH_CHECK();
+  NOLSM_TRY(pending<kMode>(a, st));
   kernel<<<2 * std::min(a.clusters, a.count), kOzThreads, Dg::kSmem, st>>>(mA, mA64, mB, g);
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
@@ -934,6 +945,13 @@ int oz_planes(int mode) { return sets(mode) * Digits<8, 8>::kD; }
 int oz_clusters(int max_n, int dev, int sms) {
   return max_n <= kOzNineBits ? active_clusters<Digits<9, 7>>(dev, sms) : active_clusters<Digits<8, 8>>(dev, sms);
 }
+
+bool oz_ready(int max_n) {
+  return max_n <= kOzNineBits ? split_fits<Digits<9, 7>, 0>() && split_fits<Digits<9, 7>, 1>()
+                              : split_fits<Digits<8, 8>, 0>() && split_fits<Digits<8, 8>, 1>();
+}
+
+nolsm_status leave_ns_oz(const OzSolve& a, cudaStream_t st) { return pending<0>(a, st); }
 
 nolsm_status launch_ns_oz(const OzSolve& a, cudaStream_t st) {
   return a.max_n <= kOzNineBits ? launch<Digits<9, 7>, 0>(a, st) : launch<Digits<8, 8>, 0>(a, st);

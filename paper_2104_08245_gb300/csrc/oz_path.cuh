@@ -39,10 +39,14 @@ struct OzSolve {
   double* Aout; double* Qout; int32_t* prep_out;
 };
 int oz_planes(int mode);
+// Whether the kernels for this dimension came out of the compiler with the registers that their split needs.
+bool oz_ready(int max_n);
 // how many clusters run at once (the scratch is sized for them)
 int oz_clusters(int max_n, int dev, int sms);
 // Leaves status[J] = kSubRefine for the submatrices k_ns_fp64 has to take.
 nolsm_status launch_ns_oz(const OzSolve& a, cudaStream_t st);
+// Leaves all of them.
+nolsm_status leave_ns_oz(const OzSolve& a, cudaStream_t st);
 // A_J in FP64 to Aout + a_off[J] and the centre columns of T_J(S)^-1 to Qout + c_off[J], prep_out[J] = kSubOk; kSubRefine
 // or kSubPending where k_prepare has to take the submatrix.
 nolsm_status launch_inverse_oz(const OzSolve& a, cudaStream_t st);

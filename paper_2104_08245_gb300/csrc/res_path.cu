@@ -1174,12 +1174,19 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_inv_res(InvSolve g) {
 }  // namespace
 
 template <typename K>
-static nolsm_status ready(K* kernel, const char* name, uint32_t smem) {
+static bool split_fits(K* kernel) {
   cudaFuncAttributes at{};
-  NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(kernel)));
-  if (at.numRegs != kRegsLaunchR) {
-    set_error("%s was built with %d registers per thread; its register split needs exactly %d", name, at.numRegs,
-              kRegsLaunchR);
+  const bool ok = cudaFuncGetAttributes(&at, reinterpret_cast<const void*>(kernel)) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok && at.numRegs == kRegsLaunchR;
+}
+
+bool inv_res_ready() { return split_fits(&k_inv_res); }
+
+template <typename K>
+static nolsm_status ready(K* kernel, const char* name, uint32_t smem) {
+  if (!split_fits(kernel)) {
+    set_error("%s was not built with the %d registers per thread that its register split needs", name, kRegsLaunchR);
     return NOLSM_ERR_UNSUPPORTED;
   }
   NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -40,5 +40,6 @@ struct InvSolve {
   uint64_t wait_ns;
 };
 nolsm_status launch_inv_res(const InvSolve& a, int sms, cudaStream_t st);
+bool inv_res_ready();
 
 }  // namespace nolsm

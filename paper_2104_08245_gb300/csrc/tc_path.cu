@@ -1355,11 +1355,15 @@ static bool formats(int precision, Fmt* main_fmt, Fmt* refine_fmt) {
 
 // The register split (setmaxnreg) assumes that the launch gives each thread regs registers; with fewer, the epilogue
 // warpgroups' increase could never be granted, so the launch is refused.
-static nolsm_status check_register_split(const void* fn, int regs) {
+static bool split_ok(const void* fn, int regs) {
   cudaFuncAttributes at{};
-  NOLSM_CUDA_TRY(cudaFuncGetAttributes(&at, fn));
-  if (at.numRegs != regs) {
-    set_error("k_ns_tc was built with %d registers per thread; its register split needs exactly %d", at.numRegs, regs);
+  const bool ok = cudaFuncGetAttributes(&at, fn) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok && at.numRegs == regs;
+}
+static nolsm_status check_register_split(const void* fn, int regs) {
+  if (!split_ok(fn, regs)) {
+    set_error("k_ns_tc was not built with the %d registers per thread that its register split needs", regs);
     return NOLSM_ERR_UNSUPPORTED;
   }
   return NOLSM_OK;
@@ -1699,6 +1703,11 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     plan->stats.launches += 1;
   }
   return NOLSM_OK;
+}
+
+bool ns_inverse_ready() {
+  return inv_res_ready() && split_ok(reinterpret_cast<const void*>(&k_ns_tc<1, 0>), Shape<0>::kRegsLaunch) &&
+         split_ok(reinterpret_cast<const void*>(&k_ns_tc<1, 1>), Shape<1>::kRegsLaunch);
 }
 
 // a2-a3 on the tensor cores for the chunk's submatrices order[0, count) (gathered into args.ws): A_J into

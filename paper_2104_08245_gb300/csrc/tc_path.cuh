@@ -31,6 +31,8 @@ struct NsInvArgs {
   int32_t max_inv;
 };
 nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_t st);
+// Whether its kernels came out of the compiler with the registers that their split needs.
+bool ns_inverse_ready();
 
 // frees the tensor-core path's workspaces held by the plan
 void tc_release(nolsm_plan* plan);

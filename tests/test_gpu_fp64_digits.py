@@ -114,3 +114,41 @@ def test_as_accurate_as_fp64_arithmetic_on_every_overlap(nl, kind, cond):
     print(f"{kind}, condition {cond}: Q {err[0]:.1e}, A {err[1]:.1e}, D {err[2]:.1e}, {int(r.iters[0])} steps")
     assert max(err) <= 2e-15 + 3.0 * cond * 2.0 ** -53
     plan.close()
+
+
+def test_without_room_for_the_digit_planes_the_fp64_kernels_take_over(nl):
+    """20 submatrices of 600 rows need some 0.4 GB with the FP64 kernels and 1 GB with the digit products; 0.52 GB are
+    left free. The density is that of a solve with room, to 1e-12."""
+    import ctypes
+
+    import torch
+    n, b = 600, 30
+    m = n // b
+    S, H = conditioned("log", n, 2, np.random.default_rng(3))
+    blocks = lambda M: np.concatenate([M[b * i:b * i + b, b * j:b * j + b].ravel() for i in range(m) for j in range(m)])  # noqa: E731
+    csr = lambda M: types.SimpleNamespace(row_ptr=np.arange(0, m * m + 1, m), col_idx=np.tile(np.arange(m), m), vals=blocks(M))  # noqa: E731
+    dsys = nl.DeviceSystem(types.SimpleNamespace(nbf=np.full(m, b), S=csr(S), H=csr(H), n_occ=1.0))
+
+    def solve():
+        plan = nl.nolsm_build_submatrices(dsys)
+        r = nl.nolsm_solve_batch(plan, MU, nl.options("fp64"))
+        assert np.all(r.sub_status.cpu().numpy() == 0)
+        D, used = plan.scatter().cpu().numpy(), plan.info().device_bytes
+        plan.close()
+        return D, used
+
+    D0, used0 = solve()
+    cuda, pool = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+    assert cuda.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert cuda.cuMemPoolTrimTo(pool, ctypes.c_size_t(0)) == 0
+    filled = torch.empty(torch.cuda.mem_get_info()[0] - 520 * 2 ** 20, dtype=torch.uint8, device="cuda")
+    try:
+        D1, used1 = solve()
+    finally:
+        del filled
+        torch.cuda.empty_cache()
+    print(f"{used0 / 2 ** 20:.0f} MB with room, {used1 / 2 ** 20:.0f} without; max|dD| = {np.max(np.abs(D1 - D0)):.1e}")
+    assert used1 < 520 * 2 ** 20 < used0
+    assert np.max(np.abs(D1 - D0)) <= 1e-12 * np.max(np.abs(D0))
