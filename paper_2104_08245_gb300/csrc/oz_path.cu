@@ -156,17 +156,6 @@ __device__ __forceinline__ void cluster_sync() {
 }
 __device__ __forceinline__ void oz_bar() { asm volatile("bar.sync 3, %0;" ::"n"(kOzEpi) : "memory"); }
 
-// K-major operand with 64-byte rows and 64-byte swizzle: 8-row atoms of 512 bytes
-__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(16 >> 4) << 16;
-  d |= (uint64_t)(512 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -367,7 +356,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                 return false;
               tc::tc_fence_after();
               const uint32_t a0 = __shfl_sync(0xffffffffu, tc::smem_u32(stage_mem + st * Dg::kStage), 0);
-              const uint64_t ad = sdesc_sw64(a0), bd = tc::sdesc_sw128(a0 + Dg::kABytes, 4096, 1024);
+              const uint64_t ad = tc::sdesc_sw64(a0, 16, 512), bd = tc::sdesc_sw128(a0 + Dg::kABytes, 4096, 1024);
               if (tc::elect_one()) {
                 for (int kk = 0; kk < 2 && 32 * ks + 16 * kk < c.n16; ++kk) {
                   const uint64_t ak = ad + ((kk * 32) >> 4), bk = bd + ((kk * 2048) >> 4);

@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(Shape<kShape>::kThreads, 1)
       sh.slot[c].cur = 0;
       begin_fetch(c);
     }
-    uint32_t kcount = 0, i = 0;
+    uint32_t i = 0;
     int s = 0;
     for (;;) {
       int pick = -1;
@@ -1446,22 +1446,21 @@ static int env_shape() {
   return -1;
 }
 
-// The launch shape of one bucket of submatrices, order[0, count) (all with n above 192, or all at most 192):
-// the one NOLSM_TC_SHAPE fixes, else the one measured faster for (mode, precision, bucket) in this process. The
-// first time, both shapes run on the bucket's largest submatrices (32 per slot of every SM: with fewer, the
+// The launch shape of the submatrices order[0, count), all with n above 192 (bucket 1): the one NOLSM_TC_SHAPE
+// fixes, else the one measured faster for (mode, precision) in this process. The
+// first time, both shapes run on the largest of them (32 per slot of every SM: with fewer, the
 // start and the tail of the launch decide; the shapes differ by 3-40 % in steady state), timed with CUDA
 // events on the stream, and the faster is kept (not when a bounded wait ran out in the measurement); the
 // results of those runs are computed again by the launches that follow. pending(order, count) resets the
 // statuses of the submatrices a launch takes.
 template <typename Pending>
-static nolsm_status bucket_shape(int mode, int precision, int bucket, bool fixed0, const TcMaps& m, TcArgs g,
-                                 const int32_t* order, int32_t count, int sms, cudaStream_t st, Pending pending,
-                                 int* out) {
-  int shape = fixed0 ? 0 : env_shape();
+static nolsm_status bucket_shape(int mode, int precision, const TcMaps& m, TcArgs g, const int32_t* order, int32_t count,
+                                 int sms, cudaStream_t st, Pending pending, int* out) {
+  int shape = env_shape();
   const int pi = precision & 7;
   if (shape < 0) {
     std::lock_guard<std::mutex> lk(g_shape_mu);
-    shape = g_shape[mode][pi][bucket];
+    shape = g_shape[mode][pi][1];
   }
   if (shape < 0) {
     g.j0 = 0;
@@ -1494,49 +1493,30 @@ static nolsm_status bucket_shape(int mode, int precision, int bucket, bool fixed
     } else {
       shape = ms[1] < ms[0] ? 1 : 0;
       std::lock_guard<std::mutex> lk(g_shape_mu);
-      g_shape[mode][pi][bucket] = shape;
+      g_shape[mode][pi][1] = shape;
     }
   }
   *out = shape;
   return NOLSM_OK;
 }
 
-// Runs the submatrices order[0, count), largest first, of which the first n_large have n above 192: each bucket
-// in its shape (bucket_shape), as one launch over both when the shapes agree (no second launch tail), else one
-// launch per bucket.
+// Runs the submatrices order[0, count), largest first, as one launch: those of more than 192 rows in the shape that
+// bucket_shape gives; E4M3 (fixed0: all dimensions) in shape 0 and groups of one.
 template <typename Pending>
-static nolsm_status run_buckets(int mode, int precision, bool fixed0, const TcMaps& m, TcArgs g, const int32_t* order,
-                                int32_t n_large, int32_t count, int mean_n, int sms, cudaStream_t st, Pending pending) {
+static nolsm_status run_largest_first(int mode, int precision, bool fixed0, const TcMaps& m, TcArgs g, const int32_t* order,
+                                      int32_t count, int mean_n, int sms, cudaStream_t st, Pending pending) {
   if (count <= 0) return NOLSM_OK;
-  int s1 = -1, s0 = -1;
-  const int g1 = fixed0 ? 1 : group_size(mean_n), g0 = 1;
-  g.group = g1;
-  if (n_large > 0) NOLSM_TRY(bucket_shape(mode, precision, 1, fixed0, m, g, order, n_large, sms, st, pending, &s1));
-  g.group = g0;
-  if (count > n_large)
-    NOLSM_TRY(bucket_shape(mode, precision, 0, fixed0, m, g, order + n_large, count - n_large, sms, st, pending, &s0));
+  int shape = 0;
+  g.group = fixed0 ? 1 : group_size(mean_n);
+  if (!fixed0) NOLSM_TRY(bucket_shape(mode, precision, m, g, order, count, sms, st, pending, &shape));
   g.j0 = 0;
-  if (n_large == 0 || n_large == count || (s1 == s0 && g1 == g0)) {
-    g.group = n_large > 0 ? g1 : g0;
-    g.order = order;
-    g.j1 = count;
-    NOLSM_TRY(pending(order, count));
-    return launch_shape(mode, n_large > 0 ? s1 : s0, m, g, sms, st);
-  }
+  g.j1 = count;
   g.order = order;
-  g.group = g1;
-  g.j1 = n_large;
-  NOLSM_TRY(pending(order, n_large));
-  NOLSM_TRY(launch_shape(mode, s1, m, g, sms, st));
-  g.order = order + n_large;
-  g.group = g0;
-  g.j1 = count - n_large;
-  NOLSM_TRY(pending(order + n_large, count - n_large));
-  return launch_shape(mode, s0, m, g, sms, st);
+  NOLSM_TRY(pending(order, count));
+  return launch_shape(mode, shape, m, g, sms, st);
 }
 
-// Bucket 0 (n <= 192) has no shape to choose (the sign but for E4M3 and the inverse run it in res_path.cu): the query
-// reports 0 once it has run.
+// Bucket 0 (n <= 192) has no shape to choose (res_path.cu): the query reports 0 once it has run.
 static void resident_shape(int mode, int precision) {
   std::lock_guard<std::mutex> lk(g_shape_mu);
   g_shape[mode][precision & 7][0] = 0;
@@ -1662,9 +1642,9 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     NOLSM_TRY(make_maps(&m, S->planes.p, S->R, S->LD, S->slots * kPlanes, f8));
     if (spec.list) {   // reruns and a bisection's later points: one launch in list order, shape 0
       NOLSM_TRY(launch_shape(0, 0, m, g, sms, st));
-    } else {           // the largest-first order in its two buckets: n above 192, the rest (E4M3 only)
-      NOLSM_TRY(run_buckets(0, o.precision, f8, m, g, S->order.as<int32_t>(), S->ord_large,
-                            f8 ? (int32_t)work : S->ord_large, S->ord_mean, sms, st, pending));
+    } else {           // E4M3: all of the order; else those above 192 rows
+      NOLSM_TRY(run_largest_first(0, o.precision, f8, m, g, S->order.as<int32_t>(), f8 ? (int32_t)work : S->ord_large,
+                                  S->ord_mean, sms, st, pending));
     }
   }
   if (resident) {
@@ -1801,7 +1781,7 @@ nolsm_status launch_ns_inverse(nolsm_plan* plan, const NsInvArgs& a, cudaStream_
       NOLSM_TRY(pending(order, count));
       return launch_shape(1, 0, m, g, sms, st);
     }
-    return run_buckets(1, NOLSM_FP16, false, m, g, order, count, count, a.mean_n, sms, st, pending);
+    return run_largest_first(1, NOLSM_FP16, false, m, g, order, count, a.mean_n, sms, st, pending);
   };
   if (a.n_large > 0) NOLSM_TRY(streamed(a.order, a.n_large, false));
   int32_t again = 0;
