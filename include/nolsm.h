@@ -526,13 +526,13 @@ nolsm_status nolsm_sign_noalloc(int32_t count, const int32_t* sub_n, const int32
  * 1 (512 threads, three epilogue groups, 128 x up to 192, a register split between warpgroups). Each solve
  * (kernel 0: sign iteration) or preparation chunk (kernel 1: inverse square root) splits its submatrices,
  * largest first, into two buckets, n above 192 (bucket 1) and the rest (bucket 0). Bucket 0 has a kernel with one
- * shape (reported as 0), but for E4M3. The first time a process
- * meets a (kernel, precision, bucket), both shapes run on that bucket's largest submatrices (32 per slot
- * of every SM), timed with CUDA events on the caller's stream, and the faster is kept for the life of the
- * process; the timed runs' results are computed again by the bucket's launch. Setting the environment
- * variable NOLSM_TC_SHAPE to "0" or "1" fixes the shape instead (read at every call); E4M3 and the reruns of
- * failed submatrices always take shape 0. Returns the shape chosen so far for (kernel, precision, bucket), or
- * -1 when none has been measured yet. Host only; thread-safe. */
+ * shape (reported as 0), but for E4M3. In bucket 1 groups of 1, 2, 4 or 8 CTAs share a submatrix, by the mean n.
+ * The first time a process meets a (kernel, precision, CTAs of a group), both shapes run on the largest
+ * submatrices (32 per slot of every SM), timed with CUDA events on the caller's stream, and the faster is kept for
+ * the life of the process; the timed runs' results are computed again by the launch that follows. Setting the
+ * environment variable NOLSM_TC_SHAPE to "0" or "1" fixes the shape instead (read at every call); E4M3 and the
+ * reruns of failed submatrices always take shape 0. Returns the shape last chosen for (kernel, precision, bucket),
+ * or -1 when none has been measured yet. Host only; thread-safe. */
 int32_t nolsm_tc_shape(int32_t kernel, int32_t precision, int32_t bucket);
 
 const char* nolsm_status_str(nolsm_status s);

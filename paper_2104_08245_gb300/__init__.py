@@ -60,9 +60,9 @@ def options(precision="fp64", **kw) -> NolsmOptions:
 
 
 def nolsm_tc_shape(kernel: str, precision, bucket: int) -> int:
-    """Launch shape chosen in this process (0 or 1, -1 while not measured) for kernel "sign" or "inverse",
+    """Launch shape last chosen in this process (0 or 1, -1 while not measured) for kernel "sign" or "inverse",
     a precision (name or value; the inverse square root always runs in "fp16") and bucket 0 (n <= 192) or
-    1 (n > 192)."""
+    1 (n > 192: measured once for each number of CTAs that share a submatrix)."""
     k = {"sign": 0, "inverse": 1}[kernel]
     p = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
     return int(_abi.load().nolsm_tc_shape(k, p, int(bucket)))

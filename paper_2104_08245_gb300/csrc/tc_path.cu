@@ -1434,11 +1434,13 @@ static nolsm_status launch_shape(int mode, int shape, const TcMaps& m, TcArgs g,
   return NOLSM_OK;
 }
 
-// The launch shape of each (mode, precision, bucket) as measured in this process (-1: not yet), and the
-// environment variable NOLSM_TC_SHAPE ("0" or "1") that fixes it instead.
+// The launch shapes of a (mode, precision) as measured in this process (-1: not yet): by the CTAs that share a submatrix
+// (1, 2, 4, 8), which decide how tiles are dealt and so which shape is the faster; the last one taken; and bucket 0's. The
+// environment variable NOLSM_TC_SHAPE ("0" or "1") fixes the shape instead.
+struct Shapes { int of_group[4] = {-1, -1, -1, -1}, last = -1, small = -1; };
 static std::mutex g_shape_mu;
-static int g_shape[2][8][2] = {{{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}},
-                               {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}}};
+static Shapes g_shape[2][8];
+static int group_index(int G) { return G >= 8 ? 3 : G >= 4 ? 2 : G >= 2 ? 1 : 0; }
 
 static int env_shape() {
   const char* e = std::getenv("NOLSM_TC_SHAPE");
@@ -1447,7 +1449,7 @@ static int env_shape() {
 }
 
 // The launch shape of the submatrices order[0, count), all with n above 192 (bucket 1): the one NOLSM_TC_SHAPE
-// fixes, else the one measured faster for (mode, precision) in this process. The
+// fixes, else the one measured faster for (mode, precision, g.group) in this process. The
 // first time, both shapes run on the largest of them (32 per slot of every SM: with fewer, the
 // start and the tail of the launch decide; the shapes differ by 3-40 % in steady state), timed with CUDA
 // events on the stream, and the faster is kept (not when a bounded wait ran out in the measurement); the
@@ -1457,10 +1459,12 @@ template <typename Pending>
 static nolsm_status bucket_shape(int mode, int precision, const TcMaps& m, TcArgs g, const int32_t* order, int32_t count,
                                  int sms, cudaStream_t st, Pending pending, int* out) {
   int shape = env_shape();
-  const int pi = precision & 7;
+  Shapes& known = g_shape[mode][precision & 7];
+  const int gi = group_index(g.group);
   if (shape < 0) {
     std::lock_guard<std::mutex> lk(g_shape_mu);
-    shape = g_shape[mode][pi][1];
+    shape = known.of_group[gi];
+    if (shape >= 0) known.last = shape;
   }
   if (shape < 0) {
     g.j0 = 0;
@@ -1493,7 +1497,7 @@ static nolsm_status bucket_shape(int mode, int precision, const TcMaps& m, TcArg
     } else {
       shape = ms[1] < ms[0] ? 1 : 0;
       std::lock_guard<std::mutex> lk(g_shape_mu);
-      g_shape[mode][pi][1] = shape;
+      known.of_group[gi] = known.last = shape;
     }
   }
   *out = shape;
@@ -1519,13 +1523,14 @@ static nolsm_status run_largest_first(int mode, int precision, bool fixed0, cons
 // Bucket 0 (n <= 192) has no shape to choose (res_path.cu): the query reports 0 once it has run.
 static void resident_shape(int mode, int precision) {
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  g_shape[mode][precision & 7][0] = 0;
+  g_shape[mode][precision & 7].small = 0;
 }
 
 int tc_shape_choice(int mode, int precision, int bucket) {
   if (mode < 0 || mode > 1 || bucket < 0 || bucket > 1) return -1;
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  return g_shape[mode][precision & 7][bucket];
+  const Shapes& known = g_shape[mode][precision & 7];
+  return bucket == 0 ? known.small : known.last;
 }
 
 nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64_t j0, int64_t j1, const SolveSpec& spec,

@@ -37,7 +37,7 @@ bool ns_inverse_ready();
 // frees the tensor-core path's workspaces held by the plan
 void tc_release(nolsm_plan* plan);
 
-// launch shape chosen in this process for (mode 0 sign / 1 inverse, precision, bucket 0: n <= 192 / 1: n > 192):
+// launch shape last chosen in this process for (mode 0 sign / 1 inverse, precision, bucket 0: n <= 192 / 1: n > 192):
 // 0 or 1, or -1 while not measured
 int tc_shape_choice(int mode, int precision, int bucket);
 
