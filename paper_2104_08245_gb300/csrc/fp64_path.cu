@@ -525,6 +525,9 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
   }
   int max_nq = 1;
   for (int64_t J = j0; J < j1; ++J) max_nq = std::max(max_nq, plan->h_nb_ptr[J + 1] - plan->h_nb_ptr[J]);
+  int dev = 0, sms = 0;
+  NOLSM_CUDA_TRY(cudaGetDevice(&dev));
+  NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t budget = (int64_t)1 << 34;  // bytes of gathered T_J(S), T_J(H0) per chunk (16 GB of the 288)
   auto done = [&](int64_t k) { return P.done[k] == kDone || (loose && P.done[k] == kDoneLoose); };
   int64_t left = 0;   // sum of n^2 over what is to be prepared
@@ -583,7 +586,7 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       if (gsm > 48 * 1024) NOLSM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
       // with few submatrices the bands of each go to several CTAs (64 of 27 bands: 43 us with one each, 14 with four)
       const unsigned spread = (unsigned)std::max<int64_t>(
-          1, std::min<int64_t>((max_nq + kGatherWarps - 1) / kGatherWarps, (16 * 152 + e - J - 1) / (e - J)));
+          1, std::min<int64_t>((max_nq + kGatherWarps - 1) / kGatherWarps, (16 * sms + e - J - 1) / (e - J)));
       kernel<<<dim3((unsigned)(e - J), spread), 32 * kGatherWarps, gsm, st>>>(g);
       return NOLSM_OK;
     };
@@ -633,9 +636,6 @@ nolsm_status prepare(nolsm_plan* plan, int64_t j0, int64_t j1, int cls, cudaStre
       // those kernels cannot run as built or their scratch does not fit on the device
       auto by_digits = [&]() -> nolsm_status {
         NOLSM_TRY(tensor_inverse(nullptr));
-        int dev = 0, sms = 0;
-        NOLSM_CUDA_TRY(cudaGetDevice(&dev));
-        NOLSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         OzSolve z{};
         z.order = plan->prep_order.as<int32_t>();
         z.count = (int32_t)(e - J);
