@@ -388,11 +388,12 @@ __global__ void __launch_bounds__(256) k_ns_fp64(NsArgs g) {
 // ------------------------------------------------------------------------------------ reductions
 // Sums of t_S and t_H over [j0, j1) in a fixed order (one block), the first failing submatrix, and
 // the work counters: sum of steps n^3 (paper convention), of the tensor products' n^3 (x3 for split
-// steps) on unpadded and padded shapes, and of steps.
+// steps) on unpadded shapes and as the MMAs run them (rows to 128, N and K to 16; E4M3, f8_main, N to 64 and K to 128),
+// and of steps.
 __global__ void __launch_bounds__(256) k_reduce(int32_t j0, int32_t j1, const double* __restrict__ tS,
                                                 const double* __restrict__ tH, const int32_t* __restrict__ status,
                                                 const int32_t* __restrict__ iters, const int32_t* __restrict__ rsteps,
-                                                const int32_t* __restrict__ sub_n, int terms_main,
+                                                const int32_t* __restrict__ sub_n, int terms_main, int f8_main,
                                                 const int32_t* __restrict__ list, int32_t count, double* out) {
   __shared__ double red[33];
   __shared__ int first[256];
@@ -409,11 +410,12 @@ __global__ void __launch_bounds__(256) k_reduce(int32_t j0, int32_t j1, const do
   for (int e = threadIdx.x; e < m; e += blockDim.x) {
     const int J = list ? list[e] : j0 + e;
     const double n = sub_n[J];
-    const double n64 = (double)((sub_n[J] + 63) & ~63), R = (double)((sub_n[J] + 127) & ~127);
-    const double prod = (double)terms_main * (iters[J] - rsteps[J]) + 3.0 * rsteps[J];
+    const double n16 = (double)((sub_n[J] + 15) & ~15), R = (double)((sub_n[J] + 127) & ~127);
+    const double nk_main = f8_main ? (double)((sub_n[J] + 63) & ~63) * R : n16 * n16;
+    const double pm = (double)terms_main * (iters[J] - rsteps[J]), pr = 3.0 * rsteps[J], prod = pm + pr;
     w0 += iters[J] * n * n * n;
     w1 += prod * n * n * n;
-    w2 += prod * R * n64 * n64;
+    w2 += R * (pm * nk_main + pr * n16 * n16);
     w3 += iters[J];
   }
   const double sa = block_sum(a, red);
@@ -814,11 +816,12 @@ nolsm_status solve_fp64(nolsm_plan* plan, double mu, const nolsm_options& o, int
   return NOLSM_OK;
 }
 
-nolsm_status reduce_traces(nolsm_plan* plan, int64_t j0, int64_t j1, int terms_main, cudaStream_t st, double* tS,
-                           double* tH, int32_t* first_bad_status, const int32_t* list, int32_t count) {
+nolsm_status reduce_traces(nolsm_plan* plan, int64_t j0, int64_t j1, int precision, cudaStream_t st, double* tS, double* tH,
+                           int32_t* first_bad_status, const int32_t* list, int32_t count) {
   k_reduce<<<1, 256, 0, st>>>((int32_t)j0, (int32_t)j1, plan->t_S.as<double>(), plan->t_H.as<double>(),
                               plan->status.as<int32_t>(), plan->iters.as<int32_t>(), plan->rsteps.as<int32_t>(),
-                              plan->sub_n.as<int32_t>(), terms_main, list, count, plan->sums.as<double>());
+                              plan->sub_n.as<int32_t>(), precision == NOLSM_FP64 ? 1 : main_terms(precision),
+                              precision == NOLSM_FP8E4M3, list, count, plan->sums.as<double>());
   NOLSM_LAUNCH_CHECK();
   plan->stats.launches += 1;
   double h[8];

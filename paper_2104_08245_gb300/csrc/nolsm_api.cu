@@ -463,7 +463,7 @@ static nolsm_status solve_impl(nolsm_plan* plan, double mu, const nolsm_options*
   mark(plan, 2, st);
   double tS = 0, tH = 0;
   int32_t bad = 0;
-  NOLSM_TRY(reduce_traces(plan, j0, j1, fp64 ? 1 : main_terms(opts->precision), st, &tS, &tH, &bad, list, count));
+  NOLSM_TRY(reduce_traces(plan, j0, j1, opts->precision, st, &tS, &tH, &bad, list, count));
   mark(plan, 3, st);
   const size_t cnt = (size_t)(j1 - j0);
   if (sub_t_S) NOLSM_CUDA_TRY(cudaMemcpyAsync(sub_t_S + j0, plan->t_S.as<double>() + j0, 8 * cnt, cudaMemcpyDeviceToDevice, st));
