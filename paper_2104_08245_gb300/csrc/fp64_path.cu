@@ -409,14 +409,13 @@ __global__ void __launch_bounds__(256) k_reduce(int32_t j0, int32_t j1, const do
   const int32_t m = list ? count : j1 - j0;
   for (int e = threadIdx.x; e < m; e += blockDim.x) {
     const int J = list ? list[e] : j0 + e;
-    const double n = sub_n[J];
-    const double n16 = (double)((sub_n[J] + 15) & ~15), R = (double)((sub_n[J] + 127) & ~127);
-    const double nk_main = f8_main ? (double)((sub_n[J] + 63) & ~63) * R : n16 * n16;
-    const double pm = (double)terms_main * (iters[J] - rsteps[J]), pr = 3.0 * rsteps[J], prod = pm + pr;
-    w0 += iters[J] * n * n * n;
-    w1 += prod * n * n * n;
-    w2 += R * (pm * nk_main + pr * n16 * n16);
-    w3 += iters[J];
+    const int64_t n = sub_n[J], n3 = n * n * n, n16 = (n + 15) & ~15, R = (n + 127) & ~127;   // whole numbers below 2^53
+    const int64_t it = iters[J], pr = 3 * rsteps[J], pm = terms_main * (it - rsteps[J]);
+    const int64_t nk = n16 * n16, nk_main = f8_main ? ((n + 63) & ~63) * R : nk;
+    w0 += (double)(it * n3);
+    w1 += (double)((pm + pr) * n3);
+    w2 += (double)(R * (pm * nk_main + pr * nk));
+    w3 += (double)it;
   }
   const double sa = block_sum(a, red);
   const double sb = block_sum(b, red);

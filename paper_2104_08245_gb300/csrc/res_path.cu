@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "nolsm_internal.cuh"
 #include "prep.cuh"
@@ -280,8 +281,9 @@ __device__ __forceinline__ void xq_exact(const uint8_t* __restrict__ X, int i, i
 
 // kFmt, kTerms: the main phase's operand format (the refinement's is FP16 in three terms). A template of it, and one site
 // each of T and of the Z blocks, because the epilogue's code has to stay in the instruction cache: with all four formats
-// at every site the code is 84 KB, against 62-74 KB.
-template <int kFmt, int kTerms>
+// at every site the code is 84 KB, against 62-74 KB. kExact: some submatrix takes xq_exact (1 % more time on 262,144 that
+// do not, with its code there).
+template <int kFmt, int kTerms, bool kExact>
 __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
   constexpr bool kOne = kFmt == FMT_F16 && kTerms == 3;   // the main format is the refinement's
   extern __shared__ uint8_t smraw[];
@@ -671,7 +673,7 @@ __global__ void __launch_bounds__(kThreadsR, 1) k_ns_res(ResSolve g) {
       const double* __restrict__ Hc = g.Hc + g.c_off[J];
       double* __restrict__ Dc = g.Dc + g.c_off[J];
       double ps = 0.0, ph = 0.0;
-      const bool exact = exact_xq(n, b);
+      const bool exact = kExact && exact_xq(n, b);
       const int units = n16 / 16, nitem = ((n + 31) / 32) * kSplit;   // of k: 16 at a time
       for (int cg = 0; cg < b; cg += 8) {
         const int cn = min(8, b - cg);
@@ -1203,8 +1205,12 @@ nolsm_status launch_ns_res(const ResSolve& a, int sms, cudaStream_t st) {
     kernel<<<std::min(sms, a.count), kThreadsR, kSmemR, st>>>(g);
     return NOLSM_OK;
   };
-  if (a.main_fmt.fmt == FMT_BF16) NOLSM_TRY(a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_BF16, 3>) : run(&k_ns_res<FMT_BF16, 1>));
-  else NOLSM_TRY(a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_F16, 3>) : run(&k_ns_res<FMT_F16, 1>));
+  auto pick = [&](auto exact) -> nolsm_status {
+    constexpr bool kE = decltype(exact)::value;
+    if (a.main_fmt.fmt == FMT_BF16) return a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_BF16, 3, kE>) : run(&k_ns_res<FMT_BF16, 1, kE>);
+    return a.main_fmt.terms > 1 ? run(&k_ns_res<FMT_F16, 3, kE>) : run(&k_ns_res<FMT_F16, 1, kE>);
+  };
+  NOLSM_TRY(a.exact_xq ? pick(std::true_type{}) : pick(std::false_type{}));
   NOLSM_LAUNCH_CHECK();
   return NOLSM_OK;
 }

@@ -17,6 +17,7 @@ struct ResSolve {
   float tol_ns, tol_accept;
   int32_t max_iter, refine_steps; const int32_t* budget;
   Fmt main_fmt;                          // a 2-byte format; the refinement's is FP16 in three terms
+  bool exact_xq;                         // some submatrix of the work sums X Q exactly (exact_xq)
   int32_t* next; int32_t* err;           // work counter (reset by the launch), timeout flag
   double* Dc; double* tS; double* tH; int32_t* iters; int32_t* status; int32_t* rsteps; int32_t* nbelow;
   uint64_t wait_ns;                      // limit of a wait of one role on another, 0: 2 s

@@ -1314,6 +1314,7 @@ struct TcState {
   int64_t ord_j0 = -1, ord_j1 = -1;
   int32_t ord_large = 0;          // how many of the cached order (a prefix) have n above 192
   int32_t ord_mean = 0;           // their mean dimension
+  bool ord_exact = false;         // some of the others sum X Q exactly
   DevBuf inv_planes, inv_flops;   // inverse mode: its own plane layout (kPlanesInv per slot), flop sums
   int iR = 0, iLD = 0, islots = 0;
 };
@@ -1580,6 +1581,9 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     while (S->ord_large < (int32_t)ord.size() && plan->h_sub_n[ord[(size_t)S->ord_large]] > 192)
       sum += plan->h_sub_n[ord[(size_t)S->ord_large++]];
     S->ord_mean = S->ord_large > 0 ? (int32_t)(sum / S->ord_large) : 0;
+    S->ord_exact = false;
+    for (size_t k = (size_t)S->ord_large; k < ord.size(); ++k)
+      S->ord_exact = S->ord_exact || exact_xq(plan->h_sub_n[(size_t)ord[k]], plan->h_sub_b[(size_t)ord[k]]);
   }
   // one CTA per SM at most, each group of them with kSlots submatrices in flight (one scratch sub-slot each)
   const int group = f8 ? 1 : group_size(S->ord_mean);   // (E4M3: a turn writes the pair that it finishes)
@@ -1663,6 +1667,7 @@ nolsm_status solve_tc(nolsm_plan* plan, double mu, const nolsm_options& o, int64
     r.tol_ns = g.tol_ns; r.tol_accept = g.tol_accept;
     r.max_iter = g.max_iter; r.refine_steps = g.refine_steps; r.budget = g.budget;
     r.main_fmt = mf;
+    r.exact_xq = S->ord_exact;
     r.next = plan->counter.as<int32_t>() + 1; r.err = g.err;
     r.Dc = g.Dc; r.tS = g.tS; r.tH = g.tH; r.iters = g.iters; r.status = g.status; r.rsteps = g.rsteps;
     r.nbelow = g.nbelow;
