@@ -52,7 +52,7 @@ typedef enum {
 /* Arithmetic of the sign-iteration products (a5/a6). The trace sums are FP64 in every mode. The overlap
  * inverse is refined to FP64 in NOLSM_FP64; the tensor-core modes factor T_J(S) in FP32, form A_J with FP32
  * solves, and refine the centre columns of T_J(S)^-1 with a double-FP32 residual (about 48 bits) to about
- * 1e-12 relative; a submatrix whose refinement does not contract, or whose overlap is too ill-conditioned
+ * 1e-12 relative (after the tensor-core inverse below 1e-10); a submatrix whose refinement does not contract, or whose overlap is too ill-conditioned
  * for the FP32 factor, is prepared again with the FP64 factorisation.
  *   NOLSM_FP64       FP64 accuracy: the products of the sign iteration and of the inverse's refinement as exact
  *                    sums of products of 8- or 9-bit digits on the tensor cores (64-bit fixed point, one exponent
@@ -136,7 +136,7 @@ typedef struct {
                             Cores" (Eqs. inv1-inv3) on the tensor cores (three-term FP16 split products),
                             T_J(S)^-1 = Z^2 / c and A_J = T_J(S)^-1 T_J(H0) as two more products; the step whose
                             ||I - Z_k Y_k||_F / sqrt(n) <= 1e-3 is the last. Either way the centre columns of
-                            T_J(S)^-1 are refined to about 1e-12 with a double-FP32 residual, and a submatrix
+                            T_J(S)^-1 are refined to below 1e-10 with a double-FP32 residual, and a submatrix
                             that fails is prepared again with the FP64 factorisation. Ignored by NOLSM_FP64 and
                             the symmetric form (which keep the Cholesky factor). */
   int64_t wait_ns;       /* tensor-core sign kernel: limit of each device-side wait of one warp role on another

@@ -15,7 +15,8 @@
 // planes [X0 hi, X0 lo, X1 hi, X1 lo, T hi, T lo], each R x LD (R = n rounded up to 128 rows, LD = n rounded up to 64
 // columns, zero padded). What bounds it: with two submatrices on every SM the planes (4 MB a submatrix at n = 650) miss
 // L2, and each product's operands come from DRAM several times over; the groups keep the planes in flight within L2
-// (512 submatrices of n = 600-713: 233 GB through DRAM before, 41 GB since; 40 -> 12.9 ms). What is left at 2.4 times
+// (512 submatrices of n = 600-713: 233 GB through DRAM before, 41 GB since; 40 -> 12.4 ms, 13.6 with the compensated
+// X Q of large submatrices, exact_xq). What is left at 2.4 times
 // the MMAs' own time is the phases' latency (first slices, last tile's epilogue, the group's meeting) and, below
 // n = 256, the start and finish of a submatrix.
 // Output tiles are 128 rows x up to 256 columns; the K dimension streams in slices of 32 through a four-stage TMA
