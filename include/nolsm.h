@@ -137,8 +137,8 @@ typedef struct {
                             T_J(S)^-1 = Z^2 / c and A_J = T_J(S)^-1 T_J(H0) as two more products; the step whose
                             ||I - Z_k Y_k||_F / sqrt(n) <= 1e-3 is the last. Either way the centre columns of
                             T_J(S)^-1 are refined to below 1e-10 with a double-FP32 residual, and a submatrix
-                            that fails is prepared again with the FP64 factorisation. Ignored by NOLSM_FP64 and
-                            the symmetric form (which keep the Cholesky factor). */
+                            that fails is prepared again with the FP64 factorisation. Ignored by NOLSM_FP64 (see
+                            there) and the symmetric form (which keeps the Cholesky factor). */
   int64_t wait_ns;       /* tensor-core sign kernel: limit of each device-side wait of one warp role on another
                             (a product's operands, its accumulator, the next descriptor), in ns; <= 0: 2 s. A
                             wait that runs out ends the kernel early: the submatrices in flight and those not
