@@ -15,7 +15,7 @@
 // planes [X0 hi, X0 lo, X1 hi, X1 lo, T hi, T lo], each R x LD (R = n rounded up to 128 rows, LD = n rounded up to 64
 // columns, zero padded). What bounds it: with two submatrices on every SM the planes (4 MB a submatrix at n = 650) miss
 // L2, and each product's operands come from DRAM several times over; the groups keep the planes in flight within L2
-// (512 submatrices of n = 600-713: 233 GB through DRAM before, 41 GB since; 40 -> 12.4 ms, 13.6 with the compensated
+// (512 submatrices of n = 600-713: 233 GB through DRAM before, 41 GB since; 40 -> 12.4 ms, 13.2 with the compensated
 // X Q of large submatrices, exact_xq). What is left at 2.4 times
 // the MMAs' own time is the phases' latency (first slices, last tile's epilogue, the group's meeting) and, below
 // n = 256, the start and finish of a submatrix.
@@ -242,38 +242,52 @@ __device__ __forceinline__ void xq_rows(const uint16_t* __restrict__ xh, const u
     e[c] = add2(e[c], add2(fma2(fma2(z, neg, t), neg, s[c]), fma2(z, neg, p)));
     s[c] = t;
   };
-  constexpr int kT = kExact ? 1 : 4;   // pieces of 32 columns together
-#pragma unroll 1
-  for (int k0 = 8 * part; k0 < kn; k0 += 32 * kT) {
-    uint4 hv[kT], lv[kT];
+  auto load = [&](int k, uint4& h, uint4& l) {   // (past the end the last piece again)
+    k = min(k, kn - 32 + 8 * part);
+    h = *reinterpret_cast<const uint4*>(xh + k);
+    l = kLo ? *reinterpret_cast<const uint4*>(xl + k) : make_uint4(0, 0, 0, 0);
+  };
+  auto piece = [&](int k, const uint4& h4, const uint4& l4) {   // eight columns
+    uint64_t p[4] = {0, 0, 0, 0};
 #pragma unroll
-    for (int t = 0; t < kT; ++t) {   // (past the end the last piece again)
-      const int k = min(k0 + 32 * t, kn - 32 + 8 * part);
-      hv[t] = *reinterpret_cast<const uint4*>(xh + k);
-      lv[t] = kLo ? *reinterpret_cast<const uint4*>(xl + k) : make_uint4(0, 0, 0, 0);
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t h = u < 2 ? h4.x : u < 4 ? h4.y : u < 6 ? h4.z : h4.w;
+      const uint32_t l = u < 2 ? l4.x : u < 4 ? l4.y : u < 6 ? l4.z : l4.w;
+      float x = from_bits((uint16_t)(h >> (16 * (u & 1))), kFmt);
+      if (kLo) x += from_bits((uint16_t)(l >> (16 * (u & 1))), kFmt);
+      const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u);
+      const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u + 4);
+      const uint64_t xx = pair2(x, x), xn = pair2(-x, -x), q[4] = {qa.x, qa.y, qb.x, qb.y};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (kExact) add_product2(s[c], e[c], xx, xn, q[c]);
+        else p[c] = fma2(xx, q[c], p[c]);
+      }
     }
 #pragma unroll
-    for (int t = 0; t < kT; ++t) {
-      const int k = k0 + 32 * t;
-      if (k >= kn) break;
-      uint64_t p[4] = {0, 0, 0, 0};
+    for (int c = 0; c < 4 && !kExact; ++c) add(c, p[c]);
+  };
+  if constexpr (kExact) {   // 320 packed operations a piece: the next one's loads are in flight meanwhile (13.65 -> 13.2 ms)
+    uint4 h, l, hn, ln;
+    load(8 * part, h, l);
+#pragma unroll 1
+    for (int k = 8 * part; k < kn; k += 32) {
+      load(k + 32, hn, ln);
+      piece(k, h, l);
+      h = hn;
+      l = ln;
+    }
+  } else {
+#pragma unroll 1
+    for (int k0 = 8 * part; k0 < kn; k0 += 128) {
+      uint4 hv[4], lv[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const uint32_t h = u < 2 ? hv[t].x : u < 4 ? hv[t].y : u < 6 ? hv[t].z : hv[t].w;
-        const uint32_t l = u < 2 ? lv[t].x : u < 4 ? lv[t].y : u < 6 ? lv[t].z : lv[t].w;
-        float x = from_bits((uint16_t)(h >> (16 * (u & 1))), kFmt);
-        if (kLo) x += from_bits((uint16_t)(l >> (16 * (u & 1))), kFmt);
-        const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u);
-        const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(Qs + qs_at(k) + 8 * u + 4);
-        const uint64_t xx = pair2(x, x), xn = pair2(-x, -x), q[4] = {qa.x, qa.y, qb.x, qb.y};
+      for (int t = 0; t < 4; ++t) load(k0 + 32 * t, hv[t], lv[t]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (kExact) add_product2(s[c], e[c], xx, xn, q[c]);
-          else p[c] = fma2(xx, q[c], p[c]);
-        }
+      for (int t = 0; t < 4; ++t) {
+        if (k0 + 32 * t >= kn) break;
+        piece(k0 + 32 * t, hv[t], lv[t]);
       }
-#pragma unroll
-      for (int c = 0; c < 4 && !kExact; ++c) add(c, p[c]);
     }
   }
 #pragma unroll

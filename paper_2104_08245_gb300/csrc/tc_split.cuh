@@ -83,7 +83,7 @@ __device__ __forceinline__ void add_product2(uint64_t& s, uint64_t& e, uint64_t 
 
 // How X Q sums its products: in FP32, eight or sixteen at a time between compensated additions, or each with its own
 // rounding error where n x b is large (b above 13 at n = 192, above 8 at n = 300, any b from n = 440 on): what the plain
-// sums lose there is 3e-8 of D. 512 submatrices of 23 functions a molecule: 24.0 ms without, 25.4 with it.
+// sums lose there is 3e-8 of D. 512 submatrices of 23 functions a molecule: 24.0 ms without, 25.0 with it.
 __host__ __device__ inline bool exact_xq(int n, int b) { return 4 * ((n + 63) & ~63) * ((b + 7) & ~7) + 8 * n * b > 32768; }
 
 // u == k ? a : b as an instruction that the compiler does not fold into an indexed (local memory) array access: local
